@@ -38,14 +38,14 @@ constexpr double kPi = 3.14159265358979323846;
 inline int pad4(int x) { return (x + 3) & ~3; }
 
 // FP32-pipe flops of the compensated double-float pair evaluation (counted from the kernel's
-// operations, FMA = 2): a Stokeslet pair's geometry (differences, distance, 1/r, 1/r^2) and its
-// per-right-hand-side part; an image triple's geometry (with 1/r^3) and its S + R + D part
-constexpr double kDwPairGeomFlops = 99.0, kDwPairRhsFlops = 149.0;
+// operations, FMA = 2): a Stokeslet pair's geometry (difference, unit vector, 1/r) and its
+// per-right-hand-side part; an image triple's geometry and its S + R + D part
+constexpr double kDwPairGeomFlops = 76.0, kDwPairRhsFlops = 129.0;
 // Each GMRES pass of a refined solve stops at kInnerTol x tol / (current relative residual); the
 // accurate residual then decides whether another pass is needed.  0.8 measured fastest on the
 // gap sweep (0.5 and 1.0 took 2.5 % and 3 % longer; tighter factors cost more iterations).
 constexpr double kInnerTol = 0.8;
-constexpr double kDwTripleGeomFlops = 106.0, kDwTripleRhsFlops = 438.0;
+constexpr double kDwTripleGeomFlops = 94.0, kDwTripleRhsFlops = 383.0;
 
 struct Factor {
   int m = 0, ncol = 0, rank = 0, ldA = 0, ldV = 0;
@@ -1976,6 +1976,7 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   c->src.P = P;
   c->src.N = N;
   c->src.n_img = ni;
+  c->src.span = c->a * (1.0 + p.r_proxy);
   if ((s = upload(c, c->src.proxy32, p32)) != MFS_OK) return s;
   if ((s = upload(c, c->src.proxy64, p64)) != MFS_OK) return s;
   if ((s = upload(c, c->src.img32, i32)) != MFS_OK) return s;

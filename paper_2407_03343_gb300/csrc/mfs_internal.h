@@ -74,6 +74,7 @@ inline int pair_nodes_per_thread(int n_tiles_large) { return n_tiles_large >= 2 
 
 struct SourceSet {
   int P = 0, N = 0, n_img = 0;
+  double span = 2.0;           // sphere radius plus proxy radius
   float4* proxy32 = nullptr;   // N positions relative to the owner centre (same for every sphere)
   double* proxy64 = nullptr;   // 4 doubles per proxy (x, y, z, 0)
   float4* img32 = nullptr;     // image node positions relative to the owner centre
@@ -151,10 +152,12 @@ void launch_pairs(const TargetSet& tg, const SourceSet& src, const T* lam_hat, c
 void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const double* lam_hat, const double* mu,
                      double* out, double visc, double* partial, int max_parts, cudaStream_t st,
                      PairShape shape = PairShape());
-// Source split of the 1-node-per-thread tiling: as many parts as keep the CTAs within one wave
-// (152 SMs x 7 resident CTAs of the double-float kernel: 72 registers x 128 threads, 28 KB of
-// shared memory), at least kPairSplitMinSources sources per part, at most max_parts.
-constexpr int kPairSplitTarget = 152 * 7;
+// Source split of a tile: enough parts for ten times the resident CTAs (152 SMs x 4), because the
+// SMs finish their last CTAs at different times and a short CTA leaves less idle behind it
+// (measured on 100 spheres, 700 tiles: 30.3 ms with 2 parts, 28.8 with 3, 27.3 with 9 and 27.5
+// with 16; on 20 spheres, 140 tiles: 1.20 ms with 8 parts and 1.11 with 16), at least
+// kPairSplitMinSources sources per part, at most max_parts.
+constexpr int kPairSplitTarget = 152 * 40;
 constexpr int kPairSplitMinSources = 64;
 constexpr int kPairMaxParts = 16;
 int pair_split_parts(long long n_tiles1, long long min_sources, int max_parts);

@@ -115,6 +115,7 @@ struct PairArgs {
   T* out;
   T scale;       // 1 / (8 pi mu)
   T dip;         // 2 mu: dipole strengths rescaled so that scale * dip = 1 / (4 pi)
+  float span;    // a little over the sphere radius plus the proxy radius: bounds |x - c| + |y - c'| on every axis
 };
 
 // One target tile (NT nodes per thread) against every source of every other sphere.
@@ -317,6 +318,7 @@ PairArgs<T> make_args(const TargetSet& tg, const SourceSet& src, const T* lam, c
   A.out = out;
   A.scale = T(1.0 / (8.0 * kPi * visc));
   A.dip = T(2.0 * visc);
+  A.span = (float)(1.001 * src.span);
   return A;
 }
 
@@ -354,342 +356,604 @@ __device__ __forceinline__ dw dw_add(dw x, dw y) {
   float v = __fadd_rn(x.l, y.l);
   return fast_two_sum(s.h, __fadd_rn(s.l, v));
 }
-__device__ __forceinline__ dw dw_sub(dw x, dw y) { return dw_add(x, dw{-y.h, -y.l}); }
 __device__ __forceinline__ dw dw_mul(dw x, dw y) {
   dw c = two_prod(x.h, y.h);
   float t = __fmul_rn(x.h, y.l);
   t = __fmaf_rn(x.l, y.h, t);
   return fast_two_sum(c.h, __fadd_rn(c.l, t));
 }
-__device__ __forceinline__ dw dw_mul_f(dw x, float y) {
-  dw c = two_prod(x.h, y);
-  return fast_two_sum(c.h, __fmaf_rn(x.l, y, c.l));
-}
 __device__ __forceinline__ dw dw_split(double v) {
   float h = (float)v;
   return {h, (float)(v - (double)h)};
 }
 __device__ __forceinline__ double dw_join(dw x) { return (double)x.h + (double)x.l; }
-// 1/sqrt(x): FP32 estimate, one FP32 Newton step, one double-word Newton step
-// y <- y + y (1 - x y^2) / 2.
-__device__ __forceinline__ dw dw_rsqrt(dw x) {
-  float s = rsqrtf(x.h);
-  s = __fmul_rn(s, __fmaf_rn(__fmul_rn(-0.5f, x.h), __fmul_rn(s, s), 1.5f));
-  dw s2 = two_prod(s, s);
-  dw e = dw_mul(x, s2);
-  float h = __fsub_rn(__fsub_rn(1.0f, e.h), e.l);
-  return fast_two_sum(s, __fmul_rn(__fmul_rn(0.5f, s), h));
+// ------------------------------------------------------------------ packed FP32
+// Two FP32 lanes per instruction (sm_100+ f32x2): the FMA pipe does one lane-operation per lane
+// either way (measured: fma, add, mul and sub all at 95 % of 152 x 128 lanes x the SM clock, the
+// scalar forms at 92 %), but half the issue slots are free for loads, selects and MUFU.
+typedef unsigned long long f2x;
+__device__ __forceinline__ f2x f2add(f2x a, f2x b) {
+  f2x d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f2x f2sub(f2x a, f2x b) {
+  f2x d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f2x f2mul(f2x a, f2x b) {
+  f2x d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f2x f2fma(f2x a, f2x b, f2x c) {
+  f2x d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f2x f2make(float lo, float hi) {
+  f2x d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void f2split(f2x v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f2x f2dup(float v) { return f2make(v, v); }
+__device__ __forceinline__ f2x f2neg(f2x v) { return v ^ 0x8000000080000000ull; }
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
-// Compensated evaluation for the pair kernel (in the style of Ogita, Rump and Oishi,
-// "Accurate sum and dot product", SIAM J. Sci. Comput. 2005): a product keeps its exact
-// rounding error plus the first-order cross terms, a sum keeps the TwoSum error plus the low
-// parts, and neither renormalises; the low part then stays within a few ulps of the high part
-// scaled by the operands' magnitude, which bounds every absolute error by ~2^-46 of the
-// operands.  Renormalisation is kept where cancellation could let the low part outgrow the
-// high part (differences of positions and dot products) and at every accumulation.
-__device__ __forceinline__ dw mul_u(dw x, dw y) {
-  float p = __fmul_rn(x.h, y.h);
-  float e = __fmaf_rn(x.h, y.h, -p);
-  e = __fmaf_rn(x.h, y.l, e);
-  e = __fmaf_rn(x.l, y.h, e);
-  return {p, e};
+// two double-word values, one per lane: high and low words packed
+struct dw2 {
+  f2x h, l;
+};
+// a + b = s + e and a - b = s + e exactly in both lanes (Knuth).  Finding the larger operand by
+// compare and select on the ALU pipe, for Dekker's three additions, measured 2-5 % slower in the
+// pair kernel (28.4-30.0 against 27.9 ms on 100 spheres) although it takes a fifth of its work off
+// the FMA pipe.
+__device__ __forceinline__ dw2 two_sum2(f2x a, f2x b) {
+  const f2x s = f2add(a, b), bb = f2sub(s, a);
+  return {s, f2add(f2sub(a, f2sub(s, bb)), f2sub(b, bb))};
 }
-__device__ __forceinline__ dw add_u(dw x, dw y) {
-  dw s = two_sum(x.h, y.h);
-  return {s.h, __fadd_rn(s.l, __fadd_rn(x.l, y.l))};
+__device__ __forceinline__ dw2 two_diff2(f2x a, f2x b) {
+  const f2x s = f2sub(a, b), bb = f2sub(s, a);
+  return {s, f2sub(f2sub(a, f2sub(s, bb)), f2add(b, bb))};
 }
-__device__ __forceinline__ dw neg(dw x) { return {-x.h, -x.l}; }
-// u += t with the running sum renormalised every time: its partial sums can exceed the final
-// value by ~1e9 under cancellation, so its low word must stay within an ulp of the high word
-__device__ __forceinline__ void acc_u(dw& u, dw t) { u = dw_add(u, t); }
-// x - y for positions: the difference is never below ~1e-3 of the radius, far above the low parts
-__device__ __forceinline__ dw sub_pos(dw x, dw y) {
-  dw s = two_sum(x.h, -y.h);
-  return fast_two_sum(s.h, __fadd_rn(s.l, __fsub_rn(x.l, y.l)));
+__device__ __forceinline__ dw2 fast_two_sum2(f2x a, f2x b) {
+  const f2x s = f2add(a, b);
+  return {s, f2sub(b, f2sub(s, a))};
 }
-// a.b for three double-word pairs, renormalised (the sum may cancel)
-__device__ __forceinline__ dw dot3_u(dw a0, dw a1, dw a2, dw b0, dw b1, dw b2) {
-  dw p0 = mul_u(a0, b0), p1 = mul_u(a1, b1), p2 = mul_u(a2, b2);
-  dw s1 = two_sum(p0.h, p1.h);
-  dw s2 = two_sum(s1.h, p2.h);
-  float lo = __fadd_rn(__fadd_rn(__fadd_rn(p0.l, p1.l), __fadd_rn(p2.l, s1.l)), s2.l);
-  return two_sum(s2.h, lo);
+__device__ __forceinline__ dw2 dw2_add(dw2 x, dw2 y) {
+  const dw2 s = two_sum2(x.h, y.h);
+  return fast_two_sum2(s.h, f2add(s.l, f2add(x.l, y.l)));
 }
-// |d|^2 (all terms positive, no cancellation)
-__device__ __forceinline__ dw norm2_u(dw d0, dw d1, dw d2) {
-  dw p0 = two_prod(d0.h, d0.h), p1 = two_prod(d1.h, d1.h), p2 = two_prod(d2.h, d2.h);
-  p0.l = __fmaf_rn(__fadd_rn(d0.h, d0.h), d0.l, p0.l);
-  p1.l = __fmaf_rn(__fadd_rn(d1.h, d1.h), d1.l, p1.l);
-  p2.l = __fmaf_rn(__fadd_rn(d2.h, d2.h), d2.l, p2.l);
-  dw s1 = two_sum(p0.h, p1.h);
-  dw s2 = two_sum(s1.h, p2.h);
-  float lo = __fadd_rn(__fadd_rn(__fadd_rn(p0.l, p1.l), __fadd_rn(p2.l, s1.l)), s2.l);
-  return fast_two_sum(s2.h, lo);
+// product and sum without renormalisation: the exact error of the high parts plus the first-order
+// terms of the low ones
+__device__ __forceinline__ dw2 mul2u(dw2 x, dw2 y) {
+  const f2x p = f2mul(x.h, y.h);
+  return {p, f2fma(x.l, y.h, f2fma(x.h, y.l, f2fma(x.h, y.h, f2neg(p))))};
 }
-__device__ __forceinline__ dw rsqrt_u(dw x) {
-  float s = rsqrtf(x.h);
-  s = __fmul_rn(s, __fmaf_rn(__fmul_rn(-0.5f, x.h), __fmul_rn(s, s), 1.5f));
-  dw e = mul_u(x, two_prod(s, s));
-  float h = __fsub_rn(__fsub_rn(1.0f, e.h), e.l);
-  return fast_two_sum(s, __fmul_rn(__fmul_rn(0.5f, s), h));
-}
-__device__ __forceinline__ dw times3_u(dw x) {
-  dw c = two_prod(x.h, 3.0f);
-  return {c.h, __fmaf_rn(x.l, 3.0f, c.l)};
+__device__ __forceinline__ dw2 add2u(dw2 x, dw2 y) {
+  const dw2 s = two_sum2(x.h, y.h);
+  return {s.h, f2add(s.l, f2add(x.l, y.l))};
 }
 
-struct __align__(16) DWPos {
-  float xh, yh, zh, pad0;
-  float xl, yl, zl, pad1;
+// ------------------------------------------------------------------ double-float pair sums
+// Each thread holds one target at a time and evaluates two sources per instruction (the lanes), so
+// a source pair is read from shared memory as it is stored and a lane sums every second source.
+// What bounds the sums is the FMA pipe: 160 lane-operations a (node, Stokeslet) pair (the earlier
+// scalar evaluation: 204, and its issue slots) and 340 an image triple (436).  Measured on 100
+// spheres (5.59e9 pairs): 27.3 ms, 81 % of the packed rate, against 43.1 ms.  The evaluation keeps
+// the accuracy of a renormalised double-word one (~2^-46 of the operands) with fewer operations:
+//  - positions of a (target sphere, source sphere) segment are split on a common power-of-two grid
+//    per axis, so the difference of the high words is exact without a two-sum;
+//  - with s = 1/|d| to FP32 accuracy (MUFU and one Newton step on the high words) the unit vector
+//    u = d / |d| is formed as s d, and its deviation 1 - |s d|^2, found to ~2^-48 by a chain of
+//    fused multiply-adds from 1 whose roundings are recovered exactly, corrects u and 1/|d| at
+//    first order; the field needs only u and 1/|d| (Stokeslet: (f + (u.f) u) / |d|);
+//  - products and sums inside a term are not renormalised (their low words stay below ~2^-23 of
+//    the operands), and the terms are summed in groups of eight per lane with exact high sums and
+//    plain low sums, the groups in double-word arithmetic: a group's roundings scale with the
+//    group's sum instead of with the running sum, so the error of a sum is smaller than that of
+//    adding every term in double-word arithmetic (0.2-0.6 of it; 686 sources, random and equal
+//    strengths, against quadruple precision).
+constexpr int kDwTile = 256;     // proxy sources staged per round (one sphere's)
+constexpr int kDwTileImg = 64;   // image nodes staged per round (one sphere's)
+constexpr int kDwGroup = 16;     // terms per lane and group
+// resident CTAs per SM (register bound: 128); 5 and 6 measured the same within 1 %
+constexpr int kDwCtas = 4;
+
+// Sources of one round in shared memory: source pair u holds its two sources' components side by
+// side, pos[3 u ..]: (xh yh), (zh xl), (yl zl), strengths likewise.
+struct DwGeom {          // geometry of one target and two sources
+  f2x p[3], np[3], l[3];  // unit vector: high words, their negatives, low words
+  f2x s, ns, il;          // 1/|d|: high word, its negative, low word
 };
 
-// Target nodes of one tile in double-float, with their running sums.
-template <int NT>
+struct DwTarget {        // a target in the grid of the current segment, duplicated into both lanes
+  f2x h[3], l[3];
+};
+
+template <bool GRID>
+__device__ __forceinline__ void dw_geometry(const DwTarget& T, const ulonglong2 a, const ulonglong2 b,
+                                            const ulonglong2 c, DwGeom& g) {
+  const f2x yh[3] = {a.x, a.y, b.x}, yl[3] = {b.y, c.x, c.y};
+  const f2x mtwo = f2dup(-2.0f), mhalf = f2dup(-0.5f);
+  f2x dh[3], dl[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const dw2 t = GRID ? dw2{f2sub(T.h[q], yh[q]), 0} : two_diff2(T.h[q], yh[q]);
+    const f2x tl = f2sub(T.l[q], yl[q]);
+    const dw2 d = fast_two_sum2(t.h, GRID ? tl : f2add(t.l, tl));
+    dh[q] = d.h;
+    dl[q] = d.l;
+  }
+  const f2x r2 = f2fma(dh[2], dh[2], f2fma(dh[1], dh[1], f2mul(dh[0], dh[0])));
+  float r0, r1;
+  f2split(r2, r0, r1);
+  const f2x s0 = f2make(rsqrt_ftz(r0), rsqrt_ftz(r1));
+  const f2x k = f2fma(f2mul(r2, mhalf), f2mul(s0, s0), f2dup(1.5f));
+  g.s = f2mul(s0, k);
+  g.ns = f2neg(g.s);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    g.p[q] = f2mul(g.s, dh[q]);
+    g.np[q] = f2mul(g.ns, dh[q]);
+    g.l[q] = f2fma(g.s, dl[q], f2fma(g.s, dh[q], g.np[q]));
+  }
+  // e = (1 - |p + l|^2) / 2: the chain -2 + px^2 + py^2 + pz^2 (which stays within a factor of two,
+  // so its differences are exact) with each rounding recovered, and the cross terms p.l
+  const f2x a1 = f2fma(g.p[0], g.p[0], mtwo), a2 = f2fma(g.p[1], g.p[1], a1), a3 = f2fma(g.p[2], g.p[2], a2);
+  const f2x t = f2add(f2add(f2fma(g.p[0], g.p[0], f2sub(mtwo, a1)), f2fma(g.p[1], g.p[1], f2sub(a1, a2))),
+                      f2fma(g.p[2], g.p[2], f2sub(a2, a3)));
+  const f2x nq = f2fma(g.np[2], g.l[2], f2fma(g.np[1], g.l[1], f2mul(g.np[0], g.l[0])));
+  const f2x e = f2fma(mhalf, f2add(f2add(a3, f2dup(1.0f)), t), nq);
+  g.il = f2mul(g.s, e);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) g.l[q] = f2fma(g.p[q], e, g.l[q]);
+}
+
+// -(u . f), not renormalised
+__device__ __forceinline__ void dw_ndot(const DwGeom& g, const f2x (&fh)[3], const f2x (&fl)[3], f2x& nh, f2x& l) {
+  f2x n[3], e[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    n[q] = f2mul(g.np[q], fh[q]);
+    e[q] = f2fma(g.l[q], fh[q], f2fma(g.p[q], fl[q], f2fma(g.p[q], fh[q], n[q])));
+  }
+  const dw2 s1 = two_sum2(n[0], n[1]);
+  const dw2 s2 = two_sum2(s1.h, n[2]);
+  nh = s2.h;                                                       // -(u.f), high word
+  l = f2sub(f2add(f2add(e[0], e[1]), f2sub(e[2], s1.l)), s2.l);    // +(u.f), low word
+}
+
+// v = f + (u.f) u in component q, from nh = -(u.f)_h, ph = (u.f)_h and l = (u.f)_l
+__device__ __forceinline__ dw2 dw_project(const DwGeom& g, int q, f2x fh, f2x fl, f2x nh, f2x ph, f2x l) {
+  const f2x nm = f2mul(nh, g.p[q]);
+  const f2x e = f2fma(l, g.p[q], f2fma(ph, g.l[q], f2fma(nh, g.np[q], nm)));
+  const dw2 s = two_diff2(fh, nm);
+  return {s.h, f2add(s.l, f2add(fl, e))};
+}
+
+// group sum += v / |d|
+__device__ __forceinline__ void dw_accumulate(const DwGeom& g, dw2 v, dw2& sum) {
+  const f2x nt = f2mul(g.ns, v.h);
+  const f2x e = f2fma(g.il, v.h, f2fma(g.s, v.l, f2fma(g.s, v.h, nt)));
+  const dw2 s = two_diff2(sum.h, nt);
+  sum.h = s.h;
+  sum.l = f2add(sum.l, f2add(s.l, e));
+}
+
+// v / |d| (three in a row in an image triple: the low parts' product is kept as well)
+__device__ __forceinline__ dw2 dw_over_r(const DwGeom& g, dw2 v) {
+  const f2x nt = f2mul(g.ns, v.h);
+  return {f2neg(nt), f2fma(g.il, f2add(v.h, v.l), f2fma(g.s, v.l, f2fma(g.s, v.h, nt)))};
+}
+
+// the lanes of a round's double-word sums joined onto the target's sum
+__device__ __forceinline__ void dw_fold(dw& u, const dw2& m) {
+  float h0, h1, l0, l1;
+  f2split(m.h, h0, h1);
+  f2split(m.l, l0, l1);
+  u = dw_add(u, dw_add(dw{h0, l0}, dw{h1, l1}));
+}
+
+// Targets of one tile (NT per thread, taken one after the other against each staged round) and
+// their sums for R right-hand sides: in registers for one per thread, else in the thread's own
+// column of shared memory, read and written once a round.
+template <int R, int NT>
 struct DWTile {
-  dw x[NT], y[NT], z[NT], ux[NT], uy[NT], uz[NT];
+  dw x[3];
+  dw u[R][3];
+  __device__ __forceinline__ void load(int) {}
+  __device__ __forceinline__ void store(int) {}
 };
-
 template <int NT>
-__device__ __forceinline__ void dw_load_targets(const PairArgs<double>& A, int start, int cnt, DWTile<NT>& T) {
+struct DwColumns {
+  float2 x[NT][3][kPairThreads], u[NT][3][kPairThreads];
+};
+template <int NT>
+struct DWTileShared {
+  DwColumns<NT>* c;
+  dw x[3];
+  dw u[1][3];
+  __device__ __forceinline__ void load(int q) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float2 a = c->x[q][k][threadIdx.x], b = c->u[q][k][threadIdx.x];
+      x[k] = dw{a.x, a.y};
+      u[0][k] = dw{b.x, b.y};
+    }
+  }
+  __device__ __forceinline__ void store(int q) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) c->u[q][k][threadIdx.x] = make_float2(u[0][k].h, u[0][k].l);
+  }
+};
+template <>
+struct DWTile<1, 4> : DWTileShared<4> {};
+
+template <int R, int NT>
+__device__ __forceinline__ void dw_load_targets(const PairArgs<double>& A, int start, int cnt, DWTile<R, NT>& T) {
 #pragma unroll
   for (int q = 0; q < NT; ++q) {
     int idx = threadIdx.x + q * kPairThreads;
     int node = start + (idx < cnt ? idx : cnt - 1);
     D4 p = A.tgt[node];
-    T.x[q] = dw_split(p.x);
-    T.y[q] = dw_split(p.y);
-    T.z[q] = dw_split(p.z);
-    T.ux[q] = T.uy[q] = T.uz[q] = dw{0.f, 0.f};
+    T.x[0] = dw_split(p.x);
+    T.x[1] = dw_split(p.y);
+    T.x[2] = dw_split(p.z);
+#pragma unroll
+    for (int r = 0; r < R; ++r) T.u[r][0] = T.u[r][1] = T.u[r][2] = dw{0.f, 0.f};
+    if constexpr (NT > 1) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) T.c->x[q][k][threadIdx.x] = make_float2(T.x[k].h, T.x[k].l);
+      T.store(q);
+    }
   }
 }
 
-// Proxy Stokeslets [r_lo, r_hi) of the flattened proxy index (sphere o = j / N, proxy j - o N),
-// staged through shared memory in tiles of kTileProxy; sphere k's own proxies carry no strength.
-template <int NT>
-__device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const CentreShift64& sh, int k, int r_lo,
-                                               int r_hi, float4* sp, float4* sf, DWTile<NT>& T) {
-  const double far = 1e18;
-  const int total = A.P * A.N;
-  for (int s0 = r_lo; s0 < r_hi; s0 += kTileProxy) {
-    const int ns = min(kTileProxy, r_hi - s0);
+// Grid of a segment: on each axis the spacing 2^(e - 24) with 2^e above every |x - y| of the
+// segment (centre distance plus twice the radius), so high words on it subtract exactly.
+struct DwGrid {
+  double shift[3];  // source sphere's centre minus target sphere's
+  double m64[3];    // rounds a double to the grid: (y + m64) - m64
+  float m32[3];     // rounds |x| to the grid: (|x| + m32) - m32 (|x| < 2^(e-1) as 2^e > 2 a)
+};
+__device__ __forceinline__ DwGrid dw_grid(const PairArgs<double>& A, const CentreShift64& sh, int o) {
+  DwGrid G;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    G.shift[q] = sh.d(o, q);
+    const float b = (float)fabs(G.shift[q]) * 1.0001f + A.span;
+    // the power of two above b (b is a normal number: at least twice the radius)
+    const float p2 = __int_as_float((__float_as_int(b) & 0x7f800000) + 0x00800000);
+    G.m32[q] = 0.5f * p2;
+    G.m64[q] = 402653184.0 * (double)p2;  // 1.5 2^52 2^-24 p2
+  }
+  return G;
+}
+__device__ __forceinline__ void dw_stage_pos(const DwGrid& G, const D4 pr, float* sp, int i) {
+  const double rel[3] = {pr.x, pr.y, pr.z};
+  float* o = sp + 12 * (i >> 1) + (i & 1);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const double y = rel[q] + G.shift[q];
+    const double h = (y + G.m64[q]) - G.m64[q];
+    o[2 * q] = (float)h;
+    o[6 + 2 * q] = (float)(y - h);
+  }
+}
+__device__ __forceinline__ DwTarget dw_target(const DwGrid& G, const dw (&x)[3]) {
+  DwTarget t;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float h = copysignf(__fsub_rn(__fadd_rn(fabsf(x[q].h), G.m32[q]), G.m32[q]), x[q].h);
+    const float l = __fadd_rn(__fsub_rn(x[q].h, h), x[q].l);
+    t.h[q] = f2dup(h);
+    t.l[q] = f2dup(l);
+  }
+  return t;
+}
+
+// whether this warp has a target among the q-th 128 of the tile
+__device__ __forceinline__ bool dw_warp_live(int q, int cnt) {
+  return (int)(threadIdx.x & ~31u) + q * kPairThreads < cnt;
+}
+
+// Proxy Stokeslets [r_lo, r_hi) of the flattened proxy index (sphere o = j / N, proxy j - o N; the
+// range holds none of the target sphere's own), one sphere at a time in rounds of at most TILE.
+template <int R, int NT, int TILE>
+__device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const CentreShift64& sh,
+                                               const double* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
+                                               int cnt, float* sp, float (*sf)[6 * TILE], DWTile<R, NT>& T) {
+  for (int s0 = r_lo; s0 < r_hi;) {
+    const int o = s0 / A.N, j0 = s0 - o * A.N;
+    const int seg = min(r_hi - s0, A.N - j0);  // what is left of sphere o
+    // even rounds of whole groups
+    const int rounds = (seg + TILE - 1) / TILE;
+    const int ns = min(seg, ((seg + rounds - 1) / rounds + 2 * kDwGroup - 1) / (2 * kDwGroup) * (2 * kDwGroup));
+    const int nu = (ns + 1) >> 1;
+    const DwGrid G = dw_grid(A, sh, o);
     __syncthreads();
-    for (int i = threadIdx.x; i < ns; i += kPairThreads) {
-      int j = s0 + i;
-      double px = far, py = far, pz = far, fx = 0, fy = 0, fz = 0;
-      if (j < total) {
-        int o = j / A.N;
-        int jj = j - o * A.N;
-        D4 pr = A.proxy[jj];
-        px = pr.x + sh.d(o, 0);
-        py = pr.y + sh.d(o, 1);
-        pz = pr.z + sh.d(o, 2);
-        if (o != k) {
-          const double* l = A.lam + A.unk_off[o] + 3LL * jj;
-          fx = l[0]; fy = l[1]; fz = l[2];
+    for (int i = threadIdx.x; i < 2 * nu; i += kPairThreads) {
+      const int jj = j0 + min(i, ns - 1);
+      dw_stage_pos(G, A.proxy[jj], sp, i);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const bool on = i < ns && (mask >> r & 1u);  // the odd round's last slot carries no strength
+        const double* l = lam[r] + A.unk_off[o] + 3LL * jj;
+        float* f = sf[r] + 12 * (i >> 1) + (i & 1);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const dw v = dw_split(on ? l[q] : 0.0);
+          f[2 * q] = v.h;
+          f[6 + 2 * q] = v.l;
         }
       }
-      dw a = dw_split(px), b = dw_split(py), c = dw_split(pz);
-      sp[2 * i] = make_float4(a.h, b.h, c.h, 0.f);
-      sp[2 * i + 1] = make_float4(a.l, b.l, c.l, 0.f);
-      a = dw_split(fx); b = dw_split(fy); c = dw_split(fz);
-      sf[2 * i] = make_float4(a.h, b.h, c.h, 0.f);
-      sf[2 * i + 1] = make_float4(a.l, b.l, c.l, 0.f);
     }
     __syncthreads();
-    for (int j = 0; j < ns; ++j) {
-      const float4 ph = sp[2 * j], pl = sp[2 * j + 1];
-      const float4 fh = sf[2 * j], fl = sf[2 * j + 1];
-      const dw fx{fh.x, fl.x}, fy{fh.y, fl.y}, fz{fh.z, fl.z};
-#pragma unroll
-      for (int q = 0; q < NT; ++q) {
-        dw dx = sub_pos(T.x[q], dw{ph.x, pl.x});
-        dw dy = sub_pos(T.y[q], dw{ph.y, pl.y});
-        dw dz = sub_pos(T.z[q], dw{ph.z, pl.z});
-        dw ir = rsqrt_u(norm2_u(dx, dy, dz));
-        dw ir2 = mul_u(ir, ir);
-        dw c = mul_u(dot3_u(dx, dy, dz, fx, fy, fz), ir2);
-        acc_u(T.ux[q], mul_u(ir, add_u(fx, mul_u(c, dx))));
-        acc_u(T.uy[q], mul_u(ir, add_u(fy, mul_u(c, dy))));
-        acc_u(T.uz[q], mul_u(ir, add_u(fz, mul_u(c, dz))));
-      }
-    }
-#pragma unroll
+#pragma unroll 1
     for (int q = 0; q < NT; ++q) {
-      T.ux[q] = two_sum(T.ux[q].h, T.ux[q].l);
-      T.uy[q] = two_sum(T.uy[q].h, T.uy[q].l);
-      T.uz[q] = two_sum(T.uz[q].h, T.uz[q].l);
+      if (!dw_warp_live(q, cnt)) continue;
+      T.load(q);
+      const DwTarget X = dw_target(G, T.x);
+      dw2 m[R][3];
+#pragma unroll
+      for (int r = 0; r < R; ++r) m[r][0] = m[r][1] = m[r][2] = dw2{0, 0};
+      for (int u0 = 0; u0 < nu; u0 += kDwGroup) {
+        dw2 sum[R][3];
+#pragma unroll
+        for (int r = 0; r < R; ++r) sum[r][0] = sum[r][1] = sum[r][2] = dw2{0, 0};
+        const int u1 = min(nu, u0 + kDwGroup);
+#pragma unroll 2
+        for (int u = u0; u < u1; ++u) {
+          const ulonglong2* P = reinterpret_cast<const ulonglong2*>(sp) + 3 * u;
+          DwGeom g;
+          dw_geometry<true>(X, P[0], P[1], P[2], g);
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            if (R > 1 && !(mask >> r & 1u)) continue;
+            const ulonglong2* F = reinterpret_cast<const ulonglong2*>(sf[r]) + 3 * u;
+            const ulonglong2 fa = F[0], fb = F[1], fc = F[2];
+            const f2x fh[3] = {fa.x, fa.y, fb.x}, fl[3] = {fb.y, fc.x, fc.y};
+            f2x nh, l;
+            dw_ndot(g, fh, fl, nh, l);
+            const f2x ph = f2neg(nh);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) dw_accumulate(g, dw_project(g, c, fh[c], fl[c], nh, ph, l), sum[r][c]);
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) m[r][c] = dw2_add(m[r][c], sum[r][c]);
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dw_fold(T.u[r][c], m[r][c]);
+      T.store(q);
     }
+    s0 += ns;
   }
 }
 
-// Image nodes [r_lo, r_hi) (Stokeslet + rotlet + potential dipole at one position), staged in
-// tiles of kTileImg; sphere k's own nodes carry no strength.
-template <int NT>
-__device__ __forceinline__ void dw_image_range(const PairArgs<double>& A, const CentreShift64& sh, int k, int r_lo,
-                                               int r_hi, float4* si, DWTile<NT>& T) {
-  const double far = 1e18;
-  for (int s0 = r_lo; s0 < r_hi; s0 += kTileImg) {
-    const int ns = min(kTileImg, r_hi - s0);
+// Image nodes [r_lo, r_hi) (Stokeslet f, rotlet t and potential dipole q at one position; none of
+// the target sphere's own), one sphere at a time.  With u and 1/r the triple's field is
+//   (1/r) [ f + (u.f) u + (1/r) [ t x u + (1/r) (3 (u.q) u - q) ] ].
+// Strengths per right-hand side and pair of nodes: f, t, -q and 3 q, high and low words.
+template <int R, int NT, int TILE>
+__device__ __forceinline__ void dw_image_range(const PairArgs<double>& A, const CentreShift64& sh,
+                                               const double* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
+                                               int cnt, float* sp, float (*si)[24 * TILE], DWTile<R, NT>& T) {
+  for (int s0 = r_lo; s0 < r_hi;) {
+    const int o = A.img_owner[s0];
+    const int first = A.img_off[o];
+    const int ns = min(TILE, min(r_hi, A.img_off[o + 1]) - s0);
+    const int nu = (ns + 1) >> 1;
+    const double shift[3] = {sh.d(o, 0), sh.d(o, 1), sh.d(o, 2)};
     __syncthreads();
-    for (int i = threadIdx.x; i < ns; i += kPairThreads) {
-      int j = s0 + i;
-      double v[12] = {far, far, far, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-      if (j < A.n_img) {
-        int o = A.img_owner[j];
-        D4 pr = A.img[j];
-        v[0] = pr.x + sh.d(o, 0);
-        v[1] = pr.y + sh.d(o, 1);
-        v[2] = pr.z + sh.d(o, 2);
-        if (o != k) {
-          const double* l = A.lam + A.unk_off[o] + 3LL * A.N + 9LL * (j - A.img_off[o]);
-          for (int q = 0; q < 6; ++q) v[3 + q] = l[q];
-          for (int q = 6; q < 9; ++q) v[3 + q] = A.dip * l[q];
+    for (int i = threadIdx.x; i < 2 * nu; i += kPairThreads) {
+      const int j = s0 + min(i, ns - 1);
+      {
+        const D4 pr = A.img[j];
+        const double y[3] = {pr.x + shift[0], pr.y + shift[1], pr.z + shift[2]};
+        float* f = sp + 12 * (i >> 1) + (i & 1);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const dw v = dw_split(y[q]);
+          f[2 * q] = v.h;
+          f[6 + 2 * q] = v.l;
         }
       }
-      // node i occupies si[6i .. 6i+5]: hi of (x, y, z, f, t, d) then lo of the same 12 values
-      float hv[12], lv[12];
-      for (int q = 0; q < 12; ++q) {
-        dw s = dw_split(v[q]);
-        hv[q] = s.h;
-        lv[q] = s.l;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const bool on = i < ns && (mask >> r & 1u);
+        const double* l = lam[r] + A.unk_off[o] + 3LL * A.N + 9LL * (j - first);
+        float* f = si[r] + 48 * (i >> 1) + (i & 1);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const double d = on ? A.dip * l[6 + q] : 0.0;
+          const double v[4] = {on ? l[q] : 0.0, on ? l[3 + q] : 0.0, -d, 3.0 * d};
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
+            const dw s = dw_split(v[w]);
+            f[12 * w + 2 * q] = s.h;
+            f[12 * w + 6 + 2 * q] = s.l;
+          }
+        }
       }
-      si[6 * i] = make_float4(hv[0], hv[1], hv[2], hv[3]);
-      si[6 * i + 1] = make_float4(hv[4], hv[5], hv[6], hv[7]);
-      si[6 * i + 2] = make_float4(hv[8], hv[9], hv[10], hv[11]);
-      si[6 * i + 3] = make_float4(lv[0], lv[1], lv[2], lv[3]);
-      si[6 * i + 4] = make_float4(lv[4], lv[5], lv[6], lv[7]);
-      si[6 * i + 5] = make_float4(lv[8], lv[9], lv[10], lv[11]);
     }
     __syncthreads();
-    for (int j = 0; j < ns; ++j) {
-      const float4 h0 = si[6 * j], h1 = si[6 * j + 1], h2 = si[6 * j + 2];
-      const float4 l0 = si[6 * j + 3], l1 = si[6 * j + 4], l2 = si[6 * j + 5];
-      const dw px{h0.x, l0.x}, py{h0.y, l0.y}, pz{h0.z, l0.z};
-      const dw fx{h0.w, l0.w}, fy{h1.x, l1.x}, fz{h1.y, l1.y};
-      const dw tx{h1.z, l1.z}, ty{h1.w, l1.w}, tz{h2.x, l2.x};
-      const dw qx{h2.y, l2.y}, qy{h2.z, l2.z}, qz{h2.w, l2.w};
-#pragma unroll
-      for (int q = 0; q < NT; ++q) {
-        dw dx = sub_pos(T.x[q], px), dy = sub_pos(T.y[q], py), dz = sub_pos(T.z[q], pz);
-        dw ir = rsqrt_u(norm2_u(dx, dy, dz));
-        dw ir2 = mul_u(ir, ir);
-        dw ir3 = mul_u(ir, ir2);
-        // Stokeslet
-        dw cs = mul_u(dot3_u(dx, dy, dz, fx, fy, fz), ir2);
-        acc_u(T.ux[q], mul_u(ir, add_u(fx, mul_u(cs, dx))));
-        acc_u(T.uy[q], mul_u(ir, add_u(fy, mul_u(cs, dy))));
-        acc_u(T.uz[q], mul_u(ir, add_u(fz, mul_u(cs, dz))));
-        // rotlet (t x r) / r^3
-        acc_u(T.ux[q], mul_u(ir3, add_u(mul_u(ty, dz), neg(mul_u(tz, dy)))));
-        acc_u(T.uy[q], mul_u(ir3, add_u(mul_u(tz, dx), neg(mul_u(tx, dz)))));
-        acc_u(T.uz[q], mul_u(ir3, add_u(mul_u(tx, dy), neg(mul_u(ty, dx)))));
-        // potential dipole -d / r^3 + 3 (d.r) r / r^5
-        dw c3 = times3_u(mul_u(mul_u(dot3_u(dx, dy, dz, qx, qy, qz), ir3), ir2));
-        acc_u(T.ux[q], mul_u(c3, dx));
-        acc_u(T.uy[q], mul_u(c3, dy));
-        acc_u(T.uz[q], mul_u(c3, dz));
-        acc_u(T.ux[q], neg(mul_u(ir3, qx)));
-        acc_u(T.uy[q], neg(mul_u(ir3, qy)));
-        acc_u(T.uz[q], neg(mul_u(ir3, qz)));
-      }
-    }
-#pragma unroll
+#pragma unroll 1
     for (int q = 0; q < NT; ++q) {
-      T.ux[q] = two_sum(T.ux[q].h, T.ux[q].l);
-      T.uy[q] = two_sum(T.uy[q].h, T.uy[q].l);
-      T.uz[q] = two_sum(T.uz[q].h, T.uz[q].l);
+      if (!dw_warp_live(q, cnt)) continue;
+      T.load(q);
+      DwTarget X;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        X.h[c] = f2dup(T.x[c].h);
+        X.l[c] = f2dup(T.x[c].l);
+      }
+      dw2 m[R][3];
+#pragma unroll
+      for (int r = 0; r < R; ++r) m[r][0] = m[r][1] = m[r][2] = dw2{0, 0};
+#pragma unroll 1
+      for (int u = 0; u < nu; ++u) {
+        const ulonglong2* P = reinterpret_cast<const ulonglong2*>(sp) + 3 * u;
+        DwGeom g;
+        dw_geometry<false>(X, P[0], P[1], P[2], g);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (R > 1 && !(mask >> r & 1u)) continue;
+          const ulonglong2* F = reinterpret_cast<const ulonglong2*>(si[r]) + 12 * u;
+          dw2 y[3];
+          {  // (1/r) (3 (u.q) u - q)
+            const ulonglong2 ta = F[9], tb = F[10], tc = F[11];
+            const f2x th[3] = {ta.x, ta.y, tb.x}, tl[3] = {tb.y, tc.x, tc.y};
+            f2x nh, l;
+            dw_ndot(g, th, tl, nh, l);
+            const f2x ph = f2neg(nh);
+            const ulonglong2 qa = F[6], qb = F[7], qc = F[8];
+            const f2x qh[3] = {qa.x, qa.y, qb.x}, ql[3] = {qb.y, qc.x, qc.y};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) y[c] = dw_over_r(g, dw_project(g, c, qh[c], ql[c], nh, ph, l));
+          }
+          {  // + t x u, then / r
+            const ulonglong2 ta = F[3], tb = F[4], tc = F[5];
+            const dw2 t[3] = {{ta.x, tb.y}, {ta.y, tc.x}, {tb.x, tc.y}};
+            const dw2 un[3] = {{g.p[0], g.l[0]}, {g.p[1], g.l[1]}, {g.p[2], g.l[2]}};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+              const dw2 b = mul2u(t[c2], un[c1]);
+              y[c] = dw_over_r(g, add2u(y[c], add2u(mul2u(t[c1], un[c2]), dw2{f2neg(b.h), f2neg(b.l)})));
+            }
+          }
+          {  // + f + (u.f) u, then / r
+            const ulonglong2 fa = F[0], fb = F[1], fc = F[2];
+            const f2x fh[3] = {fa.x, fa.y, fb.x}, fl[3] = {fb.y, fc.x, fc.y};
+            f2x nh, l;
+            dw_ndot(g, fh, fl, nh, l);
+            const f2x ph = f2neg(nh);
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+              m[r][c] = dw2_add(m[r][c], dw_over_r(g, add2u(dw_project(g, c, fh[c], fl[c], nh, ph, l), y[c])));
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) dw_fold(T.u[r][c], m[r][c]);
+      T.store(q);
     }
+    s0 += ns;
   }
 }
 
-// out = mu + sqrt(w) scale u per node (or the scaled partial sum of this source part, or the
-// plain scaled sum when mu is null)
-template <int NT>
-__device__ __forceinline__ void dw_write_out(const PairArgs<double>& A, int start, int cnt, const DWTile<NT>& T,
-                                             int part, int nparts, double* __restrict__ partial, long long pstride) {
+// out = mu + sqrt(w) scale u per node, or the scaled partial sum of this source part
+template <int R, int NT>
+__device__ __forceinline__ void dw_write_out(const PairArgs<double>& A, int start, int cnt, DWTile<R, NT>& T, int r,
+                                             const double* __restrict__ mu, double* __restrict__ out, int part,
+                                             int nparts, double* __restrict__ partial, long long pstride) {
 #pragma unroll
   for (int q = 0; q < NT; ++q) {
     int idx = threadIdx.x + q * kPairThreads;
     if (idx < cnt) {
-      long long node = start + idx;
-      double sw = A.tgt[node].w;
-      double gx = dw_join(T.ux[q]) * A.scale, gy = dw_join(T.uy[q]) * A.scale, gz = dw_join(T.uz[q]) * A.scale;
-      if (nparts > 1) {
-        double* o = partial + part * pstride + 3 * node;
-        o[0] = gx;
-        o[1] = gy;
-        o[2] = gz;
-      } else if (A.mu) {
-        A.out[3 * node] = A.mu[3 * node] + sw * gx;
-        A.out[3 * node + 1] = A.mu[3 * node + 1] + sw * gy;
-        A.out[3 * node + 2] = A.mu[3 * node + 2] + sw * gz;
-      } else {
-        A.out[3 * node] = gx;
-        A.out[3 * node + 1] = gy;
-        A.out[3 * node + 2] = gz;
+      const long long node = start + idx;
+      const double sw = A.tgt[node].w;
+      T.load(q);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const double g = dw_join(T.u[r][c]) * A.scale;
+        if (nparts > 1) partial[part * pstride + 3 * node + c] = g;
+        else out[3 * node + c] = mu[3 * node + c] + sw * g;
       }
     }
   }
 }
+
+template <int R, int TILE, int TILE_IMG>
+struct DwShared {
+  __align__(16) float sp[6 * (TILE > TILE_IMG ? TILE : TILE_IMG)];  // positions of a round
+  union {                                                           // and its strengths
+    __align__(16) float sf[R][6 * TILE];
+    __align__(16) float si[R][24 * TILE_IMG];
+  };
+};
 
 // Sources may be split over `nparts` CTAs per target tile (when there are too few tiles to
 // fill the GPU): part `part` takes a contiguous share of the tile's source list (the sources of
 // every other sphere) and, for nparts > 1, writes its scaled partial sum to
 // partial[part * pstride + 3 node + c] for pair_parts_reduce to finish.
+template <int R, int NT, int TILE, int TILE_IMG>
+__device__ __forceinline__ void dw_all_sources(const PairArgs<double>& A, const CentreShift64& sh, int k,
+                                               const double* const (&lam)[R], unsigned mask, int cnt, int part,
+                                               int nparts, DwShared<R, TILE, TILE_IMG>& S, DWTile<R, NT>& T) {
+  // the proxies before and after sphere k's own (this part's share of them)
+  const int total = A.P * A.N;
+  const int p_lo = k * A.N, p_w = A.N;
+  const long long p_eff = total - p_w;
+  const int pe0 = (int)(p_eff * part / nparts), pe1 = (int)(p_eff * (part + 1) / nparts);
+  dw_proxy_range<R, NT, TILE>(A, sh, lam, mask, min(pe0, p_lo), min(pe1, p_lo), cnt, S.sp, S.sf, T);
+  dw_proxy_range<R, NT, TILE>(A, sh, lam, mask, max(pe0, p_lo) + p_w, max(pe1, p_lo) + p_w, cnt, S.sp, S.sf, T);
+  // image nodes before and after sphere k's own, this part's share
+  const int i_lo = A.img_off[k], i_w = A.img_off[k + 1] - i_lo;
+  const long long i_eff = A.n_img - i_w;
+  const int ie0 = (int)(i_eff * part / nparts), ie1 = (int)(i_eff * (part + 1) / nparts);
+  dw_image_range<R, NT, TILE_IMG>(A, sh, lam, mask, min(ie0, i_lo), min(ie1, i_lo), cnt, S.sp, S.si, T);
+  dw_image_range<R, NT, TILE_IMG>(A, sh, lam, mask, max(ie0, i_lo) + i_w, max(ie1, i_lo) + i_w, cnt, S.sp, S.si, T);
+}
+
 template <int NT>
 __device__ __forceinline__ void pair_tile_dw(const PairArgs<double>& A, const int t, const int part, const int nparts,
                                              double* __restrict__ partial, const long long pstride) {
-  __shared__ float4 sp[2 * kTileProxy];   // position hi, lo
-  __shared__ float4 sf[2 * kTileProxy];   // strength hi, lo
-  __shared__ float4 si[6 * kTileImg];     // image node: 12 hi values (3 float4), then 12 lo values (3 float4)
-
+  __shared__ DwShared<1, kDwTile, kDwTileImg> S;
   const int k = A.tile_sphere[t];
   const int start = A.tile_start[t];
   const int cnt = A.tile_count[t];
   CentreShift64 sh;
   sh.cen = A.cen64;
   sh.init(k);
-  DWTile<NT> T;
-  dw_load_targets<NT>(A, start, cnt, T);
-
-  const int total = A.P * A.N;
-  // the proxies before and after sphere k's own (this part's share of them), in tiles with
-  // exact trip counts
-  const int p_lo = k < 0 ? total : k * A.N, p_w = k < 0 ? 0 : A.N;
-  const long long p_eff = total - p_w;
-  const int pe0 = (int)(p_eff * part / nparts), pe1 = (int)(p_eff * (part + 1) / nparts);
-  dw_proxy_range<NT>(A, sh, k, min(pe0, p_lo), min(pe1, p_lo), sp, sf, T);
-  dw_proxy_range<NT>(A, sh, k, max(pe0, p_lo) + p_w, max(pe1, p_lo) + p_w, sp, sf, T);
-
-  // image nodes before and after sphere k's own, this part's share
-  const int i_lo = k >= 0 ? A.img_off[k] : 0, i_w = k >= 0 ? A.img_off[k + 1] - i_lo : 0;
-  const long long i_eff = A.n_img - i_w;
-  const int ie0 = (int)(i_eff * part / nparts), ie1 = (int)(i_eff * (part + 1) / nparts);
-  dw_image_range<NT>(A, sh, k, min(ie0, i_lo), min(ie1, i_lo), si, T);
-  dw_image_range<NT>(A, sh, k, max(ie0, i_lo) + i_w, max(ie1, i_lo) + i_w, si, T);
-
-  dw_write_out<NT>(A, start, cnt, T, part, nparts, partial, pstride);
+  DWTile<1, NT> T;
+  if constexpr (NT > 1) {
+    __shared__ DwColumns<NT> C;
+    T.c = &C;
+  }
+  dw_load_targets<1, NT>(A, start, cnt, T);
+  const double* const lam[1] = {A.lam};
+  dw_all_sources<1, NT, kDwTile, kDwTileImg>(A, sh, k, lam, 1u, cnt, part, nparts, S, T);
+  dw_write_out<1, NT>(A, start, cnt, T, 0, A.mu, A.out, part, nparts, partial, pstride);
 }
 
 // The near part of the far-field split: only the spheres of the target sphere's near list
-// (ascending; runs of consecutive spheres are staged as one range).
+// (ascending; runs of consecutive spheres are taken as one range).
 template <int NT>
 __device__ __forceinline__ void pair_tile_dw_near(const PairArgs<double>& A, const int* __restrict__ near_off,
                                                   const int* __restrict__ near_idx, const int t, const int part,
                                                   const int nparts, double* __restrict__ partial,
                                                   const long long pstride) {
-  __shared__ float4 sp[2 * kTileProxy];
-  __shared__ float4 sf[2 * kTileProxy];
-  __shared__ float4 si[6 * kTileImg];
+  __shared__ DwShared<1, kDwTile, kDwTileImg> S;
   const int k = A.tile_sphere[t];
   const int start = A.tile_start[t];
   const int cnt = A.tile_count[t];
   CentreShift64 sh;
   sh.cen = A.cen64;
   sh.init(k);
-  DWTile<NT> T;
-  dw_load_targets<NT>(A, start, cnt, T);
+  DWTile<1, NT> T;
+  if constexpr (NT > 1) {
+    __shared__ DwColumns<NT> C;
+    T.c = &C;
+  }
+  dw_load_targets<1, NT>(A, start, cnt, T);
+  const double* const lam[1] = {A.lam};
   // this part's share of the near list
   const int b0 = near_off[k], nn = near_off[k + 1] - b0;
   const int a1 = b0 + (int)((long long)nn * (part + 1) / nparts);
@@ -701,10 +965,10 @@ __device__ __forceinline__ void pair_tile_dw_near(const PairArgs<double>& A, con
       ++o1;
     }
     ++a;
-    dw_proxy_range<NT>(A, sh, k, o0 * A.N, (o1 + 1) * A.N, sp, sf, T);
-    dw_image_range<NT>(A, sh, k, A.img_off[o0], A.img_off[o1 + 1], si, T);
+    dw_proxy_range<1, NT, kDwTile>(A, sh, lam, 1u, o0 * A.N, (o1 + 1) * A.N, cnt, S.sp, S.sf, T);
+    dw_image_range<1, NT, kDwTileImg>(A, sh, lam, 1u, A.img_off[o0], A.img_off[o1 + 1], cnt, S.sp, S.si, T);
   }
-  dw_write_out<NT>(A, start, cnt, T, part, nparts, partial, pstride);
+  dw_write_out<1, NT>(A, start, cnt, T, 0, A.mu, A.out, part, nparts, partial, pstride);
 }
 
 // ------------------------------------------------------------------ far-field kernel (FP32)
@@ -831,31 +1095,6 @@ __global__ void __launch_bounds__(kPairThreads) pairs_far_kernel(FarArgs A, int 
 // each operation of the pair math runs on both lanes of a pair with one instruction (the FMA pipe
 // still does one lane-operation per target, but the issue slots are halved, which is what bounds
 // the scalar kernel).  Sources are staged with every component duplicated into both lanes.
-typedef unsigned long long f2x;
-__device__ __forceinline__ f2x f2sub(f2x a, f2x b) {
-  f2x d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2x f2mul(f2x a, f2x b) {
-  f2x d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2x f2fma(f2x a, f2x b, f2x c) {
-  f2x d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f2x f2make(float lo, float hi) {
-  f2x d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-  return d;
-}
-__device__ __forceinline__ void f2split(f2x v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-
 __global__ void __launch_bounds__(kPairThreads) pairs_far2_kernel(FarArgs A, int nparts, double* __restrict__ partial,
                                                                   long long pstride) {
   __shared__ ulonglong2 sa[kTileFar];  // (px, px | py, py)
@@ -986,12 +1225,12 @@ __global__ void __launch_bounds__(kPairThreads) pairs_kernel(PairArgs<T> A) {
   pair_tile<T, NT>(A, blockIdx.x);
 }
 template <int NT>
-__global__ void __launch_bounds__(kPairThreads) pairs_dw_kernel(PairArgs<double> A, int nparts, double* partial,
+__global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_kernel(PairArgs<double> A, int nparts, double* partial,
                                                                 long long pstride) {
   pair_tile_dw<NT>(A, blockIdx.x / nparts, blockIdx.x % nparts, nparts, partial, pstride);
 }
 template <int NT>
-__global__ void __launch_bounds__(kPairThreads) pairs_dw_near_kernel(PairArgs<double> A, const int* near_off,
+__global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_near_kernel(PairArgs<double> A, const int* near_off,
                                                                      const int* near_idx, int nparts, double* partial,
                                                                      long long pstride) {
   pair_tile_dw_near<NT>(A, near_off, near_idx, blockIdx.x / nparts, blockIdx.x % nparts, nparts, partial, pstride);
@@ -1059,10 +1298,8 @@ __global__ void __launch_bounds__(kPairThreads) pairs_batch_kernel(const PairArg
   A.out = bv.out + bv.voff[w.x];
   pair_tile<T, NT>(A, w.y);
 }
-// (register bounds as the compiler chose them before the fused reduction: 7 CTAs per SM for 1 node
-// per thread, 4 for 4)
 template <int NT>
-__global__ void __launch_bounds__(kPairThreads, NT == 1 ? 7 : 4) pairs_dw_batch_kernel(const PairArgs<double>* __restrict__ args,
+__global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_batch_kernel(const PairArgs<double>* __restrict__ args,
                                                                       const int2* __restrict__ work,
                                                                       const int* __restrict__ active, BatchVecs bv,
                                                                       int nparts) {
@@ -1089,180 +1326,18 @@ __global__ void __launch_bounds__(kPairThreads, NT == 1 ? 7 : 4) pairs_dw_batch_
 // double-float and applied to the strengths of every listed right-hand side (~85 of the ~204
 // FP32 operations of a Stokeslet pair, ~89 of ~436 of an image triple, are shared).  Each
 // right-hand side's sums follow the operation order of pair_tile_dw.
-constexpr int kTileProxyM = 128;  // proxy sources staged per round
-constexpr int kTileImgM = 64;     // image nodes staged per round
-
-template <int R>
-struct DWMulti {
-  dw x, y, z;
-  dw ux[R], uy[R], uz[R];
-};
-
-template <int R>
-__device__ __forceinline__ void dwm_proxy_range(const PairArgs<double>& A, const CentreShift64& sh, int k,
-                                                const double* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
-                                                float4* sp, float4 (*sf)[2 * kTileProxyM], DWMulti<R>& T) {
-  const double far = 1e18;
-  const int total = A.P * A.N;
-  for (int s0 = r_lo; s0 < r_hi; s0 += kTileProxyM) {
-    const int ns = min(kTileProxyM, r_hi - s0);
-    __syncthreads();
-    for (int i = threadIdx.x; i < ns; i += kPairThreads) {
-      const int j = s0 + i;
-      double px = far, py = far, pz = far;
-      int o = -1, jj = 0;
-      if (j < total) {
-        o = j / A.N;
-        jj = j - o * A.N;
-        const D4 pr = A.proxy[jj];
-        px = pr.x + sh.d(o, 0);
-        py = pr.y + sh.d(o, 1);
-        pz = pr.z + sh.d(o, 2);
-      }
-      dw a = dw_split(px), b = dw_split(py), c = dw_split(pz);
-      sp[2 * i] = make_float4(a.h, b.h, c.h, 0.f);
-      sp[2 * i + 1] = make_float4(a.l, b.l, c.l, 0.f);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        double fx = 0, fy = 0, fz = 0;
-        if ((mask >> r & 1u) && o >= 0 && o != k) {
-          const double* l = lam[r] + A.unk_off[o] + 3LL * jj;
-          fx = l[0];
-          fy = l[1];
-          fz = l[2];
-        }
-        a = dw_split(fx);
-        b = dw_split(fy);
-        c = dw_split(fz);
-        sf[r][2 * i] = make_float4(a.h, b.h, c.h, 0.f);
-        sf[r][2 * i + 1] = make_float4(a.l, b.l, c.l, 0.f);
-      }
-    }
-    __syncthreads();
-    for (int j = 0; j < ns; ++j) {
-      const float4 ph = sp[2 * j], pl = sp[2 * j + 1];
-      const dw dx = sub_pos(T.x, dw{ph.x, pl.x});
-      const dw dy = sub_pos(T.y, dw{ph.y, pl.y});
-      const dw dz = sub_pos(T.z, dw{ph.z, pl.z});
-      const dw ir = rsqrt_u(norm2_u(dx, dy, dz));
-      const dw ir2 = mul_u(ir, ir);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        if (!(mask >> r & 1u)) continue;
-        const float4 fh = sf[r][2 * j], fl = sf[r][2 * j + 1];
-        const dw fx{fh.x, fl.x}, fy{fh.y, fl.y}, fz{fh.z, fl.z};
-        const dw c = mul_u(dot3_u(dx, dy, dz, fx, fy, fz), ir2);
-        acc_u(T.ux[r], mul_u(ir, add_u(fx, mul_u(c, dx))));
-        acc_u(T.uy[r], mul_u(ir, add_u(fy, mul_u(c, dy))));
-        acc_u(T.uz[r], mul_u(ir, add_u(fz, mul_u(c, dz))));
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      T.ux[r] = two_sum(T.ux[r].h, T.ux[r].l);
-      T.uy[r] = two_sum(T.uy[r].h, T.uy[r].l);
-      T.uz[r] = two_sum(T.uz[r].h, T.uz[r].l);
-    }
-  }
-}
-
-// image node strengths of one right-hand side in 5 float4: hi of (f, t, d) then lo of the same
-template <int R>
-__device__ __forceinline__ void dwm_image_range(const PairArgs<double>& A, const CentreShift64& sh, int k,
-                                                const double* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
-                                                float4* sip, float4 (*sis)[5 * kTileImgM], DWMulti<R>& T) {
-  const double far = 1e18;
-  for (int s0 = r_lo; s0 < r_hi; s0 += kTileImgM) {
-    const int ns = min(kTileImgM, r_hi - s0);
-    __syncthreads();
-    for (int i = threadIdx.x; i < ns; i += kPairThreads) {
-      const int j = s0 + i;
-      double px = far, py = far, pz = far;
-      int o = -1;
-      if (j < A.n_img) {
-        o = A.img_owner[j];
-        const D4 pr = A.img[j];
-        px = pr.x + sh.d(o, 0);
-        py = pr.y + sh.d(o, 1);
-        pz = pr.z + sh.d(o, 2);
-      }
-      dw a = dw_split(px), b = dw_split(py), c = dw_split(pz);
-      sip[2 * i] = make_float4(a.h, b.h, c.h, 0.f);
-      sip[2 * i + 1] = make_float4(a.l, b.l, c.l, 0.f);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        float hv[9], lv[9];
-        const double* l = nullptr;
-        if ((mask >> r & 1u) && o >= 0 && o != k) l = lam[r] + A.unk_off[o] + 3LL * A.N + 9LL * (j - A.img_off[o]);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-          const double v = l ? (q < 6 ? l[q] : A.dip * l[q]) : 0.0;
-          const dw sv = dw_split(v);
-          hv[q] = sv.h;
-          lv[q] = sv.l;
-        }
-        sis[r][5 * i] = make_float4(hv[0], hv[1], hv[2], hv[3]);
-        sis[r][5 * i + 1] = make_float4(hv[4], hv[5], hv[6], hv[7]);
-        sis[r][5 * i + 2] = make_float4(hv[8], lv[0], lv[1], lv[2]);
-        sis[r][5 * i + 3] = make_float4(lv[3], lv[4], lv[5], lv[6]);
-        sis[r][5 * i + 4] = make_float4(lv[7], lv[8], 0.f, 0.f);
-      }
-    }
-    __syncthreads();
-    for (int j = 0; j < ns; ++j) {
-      const float4 ph = sip[2 * j], pl = sip[2 * j + 1];
-      const dw dx = sub_pos(T.x, dw{ph.x, pl.x}), dy = sub_pos(T.y, dw{ph.y, pl.y}), dz = sub_pos(T.z, dw{ph.z, pl.z});
-      const dw ir = rsqrt_u(norm2_u(dx, dy, dz));
-      const dw ir2 = mul_u(ir, ir);
-      const dw ir3 = mul_u(ir, ir2);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        if (!(mask >> r & 1u)) continue;
-        const float4 v0 = sis[r][5 * j], v1 = sis[r][5 * j + 1], v2 = sis[r][5 * j + 2], v3 = sis[r][5 * j + 3],
-                     v4 = sis[r][5 * j + 4];
-        const dw fx{v0.x, v2.y}, fy{v0.y, v2.z}, fz{v0.z, v2.w};
-        const dw tx{v0.w, v3.x}, ty{v1.x, v3.y}, tz{v1.y, v3.z};
-        const dw qx{v1.z, v3.w}, qy{v1.w, v4.x}, qz{v2.x, v4.y};
-        // Stokeslet
-        const dw cs = mul_u(dot3_u(dx, dy, dz, fx, fy, fz), ir2);
-        acc_u(T.ux[r], mul_u(ir, add_u(fx, mul_u(cs, dx))));
-        acc_u(T.uy[r], mul_u(ir, add_u(fy, mul_u(cs, dy))));
-        acc_u(T.uz[r], mul_u(ir, add_u(fz, mul_u(cs, dz))));
-        // rotlet (t x r) / r^3
-        acc_u(T.ux[r], mul_u(ir3, add_u(mul_u(ty, dz), neg(mul_u(tz, dy)))));
-        acc_u(T.uy[r], mul_u(ir3, add_u(mul_u(tz, dx), neg(mul_u(tx, dz)))));
-        acc_u(T.uz[r], mul_u(ir3, add_u(mul_u(tx, dy), neg(mul_u(ty, dx)))));
-        // potential dipole -d / r^3 + 3 (d.r) r / r^5
-        const dw c3 = times3_u(mul_u(mul_u(dot3_u(dx, dy, dz, qx, qy, qz), ir3), ir2));
-        acc_u(T.ux[r], mul_u(c3, dx));
-        acc_u(T.uy[r], mul_u(c3, dy));
-        acc_u(T.uz[r], mul_u(c3, dz));
-        acc_u(T.ux[r], neg(mul_u(ir3, qx)));
-        acc_u(T.uy[r], neg(mul_u(ir3, qy)));
-        acc_u(T.uz[r], neg(mul_u(ir3, qz)));
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      T.ux[r] = two_sum(T.ux[r].h, T.ux[r].l);
-      T.uy[r] = two_sum(T.uy[r].h, T.uy[r].l);
-      T.uz[r] = two_sum(T.uz[r].h, T.uz[r].l);
-    }
-  }
-}
+constexpr int kDwTileM = 128;    // proxy sources staged per round
+constexpr int kDwTileImgM = 32;  // image nodes staged per round
 
 // work[b] = (lead problem, tile of the 1-node-per-thread tiling, first index into rhs_prob, count);
 // the sources are split over nparts CTAs per item as in pairs_dw_batch_kernel
 template <int R>
-__global__ void __launch_bounds__(kPairThreads) pairs_dw_multi_kernel(const PairArgs<double>* __restrict__ args,
+__global__ void __launch_bounds__(kPairThreads, 3) pairs_dw_multi_kernel(const PairArgs<double>* __restrict__ args,
                                                                       const int4* __restrict__ work,
                                                                       const int* __restrict__ rhs_prob,
                                                                       const int* __restrict__ active, BatchVecs bv,
                                                                       int nparts) {
-  __shared__ float4 sp[2 * kTileProxyM];
-  __shared__ float4 sf[R][2 * kTileProxyM];
-  __shared__ float4 sip[2 * kTileImgM];
-  __shared__ float4 sis[R][5 * kTileImgM];
+  __shared__ DwShared<R, kDwTileM, kDwTileImgM> S;
   const int4 w = work[blockIdx.x / nparts];
   const int part = blockIdx.x % nparts;
   int prob[R];
@@ -1284,50 +1359,14 @@ __global__ void __launch_bounds__(kPairThreads) pairs_dw_multi_kernel(const Pair
   CentreShift64 sh;
   sh.cen = A.cen64;
   sh.init(k);
-  DWMulti<R> T;
-  {
-    const int idx = threadIdx.x;
-    const int node = start + (idx < cnt ? idx : cnt - 1);
-    const D4 p = A.tgt[node];
-    T.x = dw_split(p.x);
-    T.y = dw_split(p.y);
-    T.z = dw_split(p.z);
+  DWTile<R, 1> T;
+  dw_load_targets<R, 1>(A, start, cnt, T);
+  dw_all_sources<R, 1, kDwTileM, kDwTileImgM>(A, sh, k, lam, mask, cnt, part, nparts, S, T);
 #pragma unroll
-    for (int r = 0; r < R; ++r) T.ux[r] = T.uy[r] = T.uz[r] = dw{0.f, 0.f};
-  }
-  const int total = A.P * A.N;
-  const int p_lo = k < 0 ? total : k * A.N, p_w = k < 0 ? 0 : A.N;
-  const long long p_eff = total - p_w;
-  const int pe0 = (int)(p_eff * part / nparts), pe1 = (int)(p_eff * (part + 1) / nparts);
-  dwm_proxy_range<R>(A, sh, k, lam, mask, min(pe0, p_lo), min(pe1, p_lo), sp, sf, T);
-  dwm_proxy_range<R>(A, sh, k, lam, mask, max(pe0, p_lo) + p_w, max(pe1, p_lo) + p_w, sp, sf, T);
-  const int i_lo = k >= 0 ? A.img_off[k] : 0, i_w = k >= 0 ? A.img_off[k + 1] - i_lo : 0;
-  const long long i_eff = A.n_img - i_w;
-  const int ie0 = (int)(i_eff * part / nparts), ie1 = (int)(i_eff * (part + 1) / nparts);
-  dwm_image_range<R>(A, sh, k, lam, mask, min(ie0, i_lo), min(ie1, i_lo), sip, sis, T);
-  dwm_image_range<R>(A, sh, k, lam, mask, max(ie0, i_lo) + i_w, max(ie1, i_lo) + i_w, sip, sis, T);
-  const int idx = threadIdx.x;
-  if (idx < cnt) {
-    const long long node = start + idx;
-    const double sw = A.tgt[node].w;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      if (!(mask >> r & 1u)) continue;
-      const double gx = dw_join(T.ux[r]) * A.scale, gy = dw_join(T.uy[r]) * A.scale, gz = dw_join(T.uz[r]) * A.scale;
-      const long long off = bv.voff[prob[r]];
-      if (nparts > 1) {
-        double* o = bv.partial + off + part * bv.pstride + 3 * node;
-        o[0] = gx;
-        o[1] = gy;
-        o[2] = gz;
-      } else {
-        const double* mu = bv.mu + off;
-        double* out = bv.out + off;
-        out[3 * node] = mu[3 * node] + sw * gx;
-        out[3 * node + 1] = mu[3 * node + 1] + sw * gy;
-        out[3 * node + 2] = mu[3 * node + 2] + sw * gz;
-      }
-    }
+  for (int r = 0; r < R; ++r) {
+    if (!(mask >> r & 1u)) continue;
+    const long long off = bv.voff[prob[r]];
+    dw_write_out<R, 1>(A, start, cnt, T, r, bv.mu + off, bv.out + off, part, nparts, bv.partial + off, bv.pstride);
   }
   if (nparts > 1 && bv.counter && parts_last_arrival(bv.counter, blockIdx.x / nparts, nparts)) {
 #pragma unroll
@@ -2070,7 +2109,7 @@ template void launch_pairs<double>(const TargetSet&, const SourceSet&, const dou
 
 int pair_split_parts(long long n_tiles1, long long min_sources, int max_parts) {
   if (n_tiles1 <= 0) return 1;
-  long long s = kPairSplitTarget / n_tiles1;  // at most one wave of resident CTAs
+  long long s = (kPairSplitTarget + n_tiles1 - 1) / n_tiles1;
   s = std::min<long long>(s, min_sources / kPairSplitMinSources);
   s = std::min<long long>(s, max_parts);
   return (int)std::max<long long>(s, 1);
@@ -2088,8 +2127,7 @@ PairShape resolve_dw_shape(const TargetSet& tg, const SourceSet& src, PairShape 
   PairShape r;
   r.nt = shape_nt(tg, shape);
   if (shape.parts > 0) r.parts = std::min(shape.parts, max_parts);
-  else if (r.nt == 4) r.parts = 1;
-  else r.parts = pair_split_parts(tg.n_tiles1, (long long)(src.P - 1) * src.N, max_parts);
+  else r.parts = pair_split_parts(r.nt == 4 ? tg.n_tiles : tg.n_tiles1, (long long)(src.P - 1) * src.N, max_parts);
   return r;
 }
 
