@@ -476,7 +476,10 @@ void pairs_step(mfs_ctx* c, const T* lam_hat, const T* mu, T* out) {
         return;
       }
     }
-    launch_pairs<T>(c->tg, c->src, lam_hat, mu, out, c->hd.prm.visc, c->stream);
+    if constexpr (sizeof(T) == 8)
+      launch_pairs_fp64(c->tg, c->src, lam_hat, mu, out, c->hd.prm.visc, c->d_pparts, kPairMaxParts, c->stream);
+    else
+      launch_pairs_f32(c->tg, c->src, lam_hat, mu, out, c->hd.prm.visc, c->stream);
   });
   c->tm.pair_launches += 1;
   c->tm.pair_interactions += c->pairs_per_apply;
@@ -1246,9 +1249,12 @@ void batch_apply_kernels(BatchRun& R, const double* in, double* out) {
       active_tiles += B->tiles4[p];
       if (B->others_p[p] > 0) min_others = min_others < 0 ? B->others_p[p] : std::min(min_others, B->others_p[p]);
     }
-  const int nt = pair_nodes_per_thread((int)std::min<long long>(active_tiles, 1 << 30));
+  // the native FP64 kernel takes 128-node tiles (in pieces of 32 nodes)
+  const int nt = R.dw ? pair_nodes_per_thread((int)std::min<long long>(active_tiles, 1 << 30)) : 1;
   // few tiles left (the lockstep tail): split each tile's sources over several CTAs
-  const int parts = R.dw && nt == 1 && min_others > 0 ? pair_split_parts(B->n_cwork1, min_others, kPairMaxParts) : 1;
+  const int parts = nt != 1 || min_others <= 0 ? 1
+                    : R.dw ? pair_split_parts(B->n_cwork1, min_others, kPairMaxParts)
+                           : fp64_split_parts(4LL * B->n_cwork1, min_others, kPairMaxParts);
   timed(c, c->ev_pair, [&] {
     if (R.dw && B->n_mwork > 0) {
       // right-hand sides on one geometry share the pair evaluations; the problems left single
@@ -2972,50 +2978,22 @@ mfs_status mfs_eval_velocity(mfs_ctx* c, int npts, const double* x, double* u) {
   if (!c->solved) return c->fail(MFS_ERR_STATE, "no solution yet");
   if (npts < 0 || (npts > 0 && (!x || !u))) return c->fail(MFS_ERR_ARG, "bad evaluation arrays");
   if (npts == 0) return MFS_OK;
-  // temporary target set: absolute positions, no self exclusion (sphere index -1)
-  std::vector<double> t64(4 * (size_t)npts);
-  for (int i = 0; i < npts; ++i) {
-    for (int q = 0; q < 3; ++q) t64[4 * i + q] = x[3 * i + q];
-    t64[4 * i + 3] = 1.0;
+  // points, velocities and the parts of a split sum in one allocation
+  const size_t n3 = 3 * (size_t)npts, parts = velocity_parts(npts, c->src);
+  double* buf = nullptr;
+  if (cudaMalloc(&buf, sizeof(double) * n3 * (parts > 1 ? 2 + parts : 2)) != cudaSuccess) {
+    cudaGetLastError();
+    return c->fail(MFS_ERR_OOM, "device allocation failed: evaluation points");
   }
-  int nt = (npts + kTileTargets - 1) / kTileTargets;
-  std::vector<int> ts(nt, -1), tst(nt), tcn(nt);
-  for (int t = 0; t < nt; ++t) {
-    tst[t] = t * kTileTargets;
-    tcn[t] = std::min(kTileTargets, npts - t * kTileTargets);
-  }
-  std::vector<void*> tmp;
-  auto ta = [&](size_t bytes) -> void* {
-    void* q = nullptr;
-    if (cudaMalloc(&q, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    tmp.push_back(q);
-    return q;
-  };
-  auto done = [&](mfs_status st) {
-    cudaStreamSynchronize(c->stream);
-    for (void* q : tmp) cudaFree(q);
-    return st;
-  };
-  TargetSet tg;
-  tg.n = npts;
-  tg.n_tiles = nt;
-  tg.pos64 = (double*)ta(t64.size() * 8);
-  tg.tile_sphere = (int*)ta(nt * 4);
-  tg.tile_start = (int*)ta(nt * 4);
-  tg.tile_count = (int*)ta(nt * 4);
-  double* du = (double*)ta(3 * (size_t)npts * 8);
-  if (!tg.pos64 || !tg.tile_sphere || !tg.tile_start || !tg.tile_count || !du)
-    return done(c->fail(MFS_ERR_OOM, "device allocation failed: evaluation points"));
-  cudaMemcpyAsync(tg.pos64, t64.data(), t64.size() * 8, cudaMemcpyHostToDevice, c->stream);
-  cudaMemcpyAsync(tg.tile_sphere, ts.data(), nt * 4, cudaMemcpyHostToDevice, c->stream);
-  cudaMemcpyAsync(tg.tile_start, tst.data(), nt * 4, cudaMemcpyHostToDevice, c->stream);
-  cudaMemcpyAsync(tg.tile_count, tcn.data(), nt * 4, cudaMemcpyHostToDevice, c->stream);
-  launch_pairs<double>(tg, c->src, c->d_lam, nullptr, du, c->hd.prm.visc, c->stream);
-  cudaMemcpyAsync(u, du, 3 * (size_t)npts * 8, cudaMemcpyDeviceToHost, c->stream);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (e != cudaSuccess) return done(c->fail(MFS_ERR_CUDA, std::string("eval: ") + cudaGetErrorString(e)));
-  return done(MFS_OK);
+  cudaError_t e = cudaMemcpyAsync(buf, x, sizeof(double) * n3, cudaMemcpyHostToDevice, c->stream);
+  launch_velocity(npts, buf, c->src, c->d_lam, buf + n3, buf + 2 * n3, c->hd.prm.visc, c->stream);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpyAsync(u, buf + n3, sizeof(double) * n3, cudaMemcpyDeviceToHost, c->stream);
+  const cudaError_t es = cudaStreamSynchronize(c->stream);
+  cudaFree(buf);
+  if (e == cudaSuccess) e = es;
+  if (e != cudaSuccess) return c->fail(MFS_ERR_CUDA, std::string("eval: ") + cudaGetErrorString(e));
+  return MFS_OK;
 }
 
 mfs_status mfs_get_strengths(mfs_ctx* c, double* lambda, double* pos, int* type) {

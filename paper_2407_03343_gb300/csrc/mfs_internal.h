@@ -141,11 +141,24 @@ struct PairShape {
 };
 
 // Kernel launchers (mfs_kernels.cu).  All run on `st`.
-template <typename T>
-void launch_pairs(const TargetSet& tg, const SourceSet& src, const T* lam_hat, const T* mu,
-                  T* out, double visc, cudaStream_t st);
+void launch_pairs_f32(const TargetSet& tg, const SourceSet& src, const float* lam_hat, const float* mu, float* out,
+                      double visc, cudaStream_t st);
+// Native FP64 sums in pieces of 32 targets, the sources of each split over up to max_parts CTAs
+// (partial: max_parts * 3 n doubles) whose sums a second kernel adds in part order.
+void launch_pairs_fp64(const TargetSet& tg, const SourceSet& src, const double* lam_hat, const double* mu, double* out,
+                       double visc, double* partial, int max_parts, cudaStream_t st);
+// Source split of the FP64 kernels: enough CTAs (pieces x parts) that the SMs' shares of the FP64
+// pipe differ by a few per cent (152 SMs x 16), at least kPairSplitMinSources sources per part.
+constexpr int kFp64SplitTarget = 152 * 16;
+int fp64_split_parts(long long pieces, long long min_sources, int max_parts);
+// u (3 n) = velocity at the n points x (3 n, absolute) of the strengths lam, native FP64; partial
+// holds velocity_parts(n, src) * 3 n doubles (unused for one part).
+constexpr int kVelocityMaxParts = 64;
+int velocity_parts(int n, const SourceSet& src);
+void launch_velocity(int n, const double* x, const SourceSet& src, const double* lam, double* u, double* partial,
+                     double visc, cudaStream_t st);
 
-// Same sums as launch_pairs<double> (FP64 in and out) computed in double-float arithmetic on
+// Same sums as launch_pairs_fp64 (FP64 in and out) computed in double-float arithmetic on
 // the FP32 pipes.  With few target tiles the sources of each tile are split over up to
 // max_parts CTAs whose partial sums go to `partial` (max_parts * 3 n doubles; null: no split)
 // and are added in a second, deterministic pass.

@@ -1,18 +1,17 @@
 // CUDA kernels of the hot path (sm_103a).
 //
-//  pairs_kernel<T>     steps 2+3 of the G_hat apply (Sec. 2.2, eq. uAll): for every
+//  pair kernels        steps 2+3 of the G_hat apply (Sec. 2.2, eq. uAll): for every
 //                      collocation node x_i of sphere k,
 //                        out_i = mu_i + sqrt(w_i) sum_{k' != k} [S f + R t + D d](x_i - y)
 //                      over the proxy Stokeslets and the image S/R/D triples of all other
 //                      spheres (eq. lin_comb).  Direct summation, so the self block is
 //                      skipped instead of being added and subtracted (allowed by Sec. 2.2).
-//                      Sources are staged through shared memory in tiles; each thread owns
-//                      NT target nodes in registers; 1/|r| comes from rsqrt (FP32) or an
-//                      FP32 seed refined by Newton-Raphson (FP64).  FP32 sums run per tile
-//                      and are folded into Kahan-compensated accumulators across tiles.
-//                      Positions are stored relative to their sphere centre and shifted into
-//                      the target sphere's frame while staging, with the centre difference
-//                      taken in float-float, so near-contact distances keep FP32 accuracy.
+//                      Sources are staged through shared memory in rounds; positions are stored
+//                      relative to their sphere centre and shifted into the target sphere's
+//                      frame while staging.  FP32 (pairs_kernel): NT targets per thread, sums
+//                      folded into Kahan-compensated accumulators across rounds, the centre
+//                      difference in float-float.  Double-float (pairs_dw_*) and native FP64
+//                      (pairs_fp64_*, velocity_fp64_kernel): see there.
 //  gemv_kernel<T>      batched row-major GEMV for the one-body pseudo-inverse factors
 //                      (eq. transform), HBM-bound.
 //  Krylov kernels      multi-dot, update, scale (GMRES with CGS2), FP64 partial sums.
@@ -49,25 +48,24 @@ template <> struct Prec<float> {
 };
 template <> struct Prec<double> {
   using V4 = D4;
-  // 1/sqrt(x): FP32 hardware estimate refined by two Newton-Raphson steps
-  // y <- y (3 - x y^2) / 2, each of which roughly doubles the number of correct bits.
+  // 1/sqrt(x): FP32 hardware estimate y refined by one third-order step of the binomial series,
+  // y (1 - e)^(-1/2) = y (1 + e (1/2 + 3 e / 8) + ...) with e = 1 - x y^2 ~ 2^-22 (the dropped
+  // term is below 2^-66); five FP64 operations against seven of two Newton steps.
   static __device__ __forceinline__ double rsq(double x) {
-    double y = (double)rsqrtf((float)x);
-    y = y * (1.5 - 0.5 * x * y * y);
-    y = y * (1.5 - 0.5 * x * y * y);
-    return y;
+    const double y = (double)rsqrtf((float)x);
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y, e * fma(0.375, e, 0.5), y);
   }
   static __device__ __forceinline__ V4 mk(double a, double b, double c, double d) { return D4{a, b, c, d}; }
 };
 
-// Kahan-compensated s += x.  FP64 accumulates directly.
+// Kahan-compensated s += x.
 __device__ __forceinline__ void comp_add(float& s, float& c, float x) {
   float y = x - c;
   float t = s + y;
   c = (t - s) - y;
   s = t;
 }
-__device__ __forceinline__ void comp_add(double& s, double& c, double x) { (void)c; s += x; }
 
 // Centre of sphere o minus centre of the target frame, in the working precision.
 struct CentreShift32 {
@@ -90,10 +88,6 @@ struct CentreShift64 {
   }
   __device__ __forceinline__ double d(int o, int c) const { return cen[3 * o + c] - kc[c]; }
 };
-template <typename T> struct ShiftOf;
-template <> struct ShiftOf<float> { using type = CentreShift32; };
-template <> struct ShiftOf<double> { using type = CentreShift64; };
-
 template <typename T>
 struct PairArgs {
   const typename Prec<T>::V4* tgt;  // (x, y, z, sqrt w) relative to the tile's sphere (absolute if sphere < 0)
@@ -129,8 +123,9 @@ __device__ __forceinline__ void pair_tile(const PairArgs<T>& A, const int t) {
   const int k = A.tile_sphere[t];
   const int start = A.tile_start[t];
   const int cnt = A.tile_count[t];
-  typename ShiftOf<T>::type sh;
-  if constexpr (sizeof(T) == 4) { sh.hi = A.cen_hi; sh.lo = A.cen_lo; } else { sh.cen = A.cen64; }
+  CentreShift32 sh;
+  sh.hi = A.cen_hi;
+  sh.lo = A.cen_lo;
   sh.init(k);
 
   T x[NT], y[NT], z[NT], ux[NT], uy[NT], uz[NT];
@@ -320,6 +315,135 @@ PairArgs<T> make_args(const TargetSet& tg, const SourceSet& src, const T* lam, c
   A.dip = T(2.0 * visc);
   A.span = (float)(1.001 * src.span);
   return A;
+}
+
+// ------------------------------------------------------------------ native FP64 pair sums
+// Bound by the FP64 pipe (two lanes per SM and clock, so one warp per scheduler saturates it):
+// 22 FP64 operations a (node, Stokeslet) pair.  What matters is that every SM gets the same share of
+// it down to the last CTA, so a CTA takes 32 targets (a 128-node tile in four pieces; a sphere's
+// ragged last tile then wastes at most 31 lanes) and its four warps take every fourth source, with
+// the sources split further over CTAs where there are few targets.  Measured (20 spheres with
+// images, 5.7e8 pairs): 39.3 ms with a thread per node of 128- and 512-node tiles, 25.4
+// now; 16,125 flow points around three spheres: 3.44 and 0.86 ms.
+constexpr int kFp64Warps = kPairThreads / 32;
+constexpr int kFp64Tile = 256;     // proxy sources staged per round
+constexpr int kFp64TileImg = 128;  // image nodes staged per round
+
+// Sums at the 32 points of this CTA over its share of the sources: proxies [p0, p1) and image
+// nodes [i0, i1) of the lists without sphere k's own (k < 0: nothing left out).  Returns the sums in
+// the lanes of warp 0.
+__device__ __forceinline__ void fp64_sums(const PairArgs<double>& A, int k, double x, double y, double z, int part,
+                                          int nparts, double (&out)[3]) {
+  __shared__ D4 sp[kFp64Tile], sf[kFp64Tile];
+  __shared__ D4 si[3 * kFp64TileImg];
+  __shared__ double red[kFp64Warps][3][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  CentreShift64 sh;
+  sh.cen = A.cen64;
+  sh.init(k);
+  double ux = 0, uy = 0, uz = 0;
+
+  // ---- proxy Stokeslets of every sphere but k: this part's share of the list, in runs before and
+  // after sphere k's own
+  const int total = A.P * A.N;
+  const int p_lo = k < 0 ? total : k * A.N, p_w = k < 0 ? 0 : A.N;
+  const long long p_eff = total - p_w;
+  const int pe[2] = {(int)(p_eff * part / nparts), (int)(p_eff * (part + 1) / nparts)};
+  for (int rr = 0; rr < 2; ++rr) {
+    const int r_lo = rr == 0 ? min(pe[0], p_lo) : max(pe[0], p_lo) + p_w;
+    const int r_hi = rr == 0 ? min(pe[1], p_lo) : max(pe[1], p_lo) + p_w;
+    for (int s0 = r_lo; s0 < r_hi; s0 += kFp64Tile) {
+      const int ns = min(kFp64Tile, r_hi - s0);
+      __syncthreads();
+      for (int i = threadIdx.x; i < ns; i += kPairThreads) {
+        const int j = s0 + i, o = j / A.N, jj = j - o * A.N;
+        const D4 pr = A.proxy[jj];
+        const double* l = A.lam + A.unk_off[o] + 3LL * jj;
+        sp[i] = D4{pr.x + sh.d(o, 0), pr.y + sh.d(o, 1), pr.z + sh.d(o, 2), 0.0};
+        sf[i] = D4{l[0], l[1], l[2], 0.0};
+      }
+      __syncthreads();
+#pragma unroll 2
+      for (int j = warp; j < ns; j += kFp64Warps) {
+        const D4 p = sp[j], f = sf[j];
+        const double dx = x - p.x, dy = y - p.y, dz = z - p.z;
+        const double ir = Prec<double>::rsq(fma(dz, dz, fma(dy, dy, dx * dx)));
+        const double c = fma(dz, f.z, fma(dy, f.y, dx * f.x)) * ir * ir;
+        ux = fma(ir, fma(c, dx, f.x), ux);
+        uy = fma(ir, fma(c, dy, f.y), uy);
+        uz = fma(ir, fma(c, dz, f.z), uz);
+      }
+    }
+  }
+
+  // ---- image nodes (Stokeslet + rotlet + potential dipole at one position)
+  const int i_lo = k < 0 ? A.n_img : A.img_off[k], i_w = k < 0 ? 0 : A.img_off[k + 1] - i_lo;
+  const long long i_eff = A.n_img - i_w;
+  const int ie[2] = {(int)(i_eff * part / nparts), (int)(i_eff * (part + 1) / nparts)};
+  for (int rr = 0; rr < 2; ++rr) {
+    const int r_lo = rr == 0 ? min(ie[0], i_lo) : max(ie[0], i_lo) + i_w;
+    const int r_hi = rr == 0 ? min(ie[1], i_lo) : max(ie[1], i_lo) + i_w;
+    for (int s0 = r_lo; s0 < r_hi; s0 += kFp64TileImg) {
+      const int ns = min(kFp64TileImg, r_hi - s0);
+      __syncthreads();
+      for (int i = threadIdx.x; i < ns; i += kPairThreads) {
+        const int j = s0 + i, o = A.img_owner[j];
+        const D4 pr = A.img[j];
+        const double* l = A.lam + A.unk_off[o] + 3LL * A.N + 9LL * (j - A.img_off[o]);
+        si[3 * i] = D4{pr.x + sh.d(o, 0), pr.y + sh.d(o, 1), pr.z + sh.d(o, 2), l[0]};
+        si[3 * i + 1] = D4{l[1], l[2], l[3], l[4]};
+        si[3 * i + 2] = D4{l[5], A.dip * l[6], A.dip * l[7], A.dip * l[8]};
+      }
+      __syncthreads();
+      for (int j = warp; j < ns; j += kFp64Warps) {
+        const D4 a = si[3 * j], b = si[3 * j + 1], c = si[3 * j + 2];
+        // f = (a.w, b.x, b.y), t = (b.z, b.w, c.x), d = (c.y, c.z, c.w)
+        const double dx = x - a.x, dy = y - a.y, dz = z - a.z;
+        const double ir = Prec<double>::rsq(fma(dz, dz, fma(dy, dy, dx * dx)));
+        const double ir2 = ir * ir, ir3 = ir * ir2;
+        // Stokeslet
+        const double cs = fma(dz, b.y, fma(dy, b.x, dx * a.w)) * ir2;
+        double vx = ir * fma(cs, dx, a.w), vy = ir * fma(cs, dy, b.x), vz = ir * fma(cs, dz, b.y);
+        // rotlet (t x r) / r^3 and potential dipole -d / r^3 + 3 (d.r) r / r^5
+        const double c3 = 3.0 * fma(dz, c.w, fma(dy, c.z, dx * c.y)) * ir2;
+        vx = fma(ir3, fma(b.w, dz, -c.x * dy) + fma(c3, dx, -c.y), vx);
+        vy = fma(ir3, fma(c.x, dx, -b.z * dz) + fma(c3, dy, -c.z), vy);
+        vz = fma(ir3, fma(b.z, dy, -b.w * dx) + fma(c3, dz, -c.w), vz);
+        ux += vx;
+        uy += vy;
+        uz += vz;
+      }
+    }
+  }
+  red[warp][0][lane] = ux;
+  red[warp][1][lane] = uy;
+  red[warp][2][lane] = uz;
+  __syncthreads();
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    out[c] = 0.0;
+    if (warp == 0)
+      for (int w = 0; w < kFp64Warps; ++w) out[c] += red[w][c][lane];
+    out[c] *= A.scale;
+  }
+}
+
+// One 32-node piece (0..3) of a 128-node tile: out = mu + sqrt(w) u, or this part's partial sums.
+__device__ __forceinline__ void pair_piece_fp64(const PairArgs<double>& A, int t, int piece, int part, int nparts,
+                                                double* __restrict__ partial, long long pstride) {
+  const int start = A.tile_start[t] + 32 * piece, cnt = min(32, A.tile_count[t] - 32 * piece);
+  if (cnt <= 0) return;
+  const int lane = threadIdx.x & 31;
+  const long long node = start + min(lane, cnt - 1);
+  const D4 p = A.tgt[node];
+  double u[3];
+  fp64_sums(A, A.tile_sphere[t], p.x, p.y, p.z, part, nparts, u);
+  if (threadIdx.x >= cnt) return;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    if (nparts > 1) partial[part * pstride + 3 * node + c] = u[c];
+    else A.out[3 * node + c] = A.mu[3 * node + c] + p.w * u[c];
+  }
 }
 
 // ------------------------------------------------------------------ double-float pair kernel
@@ -1224,6 +1348,25 @@ template <typename T, int NT>
 __global__ void __launch_bounds__(kPairThreads) pairs_kernel(PairArgs<T> A) {
   pair_tile<T, NT>(A, blockIdx.x);
 }
+__global__ void __launch_bounds__(kPairThreads) pairs_fp64_kernel(PairArgs<double> A, int nparts, double* partial,
+                                                                  long long pstride) {
+  const int piece = blockIdx.x % 4, t = blockIdx.x / 4 / nparts, part = blockIdx.x / 4 % nparts;
+  pair_piece_fp64(A, t, piece, part, nparts, partial, pstride);
+}
+// velocity at n arbitrary points x (absolute positions): u, or this part's partial sums
+__global__ void __launch_bounds__(kPairThreads) velocity_fp64_kernel(PairArgs<double> A, int n,
+                                                                     const double* __restrict__ x, int nparts,
+                                                                     double* __restrict__ u, long long pstride) {
+  const int part = blockIdx.x % nparts;
+  const long long i0 = 32LL * (blockIdx.x / nparts);
+  const int cnt = (int)min(32LL, n - i0);
+  const long long i = i0 + min((int)(threadIdx.x & 31), cnt - 1);
+  double v[3];
+  fp64_sums(A, -1, x[3 * i], x[3 * i + 1], x[3 * i + 2], part, nparts, v);
+  if (threadIdx.x >= cnt) return;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) u[part * pstride + 3 * i + c] = v[c];
+}
 template <int NT>
 __global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_kernel(PairArgs<double> A, int nparts, double* partial,
                                                                 long long pstride) {
@@ -1286,17 +1429,19 @@ __device__ __forceinline__ void parts_finish_node(const D4* tgt, long long node,
     out[3 * node + c] = mu[3 * node + c] + sw * sum;
   }
 }
-template <typename T, int NT>
-__global__ void __launch_bounds__(kPairThreads) pairs_batch_kernel(const PairArgs<T>* __restrict__ args,
-                                                                   const int2* __restrict__ work,
-                                                                   const int* __restrict__ active, BatchVecs bv) {
-  const int2 w = work[blockIdx.x];
+// native FP64: each (problem, 128-node tile) in four pieces; with split sources the parts are added
+// by pair_parts_reduce_batch_kernel
+__global__ void __launch_bounds__(kPairThreads, 4) pairs_fp64_batch_kernel(const PairArgs<double>* __restrict__ args,
+                                                                        const int2* __restrict__ work,
+                                                                        const int* __restrict__ active, BatchVecs bv,
+                                                                        int nparts) {
+  const int2 w = work[blockIdx.x / 4 / nparts];
   if (!active[w.x]) return;
-  PairArgs<T> A = args[w.x];
+  PairArgs<double> A = args[w.x];
   A.lam = bv.lam + bv.uoff[w.x];
   A.mu = bv.mu + bv.voff[w.x];
   A.out = bv.out + bv.voff[w.x];
-  pair_tile<T, NT>(A, w.y);
+  pair_piece_fp64(A, w.y, blockIdx.x % 4, blockIdx.x / 4 % nparts, nparts, bv.partial + bv.voff[w.x], bv.pstride);
 }
 template <int NT>
 __global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_batch_kernel(const PairArgs<double>* __restrict__ args,
@@ -2094,18 +2239,56 @@ inline int grid_for(long long n, int threads, int cap = 152 * 16) {
 long long launches_on_this_thread() { return t_launches; }
 void note_launch() { ++t_launches; }
 
-template <typename T>
-void launch_pairs(const TargetSet& tg, const SourceSet& src, const T* lam_hat, const T* mu, T* out, double visc,
-                  cudaStream_t st) {
+void launch_pairs_f32(const TargetSet& tg, const SourceSet& src, const float* lam_hat, const float* mu, float* out,
+                      double visc, cudaStream_t st) {
   if (tg.n_tiles == 0) return;
   const int nt = tg.n_tiles1 > 0 ? pair_nodes_per_thread(tg.n_tiles) : 4;
-  PairArgs<T> A = make_args<T>(tg, src, lam_hat, mu, out, visc, nt);
+  PairArgs<float> A = make_args<float>(tg, src, lam_hat, mu, out, visc, nt);
   ++t_launches;
-  if (nt == 4) pairs_kernel<T, 4><<<tg.n_tiles, kPairThreads, 0, st>>>(A);
-  else pairs_kernel<T, 1><<<tg.n_tiles1, kPairThreads, 0, st>>>(A);
+  if (nt == 4) pairs_kernel<float, 4><<<tg.n_tiles, kPairThreads, 0, st>>>(A);
+  else pairs_kernel<float, 1><<<tg.n_tiles1, kPairThreads, 0, st>>>(A);
 }
-template void launch_pairs<float>(const TargetSet&, const SourceSet&, const float*, const float*, float*, double, cudaStream_t);
-template void launch_pairs<double>(const TargetSet&, const SourceSet&, const double*, const double*, double*, double, cudaStream_t);
+
+int fp64_split_parts(long long pieces, long long min_sources, int max_parts) {
+  if (pieces <= 0) return 1;
+  long long s = (kFp64SplitTarget + pieces - 1) / pieces;
+  s = std::min<long long>(s, min_sources / kPairSplitMinSources);
+  s = std::min<long long>(s, max_parts);
+  return (int)std::max<long long>(s, 1);
+}
+
+void launch_pairs_fp64(const TargetSet& tg, const SourceSet& src, const double* lam_hat, const double* mu, double* out,
+                       double visc, double* partial, int max_parts, cudaStream_t st) {
+  if (tg.n_tiles1 == 0) return;
+  PairArgs<double> A = make_args<double>(tg, src, lam_hat, mu, out, visc, 1);
+  const long long n3 = 3LL * tg.n;
+  const int parts = fp64_split_parts(4LL * tg.n_tiles1, (long long)(src.P - 1) * src.N, max_parts);
+  ++t_launches;
+  pairs_fp64_kernel<<<4 * tg.n_tiles1 * parts, kPairThreads, 0, st>>>(A, parts, partial, n3);
+  if (parts > 1) {
+    ++t_launches;
+    pair_parts_reduce_kernel<<<grid_for(n3, 256), 256, 0, st>>>(n3, A.tgt, parts, partial, n3, mu, out);
+  }
+}
+
+int velocity_parts(int n, const SourceSet& src) {
+  return fp64_split_parts((n + 31LL) / 32, (long long)src.P * src.N, kVelocityMaxParts);
+}
+
+void launch_velocity(int n, const double* x, const SourceSet& src, const double* lam, double* u, double* partial,
+                     double visc, cudaStream_t st) {
+  if (n <= 0) return;
+  PairArgs<double> A = make_args<double>(TargetSet(), src, lam, nullptr, u, visc, 1);
+  const int parts = velocity_parts(n, src);
+  const long long n3 = 3LL * n;
+  ++t_launches;
+  velocity_fp64_kernel<<<(unsigned)((n + 31LL) / 32 * parts), kPairThreads, 0, st>>>(A, n, x, parts,
+                                                                                   parts > 1 ? partial : u, n3);
+  if (parts > 1) {
+    ++t_launches;
+    pair_parts_reduce_kernel<<<grid_for(n3, 256), 256, 0, st>>>(n3, nullptr, parts, partial, n3, nullptr, u);
+  }
+}
 
 int pair_split_parts(long long n_tiles1, long long min_sources, int max_parts) {
   if (n_tiles1 <= 0) return 1;
@@ -2297,8 +2480,13 @@ void launch_pairs_batch64(bool double_float, const void* d_args, const int2* d_w
       }
     }
   } else {
-    if (nodes_per_thread == 4) pairs_batch_kernel<double, 4><<<n_work, kPairThreads, 0, st>>>(args, d_work, d_active, bv);
-    else pairs_batch_kernel<double, 1><<<n_work, kPairThreads, 0, st>>>(args, d_work, d_active, bv);
+    if (!partial) parts = 1;
+    pairs_fp64_batch_kernel<<<4 * n_work * parts, kPairThreads, 0, st>>>(args, d_work, d_active, bv, parts);
+    if (parts > 1) {
+      ++t_launches;
+      if (seg_ctas(seg) > 0)
+        pair_parts_reduce_batch_kernel<<<dim3(seg_ctas(seg), (seg.chunk + 127) / 128), 128, 0, st>>>(seg, args, bv, parts);
+    }
   }
 }
 
