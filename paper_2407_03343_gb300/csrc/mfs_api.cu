@@ -53,29 +53,41 @@ struct Factor {
   double* V64 = nullptr;  // ncol x ldV  (V)
   float* A32 = nullptr;
   float* V32 = nullptr;
-  float2* A2 = nullptr;   // (hi, lo) float pairs of A64 and V64 for the double-float GEMV
-  float2* V2 = nullptr;
+  // rows in pairs for the double-float GEMVs: A32 a column as (a0 a1), A2 and V2 as (h0 h1 l0 l1),
+  // the (hi, lo) float pairs of A64 and V64 (a last odd row is paired with zeros)
+  float4* A2 = nullptr;
+  float4* V2 = nullptr;
   float* Q32 = nullptr;   // far field: 3 n_eq x ldQ (row-major), collocation data -> equivalent strengths
   int ldQ = 0;
 };
 
-// keep[i] is the SVD column index of the i-th retained singular triplet
-__device__ __forceinline__ float2 split2(double v) {
-  float h = (float)v;
-  return make_float2(h, (float)(v - (double)h));
+// component i % 2 of row pair i / 2, column j: the FP32 and double-float copies of an entry
+__device__ __forceinline__ void put_pair32(float* M, int ld, int i, int j, double v) {
+  M[2 * ((long long)(i >> 1) * ld + j) + (i & 1)] = (float)v;
+}
+__device__ __forceinline__ void put_pair_dw(float4* M, int ld, int i, int j, double v) {
+  const float h = (float)v;
+  float* q = reinterpret_cast<float*>(M + (long long)(i >> 1) * ld + j) + (i & 1);
+  q[0] = h;
+  q[2] = (float)(v - (double)h);
 }
 
+// keep[i] is the SVD column index of the i-th retained singular triplet; the row pairs' storage is
+// rounded up to an even number of rows
 __global__ void pack_A_kernel(int r, int m, int ld, const double* __restrict__ U, const double* __restrict__ S,
                               const int* __restrict__ keep, double* __restrict__ A64, float* __restrict__ A32,
-                              float2* __restrict__ A2) {
-  long long tot = (long long)r * ld;
+                              float4* __restrict__ A2) {
+  long long tot = (long long)((r + 1) & ~1) * ld;
   for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < tot; id += (long long)gridDim.x * blockDim.x) {
     int i = (int)(id / ld), j = (int)(id % ld);
-    int col = keep[i];
-    double v = j < m ? U[(long long)col * m + j] / S[col] : 0.0;
-    A64[id] = v;
-    A32[id] = (float)v;
-    A2[id] = split2(v);
+    double v = 0.0;
+    if (i < r) {
+      const int col = keep[i];
+      if (j < m) v = U[(long long)col * m + j] / S[col];
+      A64[id] = v;
+    }
+    put_pair32(A32, ld, i, j, v);
+    put_pair_dw(A2, ld, i, j, v);
   }
 }
 
@@ -90,14 +102,17 @@ __global__ void upper_copy_kernel(int n, const double* __restrict__ B, int ldb, 
 
 // VT is the column-major ncol x ncol matrix V^T returned by the SVD: V(row, i) = VT[row * ncol + i]
 __global__ void pack_V_kernel(int ncol, int r, int ld, const double* __restrict__ VT, const int* __restrict__ keep,
-                              double* __restrict__ V64, float* __restrict__ V32, float2* __restrict__ V2) {
-  long long tot = (long long)ncol * ld;
+                              double* __restrict__ V64, float* __restrict__ V32, float4* __restrict__ V2) {
+  long long tot = (long long)((ncol + 1) & ~1) * ld;
   for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < tot; id += (long long)gridDim.x * blockDim.x) {
     int row = (int)(id / ld), i = (int)(id % ld);
-    double v = i < r ? VT[(long long)row * ncol + keep[i]] : 0.0;
-    V64[id] = v;
-    V32[id] = (float)v;
-    V2[id] = split2(v);
+    double v = 0.0;
+    if (row < ncol) {
+      if (i < r) v = VT[(long long)row * ncol + keep[i]];
+      V64[id] = v;
+      V32[id] = (float)v;
+    }
+    put_pair_dw(V2, ld, row, i, v);
   }
 }
 
@@ -224,6 +239,7 @@ struct mfs_ctx {
   // tile shapes of the pair kernels (default: by rule; mfs_tune_pairs measures and sets them)
   PairShape shape_all, shape_near, shape_far;
   GemvBatch<float> gA32, gV32;
+  GemvBatch<float> gA2, gV2;  // double-float row pairs
   GemvBatch<double> gA64, gV64;
   long long tmp_len = 0;
   int n = 0;              // operator size 3 * n_colloc
@@ -285,6 +301,7 @@ struct mfs_ctx {
     tcA = TcGemm();
     tcQ = TcGemm();
     gA32_rest = gQ_rest = GemvBatch<float>();
+    gA2 = gV2 = GemvBatch<float>();
     tg = TargetSet();
     src = SourceSet();
     d_basis = nullptr;
@@ -413,9 +430,9 @@ void precond(mfs_ctx* c, const T* mu, T* lam_hat) {
         } else if (c->dw_fast_a) {
           launch_gemv_f32_dw(c->gA32, c->d_x2, c->d_t2, c->stream);
         } else {
-          launch_gemv_dw(Ops<T>::A(c), c->d_x2, c->d_t2, nullptr, c->stream);
+          launch_gemv_dw(c->gA2, c->d_x2, c->d_t2, nullptr, c->stream);
         }
-        launch_gemv_dw(Ops<T>::V(c), c->d_t2, nullptr, lam_hat, c->stream);
+        launch_gemv_dw(c->gV2, c->d_t2, nullptr, lam_hat, c->stream);
         return;
       }
     }
@@ -752,7 +769,12 @@ struct BatchPlan {
   int* d_active = nullptr;
   long long *d_uoff = nullptr, *d_voff = nullptr;
   GemvBatch<double> gA, gV;
-  GemvBatch<float> gA32;  // the same jobs over the FP32 copies of Sigma^+ U^T (inner MIXED solves)
+  GemvBatch<float> gA2, gV2;  // the same jobs over the double-float row pairs
+  GemvBatch<float> gA32;      // and over the FP32 copies of Sigma^+ U^T (inner MIXED solves)
+  std::vector<const void*> jmat;  // per job its factor, for the work items of the active jobs
+  int2* d_items = nullptr;        // work items of the active jobs, and of those off the tensor cores
+  int2* d_items_rest = nullptr;
+  int2* items_pin = nullptr;      // pinned staging for both
   // tensor-core step 1 of the inner MIXED solves: the spheres of every problem whose factor is
   // one store entry form the columns of one product; gA32 then covers the other jobs only
   std::shared_ptr<SharedFactor> tc_ent;  // keeps the entry (and its slices) alive with the plan
@@ -806,6 +828,7 @@ struct BatchPlan {
     if (rhs_pin) cudaFreeHost(rhs_pin);
     if (swork_pin) cudaFreeHost(swork_pin);
     if (jpin_rest) cudaFreeHost(jpin_rest);
+    if (items_pin) cudaFreeHost(items_pin);
     if (snap) cudaFreeHost(snap);
     for (void* q : gs_allocs) cudaFree(q);
     if (ev) cudaEventDestroy(ev);
@@ -893,8 +916,7 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
   // GEMV jobs: every sphere of every problem, with the problems that share a context (several
   // right-hand sides on one geometry) adjacent, so a factor matrix is read once for all of them
   std::vector<const double*> mA, mV;
-  std::vector<const float*> mA32;
-  std::vector<const float2*> mA2, mV2;
+  std::vector<const float*> mA32, mA2, mV2;
   std::vector<int> rA, cA, lA, rV, cV, lV, jp;
   std::vector<long long> xA, yA, xV, yV;
   int maxA = 0, maxV = 0;
@@ -962,9 +984,10 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
       for (int p : group) {
         mA.push_back(F.A64);
         mV.push_back(F.V64);
-        mA2.push_back(F.A2);
+        mA2.push_back(reinterpret_cast<const float*>(F.A2));
+        B->jmat.push_back(F.A64);
         mA32.push_back(F.A32);
-        mV2.push_back(F.V2);
+        mV2.push_back(reinterpret_cast<const float*>(F.V2));
         rA.push_back(F.rank); cA.push_back(F.m); lA.push_back(F.ldA);
         xA.push_back(B->voff[p] + 3LL * d.colloc_off[k]);
         yA.push_back(B->toff[p] + ptoff[p][k]);
@@ -986,8 +1009,8 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
   }
   const double** dmA = nullptr;
   const double** dmV = nullptr;
-  const float2** dmA2 = nullptr;
-  const float2** dmV2 = nullptr;
+  const float** dmA2 = nullptr;
+  const float** dmV2 = nullptr;
   const float** dmA32 = nullptr;
   int *drA, *dcA, *dlA, *drV, *dcV, *dlV, *djp;
   long long *dxA, *dyA, *dxV, *dyV;
@@ -999,8 +1022,6 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
        put(B, dyA, yA) && put(B, dxV, xV) && put(B, dyV, yV) && put(B, dmA2, mA2) && put(B, dmV2, mV2) &&
        put(B, dmA32, mA32);
   if (ok) {
-    B->gA.mat_dw = dmA2;
-    B->gV.mat_dw = dmV2;
     B->gA.mat = dmA; B->gA.rows = drA; B->gA.cols = dcA; B->gA.ld = dlA; B->gA.x_off = dxA; B->gA.y_off = dyA;
     B->gA.n_jobs = (int)mA.size(); B->gA.max_rows = maxA; B->gA.job_prob = djp; B->gA.active = B->d_active;
     B->gV.mat = dmV; B->gV.rows = drV; B->gV.cols = dcV; B->gV.ld = dlV; B->gV.x_off = dxV; B->gV.y_off = dyV;
@@ -1008,7 +1029,16 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
     B->gA32.mat = dmA32; B->gA32.rows = drA; B->gA32.cols = dcA; B->gA32.ld = dlA; B->gA32.x_off = dxA;
     B->gA32.y_off = dyA; B->gA32.n_jobs = (int)mA32.size(); B->gA32.max_rows = maxA; B->gA32.job_prob = djp;
     B->gA32.active = B->d_active;
+    B->gA32.paired = true;
+    B->gA2 = B->gA32;
+    B->gA2.mat = dmA2;
+    B->gV2 = B->gA2;
+    B->gV2.mat = dmV2;
+    B->gV2.rows = drV; B->gV2.cols = dcV; B->gV2.ld = dlV; B->gV2.x_off = dxV; B->gV2.y_off = dyV;
+    B->gV2.max_rows = maxV;
   }
+  ok = ok && (B->d_items = B->alloc<int2>(jp.size())) && (B->d_items_rest = B->alloc<int2>(jp.size())) &&
+       cudaMallocHost(&B->items_pin, sizeof(int2) * 2 * std::max<size_t>(1, jp.size())) == cudaSuccess;
   B->mwork_cap = std::max<size_t>(1, B->w1_host.size());
   ok = ok && (B->d_mwork = B->alloc<int4>(B->mwork_cap)) && (B->d_rhs = B->alloc<int>(K)) &&
        (B->d_swork1 = B->alloc<int2>(B->mwork_cap)) && (B->d_pcount = B->alloc<unsigned>(B->mwork_cap)) &&
@@ -1185,8 +1215,25 @@ mfs_status set_active(BatchRun& R, const std::vector<int>& a) {
     g->job_list = B->d_jlist;
     g->n_list = nj;
   }
-  B->gA32.job_list = B->d_jlist;
-  B->gA32.n_list = nj;
+  // work items of the double-float GEMVs: the active right-hand sides of one matrix together
+  auto set_items = [&](const int* list, int n, int2* pin, int2* dev, std::initializer_list<GemvBatch<float>*> gs,
+                       const int* d_list) -> mfs_status {
+    std::vector<int2> items;
+    const int most = gemv_items(n, list, B->jmat.data(), items);
+    std::copy(items.begin(), items.end(), pin);
+    if (!items.empty())
+      CUDA_TRY(R.c0, cudaMemcpyAsync(dev, pin, sizeof(int2) * items.size(), cudaMemcpyHostToDevice, R.st));
+    for (GemvBatch<float>* g : gs) {
+      g->job_list = d_list;
+      g->n_list = n;
+      g->items = dev;
+      g->n_items = (int)items.size();
+      g->items_max = most;
+    }
+    return MFS_OK;
+  };
+  mfs_status si = set_items(B->jpin, nj, B->items_pin, B->d_items, {&B->gA2, &B->gV2, &B->gA32}, B->d_jlist);
+  if (si != MFS_OK) return si;
   if (B->tc_ncap > 0) {
     // the FP32 GEMV covers the jobs that are not tensor columns; the columns of the active
     // problems go to the tensor-core product
@@ -1199,8 +1246,8 @@ mfs_status set_active(BatchRun& R, const std::vector<int>& a) {
         B->tc_pin[B->tc_ncap + nt] = B->tc_y_host[i];
         ++nt;
       }
-    B->gA32.job_list = B->d_jlist_rest;
-    B->gA32.n_list = nr;
+    si = set_items(B->jpin_rest, nr, B->items_pin + B->jprob_host.size(), B->d_items_rest, {&B->gA32}, B->d_jlist_rest);
+    if (si != MFS_OK) return si;
     B->tc_nact = nt;
     if (nr) CUDA_TRY(R.c0, cudaMemcpyAsync(B->d_jlist_rest, B->jpin_rest, sizeof(int) * nr, cudaMemcpyHostToDevice, R.st));
     if (nt) {
@@ -1235,9 +1282,9 @@ void batch_apply_kernels(BatchRun& R, const double* in, double* out) {
           c->tm.tc_columns += B->tc_nact;
         }
       } else {
-        launch_gemv_dw(B->gA, B->x2, B->t2, nullptr, R.st);
+        launch_gemv_dw(B->gA2, B->x2, B->t2, nullptr, R.st);
       }
-      launch_gemv_dw(B->gV, B->t2, nullptr, B->lh, R.st);
+      launch_gemv_dw(B->gV2, B->t2, nullptr, B->lh, R.st);
     } else {
       launch_gemv<double>(B->gA, in, B->tmp, R.st);
       launch_gemv<double>(B->gV, B->tmp, B->lh, R.st);
@@ -1692,8 +1739,8 @@ mfs_status batch_lockstep_impl(int K, mfs_ctx* const* ctxs, const mfs_solve_opts
     if (o.precision == MFS_MIXED) {
       // double-float factors (~2^-46 relative) instead of the FP64 pipes
       launch_split_dw(B->n_total, B->x, B->x2, R.st);
-      launch_gemv_dw(B->gA, B->x2, B->t2, nullptr, R.st);
-      launch_gemv_dw(B->gV, B->t2, nullptr, B->lam, R.st);
+      launch_gemv_dw(B->gA2, B->x2, B->t2, nullptr, R.st);
+      launch_gemv_dw(B->gV2, B->t2, nullptr, B->lam, R.st);
     } else {
       launch_gemv<double>(B->gA, B->x, B->tmp, R.st);
       launch_gemv<double>(B->gV, B->tmp, B->lam, R.st);
@@ -2308,11 +2355,12 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
       {
         std::lock_guard<std::mutex> g(mtx);
         F.A64 = (double*)falloc(sizeof(double) * (size_t)r * F.ldA);
-        F.A32 = (float*)falloc(sizeof(float) * (size_t)r * F.ldA);
+        const size_t r_even = (size_t)((r + 1) & ~1), n_even = (size_t)((ncol + 1) & ~1);
+        F.A32 = (float*)falloc(sizeof(float) * r_even * F.ldA);
         F.V64 = (double*)falloc(sizeof(double) * (size_t)ncol * F.ldV);
         F.V32 = (float*)falloc(sizeof(float) * (size_t)ncol * F.ldV);
-        F.A2 = (float2*)falloc(sizeof(float2) * (size_t)r * F.ldA);
-        F.V2 = (float2*)falloc(sizeof(float2) * (size_t)ncol * F.ldV);
+        F.A2 = (float4*)falloc(sizeof(float2) * r_even * F.ldA);
+        F.V2 = (float4*)falloc(sizeof(float2) * n_even * F.ldV);
       }
       if (!F.A64 || !F.A32 || !F.V64 || !F.V32 || !F.A2 || !F.V2) {
         fail_w(MFS_ERR_OOM, "device allocation failed: one-body factors");
@@ -2452,14 +2500,14 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   if (nf > 0) {
     std::vector<const double*> mA64(P), mV64(P);
     std::vector<const float*> mA32(P), mV32(P);
-    std::vector<const float2*> mA2(P), mV2(P);
+    std::vector<const float*> mA2(P), mV2(P);
     std::vector<int> rA(P), cA(P), lA(P), rV(P), cV(P), lV(P);
     std::vector<long long> xA(P), yA(P), xV(P), yV(P);
     int maxA = 0, maxV = 0;
     for (int k = 0; k < P; ++k) {
       const Factor& F = c->factors[d.factor_id[k]];
       mA64[k] = F.A64; mA32[k] = F.A32; mV64[k] = F.V64; mV32[k] = F.V32;
-      mA2[k] = F.A2; mV2[k] = F.V2;
+      mA2[k] = reinterpret_cast<const float*>(F.A2); mV2[k] = reinterpret_cast<const float*>(F.V2);
       rA[k] = F.rank; cA[k] = F.m; lA[k] = F.ldA;
       xA[k] = 3LL * d.colloc_off[k]; yA[k] = tmp_off[k];
       rV[k] = F.ncol; cV[k] = F.rank; lV[k] = F.ldV;
@@ -2477,31 +2525,48 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
     c->gV64.mat = dm64;
     if ((s = upload(c, dm32, mV32)) != MFS_OK) return s;
     c->gV32.mat = dm32;
-    const float2** dm2 = nullptr;
-    if ((s = upload(c, dm2, mA2)) != MFS_OK) return s;
-    c->gA64.mat_dw = dm2;
-    if ((s = upload(c, dm2, mV2)) != MFS_OK) return s;
-    c->gV64.mat_dw = dm2;
+    if ((s = upload(c, dm32, mA2)) != MFS_OK) return s;
+    c->gA2.mat = dm32;
+    if ((s = upload(c, dm32, mV2)) != MFS_OK) return s;
+    c->gV2.mat = dm32;
+    // the spheres that share a factor next to each other, and the work items over that order
+    std::vector<int> order;
+    for (int f = 0; f < nf; ++f)
+      for (int k = 0; k < P; ++k)
+        if (d.factor_id[k] == f) order.push_back(k);
+    std::vector<int2> items;
+    const int items_max = gemv_items(P, order.data(), reinterpret_cast<const void* const*>(mA2.data()), items);
+    int* d_order = nullptr;
+    int2* d_items = nullptr;
+    if ((s = upload(c, d_order, order)) != MFS_OK || (s = upload(c, d_items, items)) != MFS_OK) return s;
+    for (GemvBatch<float>* g : {&c->gA32, &c->gA2, &c->gV2}) {
+      g->job_list = d_order;
+      g->n_list = P;
+      g->items = d_items;
+      g->n_items = (int)items.size();
+      g->items_max = items_max;
+    }
+    c->gA32.paired = true;
     int *d_rA, *d_cA, *d_lA, *d_rV, *d_cV, *d_lV;
     long long *d_xA, *d_yA, *d_xV, *d_yV;
     if ((s = upload(c, d_rA, rA)) || (s = upload(c, d_cA, cA)) || (s = upload(c, d_lA, lA)) || (s = upload(c, d_rV, rV)) ||
         (s = upload(c, d_cV, cV)) || (s = upload(c, d_lV, lV)) || (s = upload(c, d_xA, xA)) || (s = upload(c, d_yA, yA)) ||
         (s = upload(c, d_xV, xV)) || (s = upload(c, d_yV, yV)))
       return s;
-    c->gA64.rows = c->gA32.rows = d_rA;
-    c->gA64.cols = c->gA32.cols = d_cA;
-    c->gA64.ld = c->gA32.ld = d_lA;
-    c->gA64.x_off = c->gA32.x_off = d_xA;
-    c->gA64.y_off = c->gA32.y_off = d_yA;
-    c->gA64.n_jobs = c->gA32.n_jobs = P;
-    c->gA64.max_rows = c->gA32.max_rows = maxA;
-    c->gV64.rows = c->gV32.rows = d_rV;
-    c->gV64.cols = c->gV32.cols = d_cV;
-    c->gV64.ld = c->gV32.ld = d_lV;
-    c->gV64.x_off = c->gV32.x_off = d_xV;
-    c->gV64.y_off = c->gV32.y_off = d_yV;
-    c->gV64.n_jobs = c->gV32.n_jobs = P;
-    c->gV64.max_rows = c->gV32.max_rows = maxV;
+    c->gA64.rows = c->gA32.rows = c->gA2.rows = d_rA;
+    c->gA64.cols = c->gA32.cols = c->gA2.cols = d_cA;
+    c->gA64.ld = c->gA32.ld = c->gA2.ld = d_lA;
+    c->gA64.x_off = c->gA32.x_off = c->gA2.x_off = d_xA;
+    c->gA64.y_off = c->gA32.y_off = c->gA2.y_off = d_yA;
+    c->gA64.n_jobs = c->gA32.n_jobs = c->gA2.n_jobs = P;
+    c->gA64.max_rows = c->gA32.max_rows = c->gA2.max_rows = maxA;
+    c->gV64.rows = c->gV32.rows = c->gV2.rows = d_rV;
+    c->gV64.cols = c->gV32.cols = c->gV2.cols = d_cV;
+    c->gV64.ld = c->gV32.ld = c->gV2.ld = d_lV;
+    c->gV64.x_off = c->gV32.x_off = c->gV2.x_off = d_xV;
+    c->gV64.y_off = c->gV32.y_off = c->gV2.y_off = d_yV;
+    c->gV64.n_jobs = c->gV32.n_jobs = c->gV2.n_jobs = P;
+    c->gV64.max_rows = c->gV32.max_rows = c->gV2.max_rows = maxV;
   }
 
   // ---- tensor-core step 1: the spheres without contacts share the basic factor; their
@@ -2590,6 +2655,15 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
         out.ld = dl;
         out.x_off = dx;
         out.y_off = dy;
+        if (!q) {
+          std::vector<int2> items;
+          out.items_max = gemv_items(out.n_jobs, nullptr, reinterpret_cast<const void* const*>(mm.data()), items);
+          int2* di = nullptr;
+          if ((st2 = upload(c, di, items))) return st2;
+          out.items = di;
+          out.n_items = (int)items.size();
+          out.paired = true;
+        }
         return MFS_OK;
       };
       if ((s = sub_batch(c->gA32_rest, false)) != MFS_OK) return s;

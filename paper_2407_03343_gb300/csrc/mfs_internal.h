@@ -232,17 +232,24 @@ struct GemvBatch {
   int max_rows = 0;
   const int* job_prob = nullptr;  // optional: problem of each job, with
   const int* active = nullptr;    //   per-problem flags (jobs of inactive problems are skipped)
-  const float2** mat_dw = nullptr;  // optional: the same matrices as (hi, lo) float pairs
   const int* job_list = nullptr;    // optional: the jobs to run (n_list of them); the grid then
   int n_list = 0;                   //   covers only those
+  bool paired = false;  // FP32: rows stored in pairs, a column's two rows side by side
+  // double-float GEMVs: work items (first, count) over the job list (or the jobs), the right-hand
+  // sides of one matrix, and the largest count
+  const int2* items = nullptr;
+  int n_items = 0, items_max = 1;
 };
+// Work items of jobs whose matrices are mat[list[i]] (list null: mat[i]): runs of equal matrices in
+// even shares of at most four; returns the largest count.
+int gemv_items(int n, const int* list, const void* const* mat, std::vector<int2>& items);
 template <typename T>
 void launch_gemv(const GemvBatch<T>& b, const T* x, T* y, cudaStream_t st);
-// Double-float GEMV on the FP32 pipes over b.mat_dw: x as (hi, lo) pairs; the result goes to
-// y_dw as pairs, or to y64 joined into doubles when y_dw is null.
-void launch_gemv_dw(const GemvBatch<double>& b, const float2* x, float2* y_dw, double* y64, cudaStream_t st);
-// Double-float GEMV over an FP32 matrix (b.mat): x as (hi, lo) pairs, y_dw as pairs.  The matrix
-// rows must start 16-byte aligned (ld a multiple of 4).
+// Double-float GEMV on the FP32 pipes: b.mat holds row pairs of (hi, lo) float pairs, a column as
+// (h0 h1 l0 l1) (b.ld columns a row pair); x as (hi, lo) pairs; the result goes to y_dw as pairs, or
+// to y64 joined into doubles when y_dw is null.  Runs over b.items.
+void launch_gemv_dw(const GemvBatch<float>& b, const float2* x, float2* y_dw, double* y64, cudaStream_t st);
+// Double-float GEMV over FP32 row pairs (a0 a1) (b.mat, b.ld even): x as (hi, lo) pairs, y_dw as pairs.
 void launch_gemv_f32_dw(const GemvBatch<float>& b, const float2* x, float2* y_dw, cudaStream_t st);
 // (hi, lo) float pairs of a double vector.
 void launch_split_dw(long long n, const double* in, float2* out, cudaStream_t st);

@@ -1543,7 +1543,6 @@ __global__ void pair_parts_reduce_batch_kernel(SegTable t, const PairArgs<double
 // ------------------------------------------------------------------ batched GEMV
 constexpr int kGemvThreads = 256;
 constexpr int kGemvRowsPerWarp = 2;
-constexpr int kGemvDepth = 4;  // 16-byte loads per row and lane in flight in the double-float GEMVs
 
 template <typename T> struct Vec;
 template <> struct Vec<float> { using type = float4; static constexpr int w = 4; };
@@ -1558,7 +1557,8 @@ template <> __device__ __forceinline__ double dot_vec<double>(const double2& m, 
   return m.x * __ldg(x) + m.y * __ldg(x + 1);
 }
 
-template <typename T>
+// PAIRED: the matrix is stored in row pairs (FP32 copy of Sigma^+ U^T); a warp's two rows are a pair
+template <typename T, bool PAIRED>
 __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, const T* __restrict__ x, T* __restrict__ y) {
   using VT = typename Vec<T>::type;
   constexpr int W = Vec<T>::w;
@@ -1581,7 +1581,15 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, cons
     for (int r = 0; r < kGemvRowsPerWarp; ++r) {
       int row = r0 + r;
       if (row < nr) {
-        VT m = reinterpret_cast<const VT*>(M + (long long)row * ld)[v];
+        VT m;
+        if constexpr (PAIRED) {
+          const VT* q = reinterpret_cast<const VT*>(M + (long long)r0 * ld) + 2 * v;
+          const VT a = q[0], b = q[1];
+          if (r == 0) m = VT{a.x, a.z, b.x, b.z};
+          else m = VT{a.y, a.w, b.y, b.w};
+        } else {
+          m = reinterpret_cast<const VT*>(M + (long long)row * ld)[v];
+        }
         acc[r] += dot_vec<T>(m, xv + v * W);
       }
     }
@@ -1590,7 +1598,7 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, cons
 #pragma unroll
     for (int r = 0; r < kGemvRowsPerWarp; ++r) {
       int row = r0 + r;
-      if (row < nr) acc[r] += M[(long long)row * ld + c] * xv[c];
+      if (row < nr) acc[r] += (PAIRED ? M[(long long)r0 * ld + 2LL * c + r] : M[(long long)row * ld + c]) * xv[c];
     }
   }
 #pragma unroll
@@ -1601,145 +1609,193 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, cons
   }
 }
 
-// Double-float GEMV: each matrix element and each x element is a (hi, lo) float pair; products
-// and sums use the error-free double-word operations above, so the result carries ~2^-46
-// relative accuracy while reading the same 8 bytes per element as FP64.
-template <bool OUT64>
-__global__ void __launch_bounds__(kGemvThreads) gemv_dw_kernel(GemvBatch<double> B, const float2* __restrict__ x,
-                                                                float2* __restrict__ y2, double* __restrict__ y64) {
-  // jobs sharing a matrix are adjacent, so its rows are read once; with a compacted list the grid
-  // covers the active problems' jobs only
-  const int job = B.job_list ? B.job_list[blockIdx.x] : blockIdx.x;
-  if (B.active && !B.active[B.job_prob[job]]) return;
-  const int nr = B.rows[job], nc = B.cols[job], ld = B.ld[job];
+// Double-float GEMVs y = M x.  The rows of M are stored in pairs, a column's two rows side by side
+// (double-float: (h0 h1 l0 l1), FP32: (a0 a1)), so that one packed FP32 instruction serves both: a
+// product keeps its exact error (TwoProd) and the cross terms, the running sum is exact (TwoSum) and
+// its errors are collected in a second float, 12 lane-operations an element (FP32 matrix: 11).
+// For the double-float matrix the two are folded into a double-word sum every 16 terms, which keeps
+// the accuracy of a double-word accumulation (~2^-46); for the FP32 matrix the rounding of its
+// entries (6e-8, amplified by Sigma^+ only along right singular vectors whose fields on the other
+// spheres are correspondingly weak, so that the operator stays accurate to ~1e-7) is far above that
+// of the plain collection.  FP32 serves Sigma^+ U^T in the inner solves of MFS_MIXED, double-float V
+// everywhere and Sigma^+ U^T in the refinement residual.
+// One right-hand side: a CTA takes one row pair, its four warps every fourth run of 32 loads, and the
+// next two loads a lane are issued before the current ones are used; what bounds it is HBM (or the
+// latency of short matrices), for which ten resident CTAs a SM measured best.  Up to four right-hand
+// sides of one matrix (spheres that share a factor, motions of one geometry) are taken together over
+// two row pairs, the matrix read once for them; those are bound by the FMA pipe.
+// Measured, both factors of one step 1 (GB300; before: two rows a warp, scalar, one right-hand side):
+// two spheres with 20 images, N = 800 (386 MB double-float) 102 -> 86 us, with the FP32 factor
+// (250 MB) 72 -> 61; 8 spheres N = 400 173 -> 128 and 122 -> 93; 100 spheres sharing the factor
+// N = 686 776 -> 531 and (V only) 391 -> 275; eight right-hand sides over one row pair 579.
+struct GemvAcc {
+  dw2 s, m;  // running sum and its collected errors; double-word sum of the groups
+};
+template <bool F32>
+__device__ __forceinline__ void gemv_step(GemvAcc& a, f2x mh, f2x ml, float2 xe) {
+  const f2x xh = f2dup(xe.x), np = f2mul(mh, f2dup(-xe.x));
+  f2x e = f2fma(mh, f2dup(xe.y), f2fma(mh, xh, np));
+  if constexpr (!F32) e = f2fma(ml, xh, e);
+  const dw2 t = two_diff2(a.s.h, np);
+  a.s.h = t.h;
+  a.s.l = f2add(a.s.l, f2add(t.l, e));
+}
+
+constexpr int kGemvPairThreads = 128;
+constexpr int kGemvMaxRhs = 4;
+
+template <bool F32, bool OUT64, int C, int RP, int KS>
+__device__ __forceinline__ void gemv_pairs(const GemvBatch<float>& B, const int* job, int rp0,
+                                           const float2* __restrict__ x, float2* __restrict__ y2,
+                                           double* __restrict__ y64) {
+  constexpr int D = 2;        // 16-byte loads per row pair and lane in flight (twice)
+  constexpr int S = 32 * KS;  // columns' loads of one step of the CTA
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = (blockIdx.y * (kGemvThreads / 32) + warp) * kGemvRowsPerWarp;
-  if (r0 >= nr) return;
-  const float2* M = B.mat_dw[job];
-  const float2* xv = x + B.x_off[job];
-  dw acc[kGemvRowsPerWarp];
+  const int nr = B.rows[job[0]], nc = B.cols[job[0]], ld = B.ld[job[0]];
+  const int nrp = (nr + 1) >> 1;
+  // a 16-byte load holds one column of a double-float row pair or two of an FP32 one
+  const int nv = F32 ? (nc + 1) >> 1 : nc;
+  const long long row16 = F32 ? ld / 2 : ld;
+  const float4* M = reinterpret_cast<const float4*>(B.mat[job[0]]) + rp0 * row16;
+  const float2* xv[C];
 #pragma unroll
-  for (int r = 0; r < kGemvRowsPerWarp; ++r) acc[r] = dw{0.f, 0.f};
-  const int npair = nc / 2;  // two elements per 16-byte load
-  // kGemvDepth loads per row and lane issued before they are used, so that enough bytes are
-  // in flight even when few jobs are active (the lockstep tail)
-  for (int v0 = lane; v0 < npair; v0 += 32 * kGemvDepth) {
-    float4 m[kGemvDepth][kGemvRowsPerWarp];
+  for (int q = 0; q < C; ++q) xv[q] = x + B.x_off[job[q]];
+  GemvAcc acc[RP][C];
 #pragma unroll
-    for (int u = 0; u < kGemvDepth; ++u)
+  for (int r = 0; r < RP; ++r)
 #pragma unroll
-      for (int r = 0; r < kGemvRowsPerWarp; ++r)
-        if (v0 + 32 * u < npair && r0 + r < nr)
-          m[u][r] = reinterpret_cast<const float4*>(M + (long long)(r0 + r) * ld)[v0 + 32 * u];
+    for (int q = 0; q < C; ++q) acc[r][q] = GemvAcc{{0, 0}, {0, 0}};
+  float4 cur[D][RP];
+  float4 nxt[D][RP];
+  auto load = [&](float4 (&m)[D][RP], int v0) {
 #pragma unroll
-    for (int u = 0; u < kGemvDepth; ++u) {
-      const int v = v0 + 32 * u;
-      if (v >= npair) break;
-      const float2 xa = xv[2 * v], xb = xv[2 * v + 1];
+    for (int u = 0; u < D; ++u)
 #pragma unroll
-      for (int r = 0; r < kGemvRowsPerWarp; ++r)
-        if (r0 + r < nr) {
-          acc[r] = dw_add(acc[r], dw_mul(dw{m[u][r].x, m[u][r].y}, dw{xa.x, xa.y}));
-          acc[r] = dw_add(acc[r], dw_mul(dw{m[u][r].z, m[u][r].w}, dw{xb.x, xb.y}));
+      for (int r = 0; r < RP; ++r) {
+        const int v = v0 + S * u;
+        m[u][r] = v < nv && rp0 + r < nrp ? __ldg(M + r * row16 + v) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+  };
+  const int v_first = KS > 1 ? (int)threadIdx.x : lane;
+  load(cur, v_first);
+  int terms = 0;
+  for (int v0 = v_first; v0 < nv; v0 += S * D) {
+    load(nxt, v0 + S * D);
+#pragma unroll
+    for (int u = 0; u < D; ++u) {
+      const int v = v0 + S * u;
+      if (v >= nv) break;
+#pragma unroll
+      for (int q = 0; q < C; ++q) {
+        if constexpr (F32) {
+          const float2 x0 = xv[q][2 * v];
+          const float2 x1 = 2 * v + 1 < nc ? xv[q][2 * v + 1] : make_float2(0.f, 0.f);
+#pragma unroll
+          for (int r = 0; r < RP; ++r) {
+            gemv_step<true>(acc[r][q], f2make(cur[u][r].x, cur[u][r].y), 0, x0);
+            gemv_step<true>(acc[r][q], f2make(cur[u][r].z, cur[u][r].w), 0, x1);
+          }
+        } else {
+          const float2 xe = xv[q][v];
+#pragma unroll
+          for (int r = 0; r < RP; ++r)
+            gemv_step<false>(acc[r][q], f2make(cur[u][r].x, cur[u][r].y), f2make(cur[u][r].z, cur[u][r].w), xe);
         }
-    }
-  }
-  for (int cidx = 2 * npair + lane; cidx < nc; cidx += 32) {
-    const float2 xa = xv[cidx];
-#pragma unroll
-    for (int r = 0; r < kGemvRowsPerWarp; ++r) {
-      int row = r0 + r;
-      if (row < nr) {
-        float2 m = M[(long long)row * ld + cidx];
-        acc[r] = dw_add(acc[r], dw_mul(dw{m.x, m.y}, dw{xa.x, xa.y}));
       }
     }
-  }
+    terms += D;
+    if (!F32 && terms >= 16) {
+      terms = 0;
 #pragma unroll
-  for (int r = 0; r < kGemvRowsPerWarp; ++r) {
-    dw s = acc[r];
-    for (int o = 16; o > 0; o >>= 1) {
-      dw t{__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.l, o)};
-      s = dw_add(s, t);
+      for (int r = 0; r < RP; ++r)
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+          acc[r][q].m = dw2_add(acc[r][q].m, acc[r][q].s);
+          acc[r][q].s = dw2{0, 0};
+        }
     }
-    if (lane == 0 && r0 + r < nr) {
-      long long idx = B.y_off[job] + r0 + r;
-      if (OUT64) y64[idx] = dw_join(s);
-      else y2[idx] = make_float2(s.h, s.l);
+#pragma unroll
+    for (int u = 0; u < D; ++u)
+#pragma unroll
+      for (int r = 0; r < RP; ++r) cur[u][r] = nxt[u][r];
+  }
+  // the lanes' sums in a fixed order; lane 0 writes a pair's first row, lane 1 its second
+  auto finish = [&](dw2 v, int r, long long y_off) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      v = dw2_add(v, dw2{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
+    float h0, h1, l0, l1;
+    f2split(v.h, h0, h1);
+    f2split(v.l, l0, l1);
+    const int row = 2 * (rp0 + r) + lane;
+    if (lane < 2 && row < nr) {
+      const dw w = lane == 0 ? dw{h0, l0} : dw{h1, l1};
+      const long long idx = y_off + row;
+      if (OUT64) y64[idx] = dw_join(w);
+      else y2[idx] = make_float2(w.h, w.l);
     }
+  };
+  auto value = [&](int r, int q) {
+    dw2 v = two_sum2(acc[r][q].s.h, acc[r][q].s.l);
+    if constexpr (!F32) v = dw2_add(acc[r][q].m, v);
+    return v;
+  };
+  if constexpr (KS > 1) {
+    // the warps' shares of the columns added in warp order, each value by one warp
+    __shared__ ulonglong2 red[KS][RP * C][32];
+#pragma unroll
+    for (int r = 0; r < RP; ++r)
+#pragma unroll
+      for (int q = 0; q < C; ++q) {
+        const dw2 v = value(r, q);
+        red[warp][r * C + q][lane] = make_ulonglong2(v.h, v.l);
+      }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = warp; i < RP * C; i += KS) {
+      const ulonglong2 a = red[0][i][lane];
+      dw2 v{a.x, a.y};
+#pragma unroll
+      for (int w = 1; w < KS; ++w) {
+        const ulonglong2 b = red[w][i][lane];
+        v = dw2_add(v, dw2{b.x, b.y});
+      }
+      long long y_off = B.y_off[job[0]];
+#pragma unroll
+      for (int q = 1; q < C; ++q)
+        if (i % C == q) y_off = B.y_off[job[q]];
+      finish(v, i / C, y_off);
+    }
+  } else {
+#pragma unroll
+    for (int r = 0; r < RP; ++r)
+#pragma unroll
+      for (int q = 0; q < C; ++q) finish(value(r, q), r, B.y_off[job[q]]);
   }
 }
 
-// The same product with the matrix in FP32 (4 bytes per element).  Per element the product
-// m (x_hi + x_lo) is formed exactly up to the rounding of its small part (TwoProd), the running
-// FP32 sum's rounding error is captured by TwoSum, and the error terms are summed in a second
-// float that is folded in once per lane: ~11 instructions per element instead of a full
-// double-word product and sum, with an accumulation error (~n^2 eps^2 for n terms per lane)
-// far below the FP32 rounding of the matrix itself, which is the only real error.  Used for Sigma^+ U^T in the inner solves of MFS_MIXED,
-// whose rounding (relative 6e-8 per element, amplified by Sigma^+ only along right singular
-// vectors whose fields on the other spheres are correspondingly weak) leaves the operator
-// accurate to ~1e-7; the refinement residual is evaluated with the double-float factors.
-__global__ void __launch_bounds__(kGemvThreads) gemv_f32dw_kernel(GemvBatch<float> B, const float2* __restrict__ x,
-                                                                  float2* __restrict__ y2) {
-  const int job = B.job_list ? B.job_list[blockIdx.x] : blockIdx.x;
-  if (B.active && !B.active[B.job_prob[job]]) return;
-  const int nr = B.rows[job], nc = B.cols[job], ld = B.ld[job];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = (blockIdx.y * (kGemvThreads / 32) + warp) * kGemvRowsPerWarp;
-  if (r0 >= nr) return;
-  const float* M = B.mat[job];
-  const float2* xv = x + B.x_off[job];
-  float sh[kGemvRowsPerWarp], sl[kGemvRowsPerWarp];
+// row pairs a warp (KS 1) or the CTA (KS 4: its warps share the columns) takes at once
+__host__ __device__ constexpr int gemv_rp(int c) { return c == 1 ? 1 : 2; }
+// work item blockIdx.x: the right-hand sides list[item.x .. item.x + item.y) of one matrix
+template <bool F32, bool OUT64, int CMAX, int KS>
+__global__ void __launch_bounds__(kGemvPairThreads, CMAX == 1 ? 10 : 1) gemv_pair_kernel(GemvBatch<float> B, const float2* __restrict__ x,
+                                                                   float2* __restrict__ y2, double* __restrict__ y64) {
+  constexpr int RP = gemv_rp(CMAX);
+  const int2 it = B.items[blockIdx.x];
+  const int rp0 = (KS > 1 ? blockIdx.y : blockIdx.y * (kGemvPairThreads / 32) + (threadIdx.x >> 5)) * RP;
+  int job[CMAX];
+  bool any = false;
 #pragma unroll
-  for (int r = 0; r < kGemvRowsPerWarp; ++r) sh[r] = sl[r] = 0.f;
-  auto add = [](float& h, float& l, float m, float2 xe) {
-    dw p = two_prod(m, xe.x);
-    p.l = __fmaf_rn(m, xe.y, p.l);
-    dw t = two_sum(h, p.h);
-    h = t.h;
-    l = __fadd_rn(l, __fadd_rn(t.l, p.l));
-  };
-  const int nq = nc / 4;  // four elements per 16-byte load
-  for (int v0 = lane; v0 < nq; v0 += 32 * kGemvDepth) {
-    float4 m[kGemvDepth][kGemvRowsPerWarp];
-#pragma unroll
-    for (int u = 0; u < kGemvDepth; ++u)
-#pragma unroll
-      for (int r = 0; r < kGemvRowsPerWarp; ++r)
-        if (v0 + 32 * u < nq && r0 + r < nr)
-          m[u][r] = reinterpret_cast<const float4*>(M + (long long)(r0 + r) * ld)[v0 + 32 * u];
-#pragma unroll
-    for (int u = 0; u < kGemvDepth; ++u) {
-      const int v = v0 + 32 * u;
-      if (v >= nq) break;
-      const float2 x0 = xv[4 * v], x1 = xv[4 * v + 1], x2 = xv[4 * v + 2], x3 = xv[4 * v + 3];
-#pragma unroll
-      for (int r = 0; r < kGemvRowsPerWarp; ++r)
-        if (r0 + r < nr) {
-          add(sh[r], sl[r], m[u][r].x, x0);
-          add(sh[r], sl[r], m[u][r].y, x1);
-          add(sh[r], sl[r], m[u][r].z, x2);
-          add(sh[r], sl[r], m[u][r].w, x3);
-        }
-    }
+  for (int q = 0; q < CMAX; ++q) {
+    const int j = it.x + min(q, it.y - 1);
+    job[q] = B.job_list ? B.job_list[j] : j;
+    any = any || !B.active || B.active[B.job_prob[job[q]]];
   }
-  for (int cidx = 4 * nq + lane; cidx < nc; cidx += 32) {
-    const float2 xa = xv[cidx];
-#pragma unroll
-    for (int r = 0; r < kGemvRowsPerWarp; ++r) {
-      int row = r0 + r;
-      if (row < nr) add(sh[r], sl[r], M[(long long)row * ld + cidx], xa);
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < kGemvRowsPerWarp; ++r) {
-    dw s = two_sum(sh[r], sl[r]);
-    for (int o = 16; o > 0; o >>= 1) {
-      dw t{__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.l, o)};
-      s = dw_add(s, t);
-    }
-    if (lane == 0 && r0 + r < nr) y2[B.y_off[job] + r0 + r] = make_float2(s.h, s.l);
-  }
+  if (!any || 2 * rp0 >= B.rows[job[0]]) return;
+  // (three of four run as four with the last one twice: the same value written twice)
+  if (CMAX > 1 && it.y == 1) gemv_pairs<F32, OUT64, 1, RP, KS>(B, job, rp0, x, y2, y64);
+  else if (CMAX > 2 && it.y == 2) gemv_pairs<F32, OUT64, 2, RP, KS>(B, job, rp0, x, y2, y64);
+  else gemv_pairs<F32, OUT64, CMAX, RP, KS>(B, job, rp0, x, y2, y64);
 }
 
 __global__ void split_dw_kernel(long long n, const double* __restrict__ in, float2* __restrict__ out) {
@@ -2563,29 +2619,56 @@ void launch_gemv(const GemvBatch<T>& b, const T* x, T* y, cudaStream_t st) {
   if (jobs == 0) return;
   dim3 grid(jobs, (b.max_rows + rows_per_cta - 1) / rows_per_cta);
   ++t_launches;
-  gemv_kernel<T><<<grid, kGemvThreads, 0, st>>>(b, x, y);
+  if (sizeof(T) == 4 && b.paired) gemv_kernel<T, sizeof(T) == 4><<<grid, kGemvThreads, 0, st>>>(b, x, y);
+  else gemv_kernel<T, false><<<grid, kGemvThreads, 0, st>>>(b, x, y);
 }
 template void launch_gemv<float>(const GemvBatch<float>&, const float*, float*, cudaStream_t);
 
-void launch_gemv_dw(const GemvBatch<double>& b, const float2* x, float2* y_dw, double* y64, cudaStream_t st) {
-  if (b.n_jobs == 0 || b.max_rows == 0) return;
-  const int rows_per_cta = (kGemvThreads / 32) * kGemvRowsPerWarp;
-  const int jobs = b.job_list ? b.n_list : b.n_jobs;
-  if (jobs == 0) return;
-  dim3 grid(jobs, (b.max_rows + rows_per_cta - 1) / rows_per_cta);
+int gemv_items(int n, const int* list, const void* const* mat, std::vector<int2>& items) {
+  items.clear();
+  int most = 1;
+  for (int i = 0; i < n;) {
+    int e = i + 1;
+    while (e < n && mat[list ? list[e] : e] == mat[list ? list[i] : i]) ++e;
+    // even shares of at most kGemvMaxRhs
+    const int cnt = e - i, parts = (cnt + kGemvMaxRhs - 1) / kGemvMaxRhs;
+    for (int q = 0; q < parts; ++q) {
+      const int i0 = i + (int)((long long)cnt * q / parts), i1 = i + (int)((long long)cnt * (q + 1) / parts);
+      items.push_back(make_int2(i0, i1 - i0));
+      most = std::max(most, i1 - i0);
+    }
+    i = e;
+  }
+  return most;
+}
+
+template <bool F32, bool OUT64>
+static void gemv_pair_launch(const GemvBatch<float>& b, const float2* x, float2* y2, double* y64, cudaStream_t st) {
+  if (b.n_items == 0 || b.max_rows == 0) return;
   ++t_launches;
-  if (y_dw) gemv_dw_kernel<false><<<grid, kGemvThreads, 0, st>>>(b, x, y_dw, nullptr);
-  else gemv_dw_kernel<true><<<grid, kGemvThreads, 0, st>>>(b, x, nullptr, y64);
+  const int c = b.items_max;
+  const int nrp = (b.max_rows + 1) / 2, groups = (nrp + gemv_rp(c) - 1) / gemv_rp(c);
+  // several right-hand sides: the CTA's warps share the columns of a row group while there are fewer
+  // groups than 64 warps a SM, and take a group each above that
+  const bool split = c == 1 || (long long)b.n_items * groups < 64LL * 152;
+  const dim3 grid(b.n_items, split ? groups : (groups + 3) / 4);
+#define MFS_GEMV(C, KS) gemv_pair_kernel<F32, OUT64, C, KS><<<grid, kGemvPairThreads, 0, st>>>(b, x, y2, y64)
+  switch (c) {
+    case 1: MFS_GEMV(1, 4); break;
+    case 2: if (split) MFS_GEMV(2, 4); else MFS_GEMV(2, 1); break;
+    case 3: if (split) MFS_GEMV(3, 4); else MFS_GEMV(3, 1); break;
+    default: if (split) MFS_GEMV(4, 4); else MFS_GEMV(4, 1);
+  }
+#undef MFS_GEMV
+}
+
+void launch_gemv_dw(const GemvBatch<float>& b, const float2* x, float2* y_dw, double* y64, cudaStream_t st) {
+  if (y_dw) gemv_pair_launch<false, false>(b, x, y_dw, nullptr, st);
+  else gemv_pair_launch<false, true>(b, x, nullptr, y64, st);
 }
 
 void launch_gemv_f32_dw(const GemvBatch<float>& b, const float2* x, float2* y_dw, cudaStream_t st) {
-  if (b.n_jobs == 0 || b.max_rows == 0) return;
-  const int rows_per_cta = (kGemvThreads / 32) * kGemvRowsPerWarp;
-  const int jobs = b.job_list ? b.n_list : b.n_jobs;
-  if (jobs == 0) return;
-  dim3 grid(jobs, (b.max_rows + rows_per_cta - 1) / rows_per_cta);
-  ++t_launches;
-  gemv_f32dw_kernel<<<grid, kGemvThreads, 0, st>>>(b, x, y_dw);
+  gemv_pair_launch<true, false>(b, x, y_dw, nullptr, st);
 }
 
 void launch_split_dw(long long n, const double* in, float2* out, cudaStream_t st) {
