@@ -1609,6 +1609,63 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, cons
   }
 }
 
+// Native FP64 y = M x, one right-hand side an item: a CTA takes kGemv64Rows rows, its four warps every
+// fourth run of 32 columns, and the next kGemv64Depth loads a row and lane are issued before the
+// current ones are used.  Bound by the FP64 pipe once enough rows are there (two lanes per SM and
+// clock, 16 bytes of matrix), by load latency below that, which is what the split of the columns and
+// the loads in flight are for.  Both factors of one step 1, before (two rows a warp, one load each in
+// flight) and now: 100 spheres N = 686 2710 -> 1775 us (the DFMA rate allows 1757), 8 spheres N = 400
+// 389 -> 188, two spheres N = 800 213 -> 117, N = 300 43 -> 26.
+constexpr int kGemv64Rows = 2, kGemv64Depth = 4, kGemv64Warps = 4;
+__global__ void __launch_bounds__(32 * kGemv64Warps) gemv64_kernel(GemvBatch<double> B, const double* __restrict__ x,
+                                                                  double* __restrict__ y) {
+  constexpr int R = kGemv64Rows, D = kGemv64Depth, S = 32 * kGemv64Warps;
+  __shared__ double red[kGemv64Warps][R][32];
+  const int job = B.job_list ? B.job_list[blockIdx.x] : blockIdx.x;
+  if (B.active && !B.active[B.job_prob[job]]) return;
+  const int nr = B.rows[job], nc = B.cols[job];
+  const int r0 = blockIdx.y * R;
+  if (r0 >= nr) return;
+  const long long ld = B.ld[job];
+  const double* M = B.mat[job] + r0 * ld;
+  const double* xv = x + B.x_off[job];
+  double acc[R], cur[D][R], nxt[D][R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) acc[r] = 0.0;
+  auto load = [&](double (&m)[D][R], int c0) {
+#pragma unroll
+    for (int u = 0; u < D; ++u)
+#pragma unroll
+      for (int r = 0; r < R; ++r) m[u][r] = c0 + S * u < nc && r0 + r < nr ? __ldg(M + r * ld + c0 + S * u) : 0.0;
+  };
+  load(cur, threadIdx.x);
+  for (int c0 = threadIdx.x; c0 < nc; c0 += S * D) {
+    load(nxt, c0 + S * D);
+#pragma unroll
+    for (int u = 0; u < D; ++u) {
+      if (c0 + S * u >= nc) break;
+      const double xe = xv[c0 + S * u];
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[r] = fma(cur[u][r], xe, acc[r]);
+    }
+#pragma unroll
+    for (int u = 0; u < D; ++u)
+#pragma unroll
+      for (int r = 0; r < R; ++r) cur[u][r] = nxt[u][r];
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int r = 0; r < R; ++r) red[warp][r][lane] = acc[r];
+  __syncthreads();
+  for (int r = warp; r < R; r += kGemv64Warps) {
+    double s = red[0][r][lane];
+#pragma unroll
+    for (int w = 1; w < kGemv64Warps; ++w) s += red[w][r][lane];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0 && r0 + r < nr) y[B.y_off[job] + r0 + r] = s;
+  }
+}
+
 // Double-float GEMVs y = M x.  The rows of M are stored in pairs, a column's two rows side by side
 // (double-float: (h0 h1 l0 l1), FP32: (a0 a1)), so that one packed FP32 instruction serves both: a
 // product keeps its exact error (TwoProd) and the cross terms, the running sum is exact (TwoSum) and
@@ -2619,7 +2676,9 @@ void launch_gemv(const GemvBatch<T>& b, const T* x, T* y, cudaStream_t st) {
   if (jobs == 0) return;
   dim3 grid(jobs, (b.max_rows + rows_per_cta - 1) / rows_per_cta);
   ++t_launches;
-  if (sizeof(T) == 4 && b.paired) gemv_kernel<T, sizeof(T) == 4><<<grid, kGemvThreads, 0, st>>>(b, x, y);
+  if constexpr (sizeof(T) == 8)
+    gemv64_kernel<<<dim3(jobs, (b.max_rows + kGemv64Rows - 1) / kGemv64Rows), 32 * kGemv64Warps, 0, st>>>(b, x, y);
+  else if (b.paired) gemv_kernel<T, true><<<grid, kGemvThreads, 0, st>>>(b, x, y);
   else gemv_kernel<T, false><<<grid, kGemvThreads, 0, st>>>(b, x, y);
 }
 template void launch_gemv<float>(const GemvBatch<float>&, const float*, float*, cudaStream_t);
