@@ -192,6 +192,7 @@ struct mfs_ctx {
   int n_sys = 0;          // GMRES system size: n, or n + 6P for the bordered mobility system
   double* d_border = nullptr;  // mobility: scaled prescribed (F_k, T_k), 6 per sphere
   double* d_pparts = nullptr;  // partial sums of the source-split pair kernel, kPairMaxParts * n
+  unsigned* d_pcount = nullptr;  // arrivals of a tile's parts (zeros between launches)
   double* d_zero = nullptr;    // 3P zeros
   // measurement
   bool prof = false;
@@ -253,7 +254,9 @@ struct mfs_ctx {
   size_t basis_bytes = 0;
   double* d_partial = nullptr;
   double* d_h = nullptr;
+  double* h_pin = nullptr;     // pinned staging of one Arnoldi step's coefficients
   int nblk = 1;
+  SegTable seg[2];             // vector chunks of the resistance and the mobility system (FP64 GMRES)
 
   mfs_status fail(mfs_status s, const std::string& m) {
     err = m;
@@ -415,11 +418,11 @@ void collect_events(mfs_ctx* c) {
 // step 1: lambda_hat = B^+ mu (two factors in turn, eq. transform); in the mixed mode the FP64
 // factors are applied in double-float arithmetic from their (hi, lo) float copies
 template <typename T>
-void precond(mfs_ctx* c, const T* mu, T* lam_hat) {
+void precond(mfs_ctx* c, const T* mu, T* lam_hat, bool x2_ready = false) {
   timed(c, c->ev_gemv, [&] {
     if constexpr (sizeof(T) == 8) {
       if (c->dw_pairs) {
-        launch_split_dw(c->n, mu, c->d_x2, c->stream);
+        if (!x2_ready) launch_split_dw(c->n, mu, c->d_x2, c->stream);
         if (c->dw_fast_a && c->tc_ncols > 0) {
           // the spheres sharing the basic factor as one product on the tensor cores
           launch_gemv_f32_dw(c->gA32_rest, c->d_x2, c->d_t2, c->stream);
@@ -452,8 +455,8 @@ void pairs_step(mfs_ctx* c, const T* lam_hat, const T* mu, T* out) {
       // near spheres directly in double-float, the far ones through their equivalent sources,
       // whose strengths q = Q mu are formed from this apply's mu
       timed(c, c->ev_pair, [&] {
-        launch_pairs_dw_near(c->tg, c->src, c->ff, lam_hat, mu, out, c->hd.prm.visc, c->d_pparts, kPairMaxParts,
-                             c->stream, c->shape_near);
+        launch_pairs_dw_near(c->tg, c->src, c->ff, lam_hat, mu, out, c->hd.prm.visc, c->d_pparts, c->d_pcount,
+                             kPairMaxParts, c->stream, c->shape_near);
       });
       timed(c, c->ev_far, [&] {
         launch_convert<double, float>(c->n, mu, 1.0, c->d_mu32, c->stream);
@@ -488,8 +491,8 @@ void pairs_step(mfs_ctx* c, const T* lam_hat, const T* mu, T* out) {
   timed(c, c->ev_pair, [&] {
     if constexpr (sizeof(T) == 8) {
       if (c->dw_pairs) {
-        launch_pairs_dw(c->tg, c->src, lam_hat, mu, out, c->hd.prm.visc, c->d_pparts, kPairMaxParts, c->stream,
-                        c->shape_all);
+        launch_pairs_dw(c->tg, c->src, lam_hat, mu, out, c->hd.prm.visc, c->d_pparts, c->d_pcount, kPairMaxParts,
+                        c->stream, c->shape_all);
         return;
       }
     }
@@ -513,10 +516,10 @@ void pairs_step(mfs_ctx* c, const T* lam_hat, const T* mu, T* out) {
   if (c->prof) c->ev_pair_kind.push_back(kind);
 }
 
-// out = G_hat mu
+// out = G_hat mu (x2_ready: d_x2 already holds mu's double-float split)
 template <typename T>
-void apply_op(mfs_ctx* c, const T* mu, T* out) {
-  precond<T>(c, mu, Ops<T>::lh(c));
+void apply_op(mfs_ctx* c, const T* mu, T* out, bool x2_ready = false) {
+  precond<T>(c, mu, Ops<T>::lh(c), x2_ready);
   pairs_step<T>(c, Ops<T>::lh(c), mu, out);
 }
 
@@ -525,8 +528,8 @@ void apply_op(mfs_ctx* c, const T* mu, T* out) {
 // (forces/torques of lambda_hat = B^+ mu by the Sec. 2.3 remark, s_F = 1/(6 pi mu a),
 // s_T = 1/(8 pi mu a^3)).
 template <typename T>
-void sys_apply(mfs_ctx* c, const T* in, T* out) {
-  apply_op<T>(c, in, out);
+void sys_apply(mfs_ctx* c, const T* in, T* out, bool x2_ready = false) {
+  apply_op<T>(c, in, out, x2_ready);
   if constexpr (sizeof(T) == 8) {
     if (c->mode == 1) {
       const double a = c->a, mu = c->hd.prm.visc;
@@ -555,8 +558,12 @@ mfs_status ensure_krylov(mfs_ctx* c, int restart) {
 // dot products of w with V[0..nvec) (FP64 partials) -> host h
 template <typename T>
 mfs_status dots(mfs_ctx* c, int nvec, const T* V, const T* w, double* h_dev) {
-  launch_multidot<T>(c->n_sys, nvec, V, c->n_sys, w, c->d_partial, c->nblk, c->stream);
-  launch_reduce_partials(nvec, c->nblk, c->d_partial, h_dev, c->stream);
+  if constexpr (sizeof(T) == 8) {
+    launch_seg_dots(c->seg[c->mode], nvec, V, c->n_sys, w, c->d_partial, h_dev, c->stream);
+  } else {
+    launch_multidot<T>(c->n_sys, nvec, V, c->n_sys, w, c->d_partial, c->nblk, c->stream);
+    launch_reduce_partials(nvec, c->nblk, c->d_partial, h_dev, c->stream);
+  }
   CHECK_LAUNCH(c);
   return MFS_OK;
 }
@@ -572,7 +579,8 @@ mfs_status gmres(mfs_ctx* c, const T* b, T* x, double tol, int restart, int max_
   const int n = c->n_sys;
   const int ldh = restart + 1;
   T* V = static_cast<T*>(c->d_basis);
-  std::vector<double> H((size_t)ldh * restart), cs(restart), sn(restart), g(ldh), hb(2 * ldh + 1), y(restart);
+  std::vector<double> H((size_t)ldh * restart), cs(restart), sn(restart), g(ldh), y(restart);
+  double* hb = c->h_pin;
   double* h1 = c->d_h;
   double* h2 = c->d_h + ldh;
   double* hn = c->d_h + 2 * ldh;
@@ -615,24 +623,35 @@ mfs_status gmres(mfs_ctx* c, const T* b, T* x, double tol, int restart, int max_
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
     int j_used = 0;
-    bool done = false;
+    bool done = false, x2_ready = false;
     for (int j = 0; j < restart; ++j) {
       T* w = V + (size_t)(j + 1) * n;
-      sys_apply<T>(c, V + (size_t)j * n, w);
+      sys_apply<T>(c, V + (size_t)j * n, w, x2_ready);
       CHECK_LAUNCH(c);
       if ((s = dots<T>(c, j + 1, V, w, h1)) != MFS_OK) return s;
-      launch_update<T>(n, j + 1, V, n, h1, -1.0, w, c->stream);
-      if ((s = dots<T>(c, j + 1, V, w, h2)) != MFS_OK) return s;
-      launch_update<T>(n, j + 1, V, n, h2, -1.0, w, c->stream);
-      if ((s = dots<T>(c, 1, w, w, hn)) != MFS_OK) return s;
-      CUDA_TRY(c, cudaMemcpyAsync(hb.data(), c->d_h, sizeof(double) * (2 * ldh + 1), cudaMemcpyDeviceToHost, c->stream));
+      if constexpr (sizeof(T) == 8) {
+        // the norm comes with the second update, and the new basis vector is scaled (and split for
+        // the next double-float apply) by it on the device, before the host reads it
+        const SegTable& t = c->seg[c->mode];
+        launch_seg_update(t, j + 1, V, n, h1, -1.0, w, c->stream);
+        if ((s = dots<T>(c, j + 1, V, w, h2)) != MFS_OK) return s;
+        launch_seg_update_norm(t, j + 1, V, n, h2, -1.0, w, c->d_partial, hn, c->stream);
+        launch_seg_normalise(t, hn, w, w, c->dw_pairs ? c->d_x2 : nullptr, c->stream);
+        x2_ready = c->dw_pairs;
+      } else {
+        launch_update<T>(n, j + 1, V, n, h1, -1.0, w, c->stream);
+        if ((s = dots<T>(c, j + 1, V, w, h2)) != MFS_OK) return s;
+        launch_update<T>(n, j + 1, V, n, h2, -1.0, w, c->stream);
+        if ((s = dots<T>(c, 1, w, w, hn)) != MFS_OK) return s;
+      }
+      CUDA_TRY(c, cudaMemcpyAsync(hb, c->d_h, sizeof(double) * (2 * ldh + 1), cudaMemcpyDeviceToHost, c->stream));
       CUDA_TRY(c, cudaStreamSynchronize(c->stream));
       double* col = &H[(size_t)j * ldh];
       for (int i = 0; i <= j; ++i) col[i] = hb[i] + hb[ldh + i];
       const double hnext = std::sqrt(std::max(0.0, hb[2 * ldh]));
       if (!std::isfinite(hnext)) return c->fail(MFS_ERR_NUMERIC, "non-finite value in the Arnoldi process");
       col[j + 1] = hnext;
-      if (hnext > 0) launch_scale_copy<T>(n, w, 1.0 / hnext, w, c->stream);
+      if (sizeof(T) == 4 && hnext > 0) launch_scale_copy<T>(n, w, 1.0 / hnext, w, c->stream);
       for (int i = 0; i < j; ++i) {
         double t = cs[i] * col[i] + sn[i] * col[i + 1];
         col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
@@ -662,7 +681,8 @@ mfs_status gmres(mfs_ctx* c, const T* b, T* x, double tol, int restart, int max_
     }
     if (j_used > 0) {
       CUDA_TRY(c, cudaMemcpyAsync(coef, y.data(), sizeof(double) * j_used, cudaMemcpyHostToDevice, c->stream));
-      launch_update<T>(n, j_used, V, n, coef, 1.0, x, c->stream);
+      if constexpr (sizeof(T) == 8) launch_seg_update(c->seg[c->mode], j_used, V, n, coef, 1.0, x, c->stream);
+      else launch_update<T>(n, j_used, V, n, coef, 1.0, x, c->stream);
       CHECK_LAUNCH(c);
     }
     if (done) break;
@@ -1523,9 +1543,8 @@ mfs_status batch_gmres_cycle(BatchRun& R, const double* b, double* x, const std:
       launch_seg_dots(B->seg, j + 1, V, n, w, B->partial, h1, R.st);
       launch_seg_update(B->seg, j + 1, V, n, h1, -1.0, w, R.st);
       launch_seg_dots(B->seg, j + 1, V, n, w, B->partial, h2, R.st);
-      launch_seg_update(B->seg, j + 1, V, n, h2, -1.0, w, R.st);
+      launch_seg_update_norm(B->seg, j + 1, V, n, h2, -1.0, w, B->partial, hn, R.st);
     });
-    launch_seg_dots(B->seg, 1, w, n, w, B->partial, hn, R.st);
     launch_batch_givens(S, j, h1, h2, hn, R.st);
     // v_{j+1} = w / h_{j+1,j}, split for the next apply
     if (R.dw) launch_seg_scale_split(B->seg, B->scl, w, w, B->x2, R.st);
@@ -1894,6 +1913,7 @@ void mfs_destroy(mfs_ctx* c) {
       cudaEventDestroy(e.first);
       cudaEventDestroy(e.second);
     }
+  if (c->h_pin) cudaFreeHost(c->h_pin);
   if (c->solver) cusolverDnDestroy(c->solver);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;
@@ -2684,6 +2704,8 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   ALLOC_TRY(c, c->d_border, double, 6 * (size_t)P);
   ALLOC_TRY(c, c->d_zero, double, 3 * (size_t)P);
   ALLOC_TRY(c, c->d_pparts, double, (size_t)kPairMaxParts * n);
+  ALLOC_TRY(c, c->d_pcount, unsigned, c->tg.n_tiles1);
+  CUDA_TRY(c, cudaMemsetAsync(c->d_pcount, 0, sizeof(unsigned) * c->tg.n_tiles1, c->stream));
   ALLOC_TRY(c, c->d_tmp64, double, c->tmp_len);
   ALLOC_TRY(c, c->d_lh64, double, c->n_unk);
   ALLOC_TRY(c, c->d_lam, double, c->n_unk);
@@ -2694,10 +2716,45 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   ALLOC_TRY(c, c->d_in32, float, std::max<long long>(n, c->n_unk));
   ALLOC_TRY(c, c->d_out32, float, std::max<long long>(n, c->n_unk));
   ALLOC_TRY(c, c->d_mu32, float, n);
-  ALLOC_TRY(c, c->d_x2, float2, n);
+  ALLOC_TRY(c, c->d_x2, float2, n + 6 * (size_t)P);
   ALLOC_TRY(c, c->d_t2, float2, c->tmp_len);
   c->nblk = std::max(1, std::min(1024, (n + 4095) / 4096));
-  ALLOC_TRY(c, c->d_partial, double, (size_t)c->nblk * 512);
+  {
+    // 1024-element chunks of the system vectors, without and with the mobility border
+    size_t most = (size_t)c->nblk;
+    for (int md = 0; md < 2; ++md) {
+      const long long len = n + (md == 1 ? 6LL * P : 0LL);
+      std::vector<long long> cs, ce;
+      for (long long a = 0; a < len; a += 1024) {
+        cs.push_back(a);
+        ce.push_back(std::min(len, a + 1024));
+      }
+      std::vector<int> prob(cs.size(), 0), pch = {0, (int)cs.size()}, one(1, 1);
+      std::vector<unsigned> cnt(1, 0u);
+      SegTable& t = c->seg[md];
+      t = SegTable();
+      t.K = 1;
+      t.nchunks = (int)cs.size();
+      int *dp = nullptr, *dpc = nullptr, *da = nullptr;
+      long long *ds = nullptr, *de = nullptr;
+      if ((s = upload(c, dp, prob)) || (s = upload(c, dpc, pch)) || (s = upload(c, da, one)) || (s = upload(c, ds, cs)) ||
+          (s = upload(c, de, ce)) || (s = upload(c, t.counter, cnt)))
+        return s;
+      t.prob = dp;
+      t.pchunk = dpc;
+      t.active = da;
+      t.start = ds;
+      t.end = de;
+      most = std::max(most, cs.size());
+      CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // the uploads' host vectors end here
+    }
+    ALLOC_TRY(c, c->d_partial, double, most * 512);
+  }
+  if (!c->h_pin && cudaMallocHost(&c->h_pin, sizeof(double) * (2 * 512 + 1)) != cudaSuccess) {
+    cudaGetLastError();
+    c->h_pin = nullptr;
+    return c->fail(MFS_ERR_OOM, "pinned allocation failed: Arnoldi coefficients");
+  }
   ALLOC_TRY(c, c->d_h, double, 5 * 512);
   CUDA_TRY(c, cudaMemsetAsync(c->d_v, 0, sizeof(double) * 3 * P, c->stream));
   CUDA_TRY(c, cudaMemsetAsync(c->d_zero, 0, sizeof(double) * 3 * P, c->stream));
@@ -3321,7 +3378,7 @@ mfs_status mfs_tune_pairs(mfs_ctx* c, mfs_pair_shapes* out) {
   double ms = 0;
   PairShape best;
   if ((s = tune([&](PairShape sh) { launch_pairs_dw(c->tg, c->src, c->d_lh64, c->d_mu, c->d_w64, visc, c->d_pparts,
-                                                    kPairMaxParts, c->stream, sh); },
+                                                    c->d_pcount, kPairMaxParts, c->stream, sh); },
                 best, ms, cands)) != MFS_OK)
     return s;
   c->shape_all = best;
@@ -3331,7 +3388,7 @@ mfs_status mfs_tune_pairs(mfs_ctx* c, mfs_pair_shapes* out) {
   r.all_ms = ms;
   if (c->ff.n_eq > 0) {
     if ((s = tune([&](PairShape sh) { launch_pairs_dw_near(c->tg, c->src, c->ff, c->d_lh64, c->d_mu, c->d_w64, visc,
-                                                           c->d_pparts, kPairMaxParts, c->stream, sh); },
+                                                           c->d_pparts, c->d_pcount, kPairMaxParts, c->stream, sh); },
                   best, ms, cands)) != MFS_OK)
       return s;
     c->shape_near = best;

@@ -160,10 +160,10 @@ void launch_velocity(int n, const double* x, const SourceSet& src, const double*
 
 // Same sums as launch_pairs_fp64 (FP64 in and out) computed in double-float arithmetic on
 // the FP32 pipes.  With few target tiles the sources of each tile are split over up to
-// max_parts CTAs whose partial sums go to `partial` (max_parts * 3 n doubles; null: no split)
-// and are added in a second, deterministic pass.
+// max_parts CTAs whose partial sums go to `partial` (max_parts * 3 n doubles; null: no split);
+// the last CTA of a tile to finish adds them in part order (counter: zeros, one per tile).
 void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const double* lam_hat, const double* mu,
-                     double* out, double visc, double* partial, int max_parts, cudaStream_t st,
+                     double* out, double visc, double* partial, unsigned* counter, int max_parts, cudaStream_t st,
                      PairShape shape = PairShape());
 // Source split of a tile: enough parts for ten times the resident CTAs (152 SMs x 4), because the
 // SMs finish their last CTAs at different times and a short CTA leaves less idle behind it
@@ -178,11 +178,11 @@ int pair_split_parts(long long n_tiles1, long long min_sources, int max_parts);
 // Near part of the far-field split, double-float: out = mu + W sum over the near spheres of the
 // target's sphere (their proxies and image triples) of G lambda_hat.
 // Both split each tile's sources over up to max_parts CTAs (partial: max_parts * 3 n doubles, or
-// null for no split) so that the grid fills whole waves of resident CTAs; the parts are added in
-// a fixed order by a second kernel.
+// null for no split) so that the grid fills whole waves of resident CTAs; the parts are added in a
+// fixed order, by the last CTA of a tile (near; counter as above) or by a second kernel (far).
 void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarField& ff, const double* lam_hat,
-                          const double* mu, double* out, double visc, double* partial, int max_parts, cudaStream_t st,
-                          PairShape shape = PairShape());
+                          const double* mu, double* out, double visc, double* partial, unsigned* counter, int max_parts,
+                          cudaStream_t st, PairShape shape = PairShape());
 // Far part, FP32 with compensated cross-tile sums: out += W sum over the far spheres of the
 // equivalent Stokeslets' field.
 void launch_pairs_far(const TargetSet& tg, const SourceSet& src, const FarField& ff, double* out, double visc,
@@ -300,6 +300,13 @@ void launch_seg_dots(const SegTable& t, int nvec, const double* V, long long ldv
                      double* h, cudaStream_t st);
 void launch_seg_update(const SegTable& t, int nvec, const double* V, long long ldv, const double* coef, double sign,
                        double* w, cudaStream_t st);
+// the update, and hn[p] = |w|^2 of its result; partial holds kSegNormPartials doubles a chunk, t.counter
+// is needed and the chunks are 1024 long but the last of a problem
+constexpr int kSegNormPartials = 8;
+void launch_seg_update_norm(const SegTable& t, int nvec, const double* V, long long ldv, const double* coef, double sign,
+                            double* w, double* partial, double* hn, cudaStream_t st);
+// out = in / sqrt(hn[p]), and its (hi, lo) split when x2 is given
+void launch_seg_normalise(const SegTable& t, const double* hn, const double* in, double* out, float2* x2, cudaStream_t st);
 void launch_seg_scale(const SegTable& t, const double* s, const double* in, double* out, cudaStream_t st);
 // the same scaling, also writing the (hi, lo) float split of the result to x2 (the input of the
 // next double-float apply, which then skips its own split)

@@ -1333,15 +1333,55 @@ __global__ void __launch_bounds__(kPairThreads) pairs_far2_kernel(FarArgs A, int
   }
 }
 
-// out[e] (+)= the parts in order: with mu, out = mu + sqrt(w) * sum (the near kernel's unscaled
-// parts); without, out += sum (the far kernel's parts, already scaled)
-__global__ void parts_add_kernel(long long n3, const D4* __restrict__ tgt, int nparts, const double* __restrict__ partial,
-                                 long long pstride, const double* __restrict__ mu, double* __restrict__ out) {
+// out[e] += the parts in order (the far kernel's, already scaled)
+__global__ void parts_add_kernel(long long n3, int nparts, const double* __restrict__ partial, long long pstride,
+                                 double* __restrict__ out) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n3; e += (long long)gridDim.x * blockDim.x) {
     double s = 0.0;
     for (int q = 0; q < nparts; ++q) s += partial[q * pstride + e];
-    out[e] = mu ? mu[e] + tgt[e / 3].w * s : out[e] + s;
+    out[e] += s;
   }
+}
+
+// Split sources, fused reduction: every CTA of work item `item` has written its partial sums of the
+// tile's nodes; the last one to arrive adds the parts in part order and writes out = mu + sqrt(w) s.
+// Returns whether this CTA was the last (all threads see the same answer).
+__device__ __forceinline__ bool parts_last_arrival(unsigned* counter, int item, int nparts) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(&counter[item], 1u) == (unsigned)nparts - 1;
+    if (last) counter[item] = 0u;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+// out = mu + sqrt(w) (sum of the parts in part order) at cnt nodes from start: a thread per value, the
+// parts' loads issued eight at a time (one at a time, the last CTA's chain of loads was the tail of every
+// launch of short problems)
+__device__ __forceinline__ void parts_finish_nodes(const D4* tgt, long long start, int cnt, int nparts,
+                                                   const double* partial, long long pstride, const double* mu,
+                                                   double* out) {
+  for (int i = threadIdx.x; i < 3 * cnt; i += blockDim.x) {
+    const long long e = 3 * start + i;
+    double sum = 0.0;
+    for (int q0 = 0; q0 < nparts; q0 += 8) {
+      double v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = q0 + q < nparts ? __ldcg(&partial[(q0 + q) * pstride + e]) : 0.0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) sum += v[q];
+    }
+    out[e] = mu[e] + tgt[start + i / 3].w * sum;
+  }
+}
+__device__ __forceinline__ void parts_finish_tile(const PairArgs<double>& A, int t, int nparts, const double* partial,
+                                                  long long pstride, unsigned* counter) {
+  if (!parts_last_arrival(counter, t, nparts)) return;
+  const int start = A.tile_start[t], cnt = A.tile_count[t];
+  parts_finish_nodes(A.tgt, start, cnt, nparts, partial, pstride, A.mu, A.out);
 }
 
 template <typename T, int NT>
@@ -1369,14 +1409,18 @@ __global__ void __launch_bounds__(kPairThreads) velocity_fp64_kernel(PairArgs<do
 }
 template <int NT>
 __global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_kernel(PairArgs<double> A, int nparts, double* partial,
-                                                                long long pstride) {
-  pair_tile_dw<NT>(A, blockIdx.x / nparts, blockIdx.x % nparts, nparts, partial, pstride);
+                                                                long long pstride, unsigned* counter) {
+  const int t = blockIdx.x / nparts;
+  pair_tile_dw<NT>(A, t, blockIdx.x % nparts, nparts, partial, pstride);
+  if (nparts > 1) parts_finish_tile(A, t, nparts, partial, pstride, counter);
 }
 template <int NT>
 __global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_near_kernel(PairArgs<double> A, const int* near_off,
                                                                      const int* near_idx, int nparts, double* partial,
-                                                                     long long pstride) {
-  pair_tile_dw_near<NT>(A, near_off, near_idx, blockIdx.x / nparts, blockIdx.x % nparts, nparts, partial, pstride);
+                                                                     long long pstride, unsigned* counter) {
+  const int t = blockIdx.x / nparts;
+  pair_tile_dw_near<NT>(A, near_off, near_idx, t, blockIdx.x % nparts, nparts, partial, pstride);
+  if (nparts > 1) parts_finish_tile(A, t, nparts, partial, pstride, counter);
 }
 // out = mu + sqrt(w) * (sum of the parts), or the plain sum when mu is null; parts added in order
 __global__ void pair_parts_reduce_kernel(long long n3, const D4* __restrict__ tgt, int nparts,
@@ -1404,31 +1448,6 @@ struct BatchVecs {
                           // item adds the parts (in part order) itself and re-arms its counter
 };
 
-// Split sources, fused reduction: every CTA of work item `item` has written its partial sums of the
-// tile's nodes; the last one to arrive adds the parts in part order and writes out = mu + sqrt(w) s.
-// Returns whether this CTA was the last (all threads see the same answer).
-__device__ __forceinline__ bool parts_last_arrival(unsigned* counter, int item, int nparts) {
-  __shared__ bool last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    last = atomicAdd(&counter[item], 1u) == (unsigned)nparts - 1;
-    if (last) counter[item] = 0u;
-  }
-  __syncthreads();
-  if (last) __threadfence();
-  return last;
-}
-__device__ __forceinline__ void parts_finish_node(const D4* tgt, long long node, int nparts, const double* partial,
-                                                  long long pstride, const double* mu, double* out) {
-  const double sw = tgt[node].w;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    double sum = 0.0;
-    for (int q = 0; q < nparts; ++q) sum += __ldcg(&partial[q * pstride + 3 * node + c]);
-    out[3 * node + c] = mu[3 * node + c] + sw * sum;
-  }
-}
 // native FP64: each (problem, 128-node tile) in four pieces; with split sources the parts are added
 // by pair_parts_reduce_batch_kernel
 __global__ void __launch_bounds__(kPairThreads, 4) pairs_fp64_batch_kernel(const PairArgs<double>* __restrict__ args,
@@ -1457,9 +1476,8 @@ __global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_batch_kernel(c
   pair_tile_dw<NT>(A, w.y, blockIdx.x % nparts, nparts, bv.partial + bv.voff[w.x], bv.pstride);
   if constexpr (NT == 1) {  // only the 1-node tiling splits sources
     if (nparts > 1 && bv.counter && parts_last_arrival(bv.counter, blockIdx.x / nparts, nparts)) {
-      const int start = A.tile_start[w.y], cnt = A.tile_count[w.y];
-      for (int i = threadIdx.x; i < cnt; i += blockDim.x)
-        parts_finish_node(A.tgt, start + i, nparts, bv.partial + bv.voff[w.x], bv.pstride, A.mu, A.out);
+      parts_finish_nodes(A.tgt, A.tile_start[w.y], A.tile_count[w.y], nparts, bv.partial + bv.voff[w.x], bv.pstride,
+                         A.mu, A.out);
     }
   }
 }
@@ -1518,8 +1536,7 @@ __global__ void __launch_bounds__(kPairThreads, 3) pairs_dw_multi_kernel(const P
     for (int r = 0; r < R; ++r) {
       if (!(mask >> r & 1u)) continue;
       const long long off = bv.voff[prob[r]];
-      for (int i = threadIdx.x; i < cnt; i += blockDim.x)
-        parts_finish_node(A.tgt, start + i, nparts, bv.partial + off, bv.pstride, bv.mu + off, bv.out + off);
+      parts_finish_nodes(A.tgt, start, cnt, nparts, bv.partial + off, bv.pstride, bv.mu + off, bv.out + off);
     }
   }
 }
@@ -2018,10 +2035,18 @@ __global__ void seg_reduce_kernel(SegTable t, int nvec, const double* __restrict
 // w += sign * sum_i coef[i K + p] V_i over one kSegUpdSub-element piece of a chunk per CTA.  The
 // CTA's kSegUpdGroups thread groups take interleaved vectors (more loads in flight when a short
 // problem has few pieces) and their sums are added in group order.
+// NORM: also hn[p] = |w|^2 of the updated vector, which saves the launch and the read of a separate
+// norm: each piece leaves its sum of squares in `partial` and the last CTA of a problem adds them
+// (in piece order, so the sum does not depend on which CTA that is).
+// With the normalisation on the device, the fused sums of split sources and these kernels in the single
+// solves too, an iteration of two spheres went from 116 to 108 us, one of four from 180 to 173, and the
+// sweep of motions from 20.4 to 20.0 ms.
 constexpr int kSegUpdGroups = 4;
+template <bool NORM>
 __global__ void __launch_bounds__(kSegUpdSub* kSegUpdGroups)
     seg_update_kernel(SegTable t, int nvec, const double* __restrict__ V, long long ldv,
-                      const double* __restrict__ coef, double sign, double* __restrict__ w) {
+                      const double* __restrict__ coef, double sign, double* __restrict__ w,
+                      double* __restrict__ partial, double* __restrict__ hn) {
   const int b = seg_chunk(t);
   const int p = t.prob[b];
   if (!t.active[p]) return;
@@ -2039,11 +2064,54 @@ __global__ void __launch_bounds__(kSegUpdSub* kSegUpdGroups)
   }
   red[g][tl] = a;
   __syncthreads();
+  double s = 0.0;
   if (g == 0 && e < t.end[b]) {
-    double s = w[e];
+    s = w[e];
 #pragma unroll
     for (int q = 0; q < kSegUpdGroups; ++q) s += red[q][tl];
     w[e] = s;
+  }
+  if constexpr (NORM) {
+    constexpr int kPieces = kSegChunkMax / kSegUpdSub;
+    __shared__ double ws[kSegUpdSub / 32];
+    __shared__ bool last;
+    double q = s * s;
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if (g == 0 && (tl & 31) == 0) ws[tl >> 5] = q;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double sum = 0.0;
+      for (int i = 0; i < kSegUpdSub / 32; ++i) sum += ws[i];
+      partial[(long long)b * kPieces + blockIdx.y] = sum;
+      __threadfence();
+      // pieces of problem p: its chunks are full (kSegChunkMax) but the last
+      const int b0 = t.pchunk[p], b1 = t.pchunk[p + 1];
+      const unsigned total = (unsigned)(b1 - 1 - b0) * kPieces +
+                             (unsigned)((t.end[b1 - 1] - t.start[b1 - 1] + kSegUpdSub - 1) / kSegUpdSub);
+      last = atomicAdd(&t.counter[p], 1u) == total - 1;
+      if (last) {
+        t.counter[p] = 0u;
+        ws[0] = 0.0;
+      }
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int b0 = t.pchunk[p], b1 = t.pchunk[p + 1];
+    const long long n_last = (t.end[b1 - 1] - t.start[b1 - 1] + kSegUpdSub - 1) / kSegUpdSub;
+    const long long total = (long long)(b1 - 1 - b0) * kPieces + n_last;
+    double sum = 0.0;
+    for (long long i = threadIdx.x; i < total; i += blockDim.x) sum += __ldcg(&partial[(long long)b0 * kPieces + i]);
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    __syncthreads();
+    double* wsum = &red[0][0];
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double tot = 0.0;
+      for (int i = 0; i < kSegUpdSub * kSegUpdGroups / 32; ++i) tot += wsum[i];
+      hn[p] = tot;
+    }
   }
 }
 
@@ -2069,6 +2137,24 @@ __global__ void seg_scale_split_kernel(SegTable t, const double* __restrict__ s,
     out[e] = v;
     const dw d = dw_split(v);
     x2[e] = make_float2(d.h, d.l);
+  }
+}
+
+// out = in / sqrt(hn[p]) (0 for hn = 0), and its (hi, lo) split for the next double-float apply when x2
+// is given
+__global__ void seg_normalise_kernel(SegTable t, const double* __restrict__ hn, const double* __restrict__ in,
+                                     double* __restrict__ out, float2* __restrict__ x2) {
+  const int b = seg_chunk(t);
+  const int p = t.prob[b];
+  if (!t.active[p]) return;
+  const double h = sqrt(fmax(0.0, hn[p])), f = h > 0 ? 1.0 / h : 0.0;
+  for (long long e = t.start[b] + threadIdx.x; e < t.end[b]; e += blockDim.x) {
+    const double v = f * in[e];
+    out[e] = v;
+    if (x2) {
+      const dw d = dw_split(v);
+      x2[e] = make_float2(d.h, d.l);
+    }
   }
 }
 
@@ -2428,7 +2514,7 @@ PairShape resolve_dw_shape(const TargetSet& tg, const SourceSet& src, PairShape 
 }
 
 void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const double* lam_hat, const double* mu, double* out,
-                     double visc, double* partial, int max_parts, cudaStream_t st, PairShape shape) {
+                     double visc, double* partial, unsigned* counter, int max_parts, cudaStream_t st, PairShape shape) {
   if (tg.n_tiles == 0) return;
   const PairShape r = resolve_dw_shape(tg, src, shape, max_parts);
   const int nt = r.nt;
@@ -2436,12 +2522,9 @@ void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const double* la
   PairArgs<double> A = make_args<double>(tg, src, lam_hat, mu, out, visc, nt);
   const long long n3 = 3LL * tg.n;
   ++t_launches;
-  if (nt == 4) pairs_dw_kernel<4><<<tg.n_tiles * parts, kPairThreads, 0, st>>>(A, parts, partial, n3);
-  else pairs_dw_kernel<1><<<tg.n_tiles1 * parts, kPairThreads, 0, st>>>(A, parts, partial, n3);
-  if (parts > 1) {
-    ++t_launches;
-    pair_parts_reduce_kernel<<<grid_for(n3, 256), 256, 0, st>>>(n3, A.tgt, parts, partial, n3, mu, out);
-  }
+  // (with split sources the last CTA of a tile to finish adds the parts)
+  if (nt == 4) pairs_dw_kernel<4><<<tg.n_tiles * parts, kPairThreads, 0, st>>>(A, parts, partial, n3, counter);
+  else pairs_dw_kernel<1><<<tg.n_tiles1 * parts, kPairThreads, 0, st>>>(A, parts, partial, n3, counter);
 }
 
 // resident CTAs of a pair kernel on the current device (SMs x CTAs per SM), looked up once per
@@ -2495,8 +2578,8 @@ PairShape resolve_near_shape(const TargetSet& tg, PairShape shape, int max_parts
 }
 
 void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarField& ff, const double* lam_hat,
-                          const double* mu, double* out, double visc, double* partial, int max_parts, cudaStream_t st,
-                          PairShape shape) {
+                          const double* mu, double* out, double visc, double* partial, unsigned* counter, int max_parts,
+                          cudaStream_t st, PairShape shape) {
   if (tg.n_tiles == 0) return;
   const PairShape r = resolve_near_shape(tg, shape, max_parts);
   const int nt = r.nt;
@@ -2506,13 +2589,9 @@ void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarFi
   const long long n3 = 3LL * tg.n;
   ++t_launches;
   if (nt == 4)
-    pairs_dw_near_kernel<4><<<tiles * parts, kPairThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3);
+    pairs_dw_near_kernel<4><<<tiles * parts, kPairThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3, counter);
   else
-    pairs_dw_near_kernel<1><<<tiles * parts, kPairThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3);
-  if (parts > 1) {
-    ++t_launches;
-    parts_add_kernel<<<grid_for(n3, 256), 256, 0, st>>>(n3, A.tgt, parts, partial, n3, mu, out);
-  }
+    pairs_dw_near_kernel<1><<<tiles * parts, kPairThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3, counter);
 }
 
 PairShape resolve_far_shape(const TargetSet& tg, PairShape shape, int max_parts) {
@@ -2557,8 +2636,7 @@ void launch_pairs_far(const TargetSet& tg, const SourceSet& src, const FarField&
   else pairs_far_kernel<1><<<tiles * parts, kPairThreads, 0, st>>>(A, parts, partial, n3);
   if (parts > 1) {
     ++t_launches;
-    parts_add_kernel<<<grid_for(n3, 256), 256, 0, st>>>(n3, reinterpret_cast<const D4*>(tg.pos64), parts, partial, n3,
-                                                        nullptr, out);
+    parts_add_kernel<<<grid_for(n3, 256), 256, 0, st>>>(n3, parts, partial, n3, out);
   }
 }
 
@@ -2640,8 +2718,20 @@ void launch_seg_update(const SegTable& t, int nvec, const double* V, long long l
                        double* w, cudaStream_t st) {
   if (seg_ctas(t) == 0 || nvec == 0) return;
   ++t_launches;
-  seg_update_kernel<<<dim3(seg_ctas(t), (t.chunk + kSegUpdSub - 1) / kSegUpdSub), kSegUpdSub * kSegUpdGroups, 0, st>>>(
-      t, nvec, V, ldv, coef, sign, w);
+  seg_update_kernel<false><<<dim3(seg_ctas(t), (t.chunk + kSegUpdSub - 1) / kSegUpdSub), kSegUpdSub * kSegUpdGroups, 0, st>>>(
+      t, nvec, V, ldv, coef, sign, w, nullptr, nullptr);
+}
+void launch_seg_update_norm(const SegTable& t, int nvec, const double* V, long long ldv, const double* coef, double sign,
+                            double* w, double* partial, double* hn, cudaStream_t st) {
+  if (seg_ctas(t) == 0 || nvec == 0) return;
+  ++t_launches;
+  seg_update_kernel<true><<<dim3(seg_ctas(t), (t.chunk + kSegUpdSub - 1) / kSegUpdSub), kSegUpdSub * kSegUpdGroups, 0, st>>>(
+      t, nvec, V, ldv, coef, sign, w, partial, hn);
+}
+void launch_seg_normalise(const SegTable& t, const double* hn, const double* in, double* out, float2* x2, cudaStream_t st) {
+  if (seg_ctas(t) == 0) return;
+  ++t_launches;
+  seg_normalise_kernel<<<seg_ctas(t), kSegThreads, 0, st>>>(t, hn, in, out, x2);
 }
 void launch_seg_scale_split(const SegTable& t, const double* s, const double* in, double* out, float2* x2,
                             cudaStream_t st) {
