@@ -191,7 +191,7 @@ struct mfs_ctx {
   int mode = 0;           // 0: resistance (velocities given), 1: mobility (forces/torques given)
   int n_sys = 0;          // GMRES system size: n, or n + 6P for the bordered mobility system
   double* d_border = nullptr;  // mobility: scaled prescribed (F_k, T_k), 6 per sphere
-  double* d_pparts = nullptr;  // partial sums of the source-split pair kernel, kPairMaxParts * n
+  double* d_pparts = nullptr;  // partial sums of the source-split pair kernels, kPairMaxParts * n
   unsigned* d_pcount = nullptr;  // arrivals of a tile's parts (zeros between launches)
   double* d_zero = nullptr;    // 3P zeros
   // measurement
@@ -249,6 +249,7 @@ struct mfs_ctx {
   double *d_tmp64 = nullptr, *d_lh64 = nullptr, *d_lam = nullptr, *d_F = nullptr, *d_T = nullptr;
   float *d_tmp32 = nullptr, *d_lh32 = nullptr, *d_in32 = nullptr, *d_out32 = nullptr, *d_mu32 = nullptr;
   float2 *d_x2 = nullptr, *d_t2 = nullptr;  // double-float staging of step 1
+  float2* d_lh2 = nullptr;                  // and its result lambda_hat, the input of the pair sums
   // Krylov workspace (lazily sized)
   void* d_basis = nullptr;
   size_t basis_bytes = 0;
@@ -435,7 +436,7 @@ void precond(mfs_ctx* c, const T* mu, T* lam_hat, bool x2_ready = false) {
         } else {
           launch_gemv_dw(c->gA2, c->d_x2, c->d_t2, nullptr, c->stream);
         }
-        launch_gemv_dw(c->gV2, c->d_t2, nullptr, lam_hat, c->stream);
+        launch_gemv_dw(c->gV2, c->d_t2, c->d_lh2, lam_hat, c->stream);
         return;
       }
     }
@@ -447,7 +448,8 @@ void precond(mfs_ctx* c, const T* mu, T* lam_hat, bool x2_ready = false) {
                                      : c->gemv_bytes32;
 }
 
-// steps 2+3 with the pair kernel of the current precision
+// steps 2+3 with the pair kernel of the current precision (double-float: of the strengths in d_lh2,
+// which step 1 leaves there)
 template <typename T>
 void pairs_step(mfs_ctx* c, const T* lam_hat, const T* mu, T* out) {
   if constexpr (sizeof(T) == 8) {
@@ -455,7 +457,7 @@ void pairs_step(mfs_ctx* c, const T* lam_hat, const T* mu, T* out) {
       // near spheres directly in double-float, the far ones through their equivalent sources,
       // whose strengths q = Q mu are formed from this apply's mu
       timed(c, c->ev_pair, [&] {
-        launch_pairs_dw_near(c->tg, c->src, c->ff, lam_hat, mu, out, c->hd.prm.visc, c->d_pparts, c->d_pcount,
+        launch_pairs_dw_near(c->tg, c->src, c->ff, c->d_lh2, mu, out, c->hd.prm.visc, c->d_pparts, c->d_pcount,
                              kPairMaxParts, c->stream, c->shape_near);
       });
       timed(c, c->ev_far, [&] {
@@ -491,7 +493,7 @@ void pairs_step(mfs_ctx* c, const T* lam_hat, const T* mu, T* out) {
   timed(c, c->ev_pair, [&] {
     if constexpr (sizeof(T) == 8) {
       if (c->dw_pairs) {
-        launch_pairs_dw(c->tg, c->src, lam_hat, mu, out, c->hd.prm.visc, c->d_pparts, c->d_pcount, kPairMaxParts,
+        launch_pairs_dw(c->tg, c->src, c->d_lh2, mu, out, c->hd.prm.visc, c->d_pparts, c->d_pcount, kPairMaxParts,
                         c->stream, c->shape_all);
         return;
       }
@@ -763,19 +765,14 @@ struct BatchPlan {
   std::vector<long long> pairs_p, proxy_p, image_p;
   std::vector<void*> allocs;
   std::vector<void*> gs_allocs;
-  void* d_args = nullptr;    // per-problem kernel arguments for 4 nodes per thread
-  void* d_args1 = nullptr;   // and for 1 node per thread
-  int2* d_work = nullptr;    // (problem, tile) lists for both tilings
-  int2* d_work1 = nullptr;
-  int n_work = 0, n_work1 = 0;
-  std::vector<int> tiles4;   // large tiles per problem, to pick the tiling of each launch
+  void* d_args1 = nullptr;   // per-problem kernel arguments (128-node tiles)
   std::vector<int> tiles1;
+  std::vector<int> pieces1;          // halves of the 128-node tiles that hold nodes
   std::vector<long long> others_p;  // proxies of the other spheres per problem (source split)
-  std::vector<int2> w4_host, w1_host;  // full work lists; the launches use the active problems' part
-  int2* d_cwork = nullptr;   // compacted (problem, tile) lists of the active problems
-  int2* d_cwork1 = nullptr;
-  int2* wpin = nullptr;      // pinned staging for them
-  int n_cwork = 0, n_cwork1 = 0;
+  std::vector<int2> w1_host;  // full (problem, tile) list; the launches use the active problems' part
+  int2* d_cwork1 = nullptr;  // the compacted list of the active problems
+  int2* wpin = nullptr;      // pinned staging for it
+  int n_cwork1 = 0;
   double* pparts = nullptr;  // source-split partial sums, kPairMaxParts * n_total
   std::vector<int> cprob_host;  // problem of each vector chunk
   std::vector<int> jprob_host;  // problem of each GEMV job
@@ -818,6 +815,7 @@ struct BatchPlan {
   int2* swork_pin = nullptr;
   unsigned* d_pcount = nullptr;  // per pair-kernel work item: arrivals of its source parts
   int n_mwork = 0, n_swork1 = 0;
+  long long n_mpieces = 0;   // halves with nodes of the tiles in d_mwork and d_swork1
   size_t mwork_cap = 0;
   std::vector<int> rhs_shared;             // per problem: right-hand sides in its pair-kernel item
   std::vector<int> leader;                 // per problem: the first problem on the same context
@@ -827,7 +825,7 @@ struct BatchPlan {
   SegTable seg;
   double *wb = nullptr, *x = nullptr, *r = nullptr, *e = nullptr, *w = nullptr, *lh = nullptr, *tmp = nullptr,
          *lam = nullptr, *partial = nullptr, *hbuf = nullptr, *coef = nullptr, *scl = nullptr;
-  float2 *x2 = nullptr, *t2 = nullptr;
+  float2 *x2 = nullptr, *t2 = nullptr, *lh2 = nullptr;
   std::vector<long long> boff;           // per problem: offset of its 3 P values in bc / F / T
   double *bc_v = nullptr, *bc_w = nullptr, *out_F = nullptr, *out_T = nullptr;
   double* basis = nullptr;
@@ -886,7 +884,6 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
   B->voff.assign(K + 1, 0);
   B->uoff.assign(K + 1, 0);
   B->toff.assign(K + 1, 0);
-  long long tiles_large = 0;
   for (int p = 0; p < K; ++p) {
     mfs_ctx* c = ctxs[p];
     B->nlen.push_back(c->n);
@@ -896,43 +893,31 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
     B->pairs_p.push_back(c->pairs_per_apply);
     B->proxy_p.push_back(c->proxy_per_apply);
     B->image_p.push_back(c->image_per_apply);
-    tiles_large += c->tg.n_tiles;
   }
   B->n_total = B->voff[K];
   B->u_total = B->uoff[K];
   B->t_total = B->toff[K];
-  (void)tiles_large;
-  // pair kernel arguments and work lists for both tilings; each launch picks the tiling from
-  // the tiles of the problems still active (the lockstep tail may hold a single problem)
+  // pair kernel arguments and the work list
   const size_t asz = pair_args64_bytes();
-  std::vector<char> args4(asz * K), args1(asz * K);
-  std::vector<int2> work4, work1;
+  std::vector<char> args1(asz * K);
+  std::vector<int2> work1;
   for (int p = 0; p < K; ++p) {
     mfs_ctx* c = ctxs[p];
-    fill_pair_args64(args4.data() + asz * p, c->tg, c->src, nullptr, nullptr, nullptr, c->hd.prm.visc, 4);
     fill_pair_args64(args1.data() + asz * p, c->tg, c->src, nullptr, nullptr, nullptr, c->hd.prm.visc, 1);
-    for (int t = 0; t < c->tg.n_tiles; ++t) work4.push_back(make_int2(p, t));
     for (int t = 0; t < c->tg.n_tiles1; ++t) work1.push_back(make_int2(p, t));
-    B->tiles4.push_back(c->tg.n_tiles);
     B->tiles1.push_back(c->tg.n_tiles1);
+    B->pieces1.push_back(c->tg.n_pieces1);
     B->others_p.push_back((long long)(c->P - 1) * c->src.N);
   }
-  B->w4_host = work4;
   B->w1_host = work1;
-  B->n_work = (int)work4.size();
-  B->n_work1 = (int)work1.size();
-  B->d_args = B->alloc<char>(args4.size());
   B->d_args1 = B->alloc<char>(args1.size());
-  bool ok = B->d_args && B->d_args1 &&
-            cudaMemcpy(B->d_args, args4.data(), args4.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
+  bool ok = B->d_args1 &&
             cudaMemcpy(B->d_args1, args1.data(), args1.size(), cudaMemcpyHostToDevice) == cudaSuccess;
-  ok = ok && put(B, B->d_work, work4) && put(B, B->d_work1, work1) && put(B, B->d_uoff, B->uoff) &&
-       put(B, B->d_voff, B->voff) && put(B, B->d_nlen, B->nlen);
+  ok = ok && put(B, B->d_uoff, B->uoff) && put(B, B->d_voff, B->voff) && put(B, B->d_nlen, B->nlen);
   B->d_active = B->alloc<int>(K);
-  B->d_cwork = B->alloc<int2>(work4.size());
   B->d_cwork1 = B->alloc<int2>(work1.size());
-  ok = ok && B->d_active && B->d_cwork && B->d_cwork1 &&
-       cudaMallocHost(&B->wpin, sizeof(int2) * std::max<size_t>(1, work4.size() + work1.size())) == cudaSuccess;
+  ok = ok && B->d_active && B->d_cwork1 &&
+       cudaMallocHost(&B->wpin, sizeof(int2) * std::max<size_t>(1, work1.size())) == cudaSuccess;
   // GEMV jobs: every sphere of every problem, with the problems that share a context (several
   // right-hand sides on one geometry) adjacent, so a factor matrix is read once for all of them
   std::vector<const double*> mA, mV;
@@ -1061,8 +1046,8 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
        cudaMallocHost(&B->items_pin, sizeof(int2) * 2 * std::max<size_t>(1, jp.size())) == cudaSuccess;
   B->mwork_cap = std::max<size_t>(1, B->w1_host.size());
   ok = ok && (B->d_mwork = B->alloc<int4>(B->mwork_cap)) && (B->d_rhs = B->alloc<int>(K)) &&
-       (B->d_swork1 = B->alloc<int2>(B->mwork_cap)) && (B->d_pcount = B->alloc<unsigned>(B->mwork_cap)) &&
-       cudaMemset(B->d_pcount, 0, sizeof(unsigned) * B->mwork_cap) == cudaSuccess &&
+       (B->d_swork1 = B->alloc<int2>(B->mwork_cap)) && (B->d_pcount = B->alloc<unsigned>(kPairPieces * B->mwork_cap)) &&
+       cudaMemset(B->d_pcount, 0, sizeof(unsigned) * kPairPieces * B->mwork_cap) == cudaSuccess &&
        cudaMallocHost(&B->mwork_pin, sizeof(int4) * B->mwork_cap) == cudaSuccess &&
        cudaMallocHost(&B->rhs_pin, sizeof(int) * K) == cudaSuccess &&
        cudaMallocHost(&B->swork_pin, sizeof(int2) * B->mwork_cap) == cudaSuccess;
@@ -1136,7 +1121,7 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
        (B->partial = B->alloc<double>((size_t)kMaxBatchVec * B->seg.nchunks)) &&
        (B->hbuf = B->alloc<double>((size_t)(2 * kMaxBatchVec + 1) * K)) &&
        (B->coef = B->alloc<double>((size_t)kMaxBatchVec * K)) && (B->scl = B->alloc<double>(K)) &&
-       (B->x2 = B->alloc<float2>(n)) && (B->t2 = B->alloc<float2>(B->t_total)) &&
+       (B->x2 = B->alloc<float2>(n)) && (B->t2 = B->alloc<float2>(B->t_total)) && (B->lh2 = B->alloc<float2>(B->u_total)) &&
        (B->pparts = B->alloc<double>((size_t)kPairMaxParts * n));
   B->boff.assign(K + 1, 0);
   for (int p = 0; p < K; ++p) B->boff[p + 1] = B->boff[p] + 3LL * ctxs[p]->P;
@@ -1179,19 +1164,16 @@ mfs_status set_active(BatchRun& R, const std::vector<int>& a) {
   if (!R.act.empty() && R.act == a) return MFS_OK;
   R.act = a;
   for (int p = 0; p < B->K; ++p) B->apin[p] = a[p];
-  int n4 = 0, n1 = 0;
-  int2* w4 = B->wpin;
-  int2* w1 = B->wpin + B->w4_host.size();
-  for (const int2& w : B->w4_host)
-    if (a[w.x]) w4[n4++] = w;
+  int n1 = 0;
+  int2* w1 = B->wpin;
   for (const int2& w : B->w1_host)
     if (a[w.x]) w1[n1++] = w;
-  B->n_cwork = n4;
   B->n_cwork1 = n1;
   // the active problems of a context in chunks of up to kPairRhs: a chunk of two or more shares
   // the pair kernel's work items, a problem alone keeps the single-problem kernel
   {
     int nm = 0, nr = 0, ns = 0;
+    B->n_mpieces = 0;
     std::vector<char> single(B->K, 0);
     B->rhs_shared.assign(B->K, 1);
     for (int L = 0; L < B->K; ++L) {
@@ -1203,6 +1185,7 @@ mfs_status set_active(BatchRun& R, const std::vector<int>& a) {
         const int cnt = (int)std::min<size_t>(kPairRhs, mem.size() - c0);
         if (cnt == 1) {
           single[mem[c0]] = 1;
+          B->n_mpieces += B->pieces1[L];
           continue;
         }
         const int r0 = nr;
@@ -1210,6 +1193,7 @@ mfs_status set_active(BatchRun& R, const std::vector<int>& a) {
           B->rhs_pin[nr++] = mem[c0 + q];
           B->rhs_shared[mem[c0 + q]] = cnt;
         }
+        B->n_mpieces += B->pieces1[L];
         for (int t = 0; t < B->tiles1[L]; ++t) B->mwork_pin[nm++] = make_int4(L, t, r0, cnt);
       }
     }
@@ -1279,7 +1263,6 @@ mfs_status set_active(BatchRun& R, const std::vector<int>& a) {
   CUDA_TRY(R.c0, cudaMemcpyAsync(B->d_active, B->apin, sizeof(int) * B->K, cudaMemcpyHostToDevice, R.st));
   if (nj) CUDA_TRY(R.c0, cudaMemcpyAsync(B->d_jlist, B->jpin, sizeof(int) * nj, cudaMemcpyHostToDevice, R.st));
   if (nc) CUDA_TRY(R.c0, cudaMemcpyAsync(B->d_cchunk, B->cpin, sizeof(int) * nc, cudaMemcpyHostToDevice, R.st));
-  if (n4) CUDA_TRY(R.c0, cudaMemcpyAsync(B->d_cwork, w4, sizeof(int2) * n4, cudaMemcpyHostToDevice, R.st));
   if (n1) CUDA_TRY(R.c0, cudaMemcpyAsync(B->d_cwork1, w1, sizeof(int2) * n1, cudaMemcpyHostToDevice, R.st));
   // the pinned staging buffers are rewritten by the next call: wait for these copies
   CUDA_TRY(R.c0, cudaStreamSynchronize(R.st));
@@ -1304,41 +1287,36 @@ void batch_apply_kernels(BatchRun& R, const double* in, double* out) {
       } else {
         launch_gemv_dw(B->gA2, B->x2, B->t2, nullptr, R.st);
       }
-      launch_gemv_dw(B->gV2, B->t2, nullptr, B->lh, R.st);
+      launch_gemv_dw(B->gV2, B->t2, B->lh2, B->lh, R.st);
     } else {
       launch_gemv<double>(B->gA, in, B->tmp, R.st);
       launch_gemv<double>(B->gV, B->tmp, B->lh, R.st);
     }
   });
-  long long active_tiles = 0, min_others = -1;
+  long long min_others = -1, active_pieces = 0;
   for (int p = 0; p < B->K; ++p)
     if (R.act[p]) {
-      active_tiles += B->tiles4[p];
+      active_pieces += B->pieces1[p];
       if (B->others_p[p] > 0) min_others = min_others < 0 ? B->others_p[p] : std::min(min_others, B->others_p[p]);
     }
-  // the native FP64 kernel takes 128-node tiles (in pieces of 32 nodes)
-  const int nt = R.dw ? pair_nodes_per_thread((int)std::min<long long>(active_tiles, 1 << 30)) : 1;
   // few tiles left (the lockstep tail): split each tile's sources over several CTAs
-  const int parts = nt != 1 || min_others <= 0 ? 1
-                    : R.dw ? pair_split_parts(B->n_cwork1, min_others, kPairMaxParts)
+  const int parts = min_others <= 0 ? 1
+                    : R.dw ? batch_split_parts(active_pieces, false, min_others, kPairMaxParts)
                            : fp64_split_parts(4LL * B->n_cwork1, min_others, kPairMaxParts);
   timed(c, c->ev_pair, [&] {
     if (R.dw && B->n_mwork > 0) {
       // right-hand sides on one geometry share the pair evaluations; the problems left single
-      // run the 1-node-per-thread kernel with the same source split, one reduction for both
-      const long long items = (long long)B->n_mwork + B->n_swork1;
-      const int mparts = min_others > 0 ? pair_split_parts(items, min_others, kPairMaxParts) : 1;
+      // run the single-problem kernel with the same source split
+      const int mparts = min_others > 0 ? batch_split_parts(B->n_mpieces, true, min_others, kPairMaxParts) : 1;
       // (with split sources the last CTA of each item adds the parts)
-      launch_pairs_multi64(B->d_args1, B->d_mwork, B->n_mwork, B->d_rhs, B->d_active, B->lh, in, out, B->d_uoff,
+      launch_pairs_multi64(B->d_args1, B->d_mwork, B->n_mwork, B->d_rhs, B->d_active, B->lh2, in, out, B->d_uoff,
                            B->d_voff, mparts, B->pparts, B->n_total, B->d_nlen, R.st, B->d_pcount);
-      launch_pairs_batch64(true, B->d_args1, B->d_swork1, B->n_swork1, B->d_active, 1, B->lh, in, out, B->d_uoff,
-                           B->d_voff, mparts, B->pparts, B->n_total, B->seg, R.st, B->d_nlen, true, B->d_pcount);
-    } else if (nt == 4)
-      launch_pairs_batch64(R.dw, B->d_args, B->d_cwork, B->n_cwork, B->d_active, 4, B->lh, in, out, B->d_uoff,
-                           B->d_voff, 1, nullptr, 0, B->seg, R.st);
-    else
-      launch_pairs_batch64(R.dw, B->d_args1, B->d_cwork1, B->n_cwork1, B->d_active, 1, B->lh, in, out, B->d_uoff,
-                           B->d_voff, parts, B->pparts, B->n_total, B->seg, R.st, B->d_nlen, false, B->d_pcount);
+      launch_pairs_batch64(true, B->d_args1, B->d_swork1, B->n_swork1, B->d_active, B->lh, B->lh2, in, out, B->d_uoff,
+                           B->d_voff, mparts, B->pparts, B->n_total, B->seg, R.st, B->d_nlen, B->d_pcount);
+    } else {
+      launch_pairs_batch64(R.dw, B->d_args1, B->d_cwork1, B->n_cwork1, B->d_active, B->lh, B->lh2, in, out, B->d_uoff,
+                           B->d_voff, parts, B->pparts, B->n_total, B->seg, R.st, B->d_nlen, B->d_pcount);
+    }
   });
   // mobility problems: the rigid motion of the border unknowns, and their force/torque rows
   // (the bordered operator of the single solves, problem by problem)
@@ -2010,6 +1988,8 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
     }
   }
   c->tg.n_tiles1 = (int)ts1.size();
+  for (int q : tcn1) c->tg.n_pieces1 += (q + kTileTargets / 8 - 1) / (kTileTargets / 8);
+  for (int q : tcn) c->tg.n_pieces4 += (q + kTileTargets / 2 - 1) / (kTileTargets / 2);
   if ((s = upload(c, c->tg.tile1_sphere, ts1)) != MFS_OK) return s;
   if ((s = upload(c, c->tg.tile1_start, tst1)) != MFS_OK) return s;
   if ((s = upload(c, c->tg.tile1_count, tcn1)) != MFS_OK) return s;
@@ -2025,12 +2005,15 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   if ((s = upload(c, c->d_sqrtw, sw)) != MFS_OK) return s;
 
   // ---- sources
-  std::vector<float4> p32(N), i32(std::max(ni, 1));
+  std::vector<float4> p32(N), p2(2 * (size_t)N), i32(std::max(ni, 1));
   std::vector<double> p64(4 * (size_t)N), i64(4 * (size_t)std::max(ni, 1), 0.0);
   for (int j = 0; j < N; ++j) {
     p32[j] = make_float4((float)d.proxy_rel[3 * j], (float)d.proxy_rel[3 * j + 1], (float)d.proxy_rel[3 * j + 2], 0.f);
     for (int q = 0; q < 3; ++q) p64[4 * j + q] = d.proxy_rel[3 * j + q];
     p64[4 * j + 3] = 0;
+    p2[2 * j] = p32[j];
+    p2[2 * j + 1] = make_float4((float)(d.proxy_rel[3 * j] - (double)p32[j].x), (float)(d.proxy_rel[3 * j + 1] - (double)p32[j].y),
+                                (float)(d.proxy_rel[3 * j + 2] - (double)p32[j].z), 0.f);
   }
   for (int j = 0; j < ni; ++j) {
     int o = d.img_owner[j];
@@ -2052,6 +2035,7 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   c->src.span = c->a * (1.0 + p.r_proxy);
   if ((s = upload(c, c->src.proxy32, p32)) != MFS_OK) return s;
   if ((s = upload(c, c->src.proxy64, p64)) != MFS_OK) return s;
+  if ((s = upload(c, c->src.proxy2, p2)) != MFS_OK) return s;
   if ((s = upload(c, c->src.img32, i32)) != MFS_OK) return s;
   if ((s = upload(c, c->src.img64, i64)) != MFS_OK) return s;
   if ((s = upload(c, c->src.img_owner, io)) != MFS_OK) return s;
@@ -2704,8 +2688,8 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   ALLOC_TRY(c, c->d_border, double, 6 * (size_t)P);
   ALLOC_TRY(c, c->d_zero, double, 3 * (size_t)P);
   ALLOC_TRY(c, c->d_pparts, double, (size_t)kPairMaxParts * n);
-  ALLOC_TRY(c, c->d_pcount, unsigned, c->tg.n_tiles1);
-  CUDA_TRY(c, cudaMemsetAsync(c->d_pcount, 0, sizeof(unsigned) * c->tg.n_tiles1, c->stream));
+  ALLOC_TRY(c, c->d_pcount, unsigned, (size_t)kPairPieces * c->tg.n_tiles1);
+  CUDA_TRY(c, cudaMemsetAsync(c->d_pcount, 0, sizeof(unsigned) * kPairPieces * c->tg.n_tiles1, c->stream));
   ALLOC_TRY(c, c->d_tmp64, double, c->tmp_len);
   ALLOC_TRY(c, c->d_lh64, double, c->n_unk);
   ALLOC_TRY(c, c->d_lam, double, c->n_unk);
@@ -2718,6 +2702,7 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   ALLOC_TRY(c, c->d_mu32, float, n);
   ALLOC_TRY(c, c->d_x2, float2, n + 6 * (size_t)P);
   ALLOC_TRY(c, c->d_t2, float2, c->tmp_len);
+  ALLOC_TRY(c, c->d_lh2, float2, c->n_unk);
   c->nblk = std::max(1, std::min(1024, (n + 4095) / 4096));
   {
     // 1024-element chunks of the system vectors, without and with the mobility border
@@ -3199,7 +3184,10 @@ static mfs_status run_step(mfs_ctx* c, int precision, int which, const double* i
     c->dw_fast_a = c->ff_pass = (precision == MFS_MIXED_PASS);
     if (which == 0) apply_op<double>(c, c->d_mu, c->d_w64);
     else if (which == 1) precond<double>(c, c->d_mu, c->d_lh64);
-    else pairs_step<double>(c, c->d_lam, c->d_mu, c->d_w64);
+    else {
+      if (c->dw_pairs) launch_split_dw(nu, c->d_lam, c->d_lh2, c->stream);
+      pairs_step<double>(c, c->d_lam, c->d_mu, c->d_w64);
+    }
     c->dw_pairs = c->dw_fast_a = c->ff_pass = false;
   } else {
     launch_convert<double, float>(len1, d1, 1.0, c->d_in32, c->stream);
@@ -3339,7 +3327,7 @@ mfs_status mfs_tune_pairs(mfs_ctx* c, mfs_pair_shapes* out) {
     }
   } evf{e0, e1};
   // inputs: the context's work buffers, zeroed (the launches' cost does not depend on the values)
-  CUDA_TRY(c, cudaMemsetAsync(c->d_lh64, 0, sizeof(double) * c->n_unk, c->stream));
+  CUDA_TRY(c, cudaMemsetAsync(c->d_lh2, 0, sizeof(float2) * c->n_unk, c->stream));
   CUDA_TRY(c, cudaMemsetAsync(c->d_mu, 0, sizeof(double) * c->n, c->stream));
   if (c->d_q) CUDA_TRY(c, cudaMemsetAsync(c->d_q, 0, sizeof(float) * 3 * (size_t)c->ff.n_eq * c->P, c->stream));
   const double visc = c->hd.prm.visc;
@@ -3377,7 +3365,7 @@ mfs_status mfs_tune_pairs(mfs_ctx* c, mfs_pair_shapes* out) {
   mfs_pair_shapes r{};
   double ms = 0;
   PairShape best;
-  if ((s = tune([&](PairShape sh) { launch_pairs_dw(c->tg, c->src, c->d_lh64, c->d_mu, c->d_w64, visc, c->d_pparts,
+  if ((s = tune([&](PairShape sh) { launch_pairs_dw(c->tg, c->src, c->d_lh2, c->d_mu, c->d_w64, visc, c->d_pparts,
                                                     c->d_pcount, kPairMaxParts, c->stream, sh); },
                 best, ms, cands)) != MFS_OK)
     return s;
@@ -3387,7 +3375,7 @@ mfs_status mfs_tune_pairs(mfs_ctx* c, mfs_pair_shapes* out) {
   r.all_parts = ra.parts;
   r.all_ms = ms;
   if (c->ff.n_eq > 0) {
-    if ((s = tune([&](PairShape sh) { launch_pairs_dw_near(c->tg, c->src, c->ff, c->d_lh64, c->d_mu, c->d_w64, visc,
+    if ((s = tune([&](PairShape sh) { launch_pairs_dw_near(c->tg, c->src, c->ff, c->d_lh2, c->d_mu, c->d_w64, visc,
                                                            c->d_pparts, c->d_pcount, kPairMaxParts, c->stream, sh); },
                   best, ms, cands)) != MFS_OK)
       return s;

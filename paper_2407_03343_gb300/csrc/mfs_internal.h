@@ -59,6 +59,7 @@ struct TargetSet {
   int n = 0;             // nodes
   int n_tiles = 0;       // tiles of up to 512 nodes (4 per thread)
   int n_tiles1 = 0;      // tiles of up to 128 nodes (1 per thread), used when there are few large tiles
+  int n_pieces4 = 0, n_pieces1 = 0;  // their halves that hold nodes (the double-float kernels' CTAs)
   float4* pos32 = nullptr;   // (x - c_k, y - c_k, z - c_k, sqrt w) per node, FP32
   double* pos64 = nullptr;   // same, 4 doubles per node
   int* tile_sphere = nullptr;
@@ -77,6 +78,7 @@ struct SourceSet {
   double span = 2.0;           // sphere radius plus proxy radius
   float4* proxy32 = nullptr;   // N positions relative to the owner centre (same for every sphere)
   double* proxy64 = nullptr;   // 4 doubles per proxy (x, y, z, 0)
+  float4* proxy2 = nullptr;    // double-float: 2 per proxy, high words then low words
   float4* img32 = nullptr;     // image node positions relative to the owner centre
   double* img64 = nullptr;     // 4 doubles per node (x, y, z, 0)
   int* img_owner = nullptr;
@@ -148,8 +150,9 @@ void launch_pairs_f32(const TargetSet& tg, const SourceSet& src, const float* la
 void launch_pairs_fp64(const TargetSet& tg, const SourceSet& src, const double* lam_hat, const double* mu, double* out,
                        double visc, double* partial, int max_parts, cudaStream_t st);
 // Source split of the FP64 kernels: enough CTAs (pieces x parts) that the SMs' shares of the FP64
-// pipe differ by a few per cent (152 SMs x 16), at least kPairSplitMinSources sources per part.
+// pipe differ by a few per cent (152 SMs x 16), at least kFp64SplitMinSources sources per part.
 constexpr int kFp64SplitTarget = 152 * 16;
+constexpr int kFp64SplitMinSources = 64;
 int fp64_split_parts(long long pieces, long long min_sources, int max_parts);
 // u (3 n) = velocity at the n points x (3 n, absolute) of the strengths lam, native FP64; partial
 // holds velocity_parts(n, src) * 3 n doubles (unused for one part).
@@ -159,28 +162,30 @@ void launch_velocity(int n, const double* x, const SourceSet& src, const double*
                      double visc, cudaStream_t st);
 
 // Same sums as launch_pairs_fp64 (FP64 in and out) computed in double-float arithmetic on
-// the FP32 pipes.  With few target tiles the sources of each tile are split over up to
+// the FP32 pipes, the strengths as (hi, lo) pairs.  With few target tiles the sources of each tile are split over up to
 // max_parts CTAs whose partial sums go to `partial` (max_parts * 3 n doubles; null: no split);
 // the last CTA of a tile to finish adds them in part order (counter: zeros, one per tile).
-void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const double* lam_hat, const double* mu,
+void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const float2* lam_hat, const double* mu,
                      double* out, double visc, double* partial, unsigned* counter, int max_parts, cudaStream_t st,
                      PairShape shape = PairShape());
-// Source split of a tile: enough parts for ten times the resident CTAs (152 SMs x 4), because the
-// SMs finish their last CTAs at different times and a short CTA leaves less idle behind it
-// (measured on 100 spheres, 700 tiles: 30.3 ms with 2 parts, 28.8 with 3, 27.3 with 9 and 27.5
-// with 16; on 20 spheres, 140 tiles: 1.20 ms with 8 parts and 1.11 with 16), at least
-// kPairSplitMinSources sources per part, at most max_parts.
-constexpr int kPairSplitTarget = 152 * 40;
-constexpr int kPairSplitMinSources = 64;
+// Source split of a launch of `items` CTAs a part: the count of parts that leaves the least work to the
+// longest SM, ceil(items x parts / resident CTAs) / parts, with the work of kPairSplitPartCost sources
+// charged per part, at least kPairSplitMinSources sources each, at most max_parts.  Against the best of
+// all shapes measured: two spheres 41.7 us (40.3 with 16 parts), 8 spheres 288 (286), 20 spheres 1097
+// (1096), 100 spheres 26.10 ms (26.09), 100 spheres of 1804 nodes 116.1 (116.1).  The rule before it, a
+// fixed count of CTAs, left 84 items of three right-hand sides on 456 resident CTAs with 6 parts, 1.1
+// waves: that sweep took 20.5 ms, 19.6 with this rule and the norm in the update.
+constexpr double kPairSplitPartCost = 16.0;
+constexpr int kPairSplitMinSources = 32;
 constexpr int kPairMaxParts = 16;
-int pair_split_parts(long long n_tiles1, long long min_sources, int max_parts);
+constexpr int kPairPieces = 2;  // arrival counters per tile or batched work item (double-float kernels)
 
 // Near part of the far-field split, double-float: out = mu + W sum over the near spheres of the
 // target's sphere (their proxies and image triples) of G lambda_hat.
 // Both split each tile's sources over up to max_parts CTAs (partial: max_parts * 3 n doubles, or
 // null for no split) so that the grid fills whole waves of resident CTAs; the parts are added in a
 // fixed order, by the last CTA of a tile (near; counter as above) or by a second kernel (far).
-void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarField& ff, const double* lam_hat,
+void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarField& ff, const float2* lam_hat,
                           const double* mu, double* out, double visc, double* partial, unsigned* counter, int max_parts,
                           cudaStream_t st, PairShape shape = PairShape());
 // Far part, FP32 with compensated cross-tile sums: out += W sum over the far spheres of the
@@ -198,26 +203,25 @@ size_t pair_args64_bytes();
 void fill_pair_args64(void* host_dst, const TargetSet& tg, const SourceSet& src, const double* lam_hat,
                       const double* mu, double* out, double visc, int nodes_per_thread);
 struct SegTable;
-// parts > 1 (double-float, 1 node per thread only): sources split as in launch_pairs_dw, the
-// partial sums in `partial` (parts slices of pstride doubles) reduced over the chunks of `seg`.
+// parts > 1: sources split as in launch_pairs_dw, the partial sums in `partial` (parts slices of
+// pstride doubles) added by the last CTA of an item (double-float; d_counter as above, kPairPieces per
+// item) or over the chunks of `seg` (native FP64).
 void launch_pairs_batch64(bool double_float, const void* d_args, const int2* d_work, int n_work, const int* d_active,
-                          int nodes_per_thread, const double* lam, const double* mu, double* out,
+                          const double* lam, const float2* lam2, const double* mu, double* out,
                           const long long* d_uoff, const long long* d_voff, int parts, double* partial,
-                          long long pstride, const SegTable& seg, cudaStream_t st, const long long* d_nlen = nullptr,
-                          bool skip_reduce = false, unsigned* d_counter = nullptr);
+                          long long pstride, const SegTable& seg, cudaStream_t st, const long long* d_nlen,
+                          unsigned* d_counter);
 // Several right-hand sides on one geometry (double-float, 1 node per thread): work[b] = (lead
 // problem, tile, first index into rhs_prob, count <= kPairRhs); each pair's Green's function is
-// formed once for all of the item's right-hand sides.  parts > 1 writes partial sums as
-// launch_pairs_batch64 does; with d_counter (zeros, one per item) the last CTA of each item adds
-// them, else the caller runs launch_pair_parts_reduce_batch once.
+// formed once for all of the item's right-hand sides.  parts > 1 and d_counter as above.
 constexpr int kPairRhs = 3;
+// Source parts of a batched launch of `items` CTAs a part (shared_rhs: of launch_pairs_multi64) by the
+// rule of kPairSplitPartCost.
+int batch_split_parts(long long items, bool shared_rhs, long long min_sources, int max_parts);
 void launch_pairs_multi64(const void* d_args1, const int4* d_work, int n_work, const int* d_rhs, const int* d_active,
-                          const double* lam, const double* mu, double* out, const long long* d_uoff,
+                          const float2* lam2, const double* mu, double* out, const long long* d_uoff,
                           const long long* d_voff, int parts, double* partial, long long pstride,
-                          const long long* d_nlen, cudaStream_t st, unsigned* d_counter = nullptr);
-void launch_pair_parts_reduce_batch(const void* d_args1, const SegTable& seg, const double* lam, const double* mu,
-                                    double* out, const long long* d_uoff, const long long* d_voff, int parts,
-                                    double* partial, long long pstride, const long long* d_nlen, cudaStream_t st);
+                          const long long* d_nlen, cudaStream_t st, unsigned* d_counter);
 
 // Batched GEMV: for every job j, y_j = M_j x_j with M_j row-major (rows_j x cols_j, leading dim ld_j).
 template <typename T>

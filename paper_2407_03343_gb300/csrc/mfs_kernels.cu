@@ -104,6 +104,8 @@ struct PairArgs {
   const float* cen_hi;
   const float* cen_lo;
   const double* cen64;
+  const float4* proxy2;  // double-float copy of proxy: high words, low words
+  const float2* lam2;    // double-float strengths (double-float kernels), in place of lam
   const T* lam;
   const T* mu;   // may be null: then out = scale * sum (no W, no identity)
   T* out;
@@ -308,6 +310,8 @@ PairArgs<T> make_args(const TargetSet& tg, const SourceSet& src, const T* lam, c
   A.cen_hi = src.cen_hi;
   A.cen_lo = src.cen_lo;
   A.cen64 = src.cen64;
+  A.proxy2 = src.proxy2;
+  A.lam2 = nullptr;
   A.lam = lam;
   A.mu = mu;
   A.out = out;
@@ -572,7 +576,7 @@ __device__ __forceinline__ dw2 add2u(dw2 x, dw2 y) {
 // a source pair is read from shared memory as it is stored and a lane sums every second source.
 // What bounds the sums is the FMA pipe: 160 lane-operations a (node, Stokeslet) pair (the earlier
 // scalar evaluation: 204, and its issue slots) and 340 an image triple (436).  Measured on 100
-// spheres (5.59e9 pairs): 27.3 ms, 81 % of the packed rate, against 43.1 ms.  The evaluation keeps
+// spheres (5.59e9 pairs): 26.1 ms, 90 % of the measured packed rate, against 43.1 ms.  The evaluation keeps
 // the accuracy of a renormalised double-word one (~2^-46 of the operands) with fewer operations:
 //  - positions of a (target sphere, source sphere) segment are split on a common power-of-two grid
 //    per axis, so the difference of the high words is exact without a two-sum;
@@ -589,8 +593,18 @@ __device__ __forceinline__ dw2 add2u(dw2 x, dw2 y) {
 constexpr int kDwTile = 256;     // proxy sources staged per round (one sphere's)
 constexpr int kDwTileImg = 64;   // image nodes staged per round (one sphere's)
 constexpr int kDwGroup = 16;     // terms per lane and group
-// resident CTAs per SM (register bound: 128); 5 and 6 measured the same within 1 %
-constexpr int kDwCtas = 4;
+// Threads of a double-float CTA: the 128-node tiles are taken in two pieces, and a piece without targets
+// ends at once, so 823 nodes a sphere run as 13 CTAs of 64 (832 places) and not as 7 of 128 (896), and
+// the last wave is made of half as long CTAs.  Measured against CTAs of 128 (same rule for the parts): 100
+// spheres 27.8 -> 26.1 ms, the dilute solve of 20 spheres 36.8 -> 35.9 ms; two spheres and the batch of
+// motions the same within 2 %.
+constexpr int kDwThreads = 64;
+constexpr int kDwPieces = kPairThreads / kDwThreads;
+static_assert(kDwPieces == kPairPieces, "arrival counters");
+// resident CTAs per SM (128 registers); 10 (96 registers) and 12 (80) were slower: 100 spheres 26.8 and
+// 26.6 ms against 26.1, two spheres 49.7 and 50.6 us against 41.8
+constexpr int kDwCtas = 8;
+constexpr int kDwMultiCtas = 6;  // of the kernel over several right-hand sides (3 x the sums; 168 registers)
 
 // Sources of one round in shared memory: source pair u holds its two sources' components side by
 // side, pos[3 u ..]: (xh yh), (zh xl), (yl zl), strengths likewise.
@@ -699,7 +713,7 @@ struct DWTile {
 };
 template <int NT>
 struct DwColumns {
-  float2 x[NT][3][kPairThreads], u[NT][3][kPairThreads];
+  float2 x[NT][3][kDwThreads], u[NT][3][kDwThreads];
 };
 template <int NT>
 struct DWTileShared {
@@ -722,11 +736,16 @@ struct DWTileShared {
 template <>
 struct DWTile<1, 4> : DWTileShared<4> {};
 
+// whether this warp has a target among the q-th kDwThreads of the piece
+__device__ __forceinline__ bool dw_warp_live(int q, int cnt) {
+  return (int)(threadIdx.x & ~31u) + q * kDwThreads < cnt;
+}
+
 template <int R, int NT>
 __device__ __forceinline__ void dw_load_targets(const PairArgs<double>& A, int start, int cnt, DWTile<R, NT>& T) {
 #pragma unroll
   for (int q = 0; q < NT; ++q) {
-    int idx = threadIdx.x + q * kPairThreads;
+    int idx = threadIdx.x + q * kDwThreads;
     int node = start + (idx < cnt ? idx : cnt - 1);
     D4 p = A.tgt[node];
     T.x[0] = dw_split(p.x);
@@ -745,39 +764,45 @@ __device__ __forceinline__ void dw_load_targets(const PairArgs<double>& A, int s
 // Grid of a segment: on each axis the spacing 2^(e - 24) with 2^e above every |x - y| of the
 // segment (centre distance plus twice the radius), so high words on it subtract exactly.
 struct DwGrid {
-  double shift[3];  // source sphere's centre minus target sphere's
-  double m64[3];    // rounds a double to the grid: (y + m64) - m64
-  float m32[3];     // rounds |x| to the grid: (|x| + m32) - m32 (|x| < 2^(e-1) as 2^e > 2 a)
+  dw shift[3];   // source sphere's centre minus target sphere's
+  float m32[3];  // 2^(e-1): rounds |x| < 2^(e-1) to the grid as (|x| + m32) - m32
 };
 __device__ __forceinline__ DwGrid dw_grid(const PairArgs<double>& A, const CentreShift64& sh, int o) {
   DwGrid G;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    G.shift[q] = sh.d(o, q);
-    const float b = (float)fabs(G.shift[q]) * 1.0001f + A.span;
-    // the power of two above b (b is a normal number: at least twice the radius)
-    const float p2 = __int_as_float((__float_as_int(b) & 0x7f800000) + 0x00800000);
-    G.m32[q] = 0.5f * p2;
-    G.m64[q] = 402653184.0 * (double)p2;  // 1.5 2^52 2^-24 p2
+    G.shift[q] = dw_split(sh.d(o, q));
+    const float b = fabsf(G.shift[q].h) * 1.0001f + A.span;
+    // half the power of two above b (b is a normal number: at least the sphere's radius)
+    G.m32[q] = 0.5f * __int_as_float((__float_as_int(b) & 0x7f800000) + 0x00800000);
   }
   return G;
 }
-__device__ __forceinline__ void dw_stage_pos(const DwGrid& G, const D4 pr, float* sp, int i) {
-  const double rel[3] = {pr.x, pr.y, pr.z};
+// x rounded to the grid (a float of 2^(e-1) and above lies on it)
+__device__ __forceinline__ float dw_on_grid(float x, float m32) {
+  const float t = fabsf(x);
+  return copysignf(t >= m32 ? t : __fsub_rn(__fadd_rn(t, m32), m32), x);
+}
+// A proxy's position in the target's frame, in FP32 operations only: with the position and the strengths
+// held in double, the sums, splits and conversions of a source were about 25 FP64 operations, 12 clocks of
+// an SM's two FP64 lanes, where 64 targets spend about 84 clocks on a source.
+__device__ __forceinline__ void dw_stage_pos(const DwGrid& G, const float4 ph, const float4 pl, float* sp, int i) {
+  const float rh[3] = {ph.x, ph.y, ph.z}, rl[3] = {pl.x, pl.y, pl.z};
   float* o = sp + 12 * (i >> 1) + (i & 1);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    const double y = rel[q] + G.shift[q];
-    const double h = (y + G.m64[q]) - G.m64[q];
-    o[2 * q] = (float)h;
-    o[6 + 2 * q] = (float)(y - h);
+    const dw s = two_sum(rh[q], G.shift[q].h);
+    const float l = __fadd_rn(s.l, __fadd_rn(rl[q], G.shift[q].l));
+    const float h = dw_on_grid(s.h, G.m32[q]);
+    o[2 * q] = h;
+    o[6 + 2 * q] = __fadd_rn(__fsub_rn(s.h, h), l);
   }
 }
 __device__ __forceinline__ DwTarget dw_target(const DwGrid& G, const dw (&x)[3]) {
   DwTarget t;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    const float h = copysignf(__fsub_rn(__fadd_rn(fabsf(x[q].h), G.m32[q]), G.m32[q]), x[q].h);
+    const float h = dw_on_grid(x[q].h, G.m32[q]);
     const float l = __fadd_rn(__fsub_rn(x[q].h, h), x[q].l);
     t.h[q] = f2dup(h);
     t.l[q] = f2dup(l);
@@ -785,16 +810,11 @@ __device__ __forceinline__ DwTarget dw_target(const DwGrid& G, const dw (&x)[3])
   return t;
 }
 
-// whether this warp has a target among the q-th 128 of the tile
-__device__ __forceinline__ bool dw_warp_live(int q, int cnt) {
-  return (int)(threadIdx.x & ~31u) + q * kPairThreads < cnt;
-}
-
 // Proxy Stokeslets [r_lo, r_hi) of the flattened proxy index (sphere o = j / N, proxy j - o N; the
 // range holds none of the target sphere's own), one sphere at a time in rounds of at most TILE.
 template <int R, int NT, int TILE>
 __device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const CentreShift64& sh,
-                                               const double* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
+                                               const float2* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
                                                int cnt, float* sp, float (*sf)[6 * TILE], DWTile<R, NT>& T) {
   for (int s0 = r_lo; s0 < r_hi;) {
     const int o = s0 / A.N, j0 = s0 - o * A.N;
@@ -805,19 +825,19 @@ __device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const 
     const int nu = (ns + 1) >> 1;
     const DwGrid G = dw_grid(A, sh, o);
     __syncthreads();
-    for (int i = threadIdx.x; i < 2 * nu; i += kPairThreads) {
+    for (int i = threadIdx.x; i < 2 * nu; i += kDwThreads) {
       const int jj = j0 + min(i, ns - 1);
-      dw_stage_pos(G, A.proxy[jj], sp, i);
+      dw_stage_pos(G, A.proxy2[2 * jj], A.proxy2[2 * jj + 1], sp, i);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const bool on = i < ns && (mask >> r & 1u);  // the odd round's last slot carries no strength
-        const double* l = lam[r] + A.unk_off[o] + 3LL * jj;
+        const float2* l = lam[r] + A.unk_off[o] + 3LL * jj;
         float* f = sf[r] + 12 * (i >> 1) + (i & 1);
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-          const dw v = dw_split(on ? l[q] : 0.0);
-          f[2 * q] = v.h;
-          f[6 + 2 * q] = v.l;
+          const float2 v = on ? l[q] : make_float2(0.f, 0.f);
+          f[2 * q] = v.x;
+          f[6 + 2 * q] = v.y;
         }
       }
     }
@@ -874,7 +894,7 @@ __device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const 
 // Strengths per right-hand side and pair of nodes: f, t, -q and 3 q, high and low words.
 template <int R, int NT, int TILE>
 __device__ __forceinline__ void dw_image_range(const PairArgs<double>& A, const CentreShift64& sh,
-                                               const double* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
+                                               const float2* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
                                                int cnt, float* sp, float (*si)[24 * TILE], DWTile<R, NT>& T) {
   for (int s0 = r_lo; s0 < r_hi;) {
     const int o = A.img_owner[s0];
@@ -883,7 +903,7 @@ __device__ __forceinline__ void dw_image_range(const PairArgs<double>& A, const 
     const int nu = (ns + 1) >> 1;
     const double shift[3] = {sh.d(o, 0), sh.d(o, 1), sh.d(o, 2)};
     __syncthreads();
-    for (int i = threadIdx.x; i < 2 * nu; i += kPairThreads) {
+    for (int i = threadIdx.x; i < 2 * nu; i += kDwThreads) {
       const int j = s0 + min(i, ns - 1);
       {
         const D4 pr = A.img[j];
@@ -899,12 +919,13 @@ __device__ __forceinline__ void dw_image_range(const PairArgs<double>& A, const 
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const bool on = i < ns && (mask >> r & 1u);
-        const double* l = lam[r] + A.unk_off[o] + 3LL * A.N + 9LL * (j - first);
+        const float2* l = lam[r] + A.unk_off[o] + 3LL * A.N + 9LL * (j - first);
+        auto at = [&](int c) { return on ? (double)l[c].x + (double)l[c].y : 0.0; };
         float* f = si[r] + 48 * (i >> 1) + (i & 1);
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-          const double d = on ? A.dip * l[6 + q] : 0.0;
-          const double v[4] = {on ? l[q] : 0.0, on ? l[3 + q] : 0.0, -d, 3.0 * d};
+          const double d = A.dip * at(6 + q);
+          const double v[4] = {at(q), at(3 + q), -d, 3.0 * d};
 #pragma unroll
           for (int w = 0; w < 4; ++w) {
             const dw s = dw_split(v[w]);
@@ -989,7 +1010,7 @@ __device__ __forceinline__ void dw_write_out(const PairArgs<double>& A, int star
                                              int nparts, double* __restrict__ partial, long long pstride) {
 #pragma unroll
   for (int q = 0; q < NT; ++q) {
-    int idx = threadIdx.x + q * kPairThreads;
+    int idx = threadIdx.x + q * kDwThreads;
     if (idx < cnt) {
       const long long node = start + idx;
       const double sw = A.tgt[node].w;
@@ -1019,7 +1040,7 @@ struct DwShared {
 // partial[part * pstride + 3 node + c] for pair_parts_reduce to finish.
 template <int R, int NT, int TILE, int TILE_IMG>
 __device__ __forceinline__ void dw_all_sources(const PairArgs<double>& A, const CentreShift64& sh, int k,
-                                               const double* const (&lam)[R], unsigned mask, int cnt, int part,
+                                               const float2* const (&lam)[R], unsigned mask, int cnt, int part,
                                                int nparts, DwShared<R, TILE, TILE_IMG>& S, DWTile<R, NT>& T) {
   // the proxies before and after sphere k's own (this part's share of them)
   const int total = A.P * A.N;
@@ -1037,12 +1058,11 @@ __device__ __forceinline__ void dw_all_sources(const PairArgs<double>& A, const 
 }
 
 template <int NT>
-__device__ __forceinline__ void pair_tile_dw(const PairArgs<double>& A, const int t, const int part, const int nparts,
-                                             double* __restrict__ partial, const long long pstride) {
+__device__ __forceinline__ void pair_tile_dw(const PairArgs<double>& A, const int t, const int start, const int cnt,
+                                             const int part, const int nparts, double* __restrict__ partial,
+                                             const long long pstride) {
   __shared__ DwShared<1, kDwTile, kDwTileImg> S;
   const int k = A.tile_sphere[t];
-  const int start = A.tile_start[t];
-  const int cnt = A.tile_count[t];
   CentreShift64 sh;
   sh.cen = A.cen64;
   sh.init(k);
@@ -1052,7 +1072,7 @@ __device__ __forceinline__ void pair_tile_dw(const PairArgs<double>& A, const in
     T.c = &C;
   }
   dw_load_targets<1, NT>(A, start, cnt, T);
-  const double* const lam[1] = {A.lam};
+  const float2* const lam[1] = {A.lam2};
   dw_all_sources<1, NT, kDwTile, kDwTileImg>(A, sh, k, lam, 1u, cnt, part, nparts, S, T);
   dw_write_out<1, NT>(A, start, cnt, T, 0, A.mu, A.out, part, nparts, partial, pstride);
 }
@@ -1061,13 +1081,11 @@ __device__ __forceinline__ void pair_tile_dw(const PairArgs<double>& A, const in
 // (ascending; runs of consecutive spheres are taken as one range).
 template <int NT>
 __device__ __forceinline__ void pair_tile_dw_near(const PairArgs<double>& A, const int* __restrict__ near_off,
-                                                  const int* __restrict__ near_idx, const int t, const int part,
-                                                  const int nparts, double* __restrict__ partial,
-                                                  const long long pstride) {
+                                                  const int* __restrict__ near_idx, const int t, const int start,
+                                                  const int cnt, const int part, const int nparts,
+                                                  double* __restrict__ partial, const long long pstride) {
   __shared__ DwShared<1, kDwTile, kDwTileImg> S;
   const int k = A.tile_sphere[t];
-  const int start = A.tile_start[t];
-  const int cnt = A.tile_count[t];
   CentreShift64 sh;
   sh.cen = A.cen64;
   sh.init(k);
@@ -1077,7 +1095,7 @@ __device__ __forceinline__ void pair_tile_dw_near(const PairArgs<double>& A, con
     T.c = &C;
   }
   dw_load_targets<1, NT>(A, start, cnt, T);
-  const double* const lam[1] = {A.lam};
+  const float2* const lam[1] = {A.lam2};
   // this part's share of the near list
   const int b0 = near_off[k], nn = near_off[k + 1] - b0;
   const int a1 = b0 + (int)((long long)nn * (part + 1) / nparts);
@@ -1377,10 +1395,17 @@ __device__ __forceinline__ void parts_finish_nodes(const D4* tgt, long long star
     out[e] = mu[e] + tgt[start + i / 3].w * sum;
   }
 }
-__device__ __forceinline__ void parts_finish_tile(const PairArgs<double>& A, int t, int nparts, const double* partial,
-                                                  long long pstride, unsigned* counter) {
-  if (!parts_last_arrival(counter, t, nparts)) return;
-  const int start = A.tile_start[t], cnt = A.tile_count[t];
+
+// The piece of a tile that work item `item` = tile x kDwPieces + piece takes; false if it has no targets.
+template <int NT>
+__device__ __forceinline__ bool dw_piece(const PairArgs<double>& A, int t, int piece, int& start, int& cnt) {
+  start = A.tile_start[t] + piece * kDwThreads * NT;
+  cnt = min(kDwThreads * NT, A.tile_count[t] - piece * kDwThreads * NT);
+  return cnt > 0;
+}
+__device__ __forceinline__ void parts_finish_piece(const PairArgs<double>& A, int item, int start, int cnt, int nparts,
+                                                   const double* partial, long long pstride, unsigned* counter) {
+  if (!parts_last_arrival(counter, item, nparts)) return;
   parts_finish_nodes(A.tgt, start, cnt, nparts, partial, pstride, A.mu, A.out);
 }
 
@@ -1408,19 +1433,23 @@ __global__ void __launch_bounds__(kPairThreads) velocity_fp64_kernel(PairArgs<do
   for (int c = 0; c < 3; ++c) u[part * pstride + 3 * i + c] = v[c];
 }
 template <int NT>
-__global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_kernel(PairArgs<double> A, int nparts, double* partial,
+__global__ void __launch_bounds__(kDwThreads, kDwCtas) pairs_dw_kernel(PairArgs<double> A, int nparts, double* partial,
                                                                 long long pstride, unsigned* counter) {
-  const int t = blockIdx.x / nparts;
-  pair_tile_dw<NT>(A, t, blockIdx.x % nparts, nparts, partial, pstride);
-  if (nparts > 1) parts_finish_tile(A, t, nparts, partial, pstride, counter);
+  const int item = blockIdx.x / nparts, t = item / kDwPieces;
+  int start, cnt;
+  if (!dw_piece<NT>(A, t, item % kDwPieces, start, cnt)) return;
+  pair_tile_dw<NT>(A, t, start, cnt, blockIdx.x % nparts, nparts, partial, pstride);
+  if (nparts > 1) parts_finish_piece(A, item, start, cnt, nparts, partial, pstride, counter);
 }
 template <int NT>
-__global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_near_kernel(PairArgs<double> A, const int* near_off,
+__global__ void __launch_bounds__(kDwThreads, kDwCtas) pairs_dw_near_kernel(PairArgs<double> A, const int* near_off,
                                                                      const int* near_idx, int nparts, double* partial,
                                                                      long long pstride, unsigned* counter) {
-  const int t = blockIdx.x / nparts;
-  pair_tile_dw_near<NT>(A, near_off, near_idx, t, blockIdx.x % nparts, nparts, partial, pstride);
-  if (nparts > 1) parts_finish_tile(A, t, nparts, partial, pstride, counter);
+  const int item = blockIdx.x / nparts, t = item / kDwPieces;
+  int start, cnt;
+  if (!dw_piece<NT>(A, t, item % kDwPieces, start, cnt)) return;
+  pair_tile_dw_near<NT>(A, near_off, near_idx, t, start, cnt, blockIdx.x % nparts, nparts, partial, pstride);
+  if (nparts > 1) parts_finish_piece(A, item, start, cnt, nparts, partial, pstride, counter);
 }
 // out = mu + sqrt(w) * (sum of the parts), or the plain sum when mu is null; parts added in order
 __global__ void pair_parts_reduce_kernel(long long n3, const D4* __restrict__ tgt, int nparts,
@@ -1436,7 +1465,8 @@ __global__ void pair_parts_reduce_kernel(long long n3, const D4* __restrict__ tg
 // The per-problem vectors are segments of concatenated ones: lam at lam + uoff[p], mu and out
 // at mu + voff[p], out + voff[p].
 struct BatchVecs {
-  const double* lam;
+  const double* lam;    // native FP64 kernel
+  const float2* lam2;   // double-float kernels
   const double* mu;
   double* out;
   const long long* uoff;
@@ -1444,8 +1474,8 @@ struct BatchVecs {
   double* partial;     // split sources: nparts slices of the concatenated vector length
   long long pstride;
   const long long* nlen;  // node rows (3 n_colloc) of each problem; a mobility problem's border follows
-  unsigned* counter;      // optional, zeros, one per work item: with split sources the last CTA of an
-                          // item adds the parts (in part order) itself and re-arms its counter
+  unsigned* counter;      // double-float: zeros, one per piece of a work item; with split sources the
+                          // last CTA of a piece adds the parts (in part order) and re-arms its counter
 };
 
 // native FP64: each (problem, 128-node tile) in four pieces; with split sources the parts are added
@@ -1462,24 +1492,22 @@ __global__ void __launch_bounds__(kPairThreads, 4) pairs_fp64_batch_kernel(const
   A.out = bv.out + bv.voff[w.x];
   pair_piece_fp64(A, w.y, blockIdx.x % 4, blockIdx.x / 4 % nparts, nparts, bv.partial + bv.voff[w.x], bv.pstride);
 }
-template <int NT>
-__global__ void __launch_bounds__(kPairThreads, kDwCtas) pairs_dw_batch_kernel(const PairArgs<double>* __restrict__ args,
+__global__ void __launch_bounds__(kDwThreads, kDwCtas) pairs_dw_batch_kernel(const PairArgs<double>* __restrict__ args,
                                                                       const int2* __restrict__ work,
                                                                       const int* __restrict__ active, BatchVecs bv,
                                                                       int nparts) {
-  const int2 w = work[blockIdx.x / nparts];
+  const int item = blockIdx.x / nparts;
+  const int2 w = work[item / kDwPieces];
   if (!active[w.x]) return;
   PairArgs<double> A = args[w.x];
-  A.lam = bv.lam + bv.uoff[w.x];
+  A.lam2 = bv.lam2 + bv.uoff[w.x];
   A.mu = bv.mu + bv.voff[w.x];
   A.out = bv.out + bv.voff[w.x];
-  pair_tile_dw<NT>(A, w.y, blockIdx.x % nparts, nparts, bv.partial + bv.voff[w.x], bv.pstride);
-  if constexpr (NT == 1) {  // only the 1-node tiling splits sources
-    if (nparts > 1 && bv.counter && parts_last_arrival(bv.counter, blockIdx.x / nparts, nparts)) {
-      parts_finish_nodes(A.tgt, A.tile_start[w.y], A.tile_count[w.y], nparts, bv.partial + bv.voff[w.x], bv.pstride,
-                         A.mu, A.out);
-    }
-  }
+  int start, cnt;
+  if (!dw_piece<1>(A, w.y, item % kDwPieces, start, cnt)) return;
+  pair_tile_dw<1>(A, w.y, start, cnt, blockIdx.x % nparts, nparts, bv.partial + bv.voff[w.x], bv.pstride);
+  if (nparts > 1)
+    parts_finish_piece(A, item, start, cnt, nparts, bv.partial + bv.voff[w.x], bv.pstride, bv.counter);
 }
 // ------------------------------------------------------------------ several right-hand sides on one geometry
 // The problems of a batch that share a context (the motions of one geometry) have the same
@@ -1495,13 +1523,14 @@ constexpr int kDwTileImgM = 32;  // image nodes staged per round
 // work[b] = (lead problem, tile of the 1-node-per-thread tiling, first index into rhs_prob, count);
 // the sources are split over nparts CTAs per item as in pairs_dw_batch_kernel
 template <int R>
-__global__ void __launch_bounds__(kPairThreads, 3) pairs_dw_multi_kernel(const PairArgs<double>* __restrict__ args,
+__global__ void __launch_bounds__(kDwThreads, kDwMultiCtas) pairs_dw_multi_kernel(const PairArgs<double>* __restrict__ args,
                                                                       const int4* __restrict__ work,
                                                                       const int* __restrict__ rhs_prob,
                                                                       const int* __restrict__ active, BatchVecs bv,
                                                                       int nparts) {
   __shared__ DwShared<R, kDwTileM, kDwTileImgM> S;
-  const int4 w = work[blockIdx.x / nparts];
+  const int item = blockIdx.x / nparts;
+  const int4 w = work[item / kDwPieces];
   const int part = blockIdx.x % nparts;
   int prob[R];
   unsigned mask = 0;
@@ -1512,13 +1541,13 @@ __global__ void __launch_bounds__(kPairThreads, 3) pairs_dw_multi_kernel(const P
   }
   if (!mask) return;
   const PairArgs<double> A = args[w.x];
-  const double* lam[R];
+  const float2* lam[R];
 #pragma unroll
-  for (int r = 0; r < R; ++r) lam[r] = bv.lam + bv.uoff[prob[r]];
+  for (int r = 0; r < R; ++r) lam[r] = bv.lam2 + bv.uoff[prob[r]];
   const int t = w.y;
   const int k = A.tile_sphere[t];
-  const int start = A.tile_start[t];
-  const int cnt = A.tile_count[t];
+  int start, cnt;
+  if (!dw_piece<1>(A, t, item % kDwPieces, start, cnt)) return;
   CentreShift64 sh;
   sh.cen = A.cen64;
   sh.init(k);
@@ -1531,7 +1560,7 @@ __global__ void __launch_bounds__(kPairThreads, 3) pairs_dw_multi_kernel(const P
     const long long off = bv.voff[prob[r]];
     dw_write_out<R, 1>(A, start, cnt, T, r, bv.mu + off, bv.out + off, part, nparts, bv.partial + off, bv.pstride);
   }
-  if (nparts > 1 && bv.counter && parts_last_arrival(bv.counter, blockIdx.x / nparts, nparts)) {
+  if (nparts > 1 && parts_last_arrival(bv.counter, item, nparts)) {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if (!(mask >> r & 1u)) continue;
@@ -1718,7 +1747,7 @@ __device__ __forceinline__ void gemv_step(GemvAcc& a, f2x mh, f2x ml, float2 xe)
 constexpr int kGemvPairThreads = 128;
 constexpr int kGemvMaxRhs = 4;
 
-template <bool F32, bool OUT64, int C, int RP, int KS>
+template <bool F32, int C, int RP, int KS>
 __device__ __forceinline__ void gemv_pairs(const GemvBatch<float>& B, const int* job, int rp0,
                                            const float2* __restrict__ x, float2* __restrict__ y2,
                                            double* __restrict__ y64) {
@@ -1805,8 +1834,8 @@ __device__ __forceinline__ void gemv_pairs(const GemvBatch<float>& B, const int*
     if (lane < 2 && row < nr) {
       const dw w = lane == 0 ? dw{h0, l0} : dw{h1, l1};
       const long long idx = y_off + row;
-      if (OUT64) y64[idx] = dw_join(w);
-      else y2[idx] = make_float2(w.h, w.l);
+      if (y64) y64[idx] = dw_join(w);
+      if (y2) y2[idx] = make_float2(w.h, w.l);
     }
   };
   auto value = [&](int r, int q) {
@@ -1851,7 +1880,7 @@ __device__ __forceinline__ void gemv_pairs(const GemvBatch<float>& B, const int*
 // row pairs a warp (KS 1) or the CTA (KS 4: its warps share the columns) takes at once
 __host__ __device__ constexpr int gemv_rp(int c) { return c == 1 ? 1 : 2; }
 // work item blockIdx.x: the right-hand sides list[item.x .. item.x + item.y) of one matrix
-template <bool F32, bool OUT64, int CMAX, int KS>
+template <bool F32, int CMAX, int KS>
 __global__ void __launch_bounds__(kGemvPairThreads, CMAX == 1 ? 10 : 1) gemv_pair_kernel(GemvBatch<float> B, const float2* __restrict__ x,
                                                                    float2* __restrict__ y2, double* __restrict__ y64) {
   constexpr int RP = gemv_rp(CMAX);
@@ -1867,9 +1896,9 @@ __global__ void __launch_bounds__(kGemvPairThreads, CMAX == 1 ? 10 : 1) gemv_pai
   }
   if (!any || 2 * rp0 >= B.rows[job[0]]) return;
   // (three of four run as four with the last one twice: the same value written twice)
-  if (CMAX > 1 && it.y == 1) gemv_pairs<F32, OUT64, 1, RP, KS>(B, job, rp0, x, y2, y64);
-  else if (CMAX > 2 && it.y == 2) gemv_pairs<F32, OUT64, 2, RP, KS>(B, job, rp0, x, y2, y64);
-  else gemv_pairs<F32, OUT64, CMAX, RP, KS>(B, job, rp0, x, y2, y64);
+  if (CMAX > 1 && it.y == 1) gemv_pairs<F32, 1, RP, KS>(B, job, rp0, x, y2, y64);
+  else if (CMAX > 2 && it.y == 2) gemv_pairs<F32, 2, RP, KS>(B, job, rp0, x, y2, y64);
+  else gemv_pairs<F32, CMAX, RP, KS>(B, job, rp0, x, y2, y64);
 }
 
 __global__ void split_dw_kernel(long long n, const double* __restrict__ in, float2* __restrict__ out) {
@@ -2451,7 +2480,7 @@ void launch_pairs_f32(const TargetSet& tg, const SourceSet& src, const float* la
 int fp64_split_parts(long long pieces, long long min_sources, int max_parts) {
   if (pieces <= 0) return 1;
   long long s = (kFp64SplitTarget + pieces - 1) / pieces;
-  s = std::min<long long>(s, min_sources / kPairSplitMinSources);
+  s = std::min<long long>(s, min_sources / kFp64SplitMinSources);
   s = std::min<long long>(s, max_parts);
   return (int)std::max<long long>(s, 1);
 }
@@ -2489,14 +2518,6 @@ void launch_velocity(int n, const double* x, const SourceSet& src, const double*
   }
 }
 
-int pair_split_parts(long long n_tiles1, long long min_sources, int max_parts) {
-  if (n_tiles1 <= 0) return 1;
-  long long s = (kPairSplitTarget + n_tiles1 - 1) / n_tiles1;
-  s = std::min<long long>(s, min_sources / kPairSplitMinSources);
-  s = std::min<long long>(s, max_parts);
-  return (int)std::max<long long>(s, 1);
-}
-
 // nodes per thread of a launch: the requested shape, else the rule (512-node tiles once they fill
 // the GPU twice; 128-node tiles only when they exist)
 static int shape_nt(const TargetSet& tg, const PairShape& shape) {
@@ -2505,31 +2526,9 @@ static int shape_nt(const TargetSet& tg, const PairShape& shape) {
   return pair_nodes_per_thread(tg.n_tiles);
 }
 
-PairShape resolve_dw_shape(const TargetSet& tg, const SourceSet& src, PairShape shape, int max_parts) {
-  PairShape r;
-  r.nt = shape_nt(tg, shape);
-  if (shape.parts > 0) r.parts = std::min(shape.parts, max_parts);
-  else r.parts = pair_split_parts(r.nt == 4 ? tg.n_tiles : tg.n_tiles1, (long long)(src.P - 1) * src.N, max_parts);
-  return r;
-}
-
-void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const double* lam_hat, const double* mu, double* out,
-                     double visc, double* partial, unsigned* counter, int max_parts, cudaStream_t st, PairShape shape) {
-  if (tg.n_tiles == 0) return;
-  const PairShape r = resolve_dw_shape(tg, src, shape, max_parts);
-  const int nt = r.nt;
-  const int parts = partial ? r.parts : 1;
-  PairArgs<double> A = make_args<double>(tg, src, lam_hat, mu, out, visc, nt);
-  const long long n3 = 3LL * tg.n;
-  ++t_launches;
-  // (with split sources the last CTA of a tile to finish adds the parts)
-  if (nt == 4) pairs_dw_kernel<4><<<tg.n_tiles * parts, kPairThreads, 0, st>>>(A, parts, partial, n3, counter);
-  else pairs_dw_kernel<1><<<tg.n_tiles1 * parts, kPairThreads, 0, st>>>(A, parts, partial, n3, counter);
-}
-
 // resident CTAs of a pair kernel on the current device (SMs x CTAs per SM), looked up once per
 // (device, kernel)
-static double resident_ctas(const void* kernel) {
+static double resident_ctas(const void* kernel, int threads = kPairThreads) {
   static std::mutex mtx;
   static std::vector<std::pair<std::pair<int, const void*>, double>> cache;
   int dev = 0;
@@ -2542,7 +2541,7 @@ static double resident_ctas(const void* kernel) {
     if (e.first.first == dev && e.first.second == kernel) return e.second;
   int per_sm = 0, sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kPairThreads, 0) != cudaSuccess || per_sm < 1) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     return 0;
   }
@@ -2550,9 +2549,51 @@ static double resident_ctas(const void* kernel) {
   return cache.back().second;
 }
 
+// (see the declaration)
+static int pair_split_parts(long long items, double wave, long long min_sources, int max_parts) {
+  if (items <= 0 || wave <= 0 || min_sources <= 0) return 1;
+  const int most = (int)std::max<long long>(1, std::min<long long>(max_parts, min_sources / kPairSplitMinSources));
+  int best = 1;
+  double best_t = 0;
+  for (int p = 1; p <= most; ++p) {
+    const double t = std::ceil((double)items * p / wave) * (1.0 / p + kPairSplitPartCost / (double)min_sources);
+    if (p == 1 || t < best_t) {
+      best_t = t;
+      best = p;
+    }
+  }
+  return best;
+}
+
+PairShape resolve_dw_shape(const TargetSet& tg, const SourceSet& src, PairShape shape, int max_parts) {
+  PairShape r;
+  // one node per thread unless four are asked for: 100 spheres of 1804 nodes 116.1 against 127.4 ms
+  r.nt = shape.nt == 4 || tg.n_tiles1 == 0 ? 4 : 1;
+  if (shape.parts > 0) r.parts = std::min(shape.parts, max_parts);
+  else r.parts = pair_split_parts(r.nt == 4 ? tg.n_pieces4 : tg.n_pieces1,
+                                  resident_ctas(r.nt == 4 ? (const void*)pairs_dw_kernel<4> : (const void*)pairs_dw_kernel<1>, kDwThreads),
+                                  (long long)(src.P - 1) * src.N, max_parts);
+  return r;
+}
+
+void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const float2* lam_hat, const double* mu, double* out,
+                     double visc, double* partial, unsigned* counter, int max_parts, cudaStream_t st, PairShape shape) {
+  if (tg.n_tiles == 0) return;
+  const PairShape r = resolve_dw_shape(tg, src, shape, max_parts);
+  const int nt = r.nt;
+  const int parts = partial ? r.parts : 1;
+  PairArgs<double> A = make_args<double>(tg, src, nullptr, mu, out, visc, nt);
+  A.lam2 = lam_hat;
+  const long long n3 = 3LL * tg.n;
+  ++t_launches;
+  // (with split sources the last CTA of a tile to finish adds the parts)
+  if (nt == 4) pairs_dw_kernel<4><<<kDwPieces * tg.n_tiles * parts, kDwThreads, 0, st>>>(A, parts, partial, n3, counter);
+  else pairs_dw_kernel<1><<<kDwPieces * tg.n_tiles1 * parts, kDwThreads, 0, st>>>(A, parts, partial, n3, counter);
+}
+
 // source parts per tile so that tiles x parts fill whole waves of the resident CTAs (ties: fewer)
-int wave_parts(long long tiles, const void* kernel, int max_parts) {
-  const double wave = resident_ctas(kernel);
+int wave_parts(long long tiles, const void* kernel, int max_parts, int threads = kPairThreads) {
+  const double wave = resident_ctas(kernel, threads);
   if (wave <= 0) return 1;
   int best = 1;
   double best_eff = 0;
@@ -2572,26 +2613,27 @@ PairShape resolve_near_shape(const TargetSet& tg, PairShape shape, int max_parts
   r.nt = shape_nt(tg, shape);
   const long long tiles = r.nt == 4 ? tg.n_tiles : tg.n_tiles1;
   r.parts = shape.parts > 0 ? std::min(shape.parts, max_parts)
-                            : wave_parts(tiles, r.nt == 4 ? (const void*)pairs_dw_near_kernel<4>
-                                                          : (const void*)pairs_dw_near_kernel<1>, max_parts);
+                            : wave_parts(kDwPieces * tiles, r.nt == 4 ? (const void*)pairs_dw_near_kernel<4>
+                                                                      : (const void*)pairs_dw_near_kernel<1>, max_parts, kDwThreads);
   return r;
 }
 
-void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarField& ff, const double* lam_hat,
+void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarField& ff, const float2* lam_hat,
                           const double* mu, double* out, double visc, double* partial, unsigned* counter, int max_parts,
                           cudaStream_t st, PairShape shape) {
   if (tg.n_tiles == 0) return;
   const PairShape r = resolve_near_shape(tg, shape, max_parts);
   const int nt = r.nt;
-  PairArgs<double> A = make_args<double>(tg, src, lam_hat, mu, out, visc, nt);
+  PairArgs<double> A = make_args<double>(tg, src, nullptr, mu, out, visc, nt);
+  A.lam2 = lam_hat;
   const long long tiles = nt == 4 ? tg.n_tiles : tg.n_tiles1;
   const int parts = partial ? r.parts : 1;
   const long long n3 = 3LL * tg.n;
   ++t_launches;
   if (nt == 4)
-    pairs_dw_near_kernel<4><<<tiles * parts, kPairThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3, counter);
+    pairs_dw_near_kernel<4><<<kDwPieces * tiles * parts, kDwThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3, counter);
   else
-    pairs_dw_near_kernel<1><<<tiles * parts, kPairThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3, counter);
+    pairs_dw_near_kernel<1><<<kDwPieces * tiles * parts, kDwThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3, counter);
 }
 
 PairShape resolve_far_shape(const TargetSet& tg, PairShape shape, int max_parts) {
@@ -2649,29 +2691,18 @@ void fill_pair_args64(void* host_dst, const TargetSet& tg, const SourceSet& src,
 }
 
 void launch_pairs_batch64(bool double_float, const void* d_args, const int2* d_work, int n_work, const int* d_active,
-                          int nodes_per_thread, const double* lam, const double* mu, double* out,
+                          const double* lam, const float2* lam2, const double* mu, double* out,
                           const long long* d_uoff, const long long* d_voff, int parts, double* partial,
                           long long pstride, const SegTable& seg, cudaStream_t st, const long long* d_nlen,
-                          bool skip_reduce, unsigned* d_counter) {
+                          unsigned* d_counter) {
   if (n_work == 0) return;
   const PairArgs<double>* args = static_cast<const PairArgs<double>*>(d_args);
-  BatchVecs bv{lam, mu, out, d_uoff, d_voff, partial, pstride, d_nlen, d_counter};
-  if (d_counter) skip_reduce = true;  // the last CTA of each item adds the parts
+  BatchVecs bv{lam, lam2, mu, out, d_uoff, d_voff, partial, pstride, d_nlen, d_counter};
+  if (!partial) parts = 1;
   ++t_launches;
-  if (double_float) {
-    if (nodes_per_thread == 4) {
-      pairs_dw_batch_kernel<4><<<n_work, kPairThreads, 0, st>>>(args, d_work, d_active, bv, 1);
-    } else {
-      if (!partial) parts = 1;
-      pairs_dw_batch_kernel<1><<<n_work * parts, kPairThreads, 0, st>>>(args, d_work, d_active, bv, parts);
-      if (parts > 1 && !skip_reduce) {
-        ++t_launches;
-        if (seg_ctas(seg) > 0)
-          pair_parts_reduce_batch_kernel<<<dim3(seg_ctas(seg), (seg.chunk + 127) / 128), 128, 0, st>>>(seg, args, bv, parts);
-      }
-    }
+  if (double_float) {  // with split sources the last CTA of each item adds the parts
+    pairs_dw_batch_kernel<<<kDwPieces * n_work * parts, kDwThreads, 0, st>>>(args, d_work, d_active, bv, parts);
   } else {
-    if (!partial) parts = 1;
     pairs_fp64_batch_kernel<<<4 * n_work * parts, kPairThreads, 0, st>>>(args, d_work, d_active, bv, parts);
     if (parts > 1) {
       ++t_launches;
@@ -2681,26 +2712,22 @@ void launch_pairs_batch64(bool double_float, const void* d_args, const int2* d_w
   }
 }
 
+int batch_split_parts(long long items, bool shared_rhs, long long min_sources, int max_parts) {
+  return pair_split_parts(items, resident_ctas(shared_rhs ? (const void*)pairs_dw_multi_kernel<kPairRhs>
+                                                                      : (const void*)pairs_dw_batch_kernel, kDwThreads),
+                          min_sources, max_parts);
+}
+
 void launch_pairs_multi64(const void* d_args1, const int4* d_work, int n_work, const int* d_rhs, const int* d_active,
-                          const double* lam, const double* mu, double* out, const long long* d_uoff,
+                          const float2* lam2, const double* mu, double* out, const long long* d_uoff,
                           const long long* d_voff, int parts, double* partial, long long pstride,
                           const long long* d_nlen, cudaStream_t st, unsigned* d_counter) {
   if (n_work == 0) return;
   if (!partial) parts = 1;
   const PairArgs<double>* args = static_cast<const PairArgs<double>*>(d_args1);
-  BatchVecs bv{lam, mu, out, d_uoff, d_voff, partial, pstride, d_nlen, d_counter};
+  BatchVecs bv{nullptr, lam2, mu, out, d_uoff, d_voff, partial, pstride, d_nlen, d_counter};
   ++t_launches;
-  pairs_dw_multi_kernel<kPairRhs><<<n_work * parts, kPairThreads, 0, st>>>(args, d_work, d_rhs, d_active, bv, parts);
-}
-
-void launch_pair_parts_reduce_batch(const void* d_args1, const SegTable& seg, const double* lam, const double* mu,
-                                    double* out, const long long* d_uoff, const long long* d_voff, int parts,
-                                    double* partial, long long pstride, const long long* d_nlen, cudaStream_t st) {
-  if (parts <= 1 || seg_ctas(seg) == 0) return;
-  const PairArgs<double>* args = static_cast<const PairArgs<double>*>(d_args1);
-  BatchVecs bv{lam, mu, out, d_uoff, d_voff, partial, pstride, d_nlen, nullptr};
-  ++t_launches;
-  pair_parts_reduce_batch_kernel<<<dim3(seg_ctas(seg), (seg.chunk + 127) / 128), 128, 0, st>>>(seg, args, bv, parts);
+  pairs_dw_multi_kernel<kPairRhs><<<kDwPieces * n_work * parts, kDwThreads, 0, st>>>(args, d_work, d_rhs, d_active, bv, parts);
 }
 
 void launch_seg_dots(const SegTable& t, int nvec, const double* V, long long ldv, const double* w, double* partial,
@@ -2791,7 +2818,7 @@ int gemv_items(int n, const int* list, const void* const* mat, std::vector<int2>
   return most;
 }
 
-template <bool F32, bool OUT64>
+template <bool F32>
 static void gemv_pair_launch(const GemvBatch<float>& b, const float2* x, float2* y2, double* y64, cudaStream_t st) {
   if (b.n_items == 0 || b.max_rows == 0) return;
   ++t_launches;
@@ -2801,7 +2828,7 @@ static void gemv_pair_launch(const GemvBatch<float>& b, const float2* x, float2*
   // groups than 64 warps a SM, and take a group each above that
   const bool split = c == 1 || (long long)b.n_items * groups < 64LL * 152;
   const dim3 grid(b.n_items, split ? groups : (groups + 3) / 4);
-#define MFS_GEMV(C, KS) gemv_pair_kernel<F32, OUT64, C, KS><<<grid, kGemvPairThreads, 0, st>>>(b, x, y2, y64)
+#define MFS_GEMV(C, KS) gemv_pair_kernel<F32, C, KS><<<grid, kGemvPairThreads, 0, st>>>(b, x, y2, y64)
   switch (c) {
     case 1: MFS_GEMV(1, 4); break;
     case 2: if (split) MFS_GEMV(2, 4); else MFS_GEMV(2, 1); break;
@@ -2812,12 +2839,11 @@ static void gemv_pair_launch(const GemvBatch<float>& b, const float2* x, float2*
 }
 
 void launch_gemv_dw(const GemvBatch<float>& b, const float2* x, float2* y_dw, double* y64, cudaStream_t st) {
-  if (y_dw) gemv_pair_launch<false, false>(b, x, y_dw, nullptr, st);
-  else gemv_pair_launch<false, true>(b, x, nullptr, y64, st);
+  gemv_pair_launch<false>(b, x, y_dw, y64, st);
 }
 
 void launch_gemv_f32_dw(const GemvBatch<float>& b, const float2* x, float2* y_dw, cudaStream_t st) {
-  gemv_pair_launch<true, false>(b, x, y_dw, nullptr, st);
+  gemv_pair_launch<true>(b, x, y_dw, nullptr, st);
 }
 
 void launch_split_dw(long long n, const double* in, float2* out, cudaStream_t st) {
@@ -2833,7 +2859,6 @@ void launch_multidot(int n, int nvec, const T* V, long long ldv, const T* w, dou
   multidot_kernel<T><<<grid, kRedThreads, 0, st>>>(n, V, ldv, w, partial, nblk);
 }
 template void launch_multidot<float>(int, int, const float*, long long, const float*, double*, int, cudaStream_t);
-template void launch_multidot<double>(int, int, const double*, long long, const double*, double*, int, cudaStream_t);
 
 void launch_reduce_partials(int nvec, int nblk, const double* partial, double* h, cudaStream_t st) {
   ++t_launches;
