@@ -650,7 +650,12 @@ __device__ __forceinline__ void dw_geometry(const DwTarget& T, const ulonglong2 
   const f2x t = f2add(f2add(f2fma(g.p[0], g.p[0], f2sub(mtwo, a1)), f2fma(g.p[1], g.p[1], f2sub(a1, a2))),
                       f2fma(g.p[2], g.p[2], f2sub(a2, a3)));
   const f2x nq = f2fma(g.np[2], g.l[2], f2fma(g.np[1], g.l[1], f2mul(g.np[0], g.l[0])));
-  const f2x e = f2fma(mhalf, f2add(f2add(a3, f2dup(1.0f)), t), nq);
+  const f2x e0 = f2fma(mhalf, f2add(f2add(a3, f2dup(1.0f)), t), nq);
+  // 1/|p + l| = 1 + e + 3/2 e^2 + ..: s is off by up to ~2e-7, so the second term reaches 6e-14, always of
+  // one sign and up to five times over in an image triple's third powers of 1/r; there it is kept (largest
+  // error of 31 proxies and 2 images a sphere 1.07e-13 -> 5.2e-14 of the absolute sum).  A Stokeslet's
+  // share of it is below the sums' other roundings (the same errors with it, 0.9 % of the time).
+  const f2x e = GRID ? e0 : f2fma(f2mul(e0, f2dup(1.5f)), e0, e0);
   g.il = f2mul(g.s, e);
 #pragma unroll
   for (int q = 0; q < 3; ++q) g.l[q] = f2fma(g.p[q], e, g.l[q]);
@@ -1037,7 +1042,7 @@ struct DwShared {
 // Sources may be split over `nparts` CTAs per target tile (when there are too few tiles to
 // fill the GPU): part `part` takes a contiguous share of the tile's source list (the sources of
 // every other sphere) and, for nparts > 1, writes its scaled partial sum to
-// partial[part * pstride + 3 node + c] for pair_parts_reduce to finish.
+// partial[part * pstride + 3 node + c] for the last part's CTA to add.
 template <int R, int NT, int TILE, int TILE_IMG>
 __device__ __forceinline__ void dw_all_sources(const PairArgs<double>& A, const CentreShift64& sh, int k,
                                                const float2* const (&lam)[R], unsigned mask, int cnt, int part,
@@ -1514,8 +1519,8 @@ __global__ void __launch_bounds__(kDwThreads, kDwCtas) pairs_dw_batch_kernel(con
 // targets and sources and differ only in their strengths.  Work item (lead problem, 128-node
 // tile, first index into the right-hand-side list, count <= kPairRhs): the position
 // differences, the distance and its powers of each (node, source) pair are formed once in
-// double-float and applied to the strengths of every listed right-hand side (~85 of the ~204
-// FP32 operations of a Stokeslet pair, ~89 of ~436 of an image triple, are shared).  Each
+// double-float and applied to the strengths of every listed right-hand side (76 of the 205 flops
+// of a Stokeslet pair and 94 of the 477 of an image triple are shared).  Each
 // right-hand side's sums follow the operation order of pair_tile_dw.
 constexpr int kDwTileM = 128;    // proxy sources staged per round
 constexpr int kDwTileImgM = 32;  // image nodes staged per round
