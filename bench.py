@@ -40,8 +40,9 @@ GOLDEN = os.path.join(ROOT, "tests", "golden", "gap_sweep_oracle.json")
 # S+R+D image triple at one node (shared distance and 1/r).  This is what `frac` is measured in.
 FLOPS_ALG = (28.0, 63.0)
 # FP32-pipe operations the double-float (compensated) kernel issues for the same pair math,
-# counted from its source: 205 per Stokeslet pair (162 lane operations) and 477 per image triple.  Their rate against the FP32 peak is `issue_frac`, a
-# measure of how busy the pipes are, not of algorithmic throughput.
+# counted from its source: 205 per Stokeslet pair and 477 per image triple.
+# Their rate against the FP32 peak is `issue_frac`, a measure of how busy the pipes are, not of
+# algorithmic throughput.
 FLOPS_ISSUED_DW = (205.0, 477.0)
 # dram__bytes_read.sum + dram__bytes_write.sum of one pairs_dw_multi_kernel<3> launch over three
 # gap-sweep geometries with their three motions each (ncu --set full on
