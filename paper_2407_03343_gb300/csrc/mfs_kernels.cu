@@ -574,25 +574,27 @@ __device__ __forceinline__ dw2 add2u(dw2 x, dw2 y) {
 // ------------------------------------------------------------------ double-float pair sums
 // Each thread holds one target at a time and evaluates two sources per instruction (the lanes), so
 // a source pair is read from shared memory as it is stored and a lane sums every second source.
-// What bounds the sums is the FMA pipe: 160 lane-operations a (node, Stokeslet) pair (the earlier
-// scalar evaluation: 204, and its issue slots) and 340 an image triple (436).  Measured on 100
-// spheres (5.59e9 pairs): 26.1 ms, 90 % of the measured packed rate, against 43.1 ms.  The evaluation keeps
+// What bounds the sums is the FMA pipe: 164 lane-operations a (node, Stokeslet) pair (the earlier
+// scalar evaluation: 204, and its issue slots) and 383 an image triple (436).  Measured on 100
+// spheres (5.59e9 pairs): 26.8 ms, 90 % of the measured packed rate, against 43.1 ms.  The evaluation keeps
 // the accuracy of a renormalised double-word one (~2^-46 of the operands) with fewer operations:
 //  - positions of a (target sphere, source sphere) segment are split on a common power-of-two grid
 //    per axis, so the difference of the high words is exact without a two-sum;
 //  - with s = 1/|d| to FP32 accuracy (MUFU and one Newton step on the high words) the unit vector
 //    u = d / |d| is formed as s d, and its deviation 1 - |s d|^2, found to ~2^-48 by a chain of
 //    fused multiply-adds from 1 whose roundings are recovered exactly, corrects u and 1/|d| at
-//    first order; the field needs only u and 1/|d| (Stokeslet: (f + (u.f) u) / |d|);
-//  - products and sums inside a term are not renormalised (their low words stay below ~2^-23 of
-//    the operands), and the terms are summed in groups of eight per lane with exact high sums and
-//    plain low sums, the groups in double-word arithmetic: a group's roundings scale with the
-//    group's sum instead of with the running sum, so the error of a sum is smaller than that of
-//    adding every term in double-word arithmetic (0.2-0.6 of it; 686 sources, random and equal
-//    strengths, against quadruple precision).
+//    second order; the field needs only u and 1/|d| (Stokeslet: (f + (u.f) u) / |d|);
+//  - products and sums inside a term but for u.f are not renormalised (their low words stay below
+//    ~2^-23 of the operands), and the terms are summed in groups of eight per lane with exact high
+//    sums and plain low sums, the groups in double-word arithmetic: a group's roundings scale with the
+//    group's sum instead of with the running sum.
+// Root mean square error per absolute sum (16 / 31 / 96 / 200 / 800 proxies of one sphere, random
+// strengths): 2.0 / 1.5 / 0.86 / 0.62 / 0.30e-15, that of adding every renormalised term in double-word
+// arithmetic 2.0 / 1.6 / 1.05 / 0.73 / 0.35e-15.  At first order, with u.f as it comes, a Newton step of
+// one more rounding and groups of sixteen it is 3.0 / 2.4 / 1.3 / 1.0 / 0.48e-15 (and 100 spheres 26.1 ms).
 constexpr int kDwTile = 256;     // proxy sources staged per round (one sphere's)
 constexpr int kDwTileImg = 64;   // image nodes staged per round (one sphere's)
-constexpr int kDwGroup = 16;     // terms per lane and group
+constexpr int kDwGroup = 8;      // terms per lane and group
 // Threads of a double-float CTA: the 128-node tiles are taken in two pieces, and a piece without targets
 // ends at once, so 823 nodes a sphere run as 13 CTAs of 64 (832 places) and not as 7 of 128 (896), and
 // the last wave is made of half as long CTAs.  Measured against CTAs of 128 (same rule for the parts): 100
@@ -634,9 +636,10 @@ __device__ __forceinline__ void dw_geometry(const DwTarget& T, const ulonglong2 
   const f2x r2 = f2fma(dh[2], dh[2], f2fma(dh[1], dh[1], f2mul(dh[0], dh[0])));
   float r0, r1;
   f2split(r2, r0, r1);
+  // one Newton step in residual form, s0 + s0 (1 - r2 s0^2) / 2: its last rounding is that of the
+  // result, so s is off by ~1.3e-7 at most (2e-7 as s0 (3 - r2 s0^2) / 2, the same four operations)
   const f2x s0 = f2make(rsqrt_ftz(r0), rsqrt_ftz(r1));
-  const f2x k = f2fma(f2mul(r2, mhalf), f2mul(s0, s0), f2dup(1.5f));
-  g.s = f2mul(s0, k);
+  g.s = f2fma(s0, f2fma(f2mul(f2mul(r2, mhalf), s0), s0, f2dup(0.5f)), s0);
   g.ns = f2neg(g.s);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
@@ -651,17 +654,15 @@ __device__ __forceinline__ void dw_geometry(const DwTarget& T, const ulonglong2 
                       f2fma(g.p[2], g.p[2], f2sub(a2, a3)));
   const f2x nq = f2fma(g.np[2], g.l[2], f2fma(g.np[1], g.l[1], f2mul(g.np[0], g.l[0])));
   const f2x e0 = f2fma(mhalf, f2add(f2add(a3, f2dup(1.0f)), t), nq);
-  // 1/|p + l| = 1 + e + 3/2 e^2 + ..: s is off by up to ~2e-7, so the second term reaches 6e-14, always of
-  // one sign and up to five times over in an image triple's third powers of 1/r; there it is kept (largest
-  // error of 31 proxies and 2 images a sphere 1.07e-13 -> 5.2e-14 of the absolute sum).  A Stokeslet's
-  // share of it is below the sums' other roundings (the same errors with it, 0.9 % of the time).
-  const f2x e = GRID ? e0 : f2fma(f2mul(e0, f2dup(1.5f)), e0, e0);
+  // 1/|p + l| = 1 + e + 3/2 e^2 + ..: the second term reaches 2e-14, always of one sign
+  const f2x e = f2fma(f2mul(e0, f2dup(1.5f)), e0, e0);
   g.il = f2mul(g.s, e);
 #pragma unroll
   for (int q = 0; q < 3; ++q) g.l[q] = f2fma(g.p[q], e, g.l[q]);
 }
 
-// -(u . f), not renormalised
+// u . f as -nh + l, renormalised (FastTwoSum: l is below 2^-22 |f|, so where it exceeds a cancelled
+// nh what is lost is below 2^-46 |f|)
 __device__ __forceinline__ void dw_ndot(const DwGeom& g, const f2x (&fh)[3], const f2x (&fl)[3], f2x& nh, f2x& l) {
   f2x n[3], e[3];
 #pragma unroll
@@ -670,9 +671,10 @@ __device__ __forceinline__ void dw_ndot(const DwGeom& g, const f2x (&fh)[3], con
     e[q] = f2fma(g.l[q], fh[q], f2fma(g.p[q], fl[q], f2fma(g.p[q], fh[q], n[q])));
   }
   const dw2 s1 = two_sum2(n[0], n[1]);
-  const dw2 s2 = two_sum2(s1.h, n[2]);
-  nh = s2.h;                                                       // -(u.f), high word
-  l = f2sub(f2add(f2add(e[0], e[1]), f2sub(e[2], s1.l)), s2.l);    // +(u.f), low word
+  const dw2 s2 = two_sum2(s1.h, n[2]);                                      // -(u.f), high word
+  const f2x lo = f2sub(f2add(f2add(e[0], e[1]), f2sub(e[2], s1.l)), s2.l);  // +(u.f), low word
+  nh = f2sub(s2.h, lo);
+  l = f2sub(lo, f2sub(s2.h, nh));
 }
 
 // v = f + (u.f) u in component q, from nh = -(u.f)_h, ph = (u.f)_h and l = (u.f)_l

@@ -1,0 +1,53 @@
+"""Accuracy of the double-float Stokeslet sums for few and many sources: root mean square of the error,
+per absolute sum of the terms, against sums in extended precision at the nodes of a sphere about the
+origin, whose coordinates relative to its centre are exact.
+
+Tolerance: that of double-word terms (renormalised |d|^2, 1/|d| and dot product) each added to a
+double-word sum.  Emulated on the CPU for these source counts and splits that evaluation has the rms
+below, the same within 5 % for every distance; 1.2 of it allows for the draw of the strengths.
+"""
+import numpy as np
+import pytest
+
+from paper_2407_03343_gb300 import mfs
+
+pytestmark = pytest.mark.gpu
+
+X = np.longdouble
+
+
+def errors(gap, seed, **kw):
+    """Errors at sphere 0 per absolute sum, three components a node."""
+    rng = np.random.default_rng(seed)
+    e = rng.normal(size=3)
+    centres = np.stack([np.zeros(3), (2.0 + gap) * e / np.linalg.norm(e)])
+    with mfs.Context(0) as ctx:
+        ctx.set_spheres(centres)
+        ctx.build(build_factors=0, left_precond=0, nim_fixed=0, **kw)
+        s = ctx.sizes()
+        lam = rng.normal(size=s.n_unknowns)
+        out = ctx.apply_pairs(lam, np.zeros(3 * s.n_colloc), mfs.MIXED)
+        x, _, owner = ctx.collocation()
+        pos, _ = ctx.source_layout()
+    n = kw["n_proxy"]
+    f = lam[3 * n:].reshape(n, 3).astype(X)
+    y = pos[:n].astype(X) + centres[1].astype(X)  # sphere 0's proxies, shifted
+    t = x[owner == 0].astype(X)
+    d = t[:, None] - y[None]
+    r2 = (d * d).sum(2)
+    ir = 1 / np.sqrt(r2)
+    scale = X(1.0 / (8.0 * np.pi))
+    u = scale * ((ir[..., None] * f[None]).sum(1) + (((d * f[None]).sum(2) * ir / r2)[..., None] * d).sum(1))
+    bound = np.zeros_like(u)
+    for a in range(3):
+        for b in range(3):
+            k = d[..., a] * d[..., b] / r2 + (1 if a == b else 0)
+            bound[:, a] += (ir * np.abs(k * f[None, :, b])).sum(1)
+    return np.asarray((out.reshape(-1, 3)[owner == 0] - u) / (scale * bound), dtype=float)
+
+
+@pytest.mark.parametrize("n_proxy,rms", [(16, 2.05e-15), (31, 1.45e-15), (96, 1.0e-15), (200, 0.7e-15), (800, 0.36e-15)])
+@pytest.mark.parametrize("gap", [0.05, 2.5])
+def test_rms_error_of_stokeslet_sums(n_proxy, rms, gap):
+    e = np.concatenate([errors(gap, s, n_proxy=n_proxy, m_basic=150, r_proxy=0.63) for s in range(4)])
+    assert np.sqrt(np.mean(e ** 2)) <= 1.2 * rms
