@@ -574,12 +574,13 @@ __device__ __forceinline__ dw2 add2u(dw2 x, dw2 y) {
 // ------------------------------------------------------------------ double-float pair sums
 // Each thread holds one target at a time and evaluates two sources per instruction (the lanes), so
 // a source pair is read from shared memory as it is stored and a lane sums every second source.
-// What bounds the sums is the FMA pipe: 164 lane-operations a (node, Stokeslet) pair (the earlier
-// scalar evaluation: 204, and its issue slots) and 383 an image triple (436).  Measured on 100
-// spheres (5.59e9 pairs): 26.8 ms, 90 % of the measured packed rate, against 43.1 ms.  The evaluation keeps
+// What bounds the sums is the FMA pipe: 164 lane-operations a (node, Stokeslet) pair, 170
+// close to the target's sphere (the earlier scalar evaluation: 204, and its issue slots) and 383 an image triple (436).  Measured on 100
+// spheres (5.59e9 pairs): 26.85 ms, 89 % of the measured packed rate, against 43.1 ms.  The evaluation keeps
 // the accuracy of a renormalised double-word one (~2^-46 of the operands) with fewer operations:
 //  - positions of a (target sphere, source sphere) segment are split on a common power-of-two grid
-//    per axis, so the difference of the high words is exact without a two-sum;
+//    per axis, so the difference of the high words is exact without a two-sum (a third word where the
+//    proxies may come close);
 //  - with s = 1/|d| to FP32 accuracy (MUFU and one Newton step on the high words) the unit vector
 //    u = d / |d| is formed as s d, and its deviation 1 - |s d|^2, found to ~2^-48 by a chain of
 //    fused multiply-adds from 1 whose roundings are recovered exactly, corrects u and 1/|d| at
@@ -589,7 +590,7 @@ __device__ __forceinline__ dw2 add2u(dw2 x, dw2 y) {
 //    sums and plain low sums, the groups in double-word arithmetic: a group's roundings scale with the
 //    group's sum instead of with the running sum.
 // Root mean square error per absolute sum (16 / 31 / 96 / 200 / 800 proxies of one sphere, random
-// strengths): 2.0 / 1.5 / 0.86 / 0.62 / 0.30e-15, that of adding every renormalised term in double-word
+// strengths): 1.8 / 1.4 / 0.80 / 0.55 / 0.28e-15, that of adding every renormalised term in double-word
 // arithmetic 2.0 / 1.6 / 1.05 / 0.73 / 0.35e-15.  At first order, with u.f as it comes, a Newton step of
 // one more rounding and groups of sixteen it is 3.0 / 2.4 / 1.3 / 1.0 / 0.48e-15 (and 100 spheres 26.1 ms).
 constexpr int kDwTile = 256;     // proxy sources staged per round (one sphere's)
@@ -616,22 +617,26 @@ struct DwGeom {          // geometry of one target and two sources
 };
 
 struct DwTarget {        // a target in the grid of the current segment, duplicated into both lanes
-  f2x h[3], l[3];
+  f2x h[3], l[3], r[3];  // (r: third words, DW_REST)
 };
 
-template <bool GRID>
+// How positions are held: double-float words; high words on the segment's grid; high and low words on
+// grids and a third word (rest: the sources' third words)
+enum { DW_FREE, DW_GRID, DW_REST };
+
+template <int FORM>
 __device__ __forceinline__ void dw_geometry(const DwTarget& T, const ulonglong2 a, const ulonglong2 b,
-                                            const ulonglong2 c, DwGeom& g) {
+                                            const ulonglong2 c, const f2x* rest, DwGeom& g) {
   const f2x yh[3] = {a.x, a.y, b.x}, yl[3] = {b.y, c.x, c.y};
   const f2x mtwo = f2dup(-2.0f), mhalf = f2dup(-0.5f);
   f2x dh[3], dl[3];
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    const dw2 t = GRID ? dw2{f2sub(T.h[q], yh[q]), 0} : two_diff2(T.h[q], yh[q]);
+    const dw2 t = FORM != DW_FREE ? dw2{f2sub(T.h[q], yh[q]), 0} : two_diff2(T.h[q], yh[q]);
     const f2x tl = f2sub(T.l[q], yl[q]);
-    const dw2 d = fast_two_sum2(t.h, GRID ? tl : f2add(t.l, tl));
+    const dw2 d = fast_two_sum2(t.h, FORM != DW_FREE ? tl : f2add(t.l, tl));
     dh[q] = d.h;
-    dl[q] = d.l;
+    dl[q] = FORM == DW_REST ? f2add(d.l, f2sub(T.r[q], rest[q])) : d.l;
   }
   const f2x r2 = f2fma(dh[2], dh[2], f2fma(dh[1], dh[1], f2mul(dh[0], dh[0])));
   float r0, r1;
@@ -769,52 +774,142 @@ __device__ __forceinline__ void dw_load_targets(const PairArgs<double>& A, int s
 }
 
 // Grid of a segment: on each axis the spacing 2^(e - 24) with 2^e above every |x - y| of the
-// segment (centre distance plus twice the radius), so high words on it subtract exactly.
+// segment (centre distance plus twice the radius), so high words on it subtract exactly.  What lies
+// below the low words, 2^(e - 49), then is an absolute error of the positions; where a proxy may come
+// closer than a quarter of 2^e to a target (centres within 3.6 radii at r_proxy 0.63) it would exceed
+// the terms' other roundings.  There the low words are put on a second grid, 2^(e - 46), and subtract
+// exactly too, and a third word holds the rest: six lane-operations more (a two-sum of double-float
+// words: 18, and twice the error).  Nodes within 0.2 of proxies at 0.97 of the surface, gap 1e-3, 31 / 96 /
+// 200 proxies: rms error 10.2 / 3.8 / 2.9e-15 of the absolute sum in two words, 2.2 / 1.1 / 0.8e-15 in three; a
+// double-float difference in the scalar evaluation 3.2 / 1.5 / 1.0e-15.  Where every segment is close it costs
+// 4 % (8 spheres of 400 proxies 295 -> 305 us), on 100 spheres 0.1 %.
 struct DwGrid {
-  dw shift[3];   // source sphere's centre minus target sphere's
-  float m32[3];  // 2^(e-1): rounds |x| < 2^(e-1) to the grid as (|x| + m32) - m32
+  dw shift[3];    // source sphere's centre minus target sphere's
+  float rest[3];  // what the split leaves of it (three words)
+  float m32[3];   // 2^(e-1): rounds |x| < 2^(e-1) to the grid as (|x| + m32) - m32
+  bool close;     // whether the segment takes three words
 };
-__device__ __forceinline__ DwGrid dw_grid(const PairArgs<double>& A, const CentreShift64& sh, int o) {
-  DwGrid G;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    G.shift[q] = dw_split(sh.d(o, q));
-    const float b = fabsf(G.shift[q].h) * 1.0001f + A.span;
-    // half the power of two above b (b is a normal number: at least the sphere's radius)
-    G.m32[q] = 0.5f * __int_as_float((__float_as_int(b) & 0x7f800000) + 0x00800000);
+// The grid of sphere o's segment, by one warp, an axis a lane: FP64 operations take 16 clocks of an SM's two
+// lanes a warp, whatever the lanes hold.
+__device__ __forceinline__ void dw_grid(const PairArgs<double>& A, const CentreShift64& sh, int o, DwGrid& G) {
+  const int lane = threadIdx.x & 31, q = min(lane, 2);
+  const double v = sh.cen[3 * o + q] - (q == 0 ? sh.kc[0] : q == 1 ? sh.kc[1] : sh.kc[2]);
+  const dw s = dw_split(v);
+  const float rest = (float)(v - dw_join(s));
+  const float b = fabsf(s.h) * 1.0001f + A.span;
+  // half the power of two above b (b is a normal number: at least the sphere's radius)
+  const float m32 = 0.5f * __int_as_float((__float_as_int(b) & 0x7f800000) + 0x00800000);
+  const float h[3] = {__shfl_sync(~0u, s.h, 0), __shfl_sync(~0u, s.h, 1), __shfl_sync(~0u, s.h, 2)};
+  const float m[3] = {__shfl_sync(~0u, m32, 0), __shfl_sync(~0u, m32, 1), __shfl_sync(~0u, m32, 2)};
+  const float gap = norm3df(h[0], h[1], h[2]) - A.span;
+  if (lane < 3) {
+    G.shift[q] = s;
+    G.rest[q] = rest;
+    G.m32[q] = m32;
+    G.close = !(fmaxf(m[0], fmaxf(m[1], m[2])) <= 2.0f * gap);
   }
-  return G;
 }
 // x rounded to the grid (a float of 2^(e-1) and above lies on it)
 __device__ __forceinline__ float dw_on_grid(float x, float m32) {
   const float t = fabsf(x);
   return copysignf(t >= m32 ? t : __fsub_rn(__fadd_rn(t, m32), m32), x);
 }
+// x rounded to the second grid, |x| up to 2^(e - 24)
+__device__ __forceinline__ float dw_on_grid2(float x, float m32) {
+  const float m = __fmul_rn(m32, 1.5f * 0x1p-22f);
+  return __fsub_rn(__fadd_rn(x, m), m);
+}
 // A proxy's position in the target's frame, in FP32 operations only: with the position and the strengths
 // held in double, the sums, splits and conversions of a source were about 25 FP64 operations, 12 clocks of
 // an SM's two FP64 lanes, where 64 targets spend about 84 clocks on a source.
-__device__ __forceinline__ void dw_stage_pos(const DwGrid& G, const float4 ph, const float4 pl, float* sp, int i) {
+__device__ __forceinline__ void dw_stage_pos(const DwGrid& G, const float4 ph, const float4 pl, float* sp, float* rest,
+                                             int i) {
   const float rh[3] = {ph.x, ph.y, ph.z}, rl[3] = {pl.x, pl.y, pl.z};
   float* o = sp + 12 * (i >> 1) + (i & 1);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     const dw s = two_sum(rh[q], G.shift[q].h);
-    const float l = __fadd_rn(s.l, __fadd_rn(rl[q], G.shift[q].l));
-    const float h = dw_on_grid(s.h, G.m32[q]);
+    float h, l;
+    if (G.close) {
+      const dw t = two_sum(rl[q], G.shift[q].l), u = two_sum(s.l, t.h), y = fast_two_sum(s.h, u.h);
+      h = dw_on_grid(y.h, G.m32[q]);
+      const dw v = two_sum(__fsub_rn(y.h, h), y.l);
+      l = dw_on_grid2(v.h, G.m32[q]);
+      rest[6 * (i >> 1) + 2 * q + (i & 1)] =
+          __fadd_rn(__fsub_rn(v.h, l), __fadd_rn(v.l, __fadd_rn(u.l, __fadd_rn(t.l, G.rest[q]))));
+    } else {
+      h = dw_on_grid(s.h, G.m32[q]);
+      l = __fadd_rn(__fsub_rn(s.h, h), __fadd_rn(s.l, __fadd_rn(rl[q], G.shift[q].l)));
+    }
     o[2 * q] = h;
-    o[6 + 2 * q] = __fadd_rn(__fsub_rn(s.h, h), l);
+    o[6 + 2 * q] = l;
   }
 }
+template <int FORM>
 __device__ __forceinline__ DwTarget dw_target(const DwGrid& G, const dw (&x)[3]) {
   DwTarget t;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     const float h = dw_on_grid(x[q].h, G.m32[q]);
-    const float l = __fadd_rn(__fsub_rn(x[q].h, h), x[q].l);
     t.h[q] = f2dup(h);
-    t.l[q] = f2dup(l);
+    if constexpr (FORM == DW_REST) {
+      const dw v = two_sum(__fsub_rn(x[q].h, h), x[q].l);
+      const float l = dw_on_grid2(v.h, G.m32[q]);
+      t.l[q] = f2dup(l);
+      t.r[q] = f2dup(__fadd_rn(__fsub_rn(v.h, l), v.l));
+    } else {
+      t.l[q] = f2dup(__fadd_rn(__fsub_rn(x[q].h, h), x[q].l));
+    }
   }
   return t;
+}
+
+// A round of nu source pairs against the targets of the piece.
+template <int R, int NT, int TILE, int FORM>
+__device__ __forceinline__ void dw_proxy_round(const DwGrid& G, unsigned mask, int nu, int cnt, const float* sp,
+                                               const float* rest, const float (*sf)[6 * TILE], DWTile<R, NT>& T) {
+#pragma unroll 1
+  for (int q = 0; q < NT; ++q) {
+    if (!dw_warp_live(q, cnt)) continue;
+    T.load(q);
+    const DwTarget X = dw_target<FORM>(G, T.x);
+    dw2 m[R][3];
+#pragma unroll
+    for (int r = 0; r < R; ++r) m[r][0] = m[r][1] = m[r][2] = dw2{0, 0};
+    for (int u0 = 0; u0 < nu; u0 += kDwGroup) {
+      dw2 sum[R][3];
+#pragma unroll
+      for (int r = 0; r < R; ++r) sum[r][0] = sum[r][1] = sum[r][2] = dw2{0, 0};
+      const int u1 = min(nu, u0 + kDwGroup);
+#pragma unroll 2
+      for (int u = u0; u < u1; ++u) {
+        const ulonglong2* P = reinterpret_cast<const ulonglong2*>(sp) + 3 * u;
+        DwGeom g;
+        dw_geometry<FORM>(X, P[0], P[1], P[2], reinterpret_cast<const f2x*>(rest) + 3 * u, g);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (R > 1 && !(mask >> r & 1u)) continue;
+          const ulonglong2* F = reinterpret_cast<const ulonglong2*>(sf[r]) + 3 * u;
+          const ulonglong2 fa = F[0], fb = F[1], fc = F[2];
+          const f2x fh[3] = {fa.x, fa.y, fb.x}, fl[3] = {fb.y, fc.x, fc.y};
+          f2x nh, l;
+          dw_ndot(g, fh, fl, nh, l);
+          const f2x ph = f2neg(nh);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) dw_accumulate(g, dw_project(g, c, fh[c], fl[c], nh, ph, l), sum[r][c]);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) m[r][c] = dw2_add(m[r][c], sum[r][c]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) dw_fold(T.u[r][c], m[r][c]);
+    T.store(q);
+  }
 }
 
 // Proxy Stokeslets [r_lo, r_hi) of the flattened proxy index (sphere o = j / N, proxy j - o N; the
@@ -822,19 +917,29 @@ __device__ __forceinline__ DwTarget dw_target(const DwGrid& G, const dw (&x)[3])
 template <int R, int NT, int TILE>
 __device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const CentreShift64& sh,
                                                const float2* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
-                                               int cnt, float* sp, float (*sf)[6 * TILE], DWTile<R, NT>& T) {
+                                               int cnt, float* sp, float (*sf)[6 * TILE], DwGrid* grids, int& segs,
+                                               DWTile<R, NT>& T) {
   for (int s0 = r_lo; s0 < r_hi;) {
     const int o = s0 / A.N, j0 = s0 - o * A.N;
     const int seg = min(r_hi - s0, A.N - j0);  // what is left of sphere o
-    // even rounds of whole groups
-    const int rounds = (seg + TILE - 1) / TILE;
+    // a new segment's grid goes to the place that was last read two segments, so two barriers, ago
+    if (s0 == r_lo || j0 == 0) {
+      ++segs;
+      if (threadIdx.x < 32) dw_grid(A, sh, o, grids[segs & 1]);
+    }
+    __syncthreads();
+    const DwGrid G = grids[segs & 1];
+    // even rounds of whole groups; third words take the place of a third of the sources
+    constexpr int kClose = 2 * TILE / 3 / (2 * kDwGroup) * (2 * kDwGroup);
+    static_assert(kClose > 0 && 9 * kClose <= 6 * TILE, "third words behind the positions");
+    float* const rest = sp + 6 * kClose;
+    const int tile = G.close ? kClose : TILE;
+    const int rounds = (seg + tile - 1) / tile;
     const int ns = min(seg, ((seg + rounds - 1) / rounds + 2 * kDwGroup - 1) / (2 * kDwGroup) * (2 * kDwGroup));
     const int nu = (ns + 1) >> 1;
-    const DwGrid G = dw_grid(A, sh, o);
-    __syncthreads();
     for (int i = threadIdx.x; i < 2 * nu; i += kDwThreads) {
       const int jj = j0 + min(i, ns - 1);
-      dw_stage_pos(G, A.proxy2[2 * jj], A.proxy2[2 * jj + 1], sp, i);
+      dw_stage_pos(G, A.proxy2[2 * jj], A.proxy2[2 * jj + 1], sp, rest, i);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const bool on = i < ns && (mask >> r & 1u);  // the odd round's last slot carries no strength
@@ -849,48 +954,8 @@ __device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const 
       }
     }
     __syncthreads();
-#pragma unroll 1
-    for (int q = 0; q < NT; ++q) {
-      if (!dw_warp_live(q, cnt)) continue;
-      T.load(q);
-      const DwTarget X = dw_target(G, T.x);
-      dw2 m[R][3];
-#pragma unroll
-      for (int r = 0; r < R; ++r) m[r][0] = m[r][1] = m[r][2] = dw2{0, 0};
-      for (int u0 = 0; u0 < nu; u0 += kDwGroup) {
-        dw2 sum[R][3];
-#pragma unroll
-        for (int r = 0; r < R; ++r) sum[r][0] = sum[r][1] = sum[r][2] = dw2{0, 0};
-        const int u1 = min(nu, u0 + kDwGroup);
-#pragma unroll 2
-        for (int u = u0; u < u1; ++u) {
-          const ulonglong2* P = reinterpret_cast<const ulonglong2*>(sp) + 3 * u;
-          DwGeom g;
-          dw_geometry<true>(X, P[0], P[1], P[2], g);
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            if (R > 1 && !(mask >> r & 1u)) continue;
-            const ulonglong2* F = reinterpret_cast<const ulonglong2*>(sf[r]) + 3 * u;
-            const ulonglong2 fa = F[0], fb = F[1], fc = F[2];
-            const f2x fh[3] = {fa.x, fa.y, fb.x}, fl[3] = {fb.y, fc.x, fc.y};
-            f2x nh, l;
-            dw_ndot(g, fh, fl, nh, l);
-            const f2x ph = f2neg(nh);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) dw_accumulate(g, dw_project(g, c, fh[c], fl[c], nh, ph, l), sum[r][c]);
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) m[r][c] = dw2_add(m[r][c], sum[r][c]);
-      }
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) dw_fold(T.u[r][c], m[r][c]);
-      T.store(q);
-    }
+    if (G.close) dw_proxy_round<R, NT, TILE, DW_REST>(G, mask, nu, cnt, sp, rest, sf, T);
+    else dw_proxy_round<R, NT, TILE, DW_GRID>(G, mask, nu, cnt, sp, rest, sf, T);
     s0 += ns;
   }
 }
@@ -960,7 +1025,7 @@ __device__ __forceinline__ void dw_image_range(const PairArgs<double>& A, const 
       for (int u = 0; u < nu; ++u) {
         const ulonglong2* P = reinterpret_cast<const ulonglong2*>(sp) + 3 * u;
         DwGeom g;
-        dw_geometry<false>(X, P[0], P[1], P[2], g);
+        dw_geometry<DW_FREE>(X, P[0], P[1], P[2], nullptr, g);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           if (R > 1 && !(mask >> r & 1u)) continue;
@@ -1039,6 +1104,7 @@ struct DwShared {
     __align__(16) float sf[R][6 * TILE];
     __align__(16) float si[R][24 * TILE_IMG];
   };
+  DwGrid grids[2];
 };
 
 // Sources may be split over `nparts` CTAs per target tile (when there are too few tiles to
@@ -1054,14 +1120,19 @@ __device__ __forceinline__ void dw_all_sources(const PairArgs<double>& A, const 
   const int p_lo = k * A.N, p_w = A.N;
   const long long p_eff = total - p_w;
   const int pe0 = (int)(p_eff * part / nparts), pe1 = (int)(p_eff * (part + 1) / nparts);
-  dw_proxy_range<R, NT, TILE>(A, sh, lam, mask, min(pe0, p_lo), min(pe1, p_lo), cnt, S.sp, S.sf, T);
-  dw_proxy_range<R, NT, TILE>(A, sh, lam, mask, max(pe0, p_lo) + p_w, max(pe1, p_lo) + p_w, cnt, S.sp, S.sf, T);
+  int segs = 0;
+#pragma unroll 1  // (one copy of the loops: with two, 8 spheres took 350 us instead of 311)
+  for (int rr = 0; rr < 2; ++rr)
+    dw_proxy_range<R, NT, TILE>(A, sh, lam, mask, rr ? max(pe0, p_lo) + p_w : min(pe0, p_lo),
+                                rr ? max(pe1, p_lo) + p_w : min(pe1, p_lo), cnt, S.sp, S.sf, S.grids, segs, T);
   // image nodes before and after sphere k's own, this part's share
   const int i_lo = A.img_off[k], i_w = A.img_off[k + 1] - i_lo;
   const long long i_eff = A.n_img - i_w;
   const int ie0 = (int)(i_eff * part / nparts), ie1 = (int)(i_eff * (part + 1) / nparts);
-  dw_image_range<R, NT, TILE_IMG>(A, sh, lam, mask, min(ie0, i_lo), min(ie1, i_lo), cnt, S.sp, S.si, T);
-  dw_image_range<R, NT, TILE_IMG>(A, sh, lam, mask, max(ie0, i_lo) + i_w, max(ie1, i_lo) + i_w, cnt, S.sp, S.si, T);
+#pragma unroll 1
+  for (int rr = 0; rr < 2; ++rr)
+    dw_image_range<R, NT, TILE_IMG>(A, sh, lam, mask, rr ? max(ie0, i_lo) + i_w : min(ie0, i_lo),
+                                    rr ? max(ie1, i_lo) + i_w : min(ie1, i_lo), cnt, S.sp, S.si, T);
 }
 
 template <int NT>
@@ -1104,6 +1175,7 @@ __device__ __forceinline__ void pair_tile_dw_near(const PairArgs<double>& A, con
   dw_load_targets<1, NT>(A, start, cnt, T);
   const float2* const lam[1] = {A.lam2};
   // this part's share of the near list
+  int segs = 0;
   const int b0 = near_off[k], nn = near_off[k + 1] - b0;
   const int a1 = b0 + (int)((long long)nn * (part + 1) / nparts);
   for (int a = b0 + (int)((long long)nn * part / nparts); a < a1;) {
@@ -1114,7 +1186,7 @@ __device__ __forceinline__ void pair_tile_dw_near(const PairArgs<double>& A, con
       ++o1;
     }
     ++a;
-    dw_proxy_range<1, NT, kDwTile>(A, sh, lam, 1u, o0 * A.N, (o1 + 1) * A.N, cnt, S.sp, S.sf, T);
+    dw_proxy_range<1, NT, kDwTile>(A, sh, lam, 1u, o0 * A.N, (o1 + 1) * A.N, cnt, S.sp, S.sf, S.grids, segs, T);
     dw_image_range<1, NT, kDwTileImg>(A, sh, lam, 1u, A.img_off[o0], A.img_off[o1 + 1], cnt, S.sp, S.si, T);
   }
   dw_write_out<1, NT>(A, start, cnt, T, 0, A.mu, A.out, part, nparts, partial, pstride);
