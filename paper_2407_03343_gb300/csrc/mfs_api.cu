@@ -2704,41 +2704,57 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   ALLOC_TRY(c, c->d_t2, float2, c->tmp_len);
   ALLOC_TRY(c, c->d_lh2, float2, c->n_unk);
   c->nblk = std::max(1, std::min(1024, (n + 4095) / 4096));
-  {
-    // 1024-element chunks of the system vectors, without and with the mobility border
-    size_t most = (size_t)c->nblk;
+  // what only a solve needs: 1024-element chunks of the system vectors, without and with the mobility border
+  // (both tables in one buffer: a transfer and an allocation each cost a build of a small context 5-10 us),
+  // the partial dots and the pinned coefficients
+  std::vector<long long> segs;
+  for (SegTable& t : c->seg) t = SegTable();
+  if (nf > 0) {
+    size_t at[2][6], most = (size_t)c->nblk;
+    int nchunks[2];
+    auto put_ints = [&](const std::vector<int>& v) {
+      const size_t o = segs.size();
+      segs.resize(o + (v.size() + 1) / 2, 0);
+      std::memcpy(segs.data() + o, v.data(), sizeof(int) * v.size());
+      return o;
+    };
     for (int md = 0; md < 2; ++md) {
       const long long len = n + (md == 1 ? 6LL * P : 0LL);
       std::vector<long long> cs, ce;
-      for (long long a = 0; a < len; a += 1024) {
-        cs.push_back(a);
-        ce.push_back(std::min(len, a + 1024));
+      for (long long q = 0; q < len; q += 1024) {
+        cs.push_back(q);
+        ce.push_back(std::min(len, q + 1024));
       }
-      std::vector<int> prob(cs.size(), 0), pch = {0, (int)cs.size()}, one(1, 1);
-      std::vector<unsigned> cnt(1, 0u);
-      SegTable& t = c->seg[md];
-      t = SegTable();
-      t.K = 1;
-      t.nchunks = (int)cs.size();
-      int *dp = nullptr, *dpc = nullptr, *da = nullptr;
-      long long *ds = nullptr, *de = nullptr;
-      if ((s = upload(c, dp, prob)) || (s = upload(c, dpc, pch)) || (s = upload(c, da, one)) || (s = upload(c, ds, cs)) ||
-          (s = upload(c, de, ce)) || (s = upload(c, t.counter, cnt)))
-        return s;
-      t.prob = dp;
-      t.pchunk = dpc;
-      t.active = da;
-      t.start = ds;
-      t.end = de;
+      nchunks[md] = (int)cs.size();
       most = std::max(most, cs.size());
-      CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // the uploads' host vectors end here
+      at[md][0] = segs.size();
+      segs.insert(segs.end(), cs.begin(), cs.end());
+      at[md][1] = segs.size();
+      segs.insert(segs.end(), ce.begin(), ce.end());
+      at[md][2] = put_ints(std::vector<int>(cs.size(), 0));       // problem of each chunk
+      at[md][3] = put_ints({0, nchunks[md]});                     // chunks of the problem
+      at[md][4] = put_ints({1});                                  // it is active
+      at[md][5] = put_ints({0});                                  // arrivals
+    }
+    long long* d = nullptr;
+    if ((s = upload(c, d, segs)) != MFS_OK) return s;
+    for (int md = 0; md < 2; ++md) {
+      SegTable& t = c->seg[md];
+      t.K = 1;
+      t.nchunks = nchunks[md];
+      t.start = d + at[md][0];
+      t.end = d + at[md][1];
+      t.prob = reinterpret_cast<const int*>(d + at[md][2]);
+      t.pchunk = reinterpret_cast<const int*>(d + at[md][3]);
+      t.active = reinterpret_cast<const int*>(d + at[md][4]);
+      t.counter = reinterpret_cast<unsigned*>(d + at[md][5]);
     }
     ALLOC_TRY(c, c->d_partial, double, most * 512);
-  }
-  if (!c->h_pin && cudaMallocHost(&c->h_pin, sizeof(double) * (2 * 512 + 1)) != cudaSuccess) {
-    cudaGetLastError();
-    c->h_pin = nullptr;
-    return c->fail(MFS_ERR_OOM, "pinned allocation failed: Arnoldi coefficients");
+    if (!c->h_pin && cudaMallocHost(&c->h_pin, sizeof(double) * (2 * 512 + 1)) != cudaSuccess) {
+      cudaGetLastError();
+      c->h_pin = nullptr;
+      return c->fail(MFS_ERR_OOM, "pinned allocation failed: Arnoldi coefficients");
+    }
   }
   ALLOC_TRY(c, c->d_h, double, 5 * 512);
   CUDA_TRY(c, cudaMemsetAsync(c->d_v, 0, sizeof(double) * 3 * P, c->stream));
