@@ -557,17 +557,35 @@ mfs_status ensure_krylov(mfs_ctx* c, int restart) {
   return MFS_OK;
 }
 
-// dot products of w with V[0..nvec) (FP64 partials) -> host h
+// whether the system vectors are short enough for the segmented kernels
+bool segmented(const mfs_ctx* c) { return c->seg[c->mode].nchunks <= kSegSingleMax; }
+
+// dot products of w with V[0..nvec) (FP64 partials) -> h on the device
 template <typename T>
 mfs_status dots(mfs_ctx* c, int nvec, const T* V, const T* w, double* h_dev) {
+  bool seg = false;
   if constexpr (sizeof(T) == 8) {
-    launch_seg_dots(c->seg[c->mode], nvec, V, c->n_sys, w, c->d_partial, h_dev, c->stream);
-  } else {
+    seg = segmented(c);
+    if (seg) launch_seg_dots(c->seg[c->mode], nvec, V, c->n_sys, w, c->d_partial, h_dev, c->stream);
+  }
+  if (!seg) {
     launch_multidot<T>(c->n_sys, nvec, V, c->n_sys, w, c->d_partial, c->nblk, c->stream);
     launch_reduce_partials(nvec, c->nblk, c->d_partial, h_dev, c->stream);
   }
   CHECK_LAUNCH(c);
   return MFS_OK;
+}
+
+// w += sign * sum_i h_i V_i
+template <typename T>
+void update(mfs_ctx* c, int nvec, const T* V, const double* h, double sign, T* w) {
+  if constexpr (sizeof(T) == 8) {
+    if (segmented(c)) {
+      launch_seg_update(c->seg[c->mode], nvec, V, c->n_sys, h, sign, w, c->stream);
+      return;
+    }
+  }
+  launch_update<T>(c->n_sys, nvec, V, c->n_sys, h, sign, w, c->stream);
 }
 
 // Restarted GMRES(m) with CGS2 Arnoldi (classical Gram-Schmidt applied twice), Givens
@@ -631,20 +649,22 @@ mfs_status gmres(mfs_ctx* c, const T* b, T* x, double tol, int restart, int max_
       sys_apply<T>(c, V + (size_t)j * n, w, x2_ready);
       CHECK_LAUNCH(c);
       if ((s = dots<T>(c, j + 1, V, w, h1)) != MFS_OK) return s;
+      update<T>(c, j + 1, V, h1, -1.0, w);
+      if ((s = dots<T>(c, j + 1, V, w, h2)) != MFS_OK) return s;
+      // FP64: the new basis vector is scaled (and split for the next double-float apply) by its norm on the
+      // device, before the host reads it; for short vectors the norm comes with the second update
+      bool norm_done = false;
       if constexpr (sizeof(T) == 8) {
-        // the norm comes with the second update, and the new basis vector is scaled (and split for
-        // the next double-float apply) by it on the device, before the host reads it
-        const SegTable& t = c->seg[c->mode];
-        launch_seg_update(t, j + 1, V, n, h1, -1.0, w, c->stream);
-        if ((s = dots<T>(c, j + 1, V, w, h2)) != MFS_OK) return s;
-        launch_seg_update_norm(t, j + 1, V, n, h2, -1.0, w, c->d_partial, hn, c->stream);
-        launch_seg_normalise(t, hn, w, w, c->dw_pairs ? c->d_x2 : nullptr, c->stream);
-        x2_ready = c->dw_pairs;
-      } else {
-        launch_update<T>(n, j + 1, V, n, h1, -1.0, w, c->stream);
-        if ((s = dots<T>(c, j + 1, V, w, h2)) != MFS_OK) return s;
-        launch_update<T>(n, j + 1, V, n, h2, -1.0, w, c->stream);
+        norm_done = segmented(c);
+        if (norm_done) launch_seg_update_norm(c->seg[c->mode], j + 1, V, n, h2, -1.0, w, c->d_partial, hn, c->stream);
+      }
+      if (!norm_done) {
+        update<T>(c, j + 1, V, h2, -1.0, w);
         if ((s = dots<T>(c, 1, w, w, hn)) != MFS_OK) return s;
+      }
+      if constexpr (sizeof(T) == 8) {
+        launch_seg_normalise(c->seg[c->mode], hn, w, w, c->dw_pairs ? c->d_x2 : nullptr, c->stream);
+        x2_ready = c->dw_pairs;
       }
       CUDA_TRY(c, cudaMemcpyAsync(hb, c->d_h, sizeof(double) * (2 * ldh + 1), cudaMemcpyDeviceToHost, c->stream));
       CUDA_TRY(c, cudaStreamSynchronize(c->stream));
@@ -683,8 +703,7 @@ mfs_status gmres(mfs_ctx* c, const T* b, T* x, double tol, int restart, int max_
     }
     if (j_used > 0) {
       CUDA_TRY(c, cudaMemcpyAsync(coef, y.data(), sizeof(double) * j_used, cudaMemcpyHostToDevice, c->stream));
-      if constexpr (sizeof(T) == 8) launch_seg_update(c->seg[c->mode], j_used, V, n, coef, 1.0, x, c->stream);
-      else launch_update<T>(n, j_used, V, n, coef, 1.0, x, c->stream);
+      update<T>(c, j_used, V, coef, 1.0, x);
       CHECK_LAUNCH(c);
     }
     if (done) break;
@@ -1111,8 +1130,8 @@ mfs_status make_plan(mfs_ctx* c0, int K, mfs_ctx* const* ctxs, const std::vector
     B->seg.active = B->d_active;
     B->seg.list = B->d_cchunk;
     B->seg.nlist = 0;
-    B->seg.counter = B->alloc<unsigned>(K);
-    ok = ok && B->seg.counter && cudaMemset(B->seg.counter, 0, sizeof(unsigned) * K) == cudaSuccess;
+    B->seg.counter = B->alloc<unsigned>((size_t)kSegCounters * K);
+    ok = ok && B->seg.counter && cudaMemset(B->seg.counter, 0, sizeof(unsigned) * kSegCounters * K) == cudaSuccess;
   }
   const long long n = B->n_total;
   ok = ok && (B->wb = B->alloc<double>(n)) && (B->x = B->alloc<double>(n)) && (B->r = B->alloc<double>(n)) &&
@@ -2734,7 +2753,7 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
       at[md][2] = put_ints(std::vector<int>(cs.size(), 0));       // problem of each chunk
       at[md][3] = put_ints({0, nchunks[md]});                     // chunks of the problem
       at[md][4] = put_ints({1});                                  // it is active
-      at[md][5] = put_ints({0});                                  // arrivals
+      at[md][5] = put_ints(std::vector<int>(kSegCounters, 0));     // arrivals
     }
     long long* d = nullptr;
     if ((s = upload(c, d, segs)) != MFS_OK) return s;

@@ -287,6 +287,12 @@ void launch_sub(int n, const double* a, const double* b, double* out, cudaStream
 // Segmented vector kernels over a concatenation of independent problems: chunk b covers
 // [start[b], end[b]) and belongs to problem prob[b]; per-problem coefficients are stored
 // vector-major, c[i * K + p].  Chunks of inactive problems do nothing.
+constexpr int kSegCounters = 32;  // arrival counters per problem
+// A single solve takes these kernels up to this many chunks and the unsegmented ones, a launch more for each
+// sum, above: there the arrivals at one counter, the 128-element CTAs of the update and their four partial sums
+// cost more than the launches.  What an iteration takes beside step 1 and the pair sums (mean of the first 60),
+// segmented / unsegmented: 14 chunks 72 / 78 us, 47: 77 / 78, 112: 104 / 93, 253: 175 / 139, 1,758: 900 / 568.
+constexpr int kSegSingleMax = 64;
 struct SegTable {
   int K = 0, nchunks = 0;
   int chunk = 1024;             // longest chunk (at most 1024 elements)
@@ -297,8 +303,8 @@ struct SegTable {
   const int* active = nullptr;
   const int* list = nullptr;    // optional: the chunks of the active problems (nlist of them); the
   int nlist = 0;                //   launches then cover only those
-  unsigned* counter = nullptr;  // optional, K zeros: the dot products are then reduced per problem by
-                                //   the last CTA of each problem instead of a second kernel
+  unsigned* counter = nullptr;  // optional, kSegCounters K zeros: the dot products are then reduced by the
+                                //   last CTA of a problem's block of vectors instead of a second kernel
 };
 void launch_seg_dots(const SegTable& t, int nvec, const double* V, long long ldv, const double* w, double* partial,
                      double* h, cudaStream_t st);

@@ -2068,6 +2068,7 @@ __device__ __forceinline__ int seg_chunk(const SegTable& t) { return t.list ? t.
 // its block, so the launch has enough CTAs to keep HBM busy even for a single short problem.
 constexpr int kSegChunkMax = 1024;
 constexpr int kSegDotVecs = 16;   // basis vectors per CTA
+static_assert(kSegCounters * kSegDotVecs >= 512, "a counter per block of basis vectors");
 constexpr int kSegUpdSub = 128;   // elements per CTA of the update (one per thread)
 __global__ void seg_dots_kernel(SegTable t, int nvec, const double* __restrict__ V, long long ldv,
                                 const double* __restrict__ w, double* __restrict__ partial, double* __restrict__ h) {
@@ -2103,24 +2104,33 @@ __global__ void seg_dots_kernel(SegTable t, int nvec, const double* __restrict__
     }
   }
   if (!t.counter) return;
-  // the last CTA of problem p to finish adds its partial dots in chunk order (so the result does
-  // not depend on which CTA that is) and re-arms the counter for the next launch
+  // The last CTA of problem p and this block of vectors adds their partial dots in chunk order (so the
+  // result does not depend on which CTA that is), a thread per vector with 16 loads in flight, and re-arms
+  // the counter for the next launch.  With one CTA for all vectors of a problem and four loads at a time an
+  // iteration of 216 spheres (507 chunks) took 592 us beside step 1 and the pair sums, this way 296.
+  unsigned* counter = t.counter + p * kSegCounters + blockIdx.y;
   __shared__ bool last;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned total = (unsigned)(t.pchunk[p + 1] - t.pchunk[p]) * gridDim.y;
-    last = atomicAdd(&t.counter[p], 1u) == total - 1;
-  }
+  const int c0 = t.pchunk[p], c1 = t.pchunk[p + 1];
+  if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == (unsigned)(c1 - c0) - 1;
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
+  const int i = blockIdx.y * kSegDotVecs + (int)threadIdx.x;
+  if (threadIdx.x < kSegDotVecs && i < i1) {
+    const double* q = partial + (long long)i * t.nchunks;
     double sum = 0.0;
-    for (int c = t.pchunk[p]; c < t.pchunk[p + 1]; ++c) sum += __ldcg(&partial[(long long)i * t.nchunks + c]);
+    for (int c = c0; c < c1; c += 16) {
+      double v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = c + u < c1 ? __ldcg(q + c + u) : 0.0;
+#pragma unroll
+      for (int u = 0; u < 16; ++u) sum += v[u];
+    }
     h[(long long)i * t.K + p] = sum;
   }
-  if (threadIdx.x == 0) t.counter[p] = 0u;
+  if (threadIdx.x == 0) *counter = 0u;
 }
 
 // h[i K + p] = sum over problem p's chunks (in order) of the partial dots of vector i
@@ -2190,9 +2200,10 @@ __global__ void __launch_bounds__(kSegUpdSub* kSegUpdGroups)
       const int b0 = t.pchunk[p], b1 = t.pchunk[p + 1];
       const unsigned total = (unsigned)(b1 - 1 - b0) * kPieces +
                              (unsigned)((t.end[b1 - 1] - t.start[b1 - 1] + kSegUpdSub - 1) / kSegUpdSub);
-      last = atomicAdd(&t.counter[p], 1u) == total - 1;
+      unsigned* counter = t.counter + p * kSegCounters;
+      last = atomicAdd(counter, 1u) == total - 1;
       if (last) {
-        t.counter[p] = 0u;
+        *counter = 0u;
         ws[0] = 0.0;
       }
     }
@@ -2249,7 +2260,15 @@ __global__ void seg_normalise_kernel(SegTable t, const double* __restrict__ hn, 
   const int b = seg_chunk(t);
   const int p = t.prob[b];
   if (!t.active[p]) return;
-  const double h = sqrt(fmax(0.0, hn[p])), f = h > 0 ? 1.0 / h : 0.0;
+  // (the root and the quotient once a CTA: by every thread they were half of the FP64 work, 34 us on 1.8e6
+  // elements, where the splits take 16)
+  __shared__ double fs;
+  if (threadIdx.x == 0) {
+    const double h = sqrt(fmax(0.0, hn[p]));
+    fs = h > 0 ? 1.0 / h : 0.0;
+  }
+  __syncthreads();
+  const double f = fs;
   for (long long e = t.start[b] + threadIdx.x; e < t.end[b]; e += blockDim.x) {
     const double v = f * in[e];
     out[e] = v;
@@ -2932,6 +2951,7 @@ void launch_multidot(int n, int nvec, const T* V, long long ldv, const T* w, dou
   multidot_kernel<T><<<grid, kRedThreads, 0, st>>>(n, V, ldv, w, partial, nblk);
 }
 template void launch_multidot<float>(int, int, const float*, long long, const float*, double*, int, cudaStream_t);
+template void launch_multidot<double>(int, int, const double*, long long, const double*, double*, int, cudaStream_t);
 
 void launch_reduce_partials(int nvec, int nblk, const double* partial, double* h, cudaStream_t st) {
   ++t_launches;
