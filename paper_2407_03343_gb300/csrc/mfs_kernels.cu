@@ -1694,30 +1694,51 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, cons
   T acc[kGemvRowsPerWarp];
 #pragma unroll
   for (int r = 0; r < kGemvRowsPerWarp; ++r) acc[r] = T(0);
-  const int nvec = nc / W;
-  for (int v = lane; v < nvec; v += 32) {
-#pragma unroll
-    for (int r = 0; r < kGemvRowsPerWarp; ++r) {
-      int row = r0 + r;
-      if (row < nr) {
-        VT m;
-        if constexpr (PAIRED) {
-          const VT* q = reinterpret_cast<const VT*>(M + (long long)r0 * ld) + 2 * v;
-          const VT a = q[0], b = q[1];
-          if (r == 0) m = VT{a.x, a.z, b.x, b.z};
-          else m = VT{a.y, a.w, b.y, b.w};
-        } else {
-          m = reinterpret_cast<const VT*>(M + (long long)row * ld)[v];
-        }
-        acc[r] += dot_vec<T>(m, xv + v * W);
+  if constexpr (PAIRED) {
+    // a 16-byte load holds two columns of the warp's row pair, so the loads of a warp are contiguous and x is
+    // read once for both rows, two elements at a time where its offset is even (loads are what bounds this; four
+    // columns a lane with the row loop of the plain layout read the matrix in two strided halves: both factors of
+    // N = 400 for 8 / 60 spheres that share them 37.5 / 222 us, now 25 / 103; from plain rows 21 / 103)
+    static_assert(sizeof(T) == 4 && kGemvRowsPerWarp == 2, "FP32 row pairs");
+    const float* pr = M + (long long)r0 * ld;
+    const float4* q = reinterpret_cast<const float4*>(pr);
+    if ((reinterpret_cast<uintptr_t>(xv) & 7) == 0) {
+      const float2* x2 = reinterpret_cast<const float2*>(xv);
+#pragma unroll 4
+      for (int v = lane; v < nc / 2; v += 32) {
+        const float4 m = __ldg(q + v);
+        const float2 xe = __ldg(x2 + v);
+        acc[0] += m.x * xe.x + m.z * xe.y;
+        acc[1] += m.y * xe.x + m.w * xe.y;
+      }
+    } else {
+#pragma unroll 4
+      for (int v = lane; v < nc / 2; v += 32) {
+        const float4 m = __ldg(q + v);
+        const float xa = __ldg(xv + 2 * v), xb = __ldg(xv + 2 * v + 1);
+        acc[0] += m.x * xa + m.z * xb;
+        acc[1] += m.y * xa + m.w * xb;
       }
     }
-  }
-  for (int c = nvec * W + lane; c < nc; c += 32) {
+    if ((nc & 1) && lane == 0) {
+      acc[0] += pr[2LL * (nc - 1)] * xv[nc - 1];
+      acc[1] += pr[2LL * (nc - 1) + 1] * xv[nc - 1];
+    }
+  } else {
+    const int nvec = nc / W;
+    for (int v = lane; v < nvec; v += 32) {
 #pragma unroll
-    for (int r = 0; r < kGemvRowsPerWarp; ++r) {
-      int row = r0 + r;
-      if (row < nr) acc[r] += (PAIRED ? M[(long long)r0 * ld + 2LL * c + r] : M[(long long)row * ld + c]) * xv[c];
+      for (int r = 0; r < kGemvRowsPerWarp; ++r) {
+        int row = r0 + r;
+        if (row < nr) acc[r] += dot_vec<T>(reinterpret_cast<const VT*>(M + (long long)row * ld)[v], xv + v * W);
+      }
+    }
+    for (int c = nvec * W + lane; c < nc; c += 32) {
+#pragma unroll
+      for (int r = 0; r < kGemvRowsPerWarp; ++r) {
+        int row = r0 + r;
+        if (row < nr) acc[r] += M[(long long)row * ld + c] * xv[c];
+      }
     }
   }
 #pragma unroll
