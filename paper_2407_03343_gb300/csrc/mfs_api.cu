@@ -342,6 +342,30 @@ mfs_status upload(mfs_ctx* c, T*& dst, const std::vector<T>& v) {
   return MFS_OK;
 }
 
+// Work items of the double-float GEMVs of a context over n jobs (of order[i]) with these matrices.  The host
+// vector ends here, so the copy is waited for.
+mfs_status set_gemv_items(mfs_ctx* c, std::initializer_list<GemvBatch<float>*> gs, int n, const int* order,
+                          const float* const* mat, int max_rows, int max_cols) {
+  const void* const* m = reinterpret_cast<const void* const*>(mat);
+  std::vector<int2> items;
+  int most = gemv_items(n, order, m, items);
+  const GemvShape sh = most > 1 ? gemv_shape(n, max_rows, max_cols) : GemvShape{kGemvMaxRhs, 0};
+  if (sh.cap < most) most = gemv_items(n, order, m, items, sh.cap);
+  int2* d = nullptr;
+  if (most > 1) {
+    mfs_status s = upload(c, d, items);
+    if (s != MFS_OK) return s;
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  }
+  for (GemvBatch<float>* g : gs) {
+    g->items = d;
+    g->n_items = (int)items.size();
+    g->items_max = most;
+    g->col_warps = sh.col_warps;
+  }
+  return MFS_OK;
+}
+
 // ------------------------------------------------------------------ operator pieces
 template <typename T> struct Ops;
 template <> struct Ops<float> {
@@ -2526,12 +2550,13 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
     std::vector<const float*> mA2(P), mV2(P);
     std::vector<int> rA(P), cA(P), lA(P), rV(P), cV(P), lV(P);
     std::vector<long long> xA(P), yA(P), xV(P), yV(P);
-    int maxA = 0, maxV = 0;
+    int maxA = 0, maxV = 0, maxC = 0;
     for (int k = 0; k < P; ++k) {
       const Factor& F = c->factors[d.factor_id[k]];
       mA64[k] = F.A64; mA32[k] = F.A32; mV64[k] = F.V64; mV32[k] = F.V32;
       mA2[k] = reinterpret_cast<const float*>(F.A2); mV2[k] = reinterpret_cast<const float*>(F.V2);
       rA[k] = F.rank; cA[k] = F.m; lA[k] = F.ldA;
+      maxC = std::max(maxC, F.m);
       xA[k] = 3LL * d.colloc_off[k]; yA[k] = tmp_off[k];
       rV[k] = F.ncol; cV[k] = F.rank; lV[k] = F.ldV;
       xV[k] = tmp_off[k]; yV[k] = d.unk_off[k];
@@ -2557,17 +2582,17 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
     for (int f = 0; f < nf; ++f)
       for (int k = 0; k < P; ++k)
         if (d.factor_id[k] == f) order.push_back(k);
-    std::vector<int2> items;
-    const int items_max = gemv_items(P, order.data(), reinterpret_cast<const void* const*>(mA2.data()), items);
-    int* d_order = nullptr;
-    int2* d_items = nullptr;
-    if ((s = upload(c, d_order, order)) != MFS_OK || (s = upload(c, d_items, items)) != MFS_OK) return s;
-    for (GemvBatch<float>* g : {&c->gA32, &c->gA2, &c->gV2}) {
-      g->job_list = d_order;
-      g->n_list = P;
-      g->items = d_items;
-      g->n_items = (int)items.size();
-      g->items_max = items_max;
+    if ((s = set_gemv_items(c, {&c->gA32, &c->gA2, &c->gV2}, P, order.data(), mA2.data(), std::max(maxA, maxV), maxC)) !=
+        MFS_OK)
+      return s;
+    // (spheres in order need no list: it would be one more load before the first of a matrix)
+    if (!std::is_sorted(order.begin(), order.end())) {
+      int* d_order = nullptr;
+      if ((s = upload(c, d_order, order)) != MFS_OK) return s;
+      for (GemvBatch<float>* g : {&c->gA32, &c->gA2, &c->gV2}) {
+        g->job_list = d_order;
+        g->n_list = P;
+      }
     }
     c->gA32.paired = true;
     int *d_rA, *d_cA, *d_lA, *d_rV, *d_cV, *d_lV;
@@ -2650,7 +2675,7 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
         std::vector<const float*> mm;
         std::vector<int> rr, cc, ll;
         std::vector<long long> xx, yy;
-        int mx = 0;
+        int mx = 0, mc = 0;
         for (int k : rest) {
           const Factor& G = c->factors[d.factor_id[k]];
           mm.push_back(q ? G.Q32 : G.A32);
@@ -2660,6 +2685,7 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
           xx.push_back(3LL * d.colloc_off[k]);
           yy.push_back(q ? 3LL * n_eq * k : tmp_off[k]);
           mx = std::max(mx, rr.back());
+          mc = std::max(mc, cc.back());
         }
         out = GemvBatch<float>();
         out.n_jobs = (int)mm.size();
@@ -2679,12 +2705,7 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
         out.x_off = dx;
         out.y_off = dy;
         if (!q) {
-          std::vector<int2> items;
-          out.items_max = gemv_items(out.n_jobs, nullptr, reinterpret_cast<const void* const*>(mm.data()), items);
-          int2* di = nullptr;
-          if ((st2 = upload(c, di, items))) return st2;
-          out.items = di;
-          out.n_items = (int)items.size();
+          if ((st2 = set_gemv_items(c, {&out}, out.n_jobs, nullptr, mm.data(), mx, mc))) return st2;
           out.paired = true;
         }
         return MFS_OK;

@@ -239,14 +239,34 @@ struct GemvBatch {
   const int* job_list = nullptr;    // optional: the jobs to run (n_list of them); the grid then
   int n_list = 0;                   //   covers only those
   bool paired = false;  // FP32: rows stored in pairs, a column's two rows side by side
-  // double-float GEMVs: work items (first, count) over the job list (or the jobs), the right-hand
-  // sides of one matrix, and the largest count
+  // double-float GEMVs: work items (first, count) over the job list (or the jobs; null: one each), the
+  // right-hand sides of one matrix, the largest count, and the warps that share the columns of a row group
+  // (0: by the number of groups)
   const int2* items = nullptr;
-  int n_items = 0, items_max = 1;
+  int n_items = 0, items_max = 1, col_warps = 0;
 };
 // Work items of jobs whose matrices are mat[list[i]] (list null: mat[i]): runs of equal matrices in
-// even shares of at most four; returns the largest count.
-int gemv_items(int n, const int* list, const void* const* mat, std::vector<int2>& items);
+// even shares of at most `cap` (at most kGemvMaxRhs); returns the largest count.
+constexpr int kGemvMaxRhs = 4;
+int gemv_items(int n, const int* list, const void* const* mat, std::vector<int2>& items, int cap = kGemvMaxRhs);
+// How the double-float GEMVs of one context take right-hand sides that share matrices: items of up to `cap`
+// of them, and col_warps as above.
+//  - Up to one wave of the single right-hand side kernel (10 CTAs of a row pair on 152 SMs) latency counts, and
+//    one right-hand side an item, four warps to its columns, is the shortest chain (3 spheres, N = 24 / 200:
+//    17.4 -> 14.6 / 22.9 -> 18.7 us for the split and both factors; 8 spheres, N = 100: 20.8 -> 18.5).
+//  - With short columns (a load or two a lane when four warps share them) and many row pairs the sums over
+//    lanes and warps are most of the work, and a row group a warp halves them: 60 spheres, N = 50 (4,500 row
+//    pairs) 26.5 -> 22.3 one right-hand side an item, 25.6-27.7 with two or four; 150, N = 50 (11,250)
+//    41.1 -> 29.4 with four, 343, N = 24 / 50 / 100 39.7 / 68.7 / 137 -> 26.9 / 46.1 / 94.9 with four,
+//    29.2 / 48.1 / 105 with one.
+//  - With longer columns two right-hand sides an item up to 5,000 row pairs (8 spheres, N = 400: 47.6 -> 43.6,
+//    with the FP32 factor 42.5 -> 37.5), which gives the chip more CTAs.
+//  - Else four right-hand sides a read and the warps by the number of groups (20 spheres, N = 100, 3,000 row
+//    pairs: 22.8, a warp a group 25-34; 60 spheres, N = 200, 1,200 columns: 72.5, a warp a group 70-77).
+struct GemvShape {
+  int cap, col_warps;
+};
+GemvShape gemv_shape(int n_jobs, int max_rows, int max_cols);
 template <typename T>
 void launch_gemv(const GemvBatch<T>& b, const T* x, T* y, cudaStream_t st);
 // Double-float GEMV on the FP32 pipes: b.mat holds row pairs of (hi, lo) float pairs, a column as

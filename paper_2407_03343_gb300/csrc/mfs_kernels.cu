@@ -1839,7 +1839,6 @@ __device__ __forceinline__ void gemv_step(GemvAcc& a, f2x mh, f2x ml, float2 xe)
 }
 
 constexpr int kGemvPairThreads = 128;
-constexpr int kGemvMaxRhs = 4;
 
 template <bool F32, int C, int RP, int KS>
 __device__ __forceinline__ void gemv_pairs(const GemvBatch<float>& B, const int* job, int rp0,
@@ -1978,7 +1977,7 @@ template <bool F32, int CMAX, int KS>
 __global__ void __launch_bounds__(kGemvPairThreads, CMAX == 1 ? 10 : 1) gemv_pair_kernel(GemvBatch<float> B, const float2* __restrict__ x,
                                                                    float2* __restrict__ y2, double* __restrict__ y64) {
   constexpr int RP = gemv_rp(CMAX);
-  const int2 it = B.items[blockIdx.x];
+  const int2 it = B.items ? B.items[blockIdx.x] : make_int2(blockIdx.x, 1);
   const int rp0 = (KS > 1 ? blockIdx.y : blockIdx.y * (kGemvPairThreads / 32) + (threadIdx.x >> 5)) * RP;
   int job[CMAX];
   bool any = false;
@@ -2913,14 +2912,21 @@ void launch_gemv(const GemvBatch<T>& b, const T* x, T* y, cudaStream_t st) {
 }
 template void launch_gemv<float>(const GemvBatch<float>&, const float*, float*, cudaStream_t);
 
-int gemv_items(int n, const int* list, const void* const* mat, std::vector<int2>& items) {
+GemvShape gemv_shape(int n_jobs, int max_rows, int max_cols) {
+  const long long pairs = (long long)n_jobs * ((max_rows + 1) / 2);
+  if (pairs <= 10 * 152) return {1, 4};
+  if (max_cols <= 640 && pairs > 4000) return {pairs <= 10000 ? 1 : kGemvMaxRhs, 1};
+  if (max_cols > 640 && pairs <= 5000) return {2, 4};
+  return {kGemvMaxRhs, 0};
+}
+
+int gemv_items(int n, const int* list, const void* const* mat, std::vector<int2>& items, int cap) {
   items.clear();
   int most = 1;
   for (int i = 0; i < n;) {
     int e = i + 1;
     while (e < n && mat[list ? list[e] : e] == mat[list ? list[i] : i]) ++e;
-    // even shares of at most kGemvMaxRhs
-    const int cnt = e - i, parts = (cnt + kGemvMaxRhs - 1) / kGemvMaxRhs;
+    const int cnt = e - i, parts = (cnt + cap - 1) / cap;
     for (int q = 0; q < parts; ++q) {
       const int i0 = i + (int)((long long)cnt * q / parts), i1 = i + (int)((long long)cnt * (q + 1) / parts);
       items.push_back(make_int2(i0, i1 - i0));
@@ -2939,11 +2945,11 @@ static void gemv_pair_launch(const GemvBatch<float>& b, const float2* x, float2*
   const int nrp = (b.max_rows + 1) / 2, groups = (nrp + gemv_rp(c) - 1) / gemv_rp(c);
   // several right-hand sides: the CTA's warps share the columns of a row group while there are fewer
   // groups than 64 warps a SM, and take a group each above that
-  const bool split = c == 1 || (long long)b.n_items * groups < 64LL * 152;
+  const bool split = b.col_warps ? b.col_warps > 1 : c == 1 || (long long)b.n_items * groups < 64LL * 152;
   const dim3 grid(b.n_items, split ? groups : (groups + 3) / 4);
 #define MFS_GEMV(C, KS) gemv_pair_kernel<F32, C, KS><<<grid, kGemvPairThreads, 0, st>>>(b, x, y2, y64)
   switch (c) {
-    case 1: MFS_GEMV(1, 4); break;
+    case 1: if (split) MFS_GEMV(1, 4); else MFS_GEMV(1, 1); break;
     case 2: if (split) MFS_GEMV(2, 4); else MFS_GEMV(2, 1); break;
     case 3: if (split) MFS_GEMV(3, 4); else MFS_GEMV(3, 1); break;
     default: if (split) MFS_GEMV(4, 4); else MFS_GEMV(4, 1);
