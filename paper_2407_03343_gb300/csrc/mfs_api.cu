@@ -2032,7 +2032,6 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   }
   c->tg.n_tiles1 = (int)ts1.size();
   for (int q : tcn1) c->tg.n_pieces1 += (q + kTileTargets / 8 - 1) / (kTileTargets / 8);
-  for (int q : tcn) c->tg.n_pieces4 += (q + kTileTargets / 2 - 1) / (kTileTargets / 2);
   if ((s = upload(c, c->tg.tile1_sphere, ts1)) != MFS_OK) return s;
   if ((s = upload(c, c->tg.tile1_start, tst1)) != MFS_OK) return s;
   if ((s = upload(c, c->tg.tile1_count, tcn1)) != MFS_OK) return s;
@@ -2498,6 +2497,8 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
         }
       }
       noff.push_back((int)nidx.size());
+      ff.near_max = std::max(ff.near_max, n_near);
+      ff.near_mean += (double)n_near / P;
       xoff.push_back((int)xidx.size());
       nfar += mk * (long long)n_eq * (P - 1 - n_near);
     }
@@ -3401,8 +3402,8 @@ mfs_status mfs_tune_pairs(mfs_ctx* c, mfs_pair_shapes* out) {
     ms = t / 2.0;
     return MFS_OK;
   };
-  // parts 0: the wave-filling rule; packed -1: the scalar far kernel
-  const std::vector<PairShape> cands = {{1, 1, 0}, {1, 0, 0}, {4, 1, 0}, {4, 0, 0}};
+  // parts 0: by the kernel's rule; packed -1: the scalar far kernel
+  const std::vector<PairShape> cands = {{1, 1, 0}, {1, 0, 0}};
   const std::vector<PairShape> far_cands = {{1, 1, 0}, {1, 0, 0}, {4, 1, 0}, {4, 0, 0}, {4, 1, -1}, {4, 0, -1}};
   auto tune = [&](auto&& launch_with, PairShape& best, double& best_ms, const std::vector<PairShape>& cs) -> mfs_status {
     best_ms = -1;
@@ -3436,7 +3437,7 @@ mfs_status mfs_tune_pairs(mfs_ctx* c, mfs_pair_shapes* out) {
                   best, ms, cands)) != MFS_OK)
       return s;
     c->shape_near = best;
-    PairShape rn = resolve_near_shape(c->tg, best, kPairMaxParts);
+    PairShape rn = resolve_near_shape(c->tg, c->src, c->ff, best, kPairMaxParts);
     r.near_nodes_per_thread = rn.nt;
     r.near_parts = rn.parts;
     r.near_ms = ms;

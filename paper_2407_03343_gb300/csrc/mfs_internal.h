@@ -59,7 +59,7 @@ struct TargetSet {
   int n = 0;             // nodes
   int n_tiles = 0;       // tiles of up to 512 nodes (4 per thread)
   int n_tiles1 = 0;      // tiles of up to 128 nodes (1 per thread), used when there are few large tiles
-  int n_pieces4 = 0, n_pieces1 = 0;  // their halves that hold nodes (the double-float kernels' CTAs)
+  int n_pieces1 = 0;     // their halves that hold nodes (the double-float kernels' CTAs)
   float4* pos32 = nullptr;   // (x - c_k, y - c_k, z - c_k, sqrt w) per node, FP32
   double* pos64 = nullptr;   // same, 4 doubles per node
   int* tile_sphere = nullptr;
@@ -100,6 +100,8 @@ struct FarField {
   float4* eq32 = nullptr;   // equivalent-source positions relative to the owner centre
   int* near_off = nullptr;  // P+1: CSR of the near spheres of each sphere, ascending
   int* near_idx = nullptr;
+  int near_max = 0;         // the longest list and the mean one
+  double near_mean = 0;
   int* excl_off = nullptr;  // P+1: the near spheres and the sphere itself, ascending (far: the rest)
   int* excl_idx = nullptr;
   const float* q = nullptr; // equivalent strengths, 3 n_eq per sphere, sphere-major
@@ -193,7 +195,8 @@ void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarFi
 void launch_pairs_far(const TargetSet& tg, const SourceSet& src, const FarField& ff, double* out, double visc,
                       double* partial, int max_parts, cudaStream_t st, PairShape shape = PairShape());
 // the shape a launch with `shape` resolves to (nodes per thread, parts), for reporting
-PairShape resolve_near_shape(const TargetSet& tg, PairShape shape, int max_parts);
+PairShape resolve_near_shape(const TargetSet& tg, const SourceSet& src, const FarField& ff, PairShape shape,
+                             int max_parts);
 PairShape resolve_far_shape(const TargetSet& tg, PairShape shape, int max_parts);
 PairShape resolve_dw_shape(const TargetSet& tg, const SourceSet& src, PairShape shape, int max_parts);
 

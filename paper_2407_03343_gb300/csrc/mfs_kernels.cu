@@ -713,64 +713,25 @@ __device__ __forceinline__ void dw_fold(dw& u, const dw2& m) {
   u = dw_add(u, dw_add(dw{h0, l0}, dw{h1, l1}));
 }
 
-// Targets of one tile (NT per thread, taken one after the other against each staged round) and
-// their sums for R right-hand sides: in registers for one per thread, else in the thread's own
-// column of shared memory, read and written once a round.
-template <int R, int NT>
+// A thread's target and its sums for R right-hand sides.
+template <int R>
 struct DWTile {
   dw x[3];
   dw u[R][3];
-  __device__ __forceinline__ void load(int) {}
-  __device__ __forceinline__ void store(int) {}
 };
-template <int NT>
-struct DwColumns {
-  float2 x[NT][3][kDwThreads], u[NT][3][kDwThreads];
-};
-template <int NT>
-struct DWTileShared {
-  DwColumns<NT>* c;
-  dw x[3];
-  dw u[1][3];
-  __device__ __forceinline__ void load(int q) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float2 a = c->x[q][k][threadIdx.x], b = c->u[q][k][threadIdx.x];
-      x[k] = dw{a.x, a.y};
-      u[0][k] = dw{b.x, b.y};
-    }
-  }
-  __device__ __forceinline__ void store(int q) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) c->u[q][k][threadIdx.x] = make_float2(u[0][k].h, u[0][k].l);
-  }
-};
-template <>
-struct DWTile<1, 4> : DWTileShared<4> {};
 
-// whether this warp has a target among the q-th kDwThreads of the piece
-__device__ __forceinline__ bool dw_warp_live(int q, int cnt) {
-  return (int)(threadIdx.x & ~31u) + q * kDwThreads < cnt;
-}
+// whether this warp has a target of the piece
+__device__ __forceinline__ bool dw_warp_live(int cnt) { return (int)(threadIdx.x & ~31u) < cnt; }
 
-template <int R, int NT>
-__device__ __forceinline__ void dw_load_targets(const PairArgs<double>& A, int start, int cnt, DWTile<R, NT>& T) {
+template <int R>
+__device__ __forceinline__ void dw_load_targets(const PairArgs<double>& A, int start, int cnt, DWTile<R>& T) {
+  const int idx = threadIdx.x;
+  const D4 p = A.tgt[start + (idx < cnt ? idx : cnt - 1)];
+  T.x[0] = dw_split(p.x);
+  T.x[1] = dw_split(p.y);
+  T.x[2] = dw_split(p.z);
 #pragma unroll
-  for (int q = 0; q < NT; ++q) {
-    int idx = threadIdx.x + q * kDwThreads;
-    int node = start + (idx < cnt ? idx : cnt - 1);
-    D4 p = A.tgt[node];
-    T.x[0] = dw_split(p.x);
-    T.x[1] = dw_split(p.y);
-    T.x[2] = dw_split(p.z);
-#pragma unroll
-    for (int r = 0; r < R; ++r) T.u[r][0] = T.u[r][1] = T.u[r][2] = dw{0.f, 0.f};
-    if constexpr (NT > 1) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) T.c->x[q][k][threadIdx.x] = make_float2(T.x[k].h, T.x[k].l);
-      T.store(q);
-    }
-  }
+  for (int r = 0; r < R; ++r) T.u[r][0] = T.u[r][1] = T.u[r][2] = dw{0.f, 0.f};
 }
 
 // Grid of a segment: on each axis the spacing 2^(e - 24) with 2^e above every |x - y| of the
@@ -865,60 +826,55 @@ __device__ __forceinline__ DwTarget dw_target(const DwGrid& G, const dw (&x)[3])
 }
 
 // A round of nu source pairs against the targets of the piece.
-template <int R, int NT, int TILE, int FORM>
+template <int R, int TILE, int FORM>
 __device__ __forceinline__ void dw_proxy_round(const DwGrid& G, unsigned mask, int nu, int cnt, const float* sp,
-                                               const float* rest, const float (*sf)[6 * TILE], DWTile<R, NT>& T) {
-#pragma unroll 1
-  for (int q = 0; q < NT; ++q) {
-    if (!dw_warp_live(q, cnt)) continue;
-    T.load(q);
-    const DwTarget X = dw_target<FORM>(G, T.x);
-    dw2 m[R][3];
+                                               const float* rest, const float (*sf)[6 * TILE], DWTile<R>& T) {
+  if (!dw_warp_live(cnt)) return;
+  const DwTarget X = dw_target<FORM>(G, T.x);
+  dw2 m[R][3];
 #pragma unroll
-    for (int r = 0; r < R; ++r) m[r][0] = m[r][1] = m[r][2] = dw2{0, 0};
-    for (int u0 = 0; u0 < nu; u0 += kDwGroup) {
-      dw2 sum[R][3];
+  for (int r = 0; r < R; ++r) m[r][0] = m[r][1] = m[r][2] = dw2{0, 0};
+  for (int u0 = 0; u0 < nu; u0 += kDwGroup) {
+    dw2 sum[R][3];
 #pragma unroll
-      for (int r = 0; r < R; ++r) sum[r][0] = sum[r][1] = sum[r][2] = dw2{0, 0};
-      const int u1 = min(nu, u0 + kDwGroup);
+    for (int r = 0; r < R; ++r) sum[r][0] = sum[r][1] = sum[r][2] = dw2{0, 0};
+    const int u1 = min(nu, u0 + kDwGroup);
 #pragma unroll 2
-      for (int u = u0; u < u1; ++u) {
-        const ulonglong2* P = reinterpret_cast<const ulonglong2*>(sp) + 3 * u;
-        DwGeom g;
-        dw_geometry<FORM>(X, P[0], P[1], P[2], reinterpret_cast<const f2x*>(rest) + 3 * u, g);
+    for (int u = u0; u < u1; ++u) {
+      const ulonglong2* P = reinterpret_cast<const ulonglong2*>(sp) + 3 * u;
+      DwGeom g;
+      dw_geometry<FORM>(X, P[0], P[1], P[2], reinterpret_cast<const f2x*>(rest) + 3 * u, g);
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          if (R > 1 && !(mask >> r & 1u)) continue;
-          const ulonglong2* F = reinterpret_cast<const ulonglong2*>(sf[r]) + 3 * u;
-          const ulonglong2 fa = F[0], fb = F[1], fc = F[2];
-          const f2x fh[3] = {fa.x, fa.y, fb.x}, fl[3] = {fb.y, fc.x, fc.y};
-          f2x nh, l;
-          dw_ndot(g, fh, fl, nh, l);
-          const f2x ph = f2neg(nh);
+      for (int r = 0; r < R; ++r) {
+        if (R > 1 && !(mask >> r & 1u)) continue;
+        const ulonglong2* F = reinterpret_cast<const ulonglong2*>(sf[r]) + 3 * u;
+        const ulonglong2 fa = F[0], fb = F[1], fc = F[2];
+        const f2x fh[3] = {fa.x, fa.y, fb.x}, fl[3] = {fb.y, fc.x, fc.y};
+        f2x nh, l;
+        dw_ndot(g, fh, fl, nh, l);
+        const f2x ph = f2neg(nh);
 #pragma unroll
-          for (int c = 0; c < 3; ++c) dw_accumulate(g, dw_project(g, c, fh[c], fl[c], nh, ph, l), sum[r][c]);
-        }
+        for (int c = 0; c < 3; ++c) dw_accumulate(g, dw_project(g, c, fh[c], fl[c], nh, ph, l), sum[r][c]);
       }
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) m[r][c] = dw2_add(m[r][c], sum[r][c]);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) dw_fold(T.u[r][c], m[r][c]);
-    T.store(q);
+      for (int c = 0; c < 3; ++c) m[r][c] = dw2_add(m[r][c], sum[r][c]);
   }
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) dw_fold(T.u[r][c], m[r][c]);
 }
 
 // Proxy Stokeslets [r_lo, r_hi) of the flattened proxy index (sphere o = j / N, proxy j - o N; the
 // range holds none of the target sphere's own), one sphere at a time in rounds of at most TILE.
-template <int R, int NT, int TILE>
+template <int R, int TILE>
 __device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const CentreShift64& sh,
                                                const float2* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
                                                int cnt, float* sp, float (*sf)[6 * TILE], DwGrid* grids, int& segs,
-                                               DWTile<R, NT>& T) {
+                                               DWTile<R>& T) {
   for (int s0 = r_lo; s0 < r_hi;) {
     const int o = s0 / A.N, j0 = s0 - o * A.N;
     const int seg = min(r_hi - s0, A.N - j0);  // what is left of sphere o
@@ -954,8 +910,8 @@ __device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const 
       }
     }
     __syncthreads();
-    if (G.close) dw_proxy_round<R, NT, TILE, DW_REST>(G, mask, nu, cnt, sp, rest, sf, T);
-    else dw_proxy_round<R, NT, TILE, DW_GRID>(G, mask, nu, cnt, sp, rest, sf, T);
+    if (G.close) dw_proxy_round<R, TILE, DW_REST>(G, mask, nu, cnt, sp, rest, sf, T);
+    else dw_proxy_round<R, TILE, DW_GRID>(G, mask, nu, cnt, sp, rest, sf, T);
     s0 += ns;
   }
 }
@@ -964,10 +920,10 @@ __device__ __forceinline__ void dw_proxy_range(const PairArgs<double>& A, const 
 // the target sphere's own), one sphere at a time.  With u and 1/r the triple's field is
 //   (1/r) [ f + (u.f) u + (1/r) [ t x u + (1/r) (3 (u.q) u - q) ] ].
 // Strengths per right-hand side and pair of nodes: f, t, -q and 3 q, high and low words.
-template <int R, int NT, int TILE>
+template <int R, int TILE>
 __device__ __forceinline__ void dw_image_range(const PairArgs<double>& A, const CentreShift64& sh,
                                                const float2* const (&lam)[R], unsigned mask, int r_lo, int r_hi,
-                                               int cnt, float* sp, float (*si)[24 * TILE], DWTile<R, NT>& T) {
+                                               int cnt, float* sp, float (*si)[24 * TILE], DWTile<R>& T) {
   for (int s0 = r_lo; s0 < r_hi;) {
     const int o = A.img_owner[s0];
     const int first = A.img_off[o];
@@ -1002,10 +958,7 @@ __device__ __forceinline__ void dw_image_range(const PairArgs<double>& A, const 
       }
     }
     __syncthreads();
-#pragma unroll 1
-    for (int q = 0; q < NT; ++q) {
-      if (!dw_warp_live(q, cnt)) continue;
-      T.load(q);
+    if (dw_warp_live(cnt)) {
       DwTarget X;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -1063,31 +1016,24 @@ __device__ __forceinline__ void dw_image_range(const PairArgs<double>& A, const 
       for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int c = 0; c < 3; ++c) dw_fold(T.u[r][c], m[r][c]);
-      T.store(q);
     }
     s0 += ns;
   }
 }
 
 // out = mu + sqrt(w) scale u per node, or the scaled partial sum of this source part
-template <int R, int NT>
-__device__ __forceinline__ void dw_write_out(const PairArgs<double>& A, int start, int cnt, DWTile<R, NT>& T, int r,
+template <int R>
+__device__ __forceinline__ void dw_write_out(const PairArgs<double>& A, int start, int cnt, const DWTile<R>& T, int r,
                                              const double* __restrict__ mu, double* __restrict__ out, int part,
                                              int nparts, double* __restrict__ partial, long long pstride) {
+  if ((int)threadIdx.x >= cnt) return;
+  const long long node = start + threadIdx.x;
+  const double sw = A.tgt[node].w;
 #pragma unroll
-  for (int q = 0; q < NT; ++q) {
-    int idx = threadIdx.x + q * kDwThreads;
-    if (idx < cnt) {
-      const long long node = start + idx;
-      const double sw = A.tgt[node].w;
-      T.load(q);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const double g = dw_join(T.u[r][c]) * A.scale;
-        if (nparts > 1) partial[part * pstride + 3 * node + c] = g;
-        else out[3 * node + c] = mu[3 * node + c] + sw * g;
-      }
-    }
+  for (int c = 0; c < 3; ++c) {
+    const double g = dw_join(T.u[r][c]) * A.scale;
+    if (nparts > 1) partial[part * pstride + 3 * node + c] = g;
+    else out[3 * node + c] = mu[3 * node + c] + sw * g;
   }
 }
 
@@ -1105,10 +1051,10 @@ struct DwShared {
 // fill the GPU): part `part` takes a contiguous share of the tile's source list (the sources of
 // every other sphere) and, for nparts > 1, writes its scaled partial sum to
 // partial[part * pstride + 3 node + c] for the last part's CTA to add.
-template <int R, int NT, int TILE, int TILE_IMG>
+template <int R, int TILE, int TILE_IMG>
 __device__ __forceinline__ void dw_all_sources(const PairArgs<double>& A, const CentreShift64& sh, int k,
                                                const float2* const (&lam)[R], unsigned mask, int cnt, int part,
-                                               int nparts, DwShared<R, TILE, TILE_IMG>& S, DWTile<R, NT>& T) {
+                                               int nparts, DwShared<R, TILE, TILE_IMG>& S, DWTile<R>& T) {
   // the proxies before and after sphere k's own (this part's share of them)
   const int total = A.P * A.N;
   const int p_lo = k * A.N, p_w = A.N;
@@ -1117,7 +1063,7 @@ __device__ __forceinline__ void dw_all_sources(const PairArgs<double>& A, const 
   int segs = 0;
 #pragma unroll 1  // (one copy of the loops: with two, 8 spheres took 350 us instead of 311)
   for (int rr = 0; rr < 2; ++rr)
-    dw_proxy_range<R, NT, TILE>(A, sh, lam, mask, rr ? max(pe0, p_lo) + p_w : min(pe0, p_lo),
+    dw_proxy_range<R, TILE>(A, sh, lam, mask, rr ? max(pe0, p_lo) + p_w : min(pe0, p_lo),
                                 rr ? max(pe1, p_lo) + p_w : min(pe1, p_lo), cnt, S.sp, S.sf, S.grids, segs, T);
   // image nodes before and after sphere k's own, this part's share
   const int i_lo = A.img_off[k], i_w = A.img_off[k + 1] - i_lo;
@@ -1125,11 +1071,10 @@ __device__ __forceinline__ void dw_all_sources(const PairArgs<double>& A, const 
   const int ie0 = (int)(i_eff * part / nparts), ie1 = (int)(i_eff * (part + 1) / nparts);
 #pragma unroll 1
   for (int rr = 0; rr < 2; ++rr)
-    dw_image_range<R, NT, TILE_IMG>(A, sh, lam, mask, rr ? max(ie0, i_lo) + i_w : min(ie0, i_lo),
+    dw_image_range<R, TILE_IMG>(A, sh, lam, mask, rr ? max(ie0, i_lo) + i_w : min(ie0, i_lo),
                                     rr ? max(ie1, i_lo) + i_w : min(ie1, i_lo), cnt, S.sp, S.si, T);
 }
 
-template <int NT>
 __device__ __forceinline__ void pair_tile_dw(const PairArgs<double>& A, const int t, const int start, const int cnt,
                                              const int part, const int nparts, double* __restrict__ partial,
                                              const long long pstride) {
@@ -1138,20 +1083,15 @@ __device__ __forceinline__ void pair_tile_dw(const PairArgs<double>& A, const in
   CentreShift64 sh;
   sh.cen = A.cen64;
   sh.init(k);
-  DWTile<1, NT> T;
-  if constexpr (NT > 1) {
-    __shared__ DwColumns<NT> C;
-    T.c = &C;
-  }
-  dw_load_targets<1, NT>(A, start, cnt, T);
+  DWTile<1> T;
+  dw_load_targets(A, start, cnt, T);
   const float2* const lam[1] = {A.lam2};
-  dw_all_sources<1, NT, kDwTile, kDwTileImg>(A, sh, k, lam, 1u, cnt, part, nparts, S, T);
-  dw_write_out<1, NT>(A, start, cnt, T, 0, A.mu, A.out, part, nparts, partial, pstride);
+  dw_all_sources<1, kDwTile, kDwTileImg>(A, sh, k, lam, 1u, cnt, part, nparts, S, T);
+  dw_write_out<1>(A, start, cnt, T, 0, A.mu, A.out, part, nparts, partial, pstride);
 }
 
 // The near part of the far-field split: only the spheres of the target sphere's near list
 // (ascending; runs of consecutive spheres are taken as one range).
-template <int NT>
 __device__ __forceinline__ void pair_tile_dw_near(const PairArgs<double>& A, const int* __restrict__ near_off,
                                                   const int* __restrict__ near_idx, const int t, const int start,
                                                   const int cnt, const int part, const int nparts,
@@ -1161,12 +1101,8 @@ __device__ __forceinline__ void pair_tile_dw_near(const PairArgs<double>& A, con
   CentreShift64 sh;
   sh.cen = A.cen64;
   sh.init(k);
-  DWTile<1, NT> T;
-  if constexpr (NT > 1) {
-    __shared__ DwColumns<NT> C;
-    T.c = &C;
-  }
-  dw_load_targets<1, NT>(A, start, cnt, T);
+  DWTile<1> T;
+  dw_load_targets(A, start, cnt, T);
   const float2* const lam[1] = {A.lam2};
   // this part's share of the near list
   int segs = 0;
@@ -1180,10 +1116,10 @@ __device__ __forceinline__ void pair_tile_dw_near(const PairArgs<double>& A, con
       ++o1;
     }
     ++a;
-    dw_proxy_range<1, NT, kDwTile>(A, sh, lam, 1u, o0 * A.N, (o1 + 1) * A.N, cnt, S.sp, S.sf, S.grids, segs, T);
-    dw_image_range<1, NT, kDwTileImg>(A, sh, lam, 1u, A.img_off[o0], A.img_off[o1 + 1], cnt, S.sp, S.si, T);
+    dw_proxy_range<1, kDwTile>(A, sh, lam, 1u, o0 * A.N, (o1 + 1) * A.N, cnt, S.sp, S.sf, S.grids, segs, T);
+    dw_image_range<1, kDwTileImg>(A, sh, lam, 1u, A.img_off[o0], A.img_off[o1 + 1], cnt, S.sp, S.si, T);
   }
-  dw_write_out<1, NT>(A, start, cnt, T, 0, A.mu, A.out, part, nparts, partial, pstride);
+  dw_write_out<1>(A, start, cnt, T, 0, A.mu, A.out, part, nparts, partial, pstride);
 }
 
 // ------------------------------------------------------------------ far-field kernel (FP32)
@@ -1470,10 +1406,9 @@ __device__ __forceinline__ void parts_finish_nodes(const D4* tgt, long long star
 }
 
 // The piece of a tile that work item `item` = tile x kDwPieces + piece takes; false if it has no targets.
-template <int NT>
 __device__ __forceinline__ bool dw_piece(const PairArgs<double>& A, int t, int piece, int& start, int& cnt) {
-  start = A.tile_start[t] + piece * kDwThreads * NT;
-  cnt = min(kDwThreads * NT, A.tile_count[t] - piece * kDwThreads * NT);
+  start = A.tile_start[t] + piece * kDwThreads;
+  cnt = min(kDwThreads, A.tile_count[t] - piece * kDwThreads);
   return cnt > 0;
 }
 __device__ __forceinline__ void parts_finish_piece(const PairArgs<double>& A, int item, int start, int cnt, int nparts,
@@ -1505,23 +1440,21 @@ __global__ void __launch_bounds__(kPairThreads) velocity_fp64_kernel(PairArgs<do
 #pragma unroll
   for (int c = 0; c < 3; ++c) u[part * pstride + 3 * i + c] = v[c];
 }
-template <int NT>
 __global__ void __launch_bounds__(kDwThreads, kDwCtas) pairs_dw_kernel(PairArgs<double> A, int nparts, double* partial,
-                                                                long long pstride, unsigned* counter) {
+                                                                       long long pstride, unsigned* counter) {
   const int item = blockIdx.x / nparts, t = item / kDwPieces;
   int start, cnt;
-  if (!dw_piece<NT>(A, t, item % kDwPieces, start, cnt)) return;
-  pair_tile_dw<NT>(A, t, start, cnt, blockIdx.x % nparts, nparts, partial, pstride);
+  if (!dw_piece(A, t, item % kDwPieces, start, cnt)) return;
+  pair_tile_dw(A, t, start, cnt, blockIdx.x % nparts, nparts, partial, pstride);
   if (nparts > 1) parts_finish_piece(A, item, start, cnt, nparts, partial, pstride, counter);
 }
-template <int NT>
 __global__ void __launch_bounds__(kDwThreads, kDwCtas) pairs_dw_near_kernel(PairArgs<double> A, const int* near_off,
                                                                      const int* near_idx, int nparts, double* partial,
                                                                      long long pstride, unsigned* counter) {
   const int item = blockIdx.x / nparts, t = item / kDwPieces;
   int start, cnt;
-  if (!dw_piece<NT>(A, t, item % kDwPieces, start, cnt)) return;
-  pair_tile_dw_near<NT>(A, near_off, near_idx, t, start, cnt, blockIdx.x % nparts, nparts, partial, pstride);
+  if (!dw_piece(A, t, item % kDwPieces, start, cnt)) return;
+  pair_tile_dw_near(A, near_off, near_idx, t, start, cnt, blockIdx.x % nparts, nparts, partial, pstride);
   if (nparts > 1) parts_finish_piece(A, item, start, cnt, nparts, partial, pstride, counter);
 }
 // out = mu + sqrt(w) * (sum of the parts), or the plain sum when mu is null; parts added in order
@@ -1577,8 +1510,8 @@ __global__ void __launch_bounds__(kDwThreads, kDwCtas) pairs_dw_batch_kernel(con
   A.mu = bv.mu + bv.voff[w.x];
   A.out = bv.out + bv.voff[w.x];
   int start, cnt;
-  if (!dw_piece<1>(A, w.y, item % kDwPieces, start, cnt)) return;
-  pair_tile_dw<1>(A, w.y, start, cnt, blockIdx.x % nparts, nparts, bv.partial + bv.voff[w.x], bv.pstride);
+  if (!dw_piece(A, w.y, item % kDwPieces, start, cnt)) return;
+  pair_tile_dw(A, w.y, start, cnt, blockIdx.x % nparts, nparts, bv.partial + bv.voff[w.x], bv.pstride);
   if (nparts > 1)
     parts_finish_piece(A, item, start, cnt, nparts, bv.partial + bv.voff[w.x], bv.pstride, bv.counter);
 }
@@ -1620,18 +1553,18 @@ __global__ void __launch_bounds__(kDwThreads, kDwMultiCtas) pairs_dw_multi_kerne
   const int t = w.y;
   const int k = A.tile_sphere[t];
   int start, cnt;
-  if (!dw_piece<1>(A, t, item % kDwPieces, start, cnt)) return;
+  if (!dw_piece(A, t, item % kDwPieces, start, cnt)) return;
   CentreShift64 sh;
   sh.cen = A.cen64;
   sh.init(k);
-  DWTile<R, 1> T;
-  dw_load_targets<R, 1>(A, start, cnt, T);
-  dw_all_sources<R, 1, kDwTileM, kDwTileImgM>(A, sh, k, lam, mask, cnt, part, nparts, S, T);
+  DWTile<R> T;
+  dw_load_targets(A, start, cnt, T);
+  dw_all_sources<R, kDwTileM, kDwTileImgM>(A, sh, k, lam, mask, cnt, part, nparts, S, T);
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     if (!(mask >> r & 1u)) continue;
     const long long off = bv.voff[prob[r]];
-    dw_write_out<R, 1>(A, start, cnt, T, r, bv.mu + off, bv.out + off, part, nparts, bv.partial + off, bv.pstride);
+    dw_write_out<R>(A, start, cnt, T, r, bv.mu + off, bv.out + off, part, nparts, bv.partial + off, bv.pstride);
   }
   if (nparts > 1 && parts_last_arrival(bv.counter, item, nparts)) {
 #pragma unroll
@@ -2640,7 +2573,7 @@ static int shape_nt(const TargetSet& tg, const PairShape& shape) {
 
 // resident CTAs of a pair kernel on the current device (SMs x CTAs per SM), looked up once per
 // (device, kernel)
-static double resident_ctas(const void* kernel, int threads = kPairThreads) {
+static double resident_ctas(const void* kernel, int threads) {
   static std::mutex mtx;
   static std::vector<std::pair<std::pair<int, const void*>, double>> cache;
   int dev = 0;
@@ -2679,11 +2612,9 @@ static int pair_split_parts(long long items, double wave, long long min_sources,
 
 PairShape resolve_dw_shape(const TargetSet& tg, const SourceSet& src, PairShape shape, int max_parts) {
   PairShape r;
-  // one node per thread unless four are asked for: 100 spheres of 1804 nodes 116.1 against 127.4 ms
-  r.nt = shape.nt == 4 || tg.n_tiles1 == 0 ? 4 : 1;
+  r.nt = 1;
   if (shape.parts > 0) r.parts = std::min(shape.parts, max_parts);
-  else r.parts = pair_split_parts(r.nt == 4 ? tg.n_pieces4 : tg.n_pieces1,
-                                  resident_ctas(r.nt == 4 ? (const void*)pairs_dw_kernel<4> : (const void*)pairs_dw_kernel<1>, kDwThreads),
+  else r.parts = pair_split_parts(tg.n_pieces1, resident_ctas((const void*)pairs_dw_kernel, kDwThreads),
                                   (long long)(src.P - 1) * src.N, max_parts);
   return r;
 }
@@ -2692,20 +2623,17 @@ void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const float2* la
                      double visc, double* partial, unsigned* counter, int max_parts, cudaStream_t st, PairShape shape) {
   if (tg.n_tiles == 0) return;
   const PairShape r = resolve_dw_shape(tg, src, shape, max_parts);
-  const int nt = r.nt;
   const int parts = partial ? r.parts : 1;
-  PairArgs<double> A = make_args<double>(tg, src, nullptr, mu, out, visc, nt);
+  PairArgs<double> A = make_args<double>(tg, src, nullptr, mu, out, visc, 1);
   A.lam2 = lam_hat;
-  const long long n3 = 3LL * tg.n;
   ++t_launches;
-  // (with split sources the last CTA of a tile to finish adds the parts)
-  if (nt == 4) pairs_dw_kernel<4><<<kDwPieces * tg.n_tiles * parts, kDwThreads, 0, st>>>(A, parts, partial, n3, counter);
-  else pairs_dw_kernel<1><<<kDwPieces * tg.n_tiles1 * parts, kDwThreads, 0, st>>>(A, parts, partial, n3, counter);
+  // (with split sources the last CTA of a piece to finish adds the parts)
+  pairs_dw_kernel<<<kDwPieces * tg.n_tiles1 * parts, kDwThreads, 0, st>>>(A, parts, partial, 3LL * tg.n, counter);
 }
 
 // source parts per tile so that tiles x parts fill whole waves of the resident CTAs (ties: fewer)
-int wave_parts(long long tiles, const void* kernel, int max_parts, int threads = kPairThreads) {
-  const double wave = resident_ctas(kernel, threads);
+static int wave_parts(long long tiles, const void* kernel, int max_parts) {
+  const double wave = resident_ctas(kernel, kPairThreads);
   if (wave <= 0) return 1;
   int best = 1;
   double best_eff = 0;
@@ -2720,13 +2648,31 @@ int wave_parts(long long tiles, const void* kernel, int max_parts, int threads =
   return best;
 }
 
-PairShape resolve_near_shape(const TargetSet& tg, PairShape shape, int max_parts) {
+// Near part: 64-target CTAs, a thread per node.  (With four from 304 512-node tiles on, 343 spheres: N = 300 at
+// centres 2.5 apart 4.99 ms against 4.65, N = 160 at 3.0 0.82 against 0.78; all pairs of 100 spheres of 1,804 nodes
+// 127.4 against 116.1.)  The parts are whole spheres of lists of uneven length, so their number is what leaves
+// the shortest sum of a resident CTA's share of the work (kPairSplitPartCost sources a part on top) and of the longest
+// CTA, which may start last: cluster of 60 spheres, N = 150, 16 parts 174 us, 4 (whole waves) 215; 125 spheres on
+// a lattice, N = 100, 6 parts 104, 1 128; 20 spheres, N = 100, 9 parts 45, 15 53 (six of them without a sphere).
+PairShape resolve_near_shape(const TargetSet& tg, const SourceSet& src, const FarField& ff, PairShape shape,
+                             int max_parts) {
   PairShape r;
-  r.nt = shape_nt(tg, shape);
-  const long long tiles = r.nt == 4 ? tg.n_tiles : tg.n_tiles1;
-  r.parts = shape.parts > 0 ? std::min(shape.parts, max_parts)
-                            : wave_parts(kDwPieces * tiles, r.nt == 4 ? (const void*)pairs_dw_near_kernel<4>
-                                                                      : (const void*)pairs_dw_near_kernel<1>, max_parts, kDwThreads);
+  r.nt = 1;
+  if (shape.parts > 0) {
+    r.parts = std::min(shape.parts, max_parts);
+    return r;
+  }
+  const double wave = resident_ctas((const void*)pairs_dw_near_kernel, kDwThreads);
+  r.parts = 1;
+  double best = 0;
+  for (int p = 1; wave > 0 && p <= std::min(max_parts, std::max(1, ff.near_max)); ++p) {
+    const double t = tg.n_pieces1 * (ff.near_mean * src.N + kPairSplitPartCost * p) / wave +
+                     (double)((ff.near_max + p - 1) / p) * src.N;
+    if (p == 1 || t < best) {
+      best = t;
+      r.parts = p;
+    }
+  }
   return r;
 }
 
@@ -2734,18 +2680,13 @@ void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarFi
                           const double* mu, double* out, double visc, double* partial, unsigned* counter, int max_parts,
                           cudaStream_t st, PairShape shape) {
   if (tg.n_tiles == 0) return;
-  const PairShape r = resolve_near_shape(tg, shape, max_parts);
-  const int nt = r.nt;
-  PairArgs<double> A = make_args<double>(tg, src, nullptr, mu, out, visc, nt);
+  const PairShape r = resolve_near_shape(tg, src, ff, shape, max_parts);
+  PairArgs<double> A = make_args<double>(tg, src, nullptr, mu, out, visc, 1);
   A.lam2 = lam_hat;
-  const long long tiles = nt == 4 ? tg.n_tiles : tg.n_tiles1;
   const int parts = partial ? r.parts : 1;
-  const long long n3 = 3LL * tg.n;
   ++t_launches;
-  if (nt == 4)
-    pairs_dw_near_kernel<4><<<kDwPieces * tiles * parts, kDwThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3, counter);
-  else
-    pairs_dw_near_kernel<1><<<kDwPieces * tiles * parts, kDwThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts, partial, n3, counter);
+  pairs_dw_near_kernel<<<kDwPieces * tg.n_tiles1 * parts, kDwThreads, 0, st>>>(A, ff.near_off, ff.near_idx, parts,
+                                                                              partial, 3LL * tg.n, counter);
 }
 
 PairShape resolve_far_shape(const TargetSet& tg, PairShape shape, int max_parts) {
