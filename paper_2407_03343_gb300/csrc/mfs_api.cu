@@ -3408,7 +3408,6 @@ mfs_status mfs_tune_pairs(mfs_ctx* c, mfs_pair_shapes* out) {
   auto tune = [&](auto&& launch_with, PairShape& best, double& best_ms, const std::vector<PairShape>& cs) -> mfs_status {
     best_ms = -1;
     for (const PairShape& sh : cs) {
-      if (sh.nt == 1 && c->tg.n_tiles1 == 0) continue;
       double ms = 0;
       mfs_status st = time_it([&] { launch_with(sh); }, ms);
       if (st != MFS_OK) return st;

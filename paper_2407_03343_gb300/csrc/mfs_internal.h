@@ -326,8 +326,8 @@ struct SegTable {
   const int* active = nullptr;
   const int* list = nullptr;    // optional: the chunks of the active problems (nlist of them); the
   int nlist = 0;                //   launches then cover only those
-  unsigned* counter = nullptr;  // optional, kSegCounters K zeros: the dot products are then reduced by the
-                                //   last CTA of a problem's block of vectors instead of a second kernel
+  unsigned* counter = nullptr;  // kSegCounters K zeros: arrivals, the last CTA of a problem's block of
+                                //   vectors adds their dot products
 };
 void launch_seg_dots(const SegTable& t, int nvec, const double* V, long long ldv, const double* w, double* partial,
                      double* h, cudaStream_t st);

@@ -74,8 +74,8 @@ struct CentreShift32 {
   float kh[3], kl[3];
   __device__ void init(int k) {
     for (int c = 0; c < 3; ++c) {
-      kh[c] = k >= 0 ? hi[3 * k + c] : 0.f;
-      kl[c] = k >= 0 ? lo[3 * k + c] : 0.f;
+      kh[c] = hi[3 * k + c];
+      kl[c] = lo[3 * k + c];
     }
   }
   __device__ __forceinline__ float d(int o, int c) const { return (hi[3 * o + c] - kh[c]) + (lo[3 * o + c] - kl[c]); }
@@ -148,8 +148,8 @@ __device__ __forceinline__ void pair_tile(const PairArgs<T>& A, const int t) {
   const int total = A.P * A.N;
   // the proxies before and after sphere k's own, in tiles with exact trip counts
   for (int rr = 0; rr < 2; ++rr) {
-  const int r_lo = rr == 0 ? 0 : (k < 0 ? total : (k + 1) * A.N);
-  const int r_hi = rr == 0 ? (k < 0 ? total : k * A.N) : total;
+  const int r_lo = rr == 0 ? 0 : (k + 1) * A.N;
+  const int r_hi = rr == 0 ? k * A.N : total;
   for (int s0 = r_lo; s0 < r_hi; s0 += kTileProxy) {
     const int ns = min(kTileProxy, r_hi - s0);
     __syncthreads();
@@ -198,7 +198,7 @@ __device__ __forceinline__ void pair_tile(const PairArgs<T>& A, const int t) {
   }
 
   // ---- image nodes (Stokeslet + rotlet + potential dipole at one position)
-  const int self_lo = k >= 0 ? A.img_off[k] : 0, self_hi = k >= 0 ? A.img_off[k + 1] : 0;
+  const int self_lo = A.img_off[k], self_hi = A.img_off[k + 1];
   for (int rr = 0; rr < 2; ++rr) {
   const int r_lo = rr == 0 ? 0 : self_hi;
   const int r_hi = rr == 0 ? self_lo : A.n_img;
@@ -272,15 +272,9 @@ __device__ __forceinline__ void pair_tile(const PairArgs<T>& A, const int t) {
       long long node = start + idx;
       T sw = A.tgt[node].w;
       T gx = (sx[q] + cx[q]) * A.scale, gy = (sy[q] + cy[q]) * A.scale, gz = (sz[q] + cz[q]) * A.scale;
-      if (A.mu) {
-        A.out[3 * node] = A.mu[3 * node] + sw * gx;
-        A.out[3 * node + 1] = A.mu[3 * node + 1] + sw * gy;
-        A.out[3 * node + 2] = A.mu[3 * node + 2] + sw * gz;
-      } else {
-        A.out[3 * node] = gx;
-        A.out[3 * node + 1] = gy;
-        A.out[3 * node + 2] = gz;
-      }
+      A.out[3 * node] = A.mu[3 * node] + sw * gx;
+      A.out[3 * node + 1] = A.mu[3 * node + 1] + sw * gy;
+      A.out[3 * node + 2] = A.mu[3 * node + 2] + sw * gz;
     }
   }
 }
@@ -1520,8 +1514,8 @@ __global__ void __launch_bounds__(kDwThreads, kDwCtas) pairs_dw_batch_kernel(con
 // targets and sources and differ only in their strengths.  Work item (lead problem, 128-node
 // tile, first index into the right-hand-side list, count <= kPairRhs): the position
 // differences, the distance and its powers of each (node, source) pair are formed once in
-// double-float and applied to the strengths of every listed right-hand side (76 of the 205 flops
-// of a Stokeslet pair and 94 of the 477 of an image triple are shared).  Each
+// double-float and applied to the strengths of every listed right-hand side (80 of the 214 flops
+// of a Stokeslet pair and 98 of the 487 of an image triple are shared).  Each
 // right-hand side's sums follow the operation order of pair_tile_dw.
 constexpr int kDwTileM = 128;    // proxy sources staged per round
 constexpr int kDwTileImgM = 32;  // image nodes staged per round
@@ -1596,24 +1590,14 @@ __global__ void pair_parts_reduce_batch_kernel(SegTable t, const PairArgs<double
 constexpr int kGemvThreads = 256;
 constexpr int kGemvRowsPerWarp = 2;
 
-template <typename T> struct Vec;
-template <> struct Vec<float> { using type = float4; static constexpr int w = 4; };
-template <> struct Vec<double> { using type = double2; static constexpr int w = 2; };
-
-template <typename T>
-__device__ __forceinline__ T dot_vec(const typename Vec<T>::type& m, const T* x);
-template <> __device__ __forceinline__ float dot_vec<float>(const float4& m, const float* x) {
+__device__ __forceinline__ float dot_vec(const float4& m, const float* x) {
   return m.x * __ldg(x) + m.y * __ldg(x + 1) + m.z * __ldg(x + 2) + m.w * __ldg(x + 3);
-}
-template <> __device__ __forceinline__ double dot_vec<double>(const double2& m, const double* x) {
-  return m.x * __ldg(x) + m.y * __ldg(x + 1);
 }
 
 // PAIRED: the matrix is stored in row pairs (FP32 copy of Sigma^+ U^T); a warp's two rows are a pair
-template <typename T, bool PAIRED>
-__global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, const T* __restrict__ x, T* __restrict__ y) {
-  using VT = typename Vec<T>::type;
-  constexpr int W = Vec<T>::w;
+template <bool PAIRED>
+__global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<float> B, const float* __restrict__ x,
+                                                            float* __restrict__ y) {
   // jobs sharing a matrix are adjacent, so its rows are read once; with a compacted list the grid
   // covers the active problems' jobs only
   const int job = B.job_list ? B.job_list[blockIdx.x] : blockIdx.x;
@@ -1622,17 +1606,17 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r0 = (blockIdx.y * (kGemvThreads / 32) + warp) * kGemvRowsPerWarp;
   if (r0 >= nr) return;
-  const T* M = B.mat[job];
-  const T* xv = x + B.x_off[job];
-  T acc[kGemvRowsPerWarp];
+  const float* M = B.mat[job];
+  const float* xv = x + B.x_off[job];
+  float acc[kGemvRowsPerWarp];
 #pragma unroll
-  for (int r = 0; r < kGemvRowsPerWarp; ++r) acc[r] = T(0);
+  for (int r = 0; r < kGemvRowsPerWarp; ++r) acc[r] = 0.f;
   if constexpr (PAIRED) {
     // a 16-byte load holds two columns of the warp's row pair, so the loads of a warp are contiguous and x is
     // read once for both rows, two elements at a time where its offset is even (loads are what bounds this; four
     // columns a lane with the row loop of the plain layout read the matrix in two strided halves: both factors of
     // N = 400 for 8 / 60 spheres that share them 37.5 / 222 us, now 25 / 103; from plain rows 21 / 103)
-    static_assert(sizeof(T) == 4 && kGemvRowsPerWarp == 2, "FP32 row pairs");
+    static_assert(kGemvRowsPerWarp == 2, "FP32 row pairs");
     const float* pr = M + (long long)r0 * ld;
     const float4* q = reinterpret_cast<const float4*>(pr);
     if ((reinterpret_cast<uintptr_t>(xv) & 7) == 0) {
@@ -1658,15 +1642,15 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, cons
       acc[1] += pr[2LL * (nc - 1) + 1] * xv[nc - 1];
     }
   } else {
-    const int nvec = nc / W;
+    const int nvec = nc / 4;
     for (int v = lane; v < nvec; v += 32) {
 #pragma unroll
       for (int r = 0; r < kGemvRowsPerWarp; ++r) {
         int row = r0 + r;
-        if (row < nr) acc[r] += dot_vec<T>(reinterpret_cast<const VT*>(M + (long long)row * ld)[v], xv + v * W);
+        if (row < nr) acc[r] += dot_vec(reinterpret_cast<const float4*>(M + (long long)row * ld)[v], xv + 4 * v);
       }
     }
-    for (int c = nvec * W + lane; c < nc; c += 32) {
+    for (int c = 4 * nvec + lane; c < nc; c += 32) {
 #pragma unroll
       for (int r = 0; r < kGemvRowsPerWarp; ++r) {
         int row = r0 + r;
@@ -1676,7 +1660,7 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<T> B, cons
   }
 #pragma unroll
   for (int r = 0; r < kGemvRowsPerWarp; ++r) {
-    T s = acc[r];
+    float s = acc[r];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0 && r0 + r < nr) y[B.y_off[job] + r0 + r] = s;
   }
@@ -2056,7 +2040,6 @@ __global__ void seg_dots_kernel(SegTable t, int nvec, const double* __restrict__
       if (i2 < i1) partial[(long long)i2 * t.nchunks + b] = d2;
     }
   }
-  if (!t.counter) return;
   // The last CTA of problem p and this block of vectors adds their partial dots in chunk order (so the
   // result does not depend on which CTA that is), a thread per vector with 16 loads in flight, and re-arms
   // the counter for the next launch.  With one CTA for all vectors of a problem and four loads at a time an
@@ -2084,17 +2067,6 @@ __global__ void seg_dots_kernel(SegTable t, int nvec, const double* __restrict__
     h[(long long)i * t.K + p] = sum;
   }
   if (threadIdx.x == 0) *counter = 0u;
-}
-
-// h[i K + p] = sum over problem p's chunks (in order) of the partial dots of vector i
-__global__ void seg_reduce_kernel(SegTable t, int nvec, const double* __restrict__ partial, double* __restrict__ h) {
-  const int p = blockIdx.x;
-  if (!t.active[p]) return;
-  for (int i = threadIdx.x; i < nvec; i += blockDim.x) {
-    double s = 0.0;
-    for (int b = t.pchunk[p]; b < t.pchunk[p + 1]; ++b) s += partial[(long long)i * t.nchunks + b];
-    h[(long long)i * t.K + p] = s;
-  }
 }
 
 // w += sign * sum_i coef[i K + p] V_i over one kSegUpdSub-element piece of a chunk per CTA.  The
@@ -2515,7 +2487,7 @@ void note_launch() { ++t_launches; }
 void launch_pairs_f32(const TargetSet& tg, const SourceSet& src, const float* lam_hat, const float* mu, float* out,
                       double visc, cudaStream_t st) {
   if (tg.n_tiles == 0) return;
-  const int nt = tg.n_tiles1 > 0 ? pair_nodes_per_thread(tg.n_tiles) : 4;
+  const int nt = pair_nodes_per_thread(tg.n_tiles);
   PairArgs<float> A = make_args<float>(tg, src, lam_hat, mu, out, visc, nt);
   ++t_launches;
   if (nt == 4) pairs_kernel<float, 4><<<tg.n_tiles, kPairThreads, 0, st>>>(A);
@@ -2563,10 +2535,9 @@ void launch_velocity(int n, const double* x, const SourceSet& src, const double*
   }
 }
 
-// nodes per thread of a launch: the requested shape, else the rule (512-node tiles once they fill
-// the GPU twice; 128-node tiles only when they exist)
+// nodes per thread of a far-field launch: the requested shape, else the rule (512-node tiles once they fill
+// the GPU twice)
 static int shape_nt(const TargetSet& tg, const PairShape& shape) {
-  if (tg.n_tiles1 == 0) return 4;
   if (shape.nt == 1 || shape.nt == 4) return shape.nt;
   return pair_nodes_per_thread(tg.n_tiles);
 }
@@ -2789,10 +2760,6 @@ void launch_seg_dots(const SegTable& t, int nvec, const double* V, long long ldv
   ++t_launches;
   seg_dots_kernel<<<dim3(seg_ctas(t), (nvec + kSegDotVecs - 1) / kSegDotVecs), kSegThreads, 0, st>>>(t, nvec, V, ldv,
                                                                                                      w, partial, h);
-  if (!t.counter) {
-    ++t_launches;
-    seg_reduce_kernel<<<t.K, 128, 0, st>>>(t, nvec, partial, h);
-  }
 }
 void launch_seg_update(const SegTable& t, int nvec, const double* V, long long ldv, const double* coef, double sign,
                        double* w, cudaStream_t st) {
@@ -2848,8 +2815,8 @@ void launch_gemv(const GemvBatch<T>& b, const T* x, T* y, cudaStream_t st) {
   ++t_launches;
   if constexpr (sizeof(T) == 8)
     gemv64_kernel<<<dim3(jobs, (b.max_rows + kGemv64Rows - 1) / kGemv64Rows), 32 * kGemv64Warps, 0, st>>>(b, x, y);
-  else if (b.paired) gemv_kernel<T, true><<<grid, kGemvThreads, 0, st>>>(b, x, y);
-  else gemv_kernel<T, false><<<grid, kGemvThreads, 0, st>>>(b, x, y);
+  else if (b.paired) gemv_kernel<true><<<grid, kGemvThreads, 0, st>>>(b, x, y);
+  else gemv_kernel<false><<<grid, kGemvThreads, 0, st>>>(b, x, y);
 }
 template void launch_gemv<float>(const GemvBatch<float>&, const float*, float*, cudaStream_t);
 
