@@ -40,10 +40,10 @@ GOLDEN = os.path.join(ROOT, "tests", "golden", "gap_sweep_oracle.json")
 # S+R+D image triple at one node (shared distance and 1/r).  This is what `frac` is measured in.
 FLOPS_ALG = (28.0, 63.0)
 # FP32-pipe operations the double-float (compensated) kernel issues for the same pair math,
-# counted from its source: 205 per Stokeslet pair and 477 per image triple.
+# counted from its source: 214 per Stokeslet pair and 487 per image triple.
 # Their rate against the FP32 peak is `issue_frac`, a measure of how busy the pipes are, not of
 # algorithmic throughput.
-FLOPS_ISSUED_DW = (205.0, 477.0)
+FLOPS_ISSUED_DW = (214.0, 487.0)
 # dram__bytes_read.sum + dram__bytes_write.sum of one pairs_dw_multi_kernel<3> launch over three
 # gap-sweep geometries with their three motions each (ncu --set full on
 # `bench.py --profile-case gemv_rhs`; 0.94 MB read, 0 written): the kernel is FP32-issue-bound
@@ -678,7 +678,7 @@ def main():
         probe = {"error": str(e)}
     fp64_peak = probe.get("fp64_dfma_tflops") or 1.0
     peak = fp32_peak if prec == "mixed" else fp64_peak
-    roofline = {"bound": "alu", "kernel": "pairs_dw_batch_kernel" if prec == "mixed" else "pairs_batch_kernel<double>",
+    roofline = {"bound": "alu", "kernel": "pairs_dw_batch_kernel" if prec == "mixed" else "pairs_fp64_batch_kernel",
                 "achieved": achieved_tflops, "peak": peak, "unit": "TFLOP/s", "frac": achieved_tflops / peak,
                 "flops_per_unit": {"stokeslet_pair": FLOPS_ALG[0], "image_triple": FLOPS_ALG[1]},
                 "units_per_launch": {"proxy_pairs": k_proxy / max(k_launch, 1),

@@ -363,10 +363,10 @@ typedef struct {
    * sphere columns they covered */
   long long tc_launches;
   long long tc_columns;
-  /* FP32-pipe flops issued by the double-float pair evaluations: 205 per (node, proxy) pair and
-   * 477 per (node, image node) triple for one right-hand side; in a batch, the right-hand sides on
-   * one geometry (R of them) share each pair's geometry (unit vector and 1/r: 76 and 94 flops),
-   * so such a pair issues 76 + 129 R (triple: 94 + 383 R).  pair_shared_rhs counts the
+  /* FP32-pipe flops issued by the double-float pair evaluations: 214 per (node, proxy) pair and
+   * 487 per (node, image node) triple for one right-hand side; in a batch, the right-hand sides on
+   * one geometry (R of them) share each pair's geometry (unit vector and 1/r: 80 and 98 flops),
+   * so such a pair issues 80 + 134 R (triple: 98 + 389 R).  pair_shared_rhs counts the
    * pair_interactions evaluated that way. */
   double pair_issued_flops;
   long long pair_shared_rhs;

@@ -40,12 +40,12 @@ inline int pad4(int x) { return (x + 3) & ~3; }
 // FP32-pipe flops of the compensated double-float pair evaluation (counted from the kernel's
 // operations, FMA = 2): a Stokeslet pair's geometry (difference, unit vector, 1/r) and its
 // per-right-hand-side part; an image triple's geometry and its S + R + D part
-constexpr double kDwPairGeomFlops = 76.0, kDwPairRhsFlops = 129.0;
+constexpr double kDwPairGeomFlops = 80.0, kDwPairRhsFlops = 134.0;
 // Each GMRES pass of a refined solve stops at kInnerTol x tol / (current relative residual); the
 // accurate residual then decides whether another pass is needed.  0.8 measured fastest on the
 // gap sweep (0.5 and 1.0 took 2.5 % and 3 % longer; tighter factors cost more iterations).
 constexpr double kInnerTol = 0.8;
-constexpr double kDwTripleGeomFlops = 94.0, kDwTripleRhsFlops = 383.0;
+constexpr double kDwTripleGeomFlops = 98.0, kDwTripleRhsFlops = 389.0;
 
 struct Factor {
   int m = 0, ncol = 0, rank = 0, ldA = 0, ldV = 0;
