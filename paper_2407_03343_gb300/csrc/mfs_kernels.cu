@@ -2622,9 +2622,12 @@ static int wave_parts(long long tiles, const void* kernel, int max_parts) {
 // Near part: 64-target CTAs, a thread per node.  (With four from 304 512-node tiles on, 343 spheres: N = 300 at
 // centres 2.5 apart 4.99 ms against 4.65, N = 160 at 3.0 0.82 against 0.78; all pairs of 100 spheres of 1,804 nodes
 // 127.4 against 116.1.)  The parts are whole spheres of lists of uneven length, so their number is what leaves
-// the shortest sum of a resident CTA's share of the work (kPairSplitPartCost sources a part on top) and of the longest
-// CTA, which may start last: cluster of 60 spheres, N = 150, 16 parts 174 us, 4 (whole waves) 215; 125 spheres on
-// a lattice, N = 100, 6 parts 104, 1 128; 20 spheres, N = 100, 9 parts 45, 15 53 (six of them without a sphere).
+// the smallest sum of a resident CTA's share of the work, kNearPartCost sources a part on top, and of half the
+// longest CTA, which one that starts last waits for.  Measured over 1 to 16 parts (taken / best / first / last): cluster
+// of 150 spheres, N = 686 3225 (8) / 3218 / 3925 / 3444 us; of 60, N = 150 172 (8) / 161 / 380 / 172; of 400, N = 300
+// 4747 (6) / 4747 / 5281 / 4888; lattices of 125, N = 100 and 343, N = 300 104 (6) / 104 / 127 / 132 and 4643 (6) / 4643 /
+// 4908 / 4766; 40 apart, N = 200 158 (12) / 151 / 292 / 176.
+constexpr double kNearPartCost = 40.0;
 PairShape resolve_near_shape(const TargetSet& tg, const SourceSet& src, const FarField& ff, PairShape shape,
                              int max_parts) {
   PairShape r;
@@ -2637,8 +2640,8 @@ PairShape resolve_near_shape(const TargetSet& tg, const SourceSet& src, const Fa
   r.parts = 1;
   double best = 0;
   for (int p = 1; wave > 0 && p <= std::min(max_parts, std::max(1, ff.near_max)); ++p) {
-    const double t = tg.n_pieces1 * (ff.near_mean * src.N + kPairSplitPartCost * p) / wave +
-                     (double)((ff.near_max + p - 1) / p) * src.N;
+    const double t = tg.n_pieces1 * (ff.near_mean * src.N + kNearPartCost * p) / wave +
+                     0.5 * ((ff.near_max + p - 1) / p) * src.N;
     if (p == 1 || t < best) {
       best = t;
       r.parts = p;
