@@ -249,7 +249,7 @@ struct mfs_ctx {
   double *d_tmp64 = nullptr, *d_lh64 = nullptr, *d_lam = nullptr, *d_F = nullptr, *d_T = nullptr;
   float *d_tmp32 = nullptr, *d_lh32 = nullptr, *d_in32 = nullptr, *d_out32 = nullptr, *d_mu32 = nullptr;
   float2 *d_x2 = nullptr, *d_t2 = nullptr;  // double-float staging of step 1
-  float2* d_lh2 = nullptr;                  // and its result lambda_hat, the input of the pair sums
+  float2* d_lh2 = nullptr;                  // and its result lambda_hat, the input of the pair sums (over d_in32)
   // Krylov workspace (lazily sized)
   void* d_basis = nullptr;
   size_t basis_bytes = 0;
@@ -2738,12 +2738,17 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
   ALLOC_TRY(c, c->d_T, double, 3 * (size_t)P);
   ALLOC_TRY(c, c->d_tmp32, float, c->tmp_len);
   ALLOC_TRY(c, c->d_lh32, float, c->n_unk);
-  ALLOC_TRY(c, c->d_in32, float, std::max<long long>(n, c->n_unk));
-  ALLOC_TRY(c, c->d_out32, float, std::max<long long>(n, c->n_unk));
+  {
+    // the FP32 mode's vectors; the double-float steps keep lambda_hat's pairs in the same place (a call runs
+    // in one precision, and carries neither to the next)
+    const long long len = (std::max<long long>(n, c->n_unk) + 1) & ~1LL;
+    ALLOC_TRY(c, c->d_in32, float, 2 * len);
+    c->d_out32 = c->d_in32 + len;
+    c->d_lh2 = reinterpret_cast<float2*>(c->d_in32);
+  }
   ALLOC_TRY(c, c->d_mu32, float, n);
   ALLOC_TRY(c, c->d_x2, float2, n + 6 * (size_t)P);
   ALLOC_TRY(c, c->d_t2, float2, c->tmp_len);
-  ALLOC_TRY(c, c->d_lh2, float2, c->n_unk);
   c->nblk = std::max(1, std::min(1024, (n + 4095) / 4096));
   // what only a solve needs: 1024-element chunks of the system vectors, without and with the mobility border
   // (both tables in one buffer: a transfer and an allocation each cost a build of a small context 5-10 us),
@@ -2767,7 +2772,7 @@ static mfs_status build_impl(mfs_ctx* c, const mfs_params* params) {
         ce.push_back(std::min(len, q + 1024));
       }
       nchunks[md] = (int)cs.size();
-      most = std::max(most, cs.size());
+      if (nchunks[md] <= kSegSingleMax) most = std::max(most, cs.size());
       at[md][0] = segs.size();
       segs.insert(segs.end(), cs.begin(), cs.end());
       at[md][1] = segs.size();
