@@ -45,10 +45,9 @@ FLOPS_ALG = (28.0, 63.0)
 # algorithmic throughput.
 FLOPS_ISSUED_DW = (214.0, 487.0)
 # dram__bytes_read.sum + dram__bytes_write.sum of one pairs_dw_multi_kernel<3> launch over three
-# gap-sweep geometries with their three motions each (ncu --set full on
-# `bench.py --profile-case gemv_rhs`; 0.94 MB read, 0 written): the kernel is FP32-issue-bound
-# and its operands stay in L2 (the single-problem kernel: 5.05 MB for an 18-problem launch)
-PAIR_DW_TRAFFIC_BYTES = 0.940e6
+# gap-sweep geometries with their three motions each (ncu on `bench.py --profile-case gemv_rhs`;
+# 1.82 MB read, 0 written): the kernel is bound by the FMA pipe and its operands stay in L2
+PAIR_DW_TRAFFIC_BYTES = 1.820e6
 
 
 def parse():
@@ -683,7 +682,7 @@ def main():
                 "flops_per_unit": {"stokeslet_pair": FLOPS_ALG[0], "image_triple": FLOPS_ALG[1]},
                 "units_per_launch": {"proxy_pairs": k_proxy / max(k_launch, 1),
                                      "image_node_pairs": k_image / max(k_launch, 1)},
-                # dram read + write of one captured launch (ncu, 18 gap-sweep problems, see profiles/)
+                # dram read + write of one captured launch (ncu, see profiles/)
                 "traffic": PAIR_DW_TRAFFIC_BYTES if prec == "mixed" else None,
                 "traffic_launch": "pairs_dw_multi_kernel<3>, 9-problem launch of --profile-case gemv_rhs"
                 if prec == "mixed" else None,

@@ -173,8 +173,8 @@ void launch_pairs_dw(const TargetSet& tg, const SourceSet& src, const float2* la
 // Source split of a launch of `items` CTAs a part: the count of parts that leaves the least work to the
 // longest SM, ceil(items x parts / resident CTAs) / parts, with the work of kPairSplitPartCost sources
 // charged per part, at least kPairSplitMinSources sources each, at most max_parts.  Against the best of
-// all shapes measured: two spheres 41.7 us (40.3 with 16 parts), 8 spheres 288 (286), 20 spheres 1097
-// (1096), 100 spheres 26.10 ms (26.09), 100 spheres of 1804 nodes 116.1 (116.1).  The rule before it, a
+// all shapes measured (with first-order terms): two spheres 41.7 us (40.3 with 16 parts), 8 spheres 288 (286),
+// 20 spheres 1097 (1096), 100 spheres 26.10 ms (26.09), 100 spheres of 1804 nodes 116.1 (116.1).  The rule before it, a
 // fixed count of CTAs, left 84 items of three right-hand sides on 456 resident CTAs with 6 parts, 1.1
 // waves: that sweep took 20.5 ms, 19.6 with this rule and the norm in the update.
 constexpr double kPairSplitPartCost = 16.0;

@@ -593,13 +593,13 @@ constexpr int kDwGroup = 8;      // terms per lane and group
 // Threads of a double-float CTA: the 128-node tiles are taken in two pieces, and a piece without targets
 // ends at once, so 823 nodes a sphere run as 13 CTAs of 64 (832 places) and not as 7 of 128 (896), and
 // the last wave is made of half as long CTAs.  Measured against CTAs of 128 (same rule for the parts): 100
-// spheres 27.8 -> 26.1 ms, the dilute solve of 20 spheres 36.8 -> 35.9 ms; two spheres and the batch of
-// motions the same within 2 %.
+// spheres 27.8 -> 26.1 ms, the dilute solve of 20 spheres 36.8 -> 35.9 ms (with first-order terms; 26.9 and
+// 35.6 now); two spheres and the batch of motions the same within 2 %.
 constexpr int kDwThreads = 64;
 constexpr int kDwPieces = kPairThreads / kDwThreads;
 static_assert(kDwPieces == kPairPieces, "arrival counters");
-// resident CTAs per SM (128 registers); 10 (96 registers) and 12 (80) were slower: 100 spheres 26.8 and
-// 26.6 ms against 26.1, two spheres 49.7 and 50.6 us against 41.8
+// resident CTAs per SM (128 registers); 10 (96 registers) and 12 (80) were slower (with first-order terms): 100
+// spheres 26.8 and 26.6 ms against 26.1, two spheres 49.7 and 50.6 us against 41.8
 constexpr int kDwCtas = 8;
 constexpr int kDwMultiCtas = 6;  // of the kernel over several right-hand sides (3 x the sums; 168 registers)
 
@@ -2076,8 +2076,8 @@ __global__ void seg_dots_kernel(SegTable t, int nvec, const double* __restrict__
 // norm: each piece leaves its sum of squares in `partial` and the last CTA of a problem adds them
 // (in piece order, so the sum does not depend on which CTA that is).
 // With the normalisation on the device, the fused sums of split sources and these kernels in the single
-// solves too, an iteration of two spheres went from 116 to 108 us, one of four from 180 to 173, and the
-// sweep of motions from 20.4 to 20.0 ms.
+// solves too (up to kSegSingleMax chunks), an iteration of two spheres went from 116 to 108 us, one of four from
+// 180 to 173, and the sweep of motions from 20.4 to 20.0 ms.
 constexpr int kSegUpdGroups = 4;
 template <bool NORM>
 __global__ void __launch_bounds__(kSegUpdSub* kSegUpdGroups)
