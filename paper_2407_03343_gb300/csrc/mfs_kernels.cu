@@ -1647,7 +1647,10 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<float> B, 
 #pragma unroll
       for (int r = 0; r < kGemvRowsPerWarp; ++r) {
         int row = r0 + r;
-        if (row < nr) acc[r] += dot_vec(reinterpret_cast<const float4*>(M + (long long)row * ld)[v], xv + 4 * v);
+        if (row < nr) {
+          const float4 m = reinterpret_cast<const float4*>(M + (long long)row * ld)[v];
+          acc[r] += dot_vec(m, xv + 4 * v);
+        }
       }
     }
     for (int c = 4 * nvec + lane; c < nc; c += 32) {
