@@ -3238,7 +3238,19 @@ static mfs_status run_step(mfs_ctx* c, int precision, int which, const double* i
   double* d1 = which == 2 ? c->d_lam : c->d_mu;
   // the operator-step entry points reuse the solution buffers; a later get_* must re-solve
   c->solved = false;
-  CUDA_TRY(c, cudaMemcpyAsync(d1, in1, sizeof(double) * len1, cudaMemcpyHostToDevice, c->stream));
+  // the double-float pairs of few strengths are formed here: their launch took 2-4 us of 40 (1,024 take 1 us)
+  constexpr int kHostSplit = 1024;
+  const bool host_split = which == 2 && nu <= kHostSplit && (precision == MFS_MIXED || precision == MFS_MIXED_PASS);
+  if (host_split) {
+    float2 pairs[kHostSplit];
+    for (long long i = 0; i < nu; ++i) {
+      const float h = (float)in1[i];
+      pairs[i] = make_float2(h, (float)(in1[i] - (double)h));
+    }
+    CUDA_TRY(c, cudaMemcpyAsync(c->d_lh2, pairs, sizeof(float2) * nu, cudaMemcpyHostToDevice, c->stream));
+  } else {
+    CUDA_TRY(c, cudaMemcpyAsync(d1, in1, sizeof(double) * len1, cudaMemcpyHostToDevice, c->stream));
+  }
   if (which == 2) CUDA_TRY(c, cudaMemcpyAsync(c->d_mu, in2, sizeof(double) * n, cudaMemcpyHostToDevice, c->stream));
   double* dout = which == 1 ? c->d_lh64 : c->d_w64;
   if (precision != MFS_FP32) {
@@ -3247,7 +3259,7 @@ static mfs_status run_step(mfs_ctx* c, int precision, int which, const double* i
     if (which == 0) apply_op<double>(c, c->d_mu, c->d_w64);
     else if (which == 1) precond<double>(c, c->d_mu, c->d_lh64);
     else {
-      if (c->dw_pairs) launch_split_dw(nu, c->d_lam, c->d_lh2, c->stream);
+      if (c->dw_pairs && !host_split) launch_split_dw(nu, c->d_lam, c->d_lh2, c->stream);
       pairs_step<double>(c, c->d_lam, c->d_mu, c->d_w64);
     }
     c->dw_pairs = c->dw_fast_a = c->ff_pass = false;

@@ -1615,7 +1615,7 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_kernel(GemvBatch<float> B, 
     // a 16-byte load holds two columns of the warp's row pair, so the loads of a warp are contiguous and x is
     // read once for both rows, two elements at a time where its offset is even (loads are what bounds this; four
     // columns a lane with the row loop of the plain layout read the matrix in two strided halves: both factors of
-    // N = 400 for 8 / 60 spheres that share them 37.5 / 222 us, now 25 / 103; from plain rows 21 / 103)
+    // N = 400 for 8 / 60 spheres that share them 37.5 / 222 us, now 21 / 79; from plain rows 21 / 103)
     static_assert(kGemvRowsPerWarp == 2, "FP32 row pairs");
     const float* pr = M + (long long)r0 * ld;
     const float4* q = reinterpret_cast<const float4*>(pr);
