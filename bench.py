@@ -212,7 +212,7 @@ def reduce_over_ranks(total_ms, pairs, device):
 def suspension_kernel_rates(device, fp32_peak):
     """Device time of one pair-kernel launch per precision on the 200-sphere suspension
     (volume fraction 0.2, ~300 near contacts, N = 800, M0 = 1600; ~1e11 pairs per launch,
-    4 target nodes per thread), discretised without the one-body factors."""
+    FP32: 4 target nodes per thread), discretised without the one-body factors."""
     from paper_2407_03343_gb300 import mfs, workloads
     ctx = mfs.Context(device)
     ctx.set_spheres(workloads.suspension(200, 0.2, seed=3))

@@ -383,13 +383,13 @@ mfs_status mfs_get_timing(mfs_ctx* ctx, mfs_timing_t* out, int reset);
  * launch runs ~0.1-0.5 s.  Allocates and frees one small device buffer. */
 mfs_status mfs_probe_alu_peak(int device, int which, double* tflops, double* ms);
 
-/* Tile shapes of the pair kernels (steps 2+3) and the autotuner that picks them.  A target tile
- * holds 512 collocation nodes (4 per thread of a 128-thread CTA) or 128 (1 per thread); a tile's
- * sources may be split over several CTAs whose partial sums a second kernel adds in a fixed
- * order.  By default the library chooses by rule (512-node tiles once they fill the GPU twice,
- * source parts that fill whole waves of resident CTAs).  mfs_tune_pairs times every candidate
- * (tile of 128 or 512 nodes x no split or the wave-filling split; for the far kernel with 512-node
- * tiles also scalar or packed two-lane FP32 instructions) of each pair-kernel family the
+/* Shapes of the pair kernels (steps 2+3) and the autotuner that picks them.  The double-float kernels
+ * take a collocation node per thread; the far field's FP32 kernel takes tiles of 512 nodes (4 per
+ * thread of a 128-thread CTA) or 128 (1 per thread).  The sources may be split over several CTAs
+ * whose partial sums are added in a fixed order.  By default the library chooses by rule (512-node
+ * tiles once they fill the GPU twice, source parts by the work of resident CTAs).  mfs_tune_pairs
+ * times every candidate (no split or the rule's; for the far kernel with either tile and with
+ * 512-node tiles also scalar or packed two-lane FP32 instructions) of each pair-kernel family the
  * context uses, on its own discretisation, with CUDA events over two launches each, keeps the
  * fastest for the context's later launches and reports them; 0 in a field means "not used by
  * this context" (e.g. the near / far kernels without the far field). */

@@ -70,7 +70,7 @@ struct TargetSet {
   int* tile1_count = nullptr;
 };
 
-// Tile size choice: 4 nodes per thread once the large tiles fill the GPU twice over.
+// Tile size choice of the FP32 kernels: 4 nodes per thread once the large tiles fill the GPU twice over.
 inline int pair_nodes_per_thread(int n_tiles_large) { return n_tiles_large >= 2 * 152 ? 4 : 1; }
 
 struct SourceSet {
@@ -136,8 +136,8 @@ size_t tc_partial_floats(const TcGemm& g, int ncols);
 void launch_tc_gemm(const TcGemm& g, int ncols, const double* x, const long long* x_off, const long long* y_off,
                     float* y32, float2* y2, float* partial, int* err, bool slice_x, cudaStream_t st);
 
-// A launch shape: nodes per thread (4: 512-node tiles, 1: 128-node tiles, 0: by rule) and source
-// parts per tile (0: the wave-filling rule, 1: no split, > 1: that many).
+// A launch shape: nodes per thread (far kernel: 4: 512-node tiles, 1: 128-node tiles, 0: by rule; the
+// double-float kernels take one) and source parts per tile (0: by rule, 1: no split, > 1: that many).
 struct PairShape {
   int nt = 0;
   int parts = 0;
@@ -184,8 +184,8 @@ constexpr int kPairPieces = 2;  // arrival counters per tile or batched work ite
 
 // Near part of the far-field split, double-float: out = mu + W sum over the near spheres of the
 // target's sphere (their proxies and image triples) of G lambda_hat.
-// Both split each tile's sources over up to max_parts CTAs (partial: max_parts * 3 n doubles, or
-// null for no split) so that the grid fills whole waves of resident CTAs; the parts are added in a
+// Near and far split each tile's sources over up to max_parts CTAs (partial: max_parts * 3 n doubles, or
+// null for no split), the far one so that the grid fills whole waves of resident CTAs; the parts are added in a
 // fixed order, by the last CTA of a tile (near; counter as above) or by a second kernel (far).
 void launch_pairs_dw_near(const TargetSet& tg, const SourceSet& src, const FarField& ff, const float2* lam_hat,
                           const double* mu, double* out, double visc, double* partial, unsigned* counter, int max_parts,
